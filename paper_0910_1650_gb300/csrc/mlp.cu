@@ -218,15 +218,6 @@ __global__ void neighbour_density_batched_kernel(const BatchProblem* __restrict_
     neighbour_row((int)(t - q.frow), nbr + q.frow * TOPK, F + q.frow * IN);
 }
 
-// Fn = (F - mu) * isd, row-major [rows x IN].
-__global__ void standardise_kernel(const float* __restrict__ F, int rows,
-                                   const float* __restrict__ P, float* Fn) {
-    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= (int64_t)rows * IN) return;
-    const int j = (int)(e % IN);
-    Fn[e] = (F[e] - P[OFF_MU + j]) * P[OFF_ISD + j];
-}
-
 // Column j of the standardisation from F [rows x IN] (one block per column,
 // float64 sums in a fixed order): mu = mean, isd = 1 / max(std, 1e-3) with the
 // population standard deviation.
@@ -257,184 +248,439 @@ __global__ void standardisation_kernel(const float* __restrict__ F, int64_t rows
     }
 }
 
-// ---- dense layers ----------------------------------------------------------------
-constexpr int TR = 64, TO = 64, TK = 16;
+// ---- the network: forward, backward and Adam ------------------------------------
+// A step of the network is bound by float32 arithmetic (activations and
+// gradients stay float32, weights are bf16: about 74000 multiply-adds per row
+// and direction), not by memory.  rows_kernel therefore takes a tile of 32
+// rows through all three layers -- and, in training, back through them -- with
+// the activations in shared memory: 128 threads own 8 rows x 8 columns of the
+// 256-wide layers each (64 accumulators against 16 shared-memory words per
+// step of k, so the FMA pipe and not shared memory is the limit), multiply in
+// packed f32x2, and prefetch the next 16 x 256 weights into registers while
+// the current ones are used.  A thread owns the same elements in every layer,
+// so the ReLU masks stay in registers.  In training the block leaves its
+// tiles' share of every gradient but W2's in one partial slot, and the rows'
+// H1 and G2 for w2_grad_kernel, which splits the rows of G2^T H1 over blocks;
+// adam_reduce_kernel adds the slots in a fixed order and takes the step.
+// A training step on 4096 rows: three launches where separate layer kernels
+// took 15 (weight gradients on at most 16 blocks, bias gradients one thread
+// per column), 80 us where they took 1752 us.  The forward pass alone on
+// 101000 rows: about 390 us where four layer launches took 870 us.
+constexpr int TR = 32;                 // rows per tile
+constexpr int RS = 36;                 // their stride in shared memory (16-byte groups, fewer bank conflicts)
+constexpr int KC = 16;                 // weights staged per step: KC x 256
+constexpr int RT = 128;                // threads of rows_kernel
+constexpr int kMaxSlots = 608;         // gradient partial slots: 4 tiles in flight per SM
+constexpr int NSMALL = NP - 2 * IN - HID * HID;   // gradients but W2's, in parameter order
+constexpr int SLOT = (NSMALL + 3) / 4 * 4;
+constexpr int W2T = 128;               // w2_grad_kernel's tile
 
-// Y[r][o] = act(sum_i X[r][i] W[o][i] + b[o]); W bf16 [out x in].
-__global__ void __launch_bounds__(256) linear_fwd_kernel(const float* __restrict__ X, int rows,
-                                                         int in, const __nv_bfloat16* __restrict__ W,
-                                                         const float* __restrict__ b, int out,
-                                                         int relu, float* Y) {
-    __shared__ float xs[TK][TR + 1], ws[TK][TO + 1];
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int r0 = blockIdx.x * TR, o0 = blockIdx.y * TO;
-    float acc[4][4] = {};
-    for (int k0 = 0; k0 < in; k0 += TK) {
-        for (int e = threadIdx.x; e < TK * TR; e += 256) {
-            const int kk = e % TK, rr = e / TK;
-            const int r = r0 + rr, k = k0 + kk;
-            xs[kk][rr] = (r < rows && k < in) ? X[(int64_t)r * in + k] : 0.f;
-            const int o = o0 + rr;
-            ws[kk][rr] = (o < out && k < in) ? __bfloat162float(W[(int64_t)o * in + k]) : 0.f;
+struct RowsSmem {
+    float ws[2][KC][HID];              // staged weights (W1: ws as [IN][HID])
+    float hs[HID * RS];                // activations / gradients of the tile, column by column
+    float xs[IN * RS];                 // standardised inputs, column by column
+    float w3[OUT][HID];
+    float ys[OUT][TR], gs[OUT][TR];
+};
+
+// Eight bf16 starting at W (16-byte aligned when vec).
+__device__ __forceinline__ uint4 load8(const __nv_bfloat16* __restrict__ W, int vec) {
+    if (vec) return __ldg(reinterpret_cast<const uint4*>(W));
+    uint32_t w[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+        w[e] = (uint32_t)__bfloat16_as_ushort(W[2 * e]) | ((uint32_t)__bfloat16_as_ushort(W[2 * e + 1]) << 16);
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+__device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
+
+// The next KC x 256 weights of W2 [256 x 256], k from k0: columns of the
+// product are W2's rows going forward (k along a row), its columns going back
+// (BACK: k is W2's row).
+template <bool BACK>
+__device__ __forceinline__ void fetch_w2(const __nv_bfloat16* __restrict__ W, int k0, int vec, uint4 (&pf)[4]) {
+    const int tid = threadIdx.x;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        if (BACK) {
+            const int e = tid + q * RT;                    // 16 rows x 32 groups of eight
+            pf[q] = load8(W + (int64_t)(k0 + (e >> 5)) * HID + 8 * (e & 31), vec);
+        } else {
+            pf[q] = load8(W + (int64_t)(tid + (q >> 1) * RT) * HID + k0 + 8 * (q & 1), vec);
         }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < TK; ++kk)
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int c = 0; c < 4; ++c)
-                    acc[a][c] = fmaf(xs[kk][ty * 4 + a], ws[kk][tx * 4 + c], acc[a][c]);
-        __syncthreads();
     }
+}
+template <bool BACK>
+__device__ __forceinline__ void put_w2(float (*ws)[HID], const uint4 (&pf)[4]) {
+    const int tid = threadIdx.x;
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        const int r = r0 + ty * 4 + a;
-        if (r >= rows) continue;
+    for (int q = 0; q < 4; ++q) {
+        const float v[8] = {bf16_lo(pf[q].x), bf16_hi(pf[q].x), bf16_lo(pf[q].y), bf16_hi(pf[q].y),
+                            bf16_lo(pf[q].z), bf16_hi(pf[q].z), bf16_lo(pf[q].w), bf16_hi(pf[q].w)};
+        if (BACK) {
+            const int e = tid + q * RT;
+            float* at = &ws[e >> 5][8 * (e & 31)];
+            *reinterpret_cast<float4*>(at) = make_float4(v[0], v[1], v[2], v[3]);
+            *reinterpret_cast<float4*>(at + 4) = make_float4(v[4], v[5], v[6], v[7]);
+        } else {
+            const int o = tid + (q >> 1) * RT;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const int o = o0 + tx * 4 + c;
-            if (o >= out) continue;
-            float v = acc[a][c] + b[o];
-            if (relu) v = fmaxf(v, 0.f);
-            Y[(int64_t)r * out + o] = v;
+            for (int j = 0; j < 8; ++j) ws[8 * (q & 1) + j][o] = v[j];
         }
     }
 }
 
-// dX[r][i] = (sum_o G[r][o] W[o][i]) * (H[r][i] > 0); W bf16 [out x in].
-__global__ void __launch_bounds__(256) linear_bwd_input_kernel(const float* __restrict__ G,
-                                                               int rows, int out,
-                                                               const __nv_bfloat16* __restrict__ W,
-                                                               int in, const float* __restrict__ H,
-                                                               float* dX) {
-    __shared__ float gs[TK][TR + 1], ws[TK][TO + 1];
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int r0 = blockIdx.x * TR, i0 = blockIdx.y * TO;
-    float acc[4][4] = {};
-    for (int o0 = 0; o0 < out; o0 += TK) {
-        for (int e = threadIdx.x; e < TK * TR; e += 256) {
-            const int oo = e % TK, rr = e / TK;
-            const int r = r0 + rr, o = o0 + oo;
-            gs[oo][rr] = (r < rows && o < out) ? G[(int64_t)r * out + o] : 0.f;
-            const int i = i0 + rr;
-            ws[oo][rr] = (o < out && i < in) ? __bfloat162float(W[(int64_t)o * in + i]) : 0.f;
-        }
-        __syncthreads();
+// acc += (column k of act) x (row k of w): this thread's rows 8 wid .. and
+// columns 2 lid + 64 j, + 1.
+__device__ __forceinline__ void rank1(const float* act, const float* w, int wid, int lid, float2 (&acc)[8][4]) {
+    const float4 a0 = *reinterpret_cast<const float4*>(act + 8 * wid);
+    const float4 a1 = *reinterpret_cast<const float4*>(act + 8 * wid + 4);
+    float2 b[4];
 #pragma unroll
-        for (int oo = 0; oo < TK; ++oo)
+    for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const float2*>(w + 64 * j + 2 * lid);
+    const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
 #pragma unroll
-            for (int a = 0; a < 4; ++a)
+    for (int r = 0; r < 8; ++r)
 #pragma unroll
-                for (int c = 0; c < 4; ++c)
-                    acc[a][c] = fmaf(gs[oo][ty * 4 + a], ws[oo][tx * 4 + c], acc[a][c]);
-        __syncthreads();
-    }
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        const int r = r0 + ty * 4 + a;
-        if (r >= rows) continue;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const int i = i0 + tx * 4 + c;
-            if (i >= in) continue;
-            const int64_t at = (int64_t)r * in + i;
-            dX[at] = H[at] > 0.f ? acc[a][c] : 0.f;
-        }
-    }
+        for (int j = 0; j < 4; ++j) acc[r][j] = __ffma2_rn(make_float2(a[r], a[r]), b[j], acc[r][j]);
 }
 
-// gW[o][i] = sum_r G[r][o] X[r][i] (rows in a fixed order); one output tile
-// per block, so the sum is deterministic.
-__global__ void __launch_bounds__(256) weight_grad_kernel(const float* __restrict__ G, int rows,
-                                                          int out, const float* __restrict__ X,
-                                                          int in, float* gW) {
-    __shared__ float gs[TK][TO + 1], xs[TK][TO + 1];
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int o0 = blockIdx.x * TO, i0 = blockIdx.y * TO;
-    float acc[4][4] = {};
-    for (int rr0 = 0; rr0 < rows; rr0 += TK) {
-        for (int e = threadIdx.x; e < TK * TO; e += 256) {
-            const int kk = e / TO, c = e % TO;
-            const int r = rr0 + kk;
-            gs[kk][c] = (r < rows && o0 + c < out) ? G[(int64_t)r * out + o0 + c] : 0.f;
-            xs[kk][c] = (r < rows && i0 + c < in) ? X[(int64_t)r * in + i0 + c] : 0.f;
-        }
-        __syncthreads();
+__device__ __forceinline__ void clear(float2 (&acc)[8][4]) {
 #pragma unroll
-        for (int kk = 0; kk < TK; ++kk)
+    for (int r = 0; r < 8; ++r)
 #pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int c = 0; c < 4; ++c)
-                    acc[a][c] = fmaf(gs[kk][ty * 4 + a], xs[kk][tx * 4 + c], acc[a][c]);
-        __syncthreads();
-    }
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        const int o = o0 + ty * 4 + a;
-        if (o >= out) continue;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const int i = i0 + tx * 4 + c;
-            if (i < in) gW[(int64_t)o * in + i] = acc[a][c];
-        }
-    }
+        for (int j = 0; j < 4; ++j) acc[r][j] = make_float2(0.f, 0.f);
 }
 
-// gb[o] = sum_r G[r][o], one thread per column, rows in order.
-__global__ void bias_grad_kernel(const float* __restrict__ G, int rows, int out, float* gb) {
-    const int o = blockIdx.x * blockDim.x + threadIdx.x;
-    if (o >= out) return;
-    float s = 0.f;
-    for (int r = 0; r < rows; ++r) s += G[(int64_t)r * out + o];
-    gb[o] = s;
-}
-
-// Per-row loss terms and dL/dY (already divided by the row count).
-__global__ void loss_kernel(const float* __restrict__ Y, const float* __restrict__ T, int rows,
-                            float* G, float* lrow) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= rows) return;
-    const float inv = 1.f / (float)rows;
-    const float d = Y[r * 3 + 0] - T[r * 3 + 0];
-    const float e = Y[r * 3 + 1] - T[r * 3 + 1];
-    const float z = Y[r * 3 + 2], t = T[r * 3 + 2];
-    const float sp = fmaxf(z, 0.f) + log1pf(expf(-fabsf(z)));     // softplus(z)
-    lrow[r] = d * d + e * e + sp - t * z;
-    G[r * 3 + 0] = 2.f * d * inv;
-    G[r * 3 + 1] = 2.f * e * inv;
-    G[r * 3 + 2] = (1.f / (1.f + expf(-z)) - t) * inv;
-}
-
-__global__ void mean_kernel(const float* __restrict__ v, int n, float* out) {
-    __shared__ double sh[1024];
-    const int per = (n + blockDim.x - 1) / blockDim.x;
-    const int lo = threadIdx.x * per, hi = min(n, lo + per);
-    double x = 0.0;
-    for (int i = lo; i < hi; ++i) x += v[i];
-    sh[threadIdx.x] = x;
+// acc = hs x W2 (or its transpose); leaves the block synchronised, hs free.
+template <bool BACK>
+__device__ __forceinline__ void layer2(RowsSmem& sm, const __nv_bfloat16* __restrict__ W, int vec, int wid, int lid,
+                                       float2 (&acc)[8][4]) {
+    uint4 pf[4];
+    clear(acc);
+    fetch_w2<BACK>(W, 0, vec, pf);
+    put_w2<BACK>(sm.ws[0], pf);
     __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
+    for (int c = 0; c < HID / KC; ++c) {
+        if (c + 1 < HID / KC) fetch_w2<BACK>(W, (c + 1) * KC, vec, pf);
+#pragma unroll
+        for (int kk = 0; kk < KC; ++kk) rank1(sm.hs + (c * KC + kk) * RS, sm.ws[c & 1][kk], wid, lid, acc);
+        if (c + 1 < HID / KC) put_w2<BACK>(sm.ws[(c + 1) & 1], pf);
         __syncthreads();
     }
-    if (threadIdx.x == 0) *out = (float)(sh[0] / (double)n);
 }
 
-// Adam with bias correction; refreshes the bf16 copy of the weights.
-__global__ void adam_kernel(float* P, const float* __restrict__ g, float* m, float* v, int64_t np,
-                            float lr, float b1, float b2, float eps, float c1, float c2,
-                            __nv_bfloat16* P16) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < np;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const float mi = b1 * m[i] + (1.f - b1) * g[i];
-        const float vi = b2 * v[i] + (1.f - b2) * g[i] * g[i];
+// The thread's 8 x 8 elements into hs, and (out != null) into row-major
+// out [rows x 256].
+__device__ __forceinline__ void put_tile(float* hs, float* out, const float2 (&v)[8][4], int wid, int lid, int64_t r0,
+                                         int rows) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        float* x = hs + (64 * j + 2 * lid) * RS + 8 * wid;
+        *reinterpret_cast<float4*>(x) = make_float4(v[0][j].x, v[1][j].x, v[2][j].x, v[3][j].x);
+        *reinterpret_cast<float4*>(x + 4) = make_float4(v[4][j].x, v[5][j].x, v[6][j].x, v[7][j].x);
+        *reinterpret_cast<float4*>(x + RS) = make_float4(v[0][j].y, v[1][j].y, v[2][j].y, v[3][j].y);
+        *reinterpret_cast<float4*>(x + RS + 4) = make_float4(v[4][j].y, v[5][j].y, v[6][j].y, v[7][j].y);
+    }
+    if (out) {
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            const int64_t row = r0 + 8 * wid + r;
+            if (row < rows)
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    *reinterpret_cast<float2*>(out + row * HID + 64 * j + 2 * lid) = v[r][j];
+        }
+    }
+}
+
+// Bias and ReLU; the mask has bit 8 r + 2 j + e for row r, column pair j, element e.
+__device__ __forceinline__ uint64_t bias_relu(float2 (&acc)[8][4], const float* __restrict__ b, int lid) {
+    uint64_t m = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const float b0 = b[64 * j + 2 * lid], b1 = b[64 * j + 2 * lid + 1];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            acc[r][j].x = fmaxf(acc[r][j].x + b0, 0.f);
+            acc[r][j].y = fmaxf(acc[r][j].y + b1, 0.f);
+            m |= (uint64_t)(acc[r][j].x > 0.f) << (8 * r + 2 * j);
+            m |= (uint64_t)(acc[r][j].y > 0.f) << (8 * r + 2 * j + 1);
+        }
+    }
+    return m;
+}
+
+struct TrainOut {
+    const float* T;           // targets [rows x 3]
+    float *H1, *G2;           // [rows x 256]
+    float* part;              // [gridDim.x][SLOT] gradients but W2's
+    double* lpart;            // [gridDim.x] summed row losses
+};
+
+template <bool TRAIN>
+__global__ void __launch_bounds__(RT) rows_kernel(const float* __restrict__ P, const __nv_bfloat16* __restrict__ P16,
+                                                  const float* __restrict__ F, int rows, int vec, float* Y,
+                                                  TrainOut t) {
+    extern __shared__ __align__(16) unsigned char rows_smem[];
+    RowsSmem& sm = *reinterpret_cast<RowsSmem*>(rows_smem);
+    const int tid = threadIdx.x, wid = tid >> 5, lid = tid & 31;
+    const int tiles = (rows + TR - 1) / TR;
+    for (int e = tid; e < OUT * HID; e += RT) (&sm.w3[0][0])[e] = __bfloat162float(P16[OFF_W3 + e]);
+    float* part = TRAIN ? t.part + (int64_t)blockIdx.x * SLOT : nullptr;
+    bool first = true;
+    double lsum = 0.0;
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const int64_t r0 = (int64_t)tile * TR;
+        __syncthreads();                                   // the previous tile is done with shared memory
+        for (int e = tid; e < TR * IN; e += RT) {
+            const int r = e / IN, k = e - r * IN;
+            sm.xs[k * RS + r] = r0 + r < rows ? (F[r0 * IN + e] - P[OFF_MU + k]) * P[OFF_ISD + k] : 0.f;
+        }
+        float* w1 = &sm.ws[0][0][0];
+        for (int e = tid; e < HID * IN; e += RT) {
+            const int k = e / HID, o = e - k * HID;
+            w1[e] = __bfloat162float(P16[OFF_W1 + o * IN + k]);
+        }
+        __syncthreads();
+        float2 acc[8][4];
+        clear(acc);
+#pragma unroll 5
+        for (int k = 0; k < IN; ++k) rank1(sm.xs + k * RS, w1 + k * HID, wid, lid, acc);
+        const uint64_t m1 = bias_relu(acc, P + OFF_B1, lid);
+        put_tile(sm.hs, TRAIN ? t.H1 : nullptr, acc, wid, lid, r0, rows);
+        __syncthreads();
+        layer2<false>(sm, P16 + OFF_W2, vec, wid, lid, acc);
+        const uint64_t m2 = bias_relu(acc, P + OFF_B2, lid);
+        put_tile(sm.hs, nullptr, acc, wid, lid, r0, rows);
+        __syncthreads();
+        if (tid < OUT * TR) {                              // warp o: output o of the 32 rows
+            float y0 = 0.f, y1 = 0.f, y2 = 0.f, y3 = 0.f;
+#pragma unroll 4
+            for (int k = 0; k < HID; k += 4) {
+                const float4 w = *reinterpret_cast<const float4*>(&sm.w3[wid][k]);
+                y0 = fmaf(sm.hs[k * RS + lid], w.x, y0);
+                y1 = fmaf(sm.hs[(k + 1) * RS + lid], w.y, y1);
+                y2 = fmaf(sm.hs[(k + 2) * RS + lid], w.z, y2);
+                y3 = fmaf(sm.hs[(k + 3) * RS + lid], w.w, y3);
+            }
+            const float y = (y0 + y1) + (y2 + y3) + P[OFF_B3 + wid];
+            if (TRAIN) sm.ys[wid][lid] = y;
+            else if (r0 + lid < rows) Y[(r0 + lid) * OUT + wid] = y;
+        }
+        if (!TRAIN) continue;
+        __syncthreads();
+        if (wid == 0) {
+            // the row's loss and dL/dY (divided by the row count)
+            const bool in = r0 + lid < rows;
+            const float inv = 1.f / (float)rows;
+            const float* tr = t.T + (r0 + (in ? lid : 0)) * OUT;
+            const float d = sm.ys[0][lid] - tr[0], e = sm.ys[1][lid] - tr[1], z = sm.ys[2][lid], tt = tr[2];
+            const float sp = fmaxf(z, 0.f) + log1pf(expf(-fabsf(z)));     // softplus(z)
+            double l = in ? (double)(d * d + e * e + sp - tt * z) : 0.0;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+            lsum += l;
+            sm.gs[0][lid] = in ? 2.f * d * inv : 0.f;
+            sm.gs[1][lid] = in ? 2.f * e * inv : 0.f;
+            sm.gs[2][lid] = in ? (1.f / (1.f + expf(-z)) - tt) * inv : 0.f;
+        }
+        __syncthreads();
+        auto add = [&](int at, float v) { part[at] = first ? v : part[at] + v; };
+        constexpr int S_B2 = OFF_B2 - HID * HID, S_W3 = OFF_W3 - HID * HID, S_B3 = OFF_B3 - HID * HID;
+        // layer 3: gW3 = G3^T H2, gb3
+#pragma unroll
+        for (int h = 0; h < HID / RT; ++h) {
+            const int c = tid + h * RT;
+            float g[OUT] = {};
+#pragma unroll
+            for (int r = 0; r < TR; r += 4) {
+                const float4 x = *reinterpret_cast<const float4*>(sm.hs + c * RS + r);
+#pragma unroll
+                for (int o = 0; o < OUT; ++o) {
+                    const float4 q = *reinterpret_cast<const float4*>(&sm.gs[o][r]);
+                    g[o] = fmaf(q.x, x.x, g[o]);
+                    g[o] = fmaf(q.y, x.y, g[o]);
+                    g[o] = fmaf(q.z, x.z, g[o]);
+                    g[o] = fmaf(q.w, x.w, g[o]);
+                }
+            }
+#pragma unroll
+            for (int o = 0; o < OUT; ++o) add(S_W3 + o * HID + c, g[o]);
+        }
+        if (tid < OUT) {
+            float g = 0.f;
+            for (int r = 0; r < TR; ++r) g += sm.gs[tid][r];
+            add(S_B3 + tid, g);
+        }
+        // G2 = (G3 W3) where H2 > 0
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            const float g0 = sm.gs[0][8 * wid + r], g1 = sm.gs[1][8 * wid + r], g2 = sm.gs[2][8 * wid + r];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int c = 64 * j + 2 * lid;
+                const float2 w0 = *reinterpret_cast<const float2*>(&sm.w3[0][c]);
+                const float2 w1v = *reinterpret_cast<const float2*>(&sm.w3[1][c]);
+                const float2 w2v = *reinterpret_cast<const float2*>(&sm.w3[2][c]);
+                const float vx = fmaf(g2, w2v.x, fmaf(g1, w1v.x, g0 * w0.x));
+                const float vy = fmaf(g2, w2v.y, fmaf(g1, w1v.y, g0 * w0.y));
+                acc[r][j] = make_float2((m2 >> (8 * r + 2 * j)) & 1 ? vx : 0.f,
+                                        (m2 >> (8 * r + 2 * j + 1)) & 1 ? vy : 0.f);
+            }
+        }
+        __syncthreads();                                   // H2 has been read
+        put_tile(sm.hs, t.G2, acc, wid, lid, r0, rows);
+        __syncthreads();
+#pragma unroll
+        for (int h = 0; h < HID / RT; ++h) {               // gb2
+            const int c = tid + h * RT;
+            float g = 0.f;
+#pragma unroll
+            for (int r = 0; r < TR; r += 4) {
+                const float4 x = *reinterpret_cast<const float4*>(sm.hs + c * RS + r);
+                g += (x.x + x.y) + (x.z + x.w);
+            }
+            add(S_B2 + c, g);
+        }
+        // G1 = (G2 W2) where H1 > 0, then gW1 = G1^T X and gb1
+        layer2<true>(sm, P16 + OFF_W2, vec, wid, lid, acc);
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                if (!((m1 >> (8 * r + 2 * j)) & 1)) acc[r][j].x = 0.f;
+                if (!((m1 >> (8 * r + 2 * j + 1)) & 1)) acc[r][j].y = 0.f;
+            }
+        put_tile(sm.hs, nullptr, acc, wid, lid, r0, rows);
+        __syncthreads();
+#pragma unroll
+        for (int h = 0; h < HID / RT; ++h) {
+            const int c = tid + h * RT;
+            float g[IN] = {}, gb = 0.f;
+#pragma unroll 2
+            for (int r = 0; r < TR; r += 4) {
+                const float4 y = *reinterpret_cast<const float4*>(sm.hs + c * RS + r);
+                gb += (y.x + y.y) + (y.z + y.w);
+#pragma unroll
+                for (int k = 0; k < IN; ++k) {
+                    const float4 x = *reinterpret_cast<const float4*>(sm.xs + k * RS + r);
+                    g[k] = fmaf(y.x, x.x, g[k]);
+                    g[k] = fmaf(y.y, x.y, g[k]);
+                    g[k] = fmaf(y.z, x.z, g[k]);
+                    g[k] = fmaf(y.w, x.w, g[k]);
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < IN; ++k) add(OFF_W1 + c * IN + k, g[k]);
+            add(OFF_B1 + c, gb);
+        }
+        first = false;
+    }
+    if (TRAIN && tid == 0) t.lpart[blockIdx.x] = lsum;
+}
+
+// Partial slot z of gW2 = G2^T H1 over rows [z * per, (z + 1) * per): one
+// 128 x 128 tile per block (grid (2, 2, splits)), 8 x 8 elements per thread.
+__global__ void __launch_bounds__(256) w2_grad_kernel(const float* __restrict__ G, const float* __restrict__ H, int rows,
+                                                      int per, float* part) {
+    __shared__ __align__(16) float gs[2][KC][W2T], hs[2][KC][W2T];
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const int o0 = blockIdx.x * W2T, i0 = blockIdx.y * W2T;
+    const int lo = blockIdx.z * per, hi = min(rows, lo + per);
+    // a chunk: 16 rows x 32 groups of four columns of G and of H, two of each per thread
+    float4 pg[2], ph[2];
+    auto fetch = [&](int r0) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int e = tid + q * 256, r = r0 + (e >> 5), c = 4 * (e & 31);
+            const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+            pg[q] = r < hi ? *reinterpret_cast<const float4*>(G + (int64_t)r * HID + o0 + c) : z;
+            ph[q] = r < hi ? *reinterpret_cast<const float4*>(H + (int64_t)r * HID + i0 + c) : z;
+        }
+    };
+    auto put = [&](int b) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int e = tid + q * 256;
+            *reinterpret_cast<float4*>(&gs[b][e >> 5][4 * (e & 31)]) = pg[q];
+            *reinterpret_cast<float4*>(&hs[b][e >> 5][4 * (e & 31)]) = ph[q];
+        }
+    };
+    float2 acc[8][4];
+    clear(acc);
+    fetch(lo);
+    put(0);
+    __syncthreads();
+    int b = 0;
+    for (int r0 = lo; r0 < hi; r0 += KC, b ^= 1) {
+        const bool more = r0 + KC < hi;
+        if (more) fetch(r0 + KC);
+#pragma unroll
+        for (int k = 0; k < KC; ++k) {
+            const float4 a0 = *reinterpret_cast<const float4*>(&gs[b][k][4 * ty]);
+            const float4 a1 = *reinterpret_cast<const float4*>(&gs[b][k][64 + 4 * ty]);
+            const float4 b0 = *reinterpret_cast<const float4*>(&hs[b][k][4 * tx]);
+            const float4 b1 = *reinterpret_cast<const float4*>(&hs[b][k][64 + 4 * tx]);
+            const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+            const float2 w[4] = {make_float2(b0.x, b0.y), make_float2(b0.z, b0.w), make_float2(b1.x, b1.y),
+                                 make_float2(b1.z, b1.w)};
+#pragma unroll
+            for (int r = 0; r < 8; ++r)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[r][j] = __ffma2_rn(make_float2(a[r], a[r]), w[j], acc[r][j]);
+        }
+        if (more) put(b ^ 1);
+        __syncthreads();
+    }
+    float* out = part + (int64_t)blockIdx.z * HID * HID;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+        float* row = out + (int64_t)(o0 + (r < 4 ? 4 * ty + r : 64 + 4 * ty + r - 4)) * HID + i0 + 4 * tx;
+        *reinterpret_cast<float4*>(row) = make_float4(acc[r][0].x, acc[r][0].y, acc[r][1].x, acc[r][1].y);
+        *reinterpret_cast<float4*>(row + 64) = make_float4(acc[r][2].x, acc[r][2].y, acc[r][3].x, acc[r][3].y);
+    }
+}
+
+// The gradient of every parameter from its partial slots (four lanes per
+// parameter take every fourth slot, then meet in a fixed tree), Adam with
+// bias correction, the bf16 copy, and (block 0) the mean loss.  mu and isd
+// are fixed: their gradient is zero.
+__global__ void __launch_bounds__(256) adam_reduce_kernel(float* P, float* m, float* v, const float* __restrict__ part,
+                                                          int slots, const float* __restrict__ w2part, int splits,
+                                                          const double* __restrict__ lpart, int rows, float lr, float b1,
+                                                          float b2, float eps, float c1, float c2, __nv_bfloat16* P16,
+                                                          float* grad, float* loss) {
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int i = (int)(t >> 2), q = (int)(t & 3);
+    float g = 0.f;
+    if (i < NP && i < OFF_MU) {
+        const bool w2 = i >= OFF_W2 && i < OFF_B2;
+        const float* at = w2 ? w2part + (i - OFF_W2) : part + (i < OFF_W2 ? i : i - HID * HID);
+        const int64_t step = w2 ? HID * HID : SLOT;
+        const int n = w2 ? splits : slots;
+#pragma unroll 8
+        for (int s = q; s < n; s += 4) g += at[s * step];
+    }
+    g += __shfl_xor_sync(0xffffffffu, g, 1);
+    g += __shfl_xor_sync(0xffffffffu, g, 2);
+    if (q == 0 && i < NP) {
+        if (grad) grad[i] = g;
+        const float mi = b1 * m[i] + (1.f - b1) * g;
+        const float vi = b2 * v[i] + (1.f - b2) * g * g;
         m[i] = mi;
         v[i] = vi;
         const float p = P[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
         P[i] = p;
         P16[i] = __float2bfloat16_rn(p);
+    }
+    if (loss && blockIdx.x == 0 && threadIdx.x < 32) {
+        double l = 0.0;
+        for (int s = threadIdx.x; s < slots; s += 32) l += lpart[s];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        if (threadIdx.x == 0) *loss = (float)(l / (double)rows);
     }
 }
 
@@ -486,33 +732,46 @@ __global__ void warm_batched_kernel(const BatchProblem* __restrict__ P, int coun
 }
 
 struct MlpWs {
-    float *Fn, *H1, *H2, *Y, *G3, *G2, *G1, *lrow, *grad;
+    float *H1, *G2, *part, *w2part;
+    double* lpart;
 };
+
+static int row_tiles(int64_t rows) { return (int)((rows + TR - 1) / TR); }
+static int grad_slots(int64_t rows) { return std::min(row_tiles(rows), kMaxSlots); }
+// Rows per split of gW2: whole KC-row chunks, and splits enough for about one
+// block per SM (four tiles of 128 x 128 each) but at least 32 rows, so that a
+// small batch is not all partial sums.
+static int w2_rows_per_split(int64_t rows) {
+    const int64_t per = std::max<int64_t>(32, (rows + 37) / 38);
+    return (int)((per + KC - 1) / KC * KC);
+}
+static int w2_splits(int64_t rows) {
+    const int per = w2_rows_per_split(rows);
+    return (int)((rows + per - 1) / per);
+}
 
 static size_t carve(void* ws, int64_t rows, MlpWs* w) {
     Carver c(ws);
-    w->Fn = c.take<float>((size_t)rows * IN);
     w->H1 = c.take<float>((size_t)rows * HID);
-    w->H2 = c.take<float>((size_t)rows * HID);
-    w->Y = c.take<float>((size_t)rows * OUT);
-    w->G3 = c.take<float>((size_t)rows * OUT);
     w->G2 = c.take<float>((size_t)rows * HID);
-    w->G1 = c.take<float>((size_t)rows * HID);
-    w->lrow = c.take<float>(rows);
-    w->grad = c.take<float>(NP);
+    w->part = c.take<float>((size_t)grad_slots(rows) * SLOT);
+    w->w2part = c.take<float>((size_t)w2_splits(rows) * HID * HID);
+    w->lpart = c.take<double>(grad_slots(rows));
     return c.used;
 }
 
-static dim3 grid2(int rows, int cols) { return dim3((rows + TR - 1) / TR, (cols + TO - 1) / TO); }
-
-static int32_t forward(const float* P, const __nv_bfloat16* P16, const float* F, int rows,
-                       const MlpWs& w, float* Y, cudaStream_t s) {
-    standardise_kernel<<<(int)(((int64_t)rows * IN + 255) / 256), 256, 0, s>>>(F, rows, P, w.Fn);
-    linear_fwd_kernel<<<grid2(rows, HID), 256, 0, s>>>(w.Fn, rows, IN, P16 + OFF_W1, P + OFF_B1, HID, 1, w.H1);
-    linear_fwd_kernel<<<grid2(rows, HID), 256, 0, s>>>(w.H1, rows, HID, P16 + OFF_W2, P + OFF_B2, HID, 1, w.H2);
-    linear_fwd_kernel<<<grid2(rows, OUT), 256, 0, s>>>(w.H2, rows, HID, P16 + OFF_W3, P + OFF_B3, OUT, 0, Y);
-    note_launches(4);
+template <bool TRAIN>
+static int32_t launch_rows(const float* P, const __nv_bfloat16* P16, const float* F, int rows, float* Y,
+                           const TrainOut& t, int grid, cudaStream_t s) {
+    AP_CUDA_TRY(cudaFuncSetAttribute(rows_kernel<TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)sizeof(RowsSmem)));
+    rows_kernel<TRAIN><<<grid, RT, sizeof(RowsSmem), s>>>(P, P16, F, rows, aligned16(P16) ? 1 : 0, Y, t);
+    note_launches(1);
     return last_error();
+}
+
+static int32_t forward(const float* P, const __nv_bfloat16* P16, const float* F, int rows, float* Y, cudaStream_t s) {
+    return launch_rows<false>(P, P16, F, rows, Y, TrainOut{}, std::min(row_tiles(rows), 8192), s);
 }
 
 }  // namespace mlp
@@ -576,9 +835,7 @@ APGB_API int32_t apl_forward(const float* P, const void* P16, const float* F, in
     AP_TRY(require_sm103());
     MlpWs w;
     AP_TRY(check_ws(ws, ws_bytes, carve(nullptr, rows, &w)));
-    carve(ws, rows, &w);
-    return forward(P, static_cast<const __nv_bfloat16*>(P16), F, (int)rows, w, Y,
-                   static_cast<cudaStream_t>(stream));
+    return forward(P, static_cast<const __nv_bfloat16*>(P16), F, (int)rows, Y, static_cast<cudaStream_t>(stream));
 }
 
 APGB_API int32_t apl_train_step(float* P, void* P16, float* M, float* V, int64_t step, float lr,
@@ -592,31 +849,16 @@ APGB_API int32_t apl_train_step(float* P, void* P16, float* M, float* V, int64_t
     MlpWs w;
     AP_TRY(check_ws(ws, ws_bytes, carve(nullptr, rows, &w)));
     carve(ws, rows, &w);
-    const int r = (int)rows;
-    const __nv_bfloat16* W16 = static_cast<const __nv_bfloat16*>(P16);
-    AP_TRY(forward(P, W16, F, r, w, w.Y, s));
-    loss_kernel<<<(r + 255) / 256, 256, 0, s>>>(w.Y, T, r, w.G3, w.lrow);
-    if (loss) mean_kernel<<<1, 1024, 0, s>>>(w.lrow, r, loss);
-    float* g = w.grad;
-    // layer 3
-    weight_grad_kernel<<<dim3(1, (HID + TO - 1) / TO), 256, 0, s>>>(w.G3, r, OUT, w.H2, HID, g + OFF_W3);
-    bias_grad_kernel<<<1, 32, 0, s>>>(w.G3, r, OUT, g + OFF_B3);
-    linear_bwd_input_kernel<<<grid2(r, HID), 256, 0, s>>>(w.G3, r, OUT, W16 + OFF_W3, HID, w.H2, w.G2);
-    // layer 2
-    weight_grad_kernel<<<dim3((HID + TO - 1) / TO, (HID + TO - 1) / TO), 256, 0, s>>>(w.G2, r, HID, w.H1, HID, g + OFF_W2);
-    bias_grad_kernel<<<(HID + 255) / 256, 256, 0, s>>>(w.G2, r, HID, g + OFF_B2);
-    linear_bwd_input_kernel<<<grid2(r, HID), 256, 0, s>>>(w.G2, r, HID, W16 + OFF_W2, HID, w.H1, w.G1);
-    // layer 1
-    weight_grad_kernel<<<dim3((HID + TO - 1) / TO, 1), 256, 0, s>>>(w.G1, r, HID, w.Fn, IN, g + OFF_W1);
-    bias_grad_kernel<<<(HID + 255) / 256, 256, 0, s>>>(w.G1, r, HID, g + OFF_B1);
-    AP_CUDA_TRY(cudaMemsetAsync(g + OFF_MU, 0, sizeof(float) * 2 * IN, s));   // fixed standardisation
-    if (grad_out) AP_CUDA_TRY(cudaMemcpyAsync(grad_out, g, sizeof(float) * NP, cudaMemcpyDeviceToDevice, s));
-    const float b1 = 0.9f, b2 = 0.999f;
+    const int r = (int)rows, slots = grad_slots(rows), per = w2_rows_per_split(rows), splits = w2_splits(rows);
+    AP_TRY(launch_rows<true>(P, static_cast<const __nv_bfloat16*>(P16), F, r, nullptr,
+                             TrainOut{T, w.H1, w.G2, w.part, w.lpart}, slots, s));
+    w2_grad_kernel<<<dim3(HID / W2T, HID / W2T, splits), 256, 0, s>>>(w.G2, w.H1, r, per, w.w2part);
     const float c1 = (float)(1.0 - std::pow(0.9, (double)step));
     const float c2 = (float)(1.0 - std::pow(0.999, (double)step));
-    adam_kernel<<<(int)((NP + 255) / 256), 256, 0, s>>>(P, g, M, V, NP, lr, b1, b2, 1e-8f, c1, c2,
-                                                        static_cast<__nv_bfloat16*>(P16));
-    note_launches(loss ? 12 : 11);
+    adam_reduce_kernel<<<(int)((4 * NP + 255) / 256), 256, 0, s>>>(P, M, V, w.part, slots, w.w2part, splits, w.lpart, r,
+                                                                   lr, 0.9f, 0.999f, 1e-8f, c1, c2,
+                                                                   static_cast<__nv_bfloat16*>(P16), grad_out, loss);
+    note_launches(2);
     return last_error();
 }
 
@@ -755,26 +997,19 @@ APGB_API int32_t apl_ap_run(const float* S, int64_t n, int64_t ld, const float* 
 namespace apgb {
 namespace mlp {
 
-constexpr int64_t kFwdChunk = 65536;     // rows per forward pass (bounds the layer scratch)
-
 static size_t carve_batch(void* ws, const int64_t* n, int32_t count, BatchProblem** table, float** F,
-                          int32_t** nbr, float** Y, void** mlp_ws, size_t* mlp_bytes) {
+                          int32_t** nbr, float** Y) {
     int64_t rows = 0;
     for (int32_t b = 0; b < count; ++b) rows += n[b];
-    MlpWs tmp;
-    const size_t mb = carve(nullptr, std::min(rows, kFwdChunk), &tmp);
     Carver c(ws);
     BatchProblem* t = c.take<BatchProblem>((size_t)count);
     float* f = c.take<float>((size_t)rows * IN);
     int32_t* nb = c.take<int32_t>((size_t)rows * TOPK);
     float* y = c.take<float>((size_t)rows * OUT);
-    void* m = c.take<char>(mb);
     if (table) *table = t;
     if (F) *F = f;
     if (nbr) *nbr = nb;
     if (Y) *Y = y;
-    if (mlp_ws) *mlp_ws = m;
-    if (mlp_bytes) *mlp_bytes = mb;
     return c.used;
 }
 
@@ -785,7 +1020,7 @@ APGB_API size_t apl_warm_start_batched_workspace_size(const int64_t* n, int32_t 
     if (!n || count < 1) return 0;
     for (int32_t b = 0; b < count; ++b)
         if (n[b] < 2 || n[b] > INT_MAX) return 0;
-    return carve_batch(nullptr, n, count, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);
+    return carve_batch(nullptr, n, count, nullptr, nullptr, nullptr, nullptr);
 }
 
 APGB_API int32_t apl_warm_start_batched(const float* S, float* R, float* A, const int64_t* offsets,
@@ -825,21 +1060,14 @@ APGB_API int32_t apl_warm_start_batched(const float* S, float* R, float* A, cons
     BatchProblem* table = nullptr;
     float *F = nullptr, *Yw = nullptr;
     int32_t* nbr = nullptr;
-    void* mws = nullptr;
-    size_t mbytes = 0;
-    carve_batch(ws, n, count, &table, &F, &nbr, &Yw, &mws, &mbytes);
+    carve_batch(ws, n, count, &table, &F, &nbr, &Yw);
     if (!Y) Y = Yw;
     AP_CUDA_TRY(cudaMemcpyAsync(table, host.data(), sizeof(BatchProblem) * count, cudaMemcpyHostToDevice, s));
     features_batched_kernel<<<(int)blocks, 256, 0, s>>>(table, count, F, nbr);
     neighbour_density_batched_kernel<<<(int)((rows + 255) / 256), 256, 0, s>>>(table, count, rows, nbr, F);
     note_launches(2);
     AP_TRY(last_error());
-    MlpWs w;
-    carve(mws, std::min(rows, kFwdChunk), &w);
-    for (int64_t lo = 0; lo < rows; lo += kFwdChunk) {
-        const int cnt = (int)std::min(kFwdChunk, rows - lo);
-        AP_TRY(forward(P, static_cast<const __nv_bfloat16*>(P16), F + lo * IN, cnt, w, Y + lo * OUT, s));
-    }
+    AP_TRY(forward(P, static_cast<const __nv_bfloat16*>(P16), F, (int)rows, Y, s));
     warm_batched_kernel<<<w0, 256, 0, s>>>(table, count, Y);
     note_launches(1);
     return last_error();

@@ -86,6 +86,33 @@ def test_gradient_matches_oracle_and_adam_step():
     assert torch.equal(P16, Pd.to(torch.bfloat16))
 
 
+@pytest.mark.parametrize("rows", [1, 31, 33, 112, 113, 19489])
+def test_step_at_tile_and_split_edges(rows):
+    """Forward and one training step where the row tiles (32), the splits of
+    W2's gradient (112 rows at 4096, at least 32) and the partial slots (608
+    tiles) end raggedly, against the oracle.  Float32 sums of at most 19489
+    terms: 1e-3 of the largest entry, as for the gradient above."""
+    P, Pd, P16 = _params(11)
+    g = np.random.default_rng(rows)
+    F = g.normal(size=(rows, 25)).astype(np.float32)
+    T = np.stack([g.normal(size=rows), np.abs(g.normal(size=rows)), (g.random(rows) < 0.2)],
+                 1).astype(np.float32)
+    Fd, Td = torch.from_numpy(F).cuda(), torch.from_numpy(T).cuda()
+    Yo, _ = omlp.forward(P, F.astype(np.float64), bf16=True)
+    assert rel_inf(capi.apl_forward(Pd, P16, Fd).cpu().numpy().astype(np.float64), Yo) <= 1e-4
+    # bf16 weights that are not 16-byte aligned take scalar loads
+    odd = torch.empty(P16.numel() + 1, dtype=torch.bfloat16, device="cuda")[1:]
+    odd.copy_(P16)
+    assert torch.equal(capi.apl_forward(Pd, odd, Fd), capi.apl_forward(Pd, P16, Fd))
+    M, V = torch.zeros_like(Pd), torch.zeros_like(Pd)
+    loss, grad = capi.apl_train_step(Pd, P16, M, V, 1, 1e-3, Fd, Td, want_grad=True)
+    Lo, Go = omlp.backward(P, F.astype(np.float64), T.astype(np.float64), bf16=True)
+    assert abs(float(loss.item()) - Lo) <= 1e-4 * abs(Lo)
+    go, gg = omlp.unpack(Go), omlp.unpack(grad.cpu().numpy().astype(np.float64))
+    for name in ("W1", "b1", "W2", "b2", "W3", "b3", "mu", "isd"):
+        assert np.abs(gg[name] - go[name]).max() <= 1e-3 * max(np.abs(go[name]).max(), 1e-30), name
+
+
 def test_warm_start_matches_oracle():
     Yh = np.array([[1.0, 2.0, 0.0], [-1.0, -3.0, 0.0], [0.5, 0.25, 1.0], [-0.9, 0.1, -2.0]],
                   dtype=np.float32)
