@@ -45,122 +45,250 @@ constexpr int64_t OFF_W1 = 0, OFF_B1 = OFF_W1 + HID * IN, OFF_W2 = OFF_B1 + HID,
 // ---- features -------------------------------------------------------------------
 constexpr int TOPK = 16;
 
-// Rows k0, k0 + kstep, ... of one problem, one row per block at a time: rows
-// of S read once; per-thread sorted top-16 (value, index) lists merged by 16
-// rounds of block arg-max ordered by (value desc, index asc).  Writes
-// features 0-22 and the 16 neighbour indices (problem-local).
-__device__ __forceinline__ void features_rows(const float* __restrict__ S, int n, int64_t ld, float scale,
-                                              float* F, int32_t* nbr, int k0, int kstep) {
-    __shared__ float hv[32];
-    __shared__ int hi[32];
-    __shared__ double s1w[32], s2w[32];
-    __shared__ int cw[32][4];
-    const int tid = threadIdx.x, lid = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
-    const float inv_scale = 1.f / scale;
+// One warp per row of one problem.  The pass is bound by reading S (twice:
+// the second time mostly from L2) and by about 25 instructions an entry, not
+// by the selection:
+//   scan 1  sums of v and v^2 (two-float accumulators, packed f32x2: float64
+//           arithmetic is scarce on this part), the four counts, and every
+//           lane's largest entry.  The 16th largest of the 32 lane maxima is
+//           a value that at least 16 entries reach;
+//   scan 2  the entries that reach it (about 22 on unordered data) go to a
+//           list in shared memory; if the list fills up it is cut to its 16
+//           best and the bar rises to the 16th of them;
+//   then each listed entry's rank is the number of better ones (larger, or
+//   equal with a lower index): ranks 0-15 are features 0-15.
+// Writes features 0-15 and 18-22, the 16 neighbour indices (problem-local)
+// and the sums, from which features_finish_row makes 16-17 with whole warps
+// of rows (a float64 division by one lane costs what 32 cost).
+// 48 problems of 200-4000 points (2.7e8 entries): 637 us (+ 29 us for the second
+// pass), where one block per row with 16 block-wide arg-max rounds and float64
+// sums took 8.1 ms.
+constexpr int kListCap = 128;      // entries listed per warp
+constexpr int kFeatWarps = 8;      // rows per block
+
+struct FeatList {
+    float v[kListCap];
+    int j[kListCap];
+    float bv[TOPK];
+    int bj[TOPK];
+};
+
+// The power of two nearest below 1 / scale, kept normal.
+__device__ __forceinline__ float unit_of(float scale) {
+    const int e = (int)(__float_as_uint(scale) >> 23);
+    return __uint_as_float((uint32_t)max(1, 253 - e) << 23);
+}
+
+// s + c += x, exactly but for c's rounding (Knuth's two-sum), two columns at a time.
+__device__ __forceinline__ void two_add(float2& s, float2& c, float2 x) {
+    const float2 mone = make_float2(-1.f, -1.f);
+    const float2 t = __fadd2_rn(s, x);
+    const float2 bp = __ffma2_rn(mone, s, t);
+    const float2 ap = __ffma2_rn(mone, bp, t);
+    c = __fadd2_rn(c, __fadd2_rn(__ffma2_rn(mone, ap, s), __ffma2_rn(mone, bp, x)));
+    s = t;
+}
+__device__ __forceinline__ void two_add1(float& s, float& c, float x) {
+    const float t = s + x, bp = t - s;
+    c += (s - (t - bp)) + (x - bp);
+    s = t;
+}
+
+// The 16 best of the list's cnt entries (cnt <= kListCap) to bv, bj, best first.
+__device__ __forceinline__ void rank_list(FeatList& L, int cnt, int lid) {
+    float v[kListCap / 32];
+    int j[kListCap / 32], rank[kListCap / 32];
+#pragma unroll
+    for (int q = 0; q < kListCap / 32; ++q) {
+        const int e = lid + 32 * q;
+        v[q] = e < cnt ? L.v[e] : -INFINITY;
+        j[q] = e < cnt ? L.j[e] : INT_MAX;
+        rank[q] = 0;
+    }
+    for (int e = 0; e < cnt; ++e) {
+        const float w = L.v[e];
+        const int i = L.j[e];
+#pragma unroll
+        for (int q = 0; q < kListCap / 32; ++q) rank[q] += w > v[q] || (w == v[q] && i < j[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < kListCap / 32; ++q)
+        if (lid + 32 * q < cnt && rank[q] < TOPK) {
+            L.bv[rank[q]] = v[q];
+            L.bj[rank[q]] = j[q];
+        }
+    __syncwarp();
+}
+
+// Four consecutive entries 4f .. 4f+3 of a row (vec: 16-byte aligned rows whose
+// stride is a multiple of 4); past the row's end: NaN, which nothing selects.
+__device__ __forceinline__ float4 row4(const float* __restrict__ row, int f, int n, int vec) {
+    if (vec) return __ldg(reinterpret_cast<const float4*>(row) + f);
+    float v[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) v[e] = 4 * f + e < n ? __ldg(row + 4 * f + e) : 0.f;
+    return make_float4(v[0], v[1], v[2], v[3]);
+}
+
+__device__ __forceinline__ void features_row(const float* __restrict__ S, int n, int64_t ld, int vec, float scale,
+                                             int k, float* F, int32_t* nbr, float4* sums, FeatList& L) {
+    const int lid = threadIdx.x & 31;
+    const float* row = S + (int64_t)k * ld;
+    const float inv_scale = 1.f / scale, unit = unit_of(scale);
     float thr[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) thr[q] = -(scale * (0.125f * (float)(1 << q)));   // exact: powers of 2
-    for (int k = k0; k < n; k += kstep) {
-        const float* row = S + (int64_t)k * ld;
-        float top[TOPK];
-        int topi[TOPK];
+    const int n4 = (n + 3) >> 2, fk = k >> 2, nfull = n >> 2;
+    float2 s1 = make_float2(0.f, 0.f), c1 = s1, s2 = s1, c2 = s1;
+    int cnt[4] = {0, 0, 0, 0};
+    float mx = -INFINITY;
+#pragma unroll 2
+    for (int f = lid; f < n4; f += 32) {
+        const float4 x = row4(row, f, n, vec);
+        float v[4] = {x.x, x.y, x.z, x.w};          // what is compared
+        float u[4] = {x.x, x.y, x.z, x.w};          // what is summed
+        if (f == fk || f >= nfull) {
 #pragma unroll
-        for (int q = 0; q < TOPK; ++q) { top[q] = -INFINITY; topi[q] = INT_MAX; }
-        double s1 = 0.0, s2 = 0.0;
-        int cnt[4] = {0, 0, 0, 0};
-        for (int j = tid; j < n; j += blockDim.x) {
-            if (j == k) continue;
-            const float v = row[j];
-            s1 += v;
-            s2 += (double)v * v;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) cnt[q] += v >= thr[q];
-            if (v > top[TOPK - 1]) {            // insertion; equal values keep the lower j first
-                float x = v;
-                int xi = j;
-#pragma unroll
-                for (int q = 0; q < TOPK; ++q) {
-                    if (x > top[q]) {
-                        const float t = top[q];
-                        const int ti = topi[q];
-                        top[q] = x; topi[q] = xi;
-                        x = t; xi = ti;
-                    }
+            for (int e = 0; e < 4; ++e)
+                if (4 * f + e == k || 4 * f + e >= n) {
+                    v[e] = -INFINITY;
+                    u[e] = 0.f;
                 }
-            }
         }
-        // block sums (fixed order: warp tree, then warps in order)
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-            s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+        for (int h = 0; h < 2; ++h) {
+            const float2 w = make_float2(u[2 * h] * unit, u[2 * h + 1] * unit);
+            const float2 p = __ffma2_rn(w, w, make_float2(0.f, 0.f));
+            const float2 e = __ffma2_rn(w, w, make_float2(-p.x, -p.y));     // w^2 = p + e exactly
+            two_add(s1, c1, w);
+            two_add(s2, c2, p);
+            c2 = __fadd2_rn(c2, e);
+        }
 #pragma unroll
-            for (int q = 0; q < 4; ++q) cnt[q] += __shfl_xor_sync(0xffffffffu, cnt[q], o);
-        }
-        if (lid == 0) {
-            s1w[wid] = s1; s2w[wid] = s2;
+        for (int e = 0; e < 4; ++e) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) cw[wid][q] = cnt[q];
+            for (int q = 0; q < 4; ++q) cnt[q] += v[e] >= thr[q];
+            mx = fmaxf(mx, v[e]);
         }
-        // 16 rounds of block arg-max over each thread's next candidate
-        int head = 0;
-        float outv[TOPK];
-        int outi[TOPK];
-        for (int r = 0; r < TOPK; ++r) {
-            float v = head < TOPK ? top[head] : -INFINITY;
-            int vi = head < TOPK ? topi[head] : INT_MAX;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const float v2 = __shfl_xor_sync(0xffffffffu, v, o);
-                const int i2 = __shfl_xor_sync(0xffffffffu, vi, o);
-                if (v2 > v || (v2 == v && i2 < vi)) { v = v2; vi = i2; }
-            }
-            if (lid == 0) { hv[wid] = v; hi[wid] = vi; }
-            __syncthreads();
-            float bv = hv[0];
-            int bi = hi[0];
-            for (int w = 1; w < nw; ++w)
-                if (hv[w] > bv || (hv[w] == bv && hi[w] < bi)) { bv = hv[w]; bi = hi[w]; }
-            if (head < TOPK && bi != INT_MAX && topi[head] == bi) ++head;
-            outv[r] = bv;
-            outi[r] = bi;
-            __syncthreads();
-        }
-        if (tid == 0) {
-            double t1 = 0.0, t2 = 0.0;
-            int c[4] = {0, 0, 0, 0};
-            for (int w = 0; w < nw; ++w) {
-                t1 += s1w[w]; t2 += s2w[w];
-                for (int q = 0; q < 4; ++q) c[q] += cw[w][q];
-            }
-            const double m = t1 / (double)(n - 1);
-            const double var = fmax(0.0, t2 / (double)(n - 1) - m * m);
-            float* f = F + (int64_t)k * IN;
-            float last = outv[0];
-            int lasti = outi[0];
-            for (int r = 0; r < TOPK; ++r) {
-                if (outv[r] == -INFINITY) { outv[r] = last; outi[r] = lasti; }  // n - 1 < 16
-                last = outv[r];
-                lasti = outi[r];
-                f[r] = outv[r] * inv_scale;
-                nbr[(int64_t)k * TOPK + r] = outi[r];
-            }
-            f[16] = (float)(m * (double)inv_scale);
-            f[17] = (float)(sqrt(var) * (double)inv_scale);
-            f[18] = row[k] * inv_scale;
-            for (int q = 0; q < 4; ++q) f[19 + q] = log1pf((float)c[q]);
-        }
-        __syncthreads();
     }
+    // the sums over the warp, in a fixed order
+    float t1 = s1.x, d1 = c1.x, t2 = s2.x, d2 = c2.x;
+    two_add1(t1, d1, s1.y);
+    two_add1(t2, d2, s2.y);
+    d1 += c1.y;
+    d2 += c2.y;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float y1 = __shfl_down_sync(0xffffffffu, t1, o), e1 = __shfl_down_sync(0xffffffffu, d1, o);
+        const float y2 = __shfl_down_sync(0xffffffffu, t2, o), e2 = __shfl_down_sync(0xffffffffu, d2, o);
+        two_add1(t1, d1, y1);
+        two_add1(t2, d2, y2);
+        d1 += e1;
+        d2 += e2;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) cnt[q] = __reduce_add_sync(0xffffffffu, cnt[q]);
+    // the 16th largest lane maximum: sort the 32 of them, largest first
+#pragma unroll
+    for (int w = 2; w <= 32; w <<= 1)
+#pragma unroll
+        for (int o = w >> 1; o > 0; o >>= 1) {
+            const float y = __shfl_xor_sync(0xffffffffu, mx, o);
+            const bool up = ((lid & w) == 0) == ((lid & o) == 0);           // this lane keeps the larger
+            mx = up ? fmaxf(mx, y) : fminf(mx, y);
+        }
+    float bar = __shfl_sync(0xffffffffu, mx, TOPK - 1);
+    int barj = INT_MAX;                             // an entry equal to bar must come before barj
+    int have = 0;
+    for (int f0 = 0; f0 < n4; f0 += 32) {
+        const int f = f0 + lid;
+        float v[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+        if (f < n4) {
+            const float4 x = row4(row, f, n, vec);
+            v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+        }
+        const bool maybe = v[0] >= bar || v[1] >= bar || v[2] >= bar || v[3] >= bar;
+        if (!__any_sync(0xffffffffu, maybe)) continue;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int j = 4 * f + e;
+            const bool in = v[e] > -INFINITY && (v[e] > bar || (v[e] == bar && j < barj)) && j != k && j < n;
+            const unsigned m = __ballot_sync(0xffffffffu, in);
+            if (in) {
+                const int at = have + __popc(m & ((1u << lid) - 1u));
+                L.v[at] = v[e];
+                L.j[at] = j;
+            }
+            have += __popc(m);
+            if (have > kListCap - 32) {             // room for the next 32: keep the best 16
+                __syncwarp();
+                rank_list(L, have, lid);
+                if (lid < TOPK) {
+                    L.v[lid] = L.bv[lid];
+                    L.j[lid] = L.bj[lid];
+                }
+                __syncwarp();
+                have = TOPK;
+                bar = L.v[TOPK - 1];
+                barj = L.j[TOPK - 1];
+            }
+        }
+    }
+    __syncwarp();
+    rank_list(L, have, lid);
+    float* out = F + (int64_t)k * IN;
+    if (lid < TOPK) {
+        // fewer than 16 others: the last one is repeated (the point itself if there is none)
+        const int r = min(lid, have - 1);
+        out[lid] = (r >= 0 ? L.bv[r] : -INFINITY) * inv_scale;
+        nbr[(int64_t)k * TOPK + lid] = r >= 0 ? L.bj[r] : k;
+    }
+    if (lid == 18) out[18] = row[k] * inv_scale;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        if (lid == 19 + q) out[19 + q] = log1pf((float)cnt[q]);
+    if (lid == 0) sums[k] = make_float4(t1, d1, t2, d2);
+    __syncwarp();
 }
 
-__global__ void features_kernel(const float* __restrict__ S, int n, int64_t ld, float scale,
-                                float* F, int32_t* nbr) {
-    features_rows(S, n, ld, scale, F, nbr, blockIdx.x, gridDim.x);
+static __device__ __forceinline__ int row_vec(const float* S, int64_t ld) {
+    return (reinterpret_cast<uintptr_t>(S) & 15) == 0 && (ld & 3) == 0;
 }
 
-// Features 23-24 of row k from the densities of its 16 neighbours.
-__device__ __forceinline__ void neighbour_row(int k, const int32_t* __restrict__ nbr, float* F) {
+__global__ void __launch_bounds__(32 * kFeatWarps) features_kernel(const float* __restrict__ S, int n, int64_t ld,
+                                                                   float scale, float* F, int32_t* nbr,
+                                                                   float4* sums) {
+    __shared__ FeatList lists[kFeatWarps];
+    const int wid = threadIdx.x >> 5, vec = row_vec(S, ld);
+    for (int k = blockIdx.x * kFeatWarps + wid; k < n; k += gridDim.x * kFeatWarps)
+        features_row(S, n, ld, vec, scale, k, F, nbr, sums, lists[wid]);
+}
+
+// Features 16-17 of row k from its sums, 23-24 from the densities of its 16
+// neighbours.  Sums out of float32's range (entries that are infinite, NaN or
+// more than about 1e18 times the scale) are taken again in float64.
+__device__ __forceinline__ void features_finish_row(const float* __restrict__ S, int64_t ld, int k, int n, float scale,
+                                                    const float4* __restrict__ sums, const int32_t* __restrict__ nbr,
+                                                    float* F) {
+    const float4 t = sums[k];
+    const double unit = (double)unit_of(scale), inv_scale = (double)(1.f / scale);
+    double a = (double)t.x + (double)t.y, b = (double)t.z + (double)t.w;
+    if (isfinite(a) && isfinite(b)) {
+        a /= unit;
+        b /= unit * unit;
+    } else {
+        a = b = 0.0;
+        for (int j = 0; j < n; ++j)
+            if (j != k) {
+                const double v = (double)S[(int64_t)k * ld + j];
+                a += v;
+                b += v * v;
+            }
+    }
+    const double m = a / (double)(n - 1);
+    const double var = fmax(0.0, b / (double)(n - 1) - m * m);
+    F[(int64_t)k * IN + 16] = (float)(m * inv_scale);
+    F[(int64_t)k * IN + 17] = (float)(sqrt(var) * inv_scale);
     const float d = F[(int64_t)k * IN + F_DENS];
     float mx = -INFINITY;
     int denser = 0;
@@ -174,9 +302,10 @@ __device__ __forceinline__ void neighbour_row(int k, const int32_t* __restrict__
     F[(int64_t)k * IN + 24] = (float)denser * (1.f / TOPK);
 }
 
-__global__ void neighbour_density_kernel(int n, const int32_t* __restrict__ nbr, float* F) {
+__global__ void features_finish_kernel(const float* __restrict__ S, int64_t ld, int n, float scale, const float4* __restrict__ sums,
+                                       const int32_t* __restrict__ nbr, float* F) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < n) neighbour_row(k, nbr, F);
+    if (k < n) features_finish_row(S, ld, k, n, scale, sums, nbr, F);
 }
 
 // ---- the same over a batch of problems (feature rows of problem b from frow) ----
@@ -188,7 +317,7 @@ struct BatchProblem {
     int n;
     float scale;
     int b0, nb;             // feature blocks: [b0, b0 + nb)
-    int w0;                 // warm-start blocks: [w0, w0 + n), one per row
+    int w0;                 // first warm-start block (kWarmRows rows each)
     int pad;
 };
 
@@ -203,19 +332,26 @@ __device__ __forceinline__ int batch_problem_of(const BatchProblem* P, int count
     return lo;
 }
 
-__global__ void features_batched_kernel(const BatchProblem* __restrict__ P, int count, float* F, int32_t* nbr) {
+__global__ void __launch_bounds__(32 * kFeatWarps) features_batched_kernel(const BatchProblem* __restrict__ P, int count,
+                                                                           float* F, int32_t* nbr, float4* sums) {
+    __shared__ FeatList lists[kFeatWarps];
     const int b = batch_problem_of(P, count, blockIdx.x, [](const BatchProblem& q) { return (int64_t)q.b0; });
     const BatchProblem& q = P[b];
-    features_rows(q.S, q.n, q.ld, q.scale, F + q.frow * IN, nbr + q.frow * TOPK, blockIdx.x - q.b0, q.nb);
+    const int wid = threadIdx.x >> 5;
+    const int k = (blockIdx.x - q.b0) * kFeatWarps + wid;
+    if (k < q.n)
+        features_row(q.S, q.n, q.ld, row_vec(q.S, q.ld), q.scale, k, F + q.frow * IN, nbr + q.frow * TOPK,
+                     sums + q.frow, lists[wid]);
 }
 
-__global__ void neighbour_density_batched_kernel(const BatchProblem* __restrict__ P, int count, int64_t rows,
-                                                 const int32_t* __restrict__ nbr, float* F) {
+__global__ void features_finish_batched_kernel(const BatchProblem* __restrict__ P, int count, int64_t rows,
+                                               const float4* __restrict__ sums, const int32_t* __restrict__ nbr,
+                                               float* F) {
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (t >= rows) return;
     const int b = batch_problem_of(P, count, t, [](const BatchProblem& q) { return q.frow; });
     const BatchProblem& q = P[b];
-    neighbour_row((int)(t - q.frow), nbr + q.frow * TOPK, F + q.frow * IN);
+    features_finish_row(q.S, q.ld, (int)(t - q.frow), q.n, q.scale, sums + q.frow, nbr + q.frow * TOPK, F + q.frow * IN);
 }
 
 // Column j of the standardisation from F [rows x IN] (one block per column,
@@ -714,21 +850,43 @@ __global__ void warm_columns_kernel(const float* __restrict__ Y, int n, float sc
     }
 }
 
-// The warm start of every problem of a batch: one block per row i of problem
-// b; R(i,:) = 0 and A(i,:) the column-constant availabilities of b's
-// predictions (as warm_columns_kernel).
-__global__ void warm_batched_kernel(const BatchProblem* __restrict__ P, int count, const float* __restrict__ Y) {
+// The warm start of every problem of a batch: kWarmRows rows i of problem b per
+// block; R(i,:) = 0 and A(i,:) the column-constant availabilities of b's
+// predictions (as warm_columns_kernel).  Bound by writing R and A: a thread
+// makes its columns' values once and writes them to every row of the block,
+// 16 bytes at a time where the rows allow (2.7e8 entries: 355 us; one row per
+// block and scalar stores took 486 us).
+constexpr int kWarmRows = 16;
+
+__global__ void __launch_bounds__(256) warm_batched_kernel(const BatchProblem* __restrict__ P, int count,
+                                                           const float* __restrict__ Y) {
     const int b = batch_problem_of(P, count, blockIdx.x, [](const BatchProblem& q) { return (int64_t)q.w0; });
     const BatchProblem& q = P[b];
-    const int i = blockIdx.x - q.w0;
+    const int i0 = (blockIdx.x - q.w0) * kWarmRows, i1 = min(q.n, i0 + kWarmRows);
     const float* y = Y + q.frow * OUT;
-    float* rr = q.R + (int64_t)i * q.ld;
-    float* ar = q.A + (int64_t)i * q.ld;
-    for (int k = threadIdx.x; k < q.n; k += blockDim.x) {
-        const float ch = y[k * 3 + 0], ah = y[k * 3 + 1];
-        rr[k] = 0.f;
-        ar[k] = (k == i) ? fmaxf(0.f, ah * q.scale) : fminf(0.f, ch * q.scale);
+    const float scale = q.scale;
+    auto value = [&](int i, int k) {
+        return (k == i) ? fmaxf(0.f, y[k * 3 + 1] * scale) : fminf(0.f, y[k * 3] * scale);
+    };
+    int done = 0;                       // columns written by the vector path
+    if (row_vec(q.R, q.ld) && row_vec(q.A, q.ld)) {
+        for (int f = threadIdx.x; f < q.n >> 2; f += blockDim.x) {
+            const int k = 4 * f;
+            const float4 c = make_float4(value(-1, k), value(-1, k + 1), value(-1, k + 2), value(-1, k + 3));
+            for (int i = i0; i < i1; ++i) {
+                float4 v = c;
+                if ((i >> 2) == f) v = make_float4(value(i, k), value(i, k + 1), value(i, k + 2), value(i, k + 3));
+                reinterpret_cast<float4*>(q.R + (int64_t)i * q.ld)[f] = make_float4(0.f, 0.f, 0.f, 0.f);
+                reinterpret_cast<float4*>(q.A + (int64_t)i * q.ld)[f] = v;
+            }
+        }
+        done = q.n & ~3;
     }
+    for (int k = done + threadIdx.x; k < q.n; k += blockDim.x)
+        for (int i = i0; i < i1; ++i) {
+            q.R[(int64_t)i * q.ld + k] = 0.f;
+            q.A[(int64_t)i * q.ld + k] = value(i, k);
+        }
 }
 
 struct MlpWs {
@@ -786,6 +944,7 @@ APGB_API size_t apl_features_workspace_size(int64_t n) {
     if (n < 2 || n > INT_MAX) return 0;
     Carver c(nullptr);
     c.take<int32_t>((size_t)n * TOPK);
+    c.take<float4>((size_t)n);
     return c.used;
 }
 
@@ -797,8 +956,10 @@ APGB_API int32_t apl_features(const float* S, int64_t n, int64_t ld, float scale
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     Carver c(ws);
     int32_t* nbr = c.take<int32_t>((size_t)n * TOPK);
-    features_kernel<<<(int)std::min<int64_t>(n, 65535), 256, 0, s>>>(S, (int)n, ld, scale, F, nbr);
-    neighbour_density_kernel<<<(int)((n + 255) / 256), 256, 0, s>>>((int)n, nbr, F);
+    float4* sums = c.take<float4>((size_t)n);
+    features_kernel<<<(int)std::min<int64_t>((n + kFeatWarps - 1) / kFeatWarps, 65535), 32 * kFeatWarps, 0, s>>>(
+        S, (int)n, ld, scale, F, nbr, sums);
+    features_finish_kernel<<<(int)((n + 255) / 256), 256, 0, s>>>(S, ld, (int)n, scale, sums, nbr, F);
     note_launches(2);
     return last_error();
 }
@@ -998,14 +1159,16 @@ namespace apgb {
 namespace mlp {
 
 static size_t carve_batch(void* ws, const int64_t* n, int32_t count, BatchProblem** table, float** F,
-                          int32_t** nbr, float** Y) {
+                          int32_t** nbr, float4** sums, float** Y) {
     int64_t rows = 0;
     for (int32_t b = 0; b < count; ++b) rows += n[b];
     Carver c(ws);
     BatchProblem* t = c.take<BatchProblem>((size_t)count);
     float* f = c.take<float>((size_t)rows * IN);
     int32_t* nb = c.take<int32_t>((size_t)rows * TOPK);
+    float4* sm = c.take<float4>((size_t)rows);
     float* y = c.take<float>((size_t)rows * OUT);
+    if (sums) *sums = sm;
     if (table) *table = t;
     if (F) *F = f;
     if (nbr) *nbr = nb;
@@ -1020,7 +1183,7 @@ APGB_API size_t apl_warm_start_batched_workspace_size(const int64_t* n, int32_t 
     if (!n || count < 1) return 0;
     for (int32_t b = 0; b < count; ++b)
         if (n[b] < 2 || n[b] > INT_MAX) return 0;
-    return carve_batch(nullptr, n, count, nullptr, nullptr, nullptr, nullptr);
+    return carve_batch(nullptr, n, count, nullptr, nullptr, nullptr, nullptr, nullptr);
 }
 
 APGB_API int32_t apl_warm_start_batched(const float* S, float* R, float* A, const int64_t* offsets,
@@ -1043,7 +1206,7 @@ APGB_API int32_t apl_warm_start_batched(const float* S, float* R, float* A, cons
         q.frow = rows;
         q.n = (int)n[b];
         q.scale = scale[b];
-        q.nb = (int)std::min<int64_t>(n[b], 1024);
+        q.nb = (int)((n[b] + kFeatWarps - 1) / kFeatWarps);
         q.b0 = (int)blocks;
         blocks += q.nb;
         rows += n[b];
@@ -1052,7 +1215,7 @@ APGB_API int32_t apl_warm_start_batched(const float* S, float* R, float* A, cons
     int w0 = 0;
     for (int32_t b = 0; b < count; ++b) {
         host[b].w0 = w0;
-        w0 += host[b].n;
+        w0 += (host[b].n + kWarmRows - 1) / kWarmRows;
     }
     AP_TRY(require_sm103());
     AP_TRY(check_ws(ws, ws_bytes, need));
@@ -1060,11 +1223,12 @@ APGB_API int32_t apl_warm_start_batched(const float* S, float* R, float* A, cons
     BatchProblem* table = nullptr;
     float *F = nullptr, *Yw = nullptr;
     int32_t* nbr = nullptr;
-    carve_batch(ws, n, count, &table, &F, &nbr, &Yw);
+    float4* sums = nullptr;
+    carve_batch(ws, n, count, &table, &F, &nbr, &sums, &Yw);
     if (!Y) Y = Yw;
     AP_CUDA_TRY(cudaMemcpyAsync(table, host.data(), sizeof(BatchProblem) * count, cudaMemcpyHostToDevice, s));
-    features_batched_kernel<<<(int)blocks, 256, 0, s>>>(table, count, F, nbr);
-    neighbour_density_batched_kernel<<<(int)((rows + 255) / 256), 256, 0, s>>>(table, count, rows, nbr, F);
+    features_batched_kernel<<<(int)blocks, 32 * kFeatWarps, 0, s>>>(table, count, F, nbr, sums);
+    features_finish_batched_kernel<<<(int)((rows + 255) / 256), 256, 0, s>>>(table, count, rows, sums, nbr, F);
     note_launches(2);
     AP_TRY(last_error());
     AP_TRY(forward(P, static_cast<const __nv_bfloat16*>(P16), F, (int)rows, Y, s));

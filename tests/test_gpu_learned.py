@@ -52,6 +52,56 @@ def test_features_match_oracle(n):
     assert np.array_equal(F[:, 24], Fo[:, 24])
 
 
+@pytest.mark.parametrize("ld_pad", [0, 1])
+@pytest.mark.parametrize("kind,n", [("equal", 129), ("equal", 700), ("ascending", 701), ("steps", 1030),
+                                    ("mixture", 2), ("mixture", 33), ("masked", 300), ("huge", 260)])
+def test_features_selection_edges(kind, n, ld_pad):
+    """Rows where the selection's list fills up or ties decide (all entries
+    equal, each larger than the one before, few distinct values), fewer than
+    16 others, entries at -inf, and values whose squares leave float32's
+    range; rows 16-byte aligned or not.  Counts and order against the oracle
+    (values as float32), moments within float32 rounding."""
+    g = np.random.default_rng(n)
+    if kind == "equal":
+        S = np.full((n, n), -1.0)
+    elif kind == "ascending":
+        S = np.tile(-(n - np.arange(n)) * 0.01, (n, 1))
+    elif kind == "steps":
+        S = -np.floor(g.uniform(0, 6, (n, n)))
+    else:
+        S = oap.build_similarity(synth.gaussian_mixture(n, 5, 2, n, 4.0, 1.0)[0])[0]
+    if kind == "huge":
+        S = S * 1e25
+    S = S.astype(np.float32).astype(np.float64)
+    scale = float(np.float32(np.median(-S[~np.eye(n, dtype=bool)])))
+    if kind == "masked":
+        S[g.random((n, n)) < 0.97] = -np.inf
+        np.fill_diagonal(S, -scale)
+    ld = capi.padded_ld(n) + ld_pad
+    base = torch.full((n, ld), float("nan"), dtype=torch.float32, device="cuda")
+    base[:, :n] = torch.from_numpy(S.astype(np.float32)).cuda()
+    F = capi.apl_features(base[:, :n], scale).cpu().numpy().astype(np.float64)
+    D = S.copy()
+    np.fill_diagonal(D, -np.inf)
+    order = np.argsort(-D, axis=1, kind="stable")[:, :16]
+    finite = np.isfinite(D).sum(1)
+    order = np.take_along_axis(order, np.minimum(np.arange(order.shape[1])[None, :], finite[:, None] - 1), 1)
+    if order.shape[1] < 16:
+        order = np.concatenate([order, np.repeat(order[:, -1:], 16 - order.shape[1], 1)], 1)
+    top = np.take_along_axis(D, order, 1)
+    assert np.allclose(F[:, :16], top / scale, rtol=3e-7, atol=0)
+    cnt = np.stack([(D >= -np.float64(np.float32(scale) * np.float32(q))).sum(1)
+                    for q in (0.125, 0.25, 0.5, 1.0)], 1)
+    assert np.abs(F[:, 19:23] - np.log1p(cnt)).max() <= 1e-6
+    dens = F[:, 20]
+    assert np.array_equal(F[:, 24], (dens[order] > dens[:, None]).mean(1))
+    if kind == "masked":
+        assert np.all(np.isneginf(F[:, 16])) and np.all(F[:, 17] == 0)
+    else:
+        off = S[~np.eye(n, dtype=bool)].reshape(n, n - 1)
+        assert rel_inf(F[:, 16:18], np.stack([off.mean(1), off.std(1)], 1) / scale) <= 1e-6
+
+
 def test_forward_matches_oracle():
     P, Pd, P16 = _params()
     F = np.random.default_rng(7).normal(size=(1000, 25)).astype(np.float32)
