@@ -8,9 +8,9 @@
 //      (of the bf16-rounded rows for the tensor-core path);
 //   3. S = 2 Xc Xc^T - |x_i|^2 - |x_k|^2 clamped to <= 0 (SIMT float32 GEMM
 //      here, tcgen05 GEMM in tc_gemm.cu);
-//   4. preference: exact median of the n(n-1) off-diagonal values by a
-//      three-pass radix select on order-preserving 32-bit keys (11/11/10
-//      bits), both middle order statistics at once;
+//   4. preference: exact median of the n(n-1) off-diagonal values, both middle
+//      order statistics at once, on order-preserving 32-bit keys: a sampled
+//      bracket, one pass over S, and radix digits over what it encloses;
 //   5. diagonal <- p, then s <- s + noise_rel*|s|*u(i,k) on every entry.
 #include <algorithm>
 #include <mutex>
@@ -259,154 +259,429 @@ __device__ __forceinline__ float key_float(uint32_t k) {
     return __uint_as_float(u);
 }
 
+// The two middle order statistics of the n(n-1) off-diagonal entries of S, in
+// one pass over S.  16384 entries drawn at random bracket the median
+// (sample_kernel): the sample's order statistics 288 either side of its
+// middle (4.5 standard deviations of a median's rank) enclose the wanted ranks
+// but for about 1 matrix in 10^5.  bracket_pass reads S once, counts the
+// entries below the bracket and copies those inside it (3.5 % on average) to
+// a buffer; digit_kernel then selects by radix passes of 11 bits over the
+// buffer, starting at the bracket's own highest bit.  Where the bracket missed
+// or the buffer overflowed (a large share of equal entries), the digit passes
+// read S itself from the top bit, so the result is exact either way.  The
+// decision stays on the device.  20000 points (1.6 GB): 445 us, of which the
+// pass is 374, the digits 52 and the sample 18, where three radix passes over
+// S took 1025 us; 1000 points: 62 us where they took 144 us (16 blocks, most of
+// the time waiting on shared-memory atomics).
+constexpr int kSampleThreads = 1024;
+constexpr int kSamplePer = 16;          // entries drawn per thread
+constexpr int kSample = kSampleThreads * kSamplePer, kSampleHalfWidth = 288;
+constexpr int kSampleBins = 1024;       // two digits of 10 bits settle the bracket
+constexpr int kChunk = 512;             // buffer entries a warp takes at a time (its hits of one step, at most)
+constexpr int kPassWarps = 8;           // warps per block of the pass
+
 struct SelectState {
-    uint32_t prefix[2];
+    uint32_t lo, range;       // the bracket: keys lo .. lo + range
+    uint32_t prefix[2];       // known digits of (key - lo) of the two order statistics
     uint32_t known_mask;
-    int32_t  pad;
-    uint64_t rank[2];
+    int32_t  direct;          // the digit passes read S (lo = 0), not the buffer
+    uint64_t rank[2];         // ranks left inside the prefix
+    unsigned long long less, inside, slots;   // entries below and inside the bracket; buffer taken
+    unsigned ticket;          // blocks of a digit pass that have finished
+    int32_t  bits;            // of range + 1: where the digits start
 };
 
-// Pass: histogram of the digit at `shift` among entries whose known high bits
-// match each target's prefix.
-// Histogram of digit (key >> shift) & (2^bits - 1) over the off-diagonal keys
-// that match each order statistic's known prefix.  While both statistics
-// share their prefix (always in the first pass, usually later), one histogram
-// serves both.  VEC: rows read as float4 (S 16-byte aligned, lds % 4 == 0).
-// Block bx of gx blocks (rows bx, bx + gx, ...).
+// One selection: a problem's S, its buffer and its blocks in the launch.
+struct Select {
+    const float* S;
+    int64_t lds;
+    int n;
+    int b0, nb;               // blocks [b0, b0 + nb) of the pass
+    int d0, dn;               // blocks [d0, d0 + dn) of a digit pass
+    SelectState* st;
+    unsigned long long* hist; // 2 x 2048 bins
+    uint32_t* cand;           // the buffer, cap entries
+    unsigned long long cap;
+    float* pref;
+};
+
+// Blocks of the pass over S: about 32K entries each, at most 8 blocks per SM; half
+// of them for the digits of the buffer.
+static int pass_blocks(int n) {
+    return (int)std::max<int64_t>(1, std::min<int64_t>(1216, ((int64_t)n * n + 32767) / 32768));
+}
+static int digit_blocks(int n) { return std::max(1, pass_blocks(n) / 2); }
+// A 16th of the entries (the bracket holds 3.5 % on average), and every warp's last chunk.
+static unsigned long long cand_cap(int n) {
+    return (unsigned long long)n * (unsigned long long)n / 16 + (unsigned long long)pass_blocks(n) * kPassWarps * kChunk;
+}
+
+// The bracket of one problem (one block of kSampleThreads): kSample entries at
+// seeded random places off the diagonal, and the keys around the two ranks by
+// two radix passes of 10 bits below the sample's own highest differing bit
+// (the digits spread: a fixed top byte would put nearly every entry in one
+// bin, whose shared-memory atomics wait for one another).  What the digits
+// leave open widens the bracket.  The state and histograms start from here.
+__device__ __forceinline__ void sample_block(const Select& q) {
+    __shared__ unsigned int h[2][kSampleBins];
+    __shared__ unsigned int wsum[32];
+    __shared__ uint32_t wmin[32], wmax[32];
+    __shared__ int found[2];
+    __shared__ unsigned int rem[2];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    uint32_t key[kSamplePer];
+    uint32_t kmin = 0xffffffffu, kmax = 0;
+#pragma unroll
+    for (int e = 0; e < kSamplePer; ++e) {
+        const uint64_t u = splitmix64_at(0x6d656469616eull, (uint64_t)(e * kSampleThreads + t) + 1);
+        const int i = (int)(((u >> 32) * (uint64_t)q.n) >> 32);
+        int k = (int)(((u & 0xffffffffull) * (uint64_t)(q.n - 1)) >> 32);
+        k += k >= i;
+        key[e] = float_key(__ldg(q.S + (int64_t)i * q.lds + k));
+    }
+#pragma unroll
+    for (int e = 0; e < kSamplePer; ++e) {
+        kmin = min(kmin, key[e]);
+        kmax = max(kmax, key[e]);
+    }
+    kmin = __reduce_min_sync(0xffffffffu, kmin);
+    kmax = __reduce_max_sync(0xffffffffu, kmax);
+    if (lane == 0) { wmin[warp] = kmin; wmax[warp] = kmax; }
+    for (int b = t; b < 4096; b += kSampleThreads) q.hist[b] = 0;
+    __syncthreads();
+    kmin = __reduce_min_sync(0xffffffffu, wmin[lane]);
+    kmax = __reduce_max_sync(0xffffffffu, wmax[lane]);
+    const int bits = 32 - __clz((int)(kmax - kmin));
+    uint32_t pre[2] = {0, 0}, km = 0;
+    unsigned int rank[2] = {kSample / 2 - kSampleHalfWidth, kSample / 2 + kSampleHalfWidth};
+    int shift = bits;
+#pragma unroll
+    for (int pass = 0; pass < 2; ++pass) {
+        const int width = min(10, shift);
+        shift -= width;
+        const uint32_t dm = (1u << width) - 1u;
+        h[0][t] = 0;
+        h[1][t] = 0;
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < kSamplePer; ++e) {
+            const uint32_t rel = key[e] - kmin, dg = (rel >> shift) & dm;
+            if ((rel & km) == pre[0]) atomicAdd(&h[0][dg], 1u);
+            if ((rel & km) == pre[1]) atomicAdd(&h[1][dg], 1u);
+        }
+        __syncthreads();
+        // thread t owns bin t of both histograms (each at most kSample: 15 bits),
+        // scanned together in one word
+        const unsigned int own = h[0][t] | (h[1][t] << 16);
+        unsigned int x = own;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned int y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) wsum[warp] = x;
+        __syncthreads();
+        unsigned int w = wsum[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned int y = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += y;
+        }
+        const unsigned int before = __shfl_sync(0xffffffffu, w, warp > 0 ? warp - 1 : 0);
+        x += (warp > 0 ? before : 0u) - own;                // exclusive
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const unsigned int lo = (x >> (16 * j)) & 0xffffu, c = (own >> (16 * j)) & 0xffffu;
+            if (rank[j] >= lo && rank[j] < lo + c) {
+                found[j] = t;
+                rem[j] = rank[j] - lo;
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            pre[j] |= (uint32_t)found[j] << shift;
+            rank[j] = rem[j];
+        }
+        km |= dm << shift;
+        __syncthreads();
+    }
+    if (t == 0) {
+        SelectState s{};
+        s.lo = kmin + pre[0];
+        s.range = (pre[1] | ((1u << shift) - 1u)) - pre[0];
+        const uint64_t m = (uint64_t)q.n * (uint64_t)(q.n - 1);
+        s.rank[0] = (m - 1) / 2;
+        s.rank[1] = m / 2;
+        *q.st = s;
+    }
+}
+
+// Four consecutive entries 4f .. 4f+3 of a row; entries past its end read as 0.
 template <bool VEC>
-__device__ __forceinline__ void radix_hist_rows(const float* __restrict__ S, int n, int64_t lds,
-                                                int shift, int bits, const SelectState* __restrict__ st,
-                                                unsigned long long* hist, int bx, int gx) {
+__device__ __forceinline__ float4 entries4(const float* __restrict__ row, int f, int n) {
+    if constexpr (VEC) {
+        return __ldg(reinterpret_cast<const float4*>(row) + f);
+    } else {
+        float v[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[e] = 4 * f + e < n ? __ldg(row + 4 * f + e) : 0.f;
+        return make_float4(v[0], v[1], v[2], v[3]);
+    }
+}
+
+// The pass over S: warps take rows in turn; block bx of gx.  A step is 512
+// entries of a row, 16 per lane: two float comparisons each settle all but
+// the bracket's own; these (3.5 %) are looked at again as keys, so that NaN
+// and signed zeros fall where their keys do, and written behind one another
+// by a scan of the lanes' counts.  About 9 instructions an entry, so the pass
+// runs at the rate S can be read.
+template <bool VEC>
+__device__ __forceinline__ void bracket_pass(const Select& q, int bx, int gx) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t lo = q.st->lo, range = q.st->range;
+    const float flo = key_float(lo), fhi = key_float(lo + range);
+    const int n = q.n, n4 = (n + 3) >> 2, nfull = n >> 2;
+    unsigned less = 0, inside = 0;
+    // the warp's current chunk of the buffer: entries [at, end)
+    unsigned long long at = 0, end = 0;
+    bool full = false;
+    for (int i = bx * kPassWarps + (threadIdx.x >> 5); i < n; i += gx * kPassWarps) {
+        const float* row = q.S + (int64_t)i * q.lds;
+        const int fi = i >> 2;
+        for (int f0 = 0; f0 < n4; f0 += 128) {
+            float4 x[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int f = f0 + 32 * u + lane;
+                x[u] = f < n4 ? entries4<VEC>(row, f, n) : make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
+            }
+            unsigned mask = 0;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int f = f0 + 32 * u + lane;
+                float v[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
+                if (f == fi || f >= nfull) {
+                    // the diagonal and what lies past the row's end: above every finite bracket
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if (4 * f + e == i || 4 * f + e >= n) v[e] = INFINITY;
+                }
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const bool below = v[e] < flo;
+                    less += below;
+                    if (!below && !(v[e] > fhi)) mask |= 1u << (4 * u + e);
+                }
+            }
+            if (!__any_sync(0xffffffffu, mask != 0)) continue;
+            // the candidates again, as keys
+            unsigned keep = 0;
+            for (unsigned m = mask; m; m &= m - 1) {
+                const int b = __ffs((int)m) - 1, k = 4 * (f0 + 32 * (b >> 2) + lane) + (b & 3);
+                if (k == i || k >= n) continue;
+                const uint32_t key = float_key(__ldg(row + k));
+                if (key - lo <= range) keep |= 1u << b;
+                else less += key < lo;
+            }
+            const int own = __popc(keep);
+            int incl = own;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            const int total = __shfl_sync(0xffffffffu, incl, 31);
+            inside += total;
+            if (full || total == 0) continue;
+            unsigned long long pos = at + (incl - own), fresh = 0;
+            if (at + total > end) {                         // the entries past `end` open a new chunk
+                if (lane == 0) fresh = atomicAdd(&q.st->slots, (unsigned long long)kChunk);
+                fresh = __shfl_sync(0xffffffffu, fresh, 0);
+                if (fresh + kChunk > q.cap) {
+                    full = true;                            // the digit passes will read S
+                    continue;
+                }
+            }
+            for (unsigned m = keep; m; m &= m - 1, ++pos) {
+                const int b = __ffs((int)m) - 1, k = 4 * (f0 + 32 * (b >> 2) + lane) + (b & 3);
+                q.cand[pos < end ? pos : fresh + (pos - end)] = float_key(__ldg(row + k)) - lo;
+            }
+            if (at + total > end) {
+                at = fresh + (at + total - end);
+                end = fresh + kChunk;
+            } else {
+                at += total;
+            }
+        }
+    }
+    for (unsigned long long x = at + lane; x < end; x += 32) q.cand[x] = 0xffffffffu;   // beyond every range
+    less = __reduce_add_sync(0xffffffffu, less);
+    if (lane == 0) {
+        if (less) atomicAdd(&q.st->less, (unsigned long long)less);
+        if (inside) atomicAdd(&q.st->inside, (unsigned long long)inside);
+    }
+}
+
+// The bin of a histogram of at most 2048 counts that holds rank r, and the
+// rank left inside it (a block of 256 threads, eight bins each).
+__device__ __forceinline__ void find_bin(const unsigned long long* h, int nb, unsigned long long r,
+                                         unsigned long long* wsum, int* found, unsigned long long* rem) {
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    unsigned long long c[8], own = 0;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) c[e] = 8 * t + e < nb ? __ldcg(h + 8 * t + e) : 0ull;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) own += c[e];
+    unsigned long long x = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    __syncthreads();
+    if (lane == 31) wsum[warp] = x;
+    __syncthreads();
+    unsigned long long at = x - own;
+    for (int w = 0; w < warp; ++w) at += wsum[w];
+    if (r >= at && r < at + own) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            if (r >= at && r < at + c[e]) {
+                *found = 8 * t + e;
+                *rem = r - at;
+            }
+            at += c[e];
+        }
+    }
+    __syncthreads();
+}
+
+// Digit pass p (0, 1, 2): block bx of gx counts the digit of the entries that
+// match each order statistic's known prefix (one histogram serves both while
+// they share it); the last block to finish finds the two bins and advances
+// the state.
+template <bool VEC>
+__device__ __forceinline__ void digit_pass(const Select& q, int p, int bx, int gx) {
     __shared__ unsigned int h[2][2048];
-    const int nb = 1 << bits;
+    __shared__ unsigned long long wsum[32], rem[2];
+    __shared__ int found[2];
+    __shared__ bool last;
+    SelectState* st = q.st;
+    // pass 0 settles what the bracket gave (every block reads the same values;
+    // the last one writes them)
+    uint32_t lo = st->lo, range = st->range;
+    bool direct = st->direct != 0;
+    uint64_t r0 = st->rank[0], r1 = st->rank[1];
+    int bits = st->bits;
+    if (p == 0) {
+        const unsigned long long less = st->less, inside = st->inside;
+        // a full buffer is one whose chunks passed its end; a bracket up to the
+        // largest key would leave the unused entries' mark inside it
+        direct = st->slots > q.cap || r0 < less || r1 >= less + inside || range == 0xffffffffu;
+        if (direct) {
+            lo = 0;
+            range = 0xffffffffu;
+        } else {
+            r0 -= less;
+            r1 -= less;
+        }
+        bits = 32 - __clz((int)range);
+    }
+    const int top = bits - 11 * p;                      // bits still unknown
+    if (top <= 0 && p > 0) return;
+    const int shift = max(0, top - 11), width = max(0, min(11, top)), nb = 1 << width;
+    const uint32_t dm = (uint32_t)nb - 1u;
+    const uint32_t km = p == 0 ? 0u : st->known_mask, p0 = p == 0 ? 0u : st->prefix[0], p1 = p == 0 ? 0u : st->prefix[1];
+    const bool same = p0 == p1;
     for (int b = threadIdx.x; b < 2 * 2048; b += blockDim.x) (&h[0][0])[b] = 0;
     __syncthreads();
-    const uint32_t km = st->known_mask, p0 = st->prefix[0], p1 = st->prefix[1];
-    const bool same = p0 == p1;
-    const uint32_t dm = (uint32_t)nb - 1u;
-    auto count = [&](float v) {
-        const uint32_t key = float_key(v);
-        const uint32_t dg = (key >> shift) & dm;
-        if ((key & km) == p0) atomicAdd(&h[0][dg], 1u);
-        if (!same && (key & km) == p1) atomicAdd(&h[1][dg], 1u);
+    auto count = [&](uint32_t rel) {
+        const uint32_t dg = (rel >> shift) & dm;
+        if ((rel & km) == p0) atomicAdd(&h[0][dg], 1u);
+        if (!same && (rel & km) == p1) atomicAdd(&h[1][dg], 1u);
     };
-    for (int i = bx; i < n; i += gx) {
-        const float* row = S + (int64_t)i * lds;
-        if (VEC) {
-            const float4* row4 = reinterpret_cast<const float4*>(row);
-            const int n4 = (n + 3) >> 2;
-            for (int k4 = threadIdx.x; k4 < n4; k4 += blockDim.x) {
-                const float4 v = row4[k4];
-                const int k = 4 * k4;
-                if (k != i && k < n) count(v.x);
-                if (k + 1 != i && k + 1 < n) count(v.y);
-                if (k + 2 != i && k + 2 < n) count(v.z);
-                if (k + 3 != i && k + 3 < n) count(v.w);
+    if (!direct) {
+        const unsigned long long slots = st->slots;
+        const uint4* c4 = reinterpret_cast<const uint4*>(q.cand);      // slots is a multiple of kChunk
+        const unsigned long long n4 = slots / 4, step = (unsigned long long)gx * blockDim.x;
+        for (unsigned long long x0 = (unsigned long long)bx * blockDim.x + threadIdx.x; x0 < n4; x0 += 4 * step) {
+            uint4 v[4];                     // four loads in flight before the first count
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                v[u] = x0 + u * step < n4 ? __ldg(c4 + x0 + u * step)
+                                          : make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (v[u].x <= range) count(v[u].x);
+                if (v[u].y <= range) count(v[u].y);
+                if (v[u].z <= range) count(v[u].z);
+                if (v[u].w <= range) count(v[u].w);
             }
-        } else {
-            for (int k = threadIdx.x; k < n; k += blockDim.x)
-                if (k != i) count(row[k]);
+        }
+    } else {
+        const int n4 = (q.n + 3) >> 2;
+        for (int i = bx; i < q.n; i += gx) {
+            const float* row = q.S + (int64_t)i * q.lds;
+            for (int f = threadIdx.x; f < n4; f += blockDim.x) {
+                const float4 x = entries4<VEC>(row, f, q.n);
+                const float v[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (4 * f + e < q.n && 4 * f + e != i) count(float_key(v[e]));
+            }
         }
     }
     __syncthreads();
     for (int b = threadIdx.x; b < nb; b += blockDim.x) {
         const unsigned int c0 = h[0][b], c1 = same ? c0 : h[1][b];
-        if (c0) atomicAdd(&hist[b], (unsigned long long)c0);
-        if (c1) atomicAdd(&hist[2048 + b], (unsigned long long)c1);
+        if (c0) atomicAdd(&q.hist[b], (unsigned long long)c0);
+        if (c1) atomicAdd(&q.hist[2048 + b], (unsigned long long)c1);
     }
-}
-
-template <bool VEC>
-__global__ void __launch_bounds__(256) radix_hist_kernel(const float* __restrict__ S, int n,
-                                                         int64_t lds, int shift, int bits,
-                                                         const SelectState* __restrict__ st,
-                                                         unsigned long long* hist) {
-    radix_hist_rows<VEC>(S, n, lds, shift, bits, st, hist, blockIdx.x, gridDim.x);
-}
-
-// For each order statistic: the bin holding its remaining rank (a block-wide
-// exclusive scan of the counts; each of the 1024 threads owns 2 bins), then
-// the prefix, rank and known-digit mask are advanced and the histograms
-// cleared for the next pass.
-__device__ __forceinline__ void radix_scan_block(SelectState* st, unsigned long long* hist,
-                                                 int shift, int bits) {
-    const int nb = 1 << bits;
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    __shared__ unsigned long long wsum[32];
-    __shared__ int found[2];
-    __shared__ unsigned long long rem[2];
-    if (t < 2) {
-        found[t] = nb - 1;          // kept only if the counts were inconsistent
-        rem[t] = st->rank[t];
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(&st->ticket, 1u) == (unsigned)gx - 1u;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    if (threadIdx.x < 2) {
+        found[threadIdx.x] = nb - 1;                    // kept only if the counts were inconsistent
+        rem[threadIdx.x] = 0;
     }
     __syncthreads();
-    for (int j = 0; j < 2; ++j) {
-        const unsigned long long* h = hist + 2048 * j;
-        const unsigned long long r = st->rank[j];
-        const int b0 = 2 * t;
-        const unsigned long long c0 = b0 < nb ? h[b0] : 0ull, c1 = b0 + 1 < nb ? h[b0 + 1] : 0ull;
-        unsigned long long x = c0 + c1;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) wsum[warp] = x;
-        __syncthreads();
-        if (warp == 0) {
-            unsigned long long v = wsum[lane];
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned long long y = __shfl_up_sync(0xffffffffu, v, o);
-                if (lane >= o) v += y;
-            }
-            wsum[lane] = v;
-        }
-        __syncthreads();
-        const unsigned long long base = (warp > 0 ? wsum[warp - 1] : 0ull) + x - (c0 + c1);
-        if (r >= base && r < base + c0) {
-            found[j] = b0;
-            rem[j] = r - base;
-        } else if (r >= base + c0 && r < base + c0 + c1) {
-            found[j] = b0 + 1;
-            rem[j] = r - base - c0;
-        }
-        __syncthreads();
-    }
-    if (t < 2) {
-        st->prefix[t] |= (uint32_t)found[t] << shift;
-        st->rank[t] = rem[t];
-    }
-    if (t == 0) st->known_mask |= (uint32_t)(nb - 1) << shift;
-    for (int b = t; b < 2 * 2048; b += blockDim.x) hist[b] = 0;
-}
-
-__global__ void __launch_bounds__(1024) radix_scan_kernel(SelectState* st, unsigned long long* hist,
-                                                          int shift, int bits) {
-    radix_scan_block(st, hist, shift, bits);
-}
-
-// The two middle order statistics of the n(n-1) off-diagonal entries:
-// ranks (m-1)/2 and m/2, m = n(n-1).
-__device__ __forceinline__ void select_init_block(SelectState* st, unsigned long long* hist, int n) {
-    const uint64_t m = (uint64_t)n * (uint64_t)(n - 1);
-    for (int x = threadIdx.x; x < 4096; x += blockDim.x) hist[x] = 0;
+    find_bin(q.hist, nb, r0, wsum, &found[0], &rem[0]);
+    find_bin(q.hist + 2048, nb, r1, wsum, &found[1], &rem[1]);
+    for (int b = threadIdx.x; b < 2 * 2048; b += blockDim.x) q.hist[b] = 0;
     if (threadIdx.x == 0) {
-        st->prefix[0] = st->prefix[1] = 0;
-        st->known_mask = 0;
-        st->rank[0] = (m - 1) / 2;
-        st->rank[1] = m / 2;
+        st->lo = lo;
+        st->range = range;
+        st->direct = direct ? 1 : 0;
+        st->bits = bits;
+        st->prefix[0] = p0 | ((uint32_t)found[0] << shift);
+        st->prefix[1] = p1 | ((uint32_t)found[1] << shift);
+        st->known_mask = km | (dm << shift);
+        st->rank[0] = rem[0];
+        st->rank[1] = rem[1];
+        st->ticket = 0;
     }
-}
-
-__global__ void select_init_kernel(SelectState* st, unsigned long long* hist, int n) {
-    select_init_block(st, hist, n);
 }
 
 __device__ __forceinline__ float select_result(const SelectState* st) {
-    const double a = (double)key_float(st->prefix[0]);
-    const double b = (double)key_float(st->prefix[1]);
+    const double a = (double)key_float(st->lo + st->prefix[0]);
+    const double b = (double)key_float(st->lo + st->prefix[1]);
     return (float)(0.5 * (a + b));
+}
+
+__global__ void __launch_bounds__(kSampleThreads) sample_kernel(Select q) { sample_block(q); }
+
+template <bool VEC>
+__global__ void __launch_bounds__(32 * kPassWarps, 4) bracket_kernel(Select q) {
+    bracket_pass<VEC>(q, blockIdx.x, gridDim.x);
+}
+
+template <bool VEC>
+__global__ void __launch_bounds__(256) digit_kernel(Select q, int p) {
+    digit_pass<VEC>(q, p, blockIdx.x, gridDim.x);
 }
 
 __global__ void select_finish_kernel(const SelectState* st, float* pref) {
@@ -414,11 +689,14 @@ __global__ void select_finish_kernel(const SelectState* st, float* pref) {
 }
 
 // ---- 5. diagonal and tie-break noise -----------------------------------------------
-// p(i) from a device vector, a device scalar or a by-value scalar (in that order).
+// p(i) from a device vector, a finished selection (whose result goes to pref)
+// or a by-value scalar (in that order).
 __global__ void diag_kernel(float* S, int n, int64_t lds, const float* __restrict__ pvec,
-                            const float* __restrict__ pdev, float pval) {
+                            const SelectState* __restrict__ st, float* pref, float pval) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) S[(int64_t)i * lds + i] = pvec ? pvec[i] : pdev ? *pdev : pval;
+    const float p = st ? select_result(st) : pval;
+    if (st && i == 0) *pref = p;
+    if (i < n) S[(int64_t)i * lds + i] = pvec ? pvec[i] : p;
 }
 
 __global__ void noise_kernel(float* S, int n, int64_t lds, double rel, uint64_t seed) {
@@ -440,6 +718,7 @@ struct SimWs {
     float* nrm;
     SelectState* sel;
     unsigned long long* hist;
+    uint32_t* cand;
     float* pref;
     int32_t* err;
 };
@@ -452,12 +731,6 @@ static int pad_dim(int d) { return (d + 63) / 64 * 64; }
 // Row blocks of the column means: 256 rows, or more so that there are at most
 // 2048 blocks (the float64 combine of the partials is sequential per column).
 static int64_t mean_rows(int64_t n) { return std::max<int64_t>(kMeanRows, (n + 2047) / 2048); }
-// Histogram blocks of the median: about 64K entries each (a block clears and
-// flushes up to 4096 bins, which one row of a small problem would not repay),
-// at most 4096.
-static int hist_blocks(int n) {
-    return (int)std::max<int64_t>(1, std::min<int64_t>(4096, ((int64_t)n * n + 65535) / 65536));
-}
 static int mean_blocks(int64_t n) { return (int)((n + mean_rows(n) - 1) / mean_rows(n)); }
 
 size_t column_mean_part_doubles(int64_t n, int d) { return (size_t)mean_blocks(n) * (size_t)d; }
@@ -480,25 +753,28 @@ static size_t carve_sim(void* ws, int64_t n, int64_t d, SimWs* w) {
     w->nrm = c.take<float>(npad);
     w->sel = c.take<SelectState>(1);
     w->hist = c.take<unsigned long long>(4096);
+    w->cand = c.take<uint32_t>(cand_cap((int)n));
     w->pref = c.take<float>(1);
     w->err = c.take<int32_t>(1);
     return c.used;
 }
 
-int32_t median_offdiag(const float* S, int n, int64_t lds, SelectState* sel,
-                       unsigned long long* hist, float* pref, cudaStream_t s) {
-    select_init_kernel<<<1, 256, 0, s>>>(sel, hist, n);
-    const int grid = hist_blocks(n);
-    const int shifts[3] = {21, 10, 0}, bits[3] = {11, 11, 10};
+// Enqueues the selection of the two middle order statistics of S's off-diagonal
+// entries; select_result reads them from sel.
+static int32_t median_offdiag(const float* S, int n, int64_t lds, SelectState* sel, unsigned long long* hist,
+                              uint32_t* cand, cudaStream_t s) {
+    const int grid = pass_blocks(n);
+    const int dgrid = digit_blocks(n);
+    const Select q{S, lds, n, 0, grid, 0, dgrid, sel, hist, cand, cand_cap(n), nullptr};
+    const bool vec = aligned16(S) && (lds & 3) == 0;
+    sample_kernel<<<1, kSampleThreads, 0, s>>>(q);
+    if (vec) bracket_kernel<true><<<grid, 32 * kPassWarps, 0, s>>>(q);
+    else bracket_kernel<false><<<grid, 32 * kPassWarps, 0, s>>>(q);
     for (int p = 0; p < 3; ++p) {
-        if (aligned16(S) && (lds & 3) == 0)
-            radix_hist_kernel<true><<<grid, 256, 0, s>>>(S, n, lds, shifts[p], bits[p], sel, hist);
-        else
-            radix_hist_kernel<false><<<grid, 256, 0, s>>>(S, n, lds, shifts[p], bits[p], sel, hist);
-        radix_scan_kernel<<<1, 1024, 0, s>>>(sel, hist, shifts[p], bits[p]);
+        if (vec) digit_kernel<true><<<dgrid, 256, 0, s>>>(q, p);
+        else digit_kernel<false><<<dgrid, 256, 0, s>>>(q, p);
     }
-    select_finish_kernel<<<1, 1, 0, s>>>(sel, pref);
-    note_launches(8);
+    note_launches(5);
     return last_error();
 }
 
@@ -518,14 +794,11 @@ struct SimProblem {
     int nb;                 // column-sum blocks
     int part_b0;            // first column-sum block of the problem in the batched grid
     int centre_b0, centre_nb;
-    int hist_b0, hist_nb;
+    Select sel;             // the median's selection (its blocks in the passes included)
     double* part;
     float* mean;
     void* xc;
     float* nrm;
-    SelectState* sel;
-    unsigned long long* hist;
-    float* pref;
     int64_t roff;           // first row of the problem in the centred-feature arena
 };
 
@@ -569,32 +842,30 @@ __global__ void centre_batched_kernel(const SimProblem* __restrict__ P, int coun
 }
 
 // grid (problems)
-__global__ void select_init_batched_kernel(const SimProblem* __restrict__ P) {
-    const SimProblem& q = P[blockIdx.x];
-    select_init_block(q.sel, q.hist, q.n);
+__global__ void __launch_bounds__(kSampleThreads) sample_batched_kernel(const SimProblem* __restrict__ P) {
+    sample_block(P[blockIdx.x].sel);
 }
 
-// grid (sum of histogram blocks)
+// grid (sum of the problems' pass blocks)
 template <bool VEC>
-__global__ void __launch_bounds__(256) radix_hist_batched_kernel(const SimProblem* __restrict__ P, int count,
-                                                                 int shift, int bits) {
-    const int b = sim_problem_of(P, count, blockIdx.x, [](const SimProblem& q) { return q.hist_b0; });
-    const SimProblem& q = P[b];
-    radix_hist_rows<VEC>(q.S, q.n, q.lds, shift, bits, q.sel, q.hist, blockIdx.x - q.hist_b0, q.hist_nb);
+__global__ void __launch_bounds__(32 * kPassWarps, 4) bracket_batched_kernel(const SimProblem* __restrict__ P, int count) {
+    const int b = sim_problem_of(P, count, blockIdx.x, [](const SimProblem& q) { return q.sel.b0; });
+    const Select q = P[b].sel;
+    bracket_pass<VEC>(q, blockIdx.x - q.b0, q.nb);
 }
 
-// grid (problems), 1024 threads
-__global__ void __launch_bounds__(1024) radix_scan_batched_kernel(const SimProblem* __restrict__ P, int shift,
-                                                                  int bits) {
-    const SimProblem& q = P[blockIdx.x];
-    radix_scan_block(q.sel, q.hist, shift, bits);
+template <bool VEC>
+__global__ void __launch_bounds__(256) digit_batched_kernel(const SimProblem* __restrict__ P, int count, int p) {
+    const int b = sim_problem_of(P, count, blockIdx.x, [](const SimProblem& q) { return q.sel.d0; });
+    const Select q = P[b].sel;
+    digit_pass<VEC>(q, p, blockIdx.x - q.d0, q.dn);
 }
 
 // grid (problems, y); the median (median = 1) or the scalar p onto the diagonal
 __global__ void diag_batched_kernel(const SimProblem* __restrict__ P, int median, float pval) {
     const SimProblem& q = P[blockIdx.x];
-    const float p = median ? select_result(q.sel) : pval;
-    if (median && blockIdx.y == 0 && threadIdx.x == 0) *q.pref = p;
+    const float p = median ? select_result(q.sel.st) : pval;
+    if (median && blockIdx.y == 0 && threadIdx.x == 0) *q.sel.pref = p;
     for (int i = blockIdx.y * blockDim.x + threadIdx.x; i < q.n; i += gridDim.y * blockDim.x)
         q.S[(int64_t)i * q.lds + i] = p;
 }
@@ -639,12 +910,12 @@ static int32_t similarity_enqueue(const float* X, int ni, int di, int64_t ldx, f
                                   err, s));
     }
     if (pref_mode == AP_PREF_MEDIAN) {
-        AP_TRY(median_offdiag(S, ni, lds, w.sel, w.hist, pref_dev, s));
-        diag_kernel<<<(ni + 255) / 256, 256, 0, s>>>(S, ni, lds, nullptr, pref_dev, 0.f);
+        AP_TRY(median_offdiag(S, ni, lds, w.sel, w.hist, w.cand, s));
+        diag_kernel<<<(ni + 255) / 256, 256, 0, s>>>(S, ni, lds, nullptr, w.sel, pref_dev, 0.f);
     } else if (pref_mode == AP_PREF_SCALAR) {
-        diag_kernel<<<(ni + 255) / 256, 256, 0, s>>>(S, ni, lds, nullptr, nullptr, pref[0]);
+        diag_kernel<<<(ni + 255) / 256, 256, 0, s>>>(S, ni, lds, nullptr, nullptr, nullptr, pref[0]);
     } else {
-        diag_kernel<<<(ni + 255) / 256, 256, 0, s>>>(S, ni, lds, pref, nullptr, 0.f);
+        diag_kernel<<<(ni + 255) / 256, 256, 0, s>>>(S, ni, lds, pref, nullptr, nullptr, 0.f);
     }
     if (noise_rel > 0.0) {
         noise_kernel<<<std::min(ni, 8192), 256, 0, s>>>(S, ni, lds, noise_rel, seed);
@@ -737,7 +1008,7 @@ static size_t carve_batched(void* ws, const int64_t* n, int32_t count, int64_t d
     unsigned char* xc_arena = c.take<unsigned char>((size_t)rows * dpad * esz);
     float* nrm_arena = c.take<float>((size_t)rows);
     void* tab = c.take<unsigned char>(tc_grouped_table_bytes(n, count));
-    int part_b0 = 0, centre_b0 = 0, hist_b0 = 0;
+    int part_b0 = 0, centre_b0 = 0, pass_b0 = 0, digit_b0 = 0;
     int64_t roff = 0;
     for (int32_t b = 0; b < count; ++b) {
         SimProblem q{};
@@ -750,18 +1021,24 @@ static size_t carve_batched(void* ws, const int64_t* n, int32_t count, int64_t d
         q.centre_nb = std::min((q.npad + 7) / 8, 65535);
         q.centre_b0 = centre_b0;
         centre_b0 += q.centre_nb;
-        q.hist_nb = hist_blocks(q.n);
-        q.hist_b0 = hist_b0;
-        hist_b0 += q.hist_nb;
+        q.sel.n = q.n;
+        q.sel.nb = pass_blocks(q.n);
+        q.sel.b0 = pass_b0;
+        pass_b0 += q.sel.nb;
+        q.sel.dn = digit_blocks(q.n);
+        q.sel.d0 = digit_b0;
+        digit_b0 += q.sel.dn;
         q.part = c.take<double>((size_t)q.nb * d);
         q.mean = c.take<float>((size_t)d);
         q.roff = roff;
         q.xc = xc_arena ? xc_arena + (size_t)roff * dpad * esz : nullptr;
         q.nrm = nrm_arena ? nrm_arena + roff : nullptr;
         roff += q.npad;
-        q.sel = c.take<SelectState>(1);
-        q.hist = c.take<unsigned long long>(4096);
-        q.pref = pv ? pv + b : nullptr;
+        q.sel.st = c.take<SelectState>(1);
+        q.sel.hist = c.take<unsigned long long>(4096);
+        q.sel.cap = cand_cap(q.n);
+        q.sel.cand = c.take<uint32_t>(q.sel.cap);
+        q.sel.pref = pv ? pv + b : nullptr;
         if (host) (*host)[b] = q;
     }
     if (table) *table = t;
@@ -817,14 +1094,17 @@ APGB_API int32_t ap_similarity_batched(const float* X, const int64_t* xoff, cons
     float* prefs = nullptr;
     void* tables = nullptr;
     carve_batched(ws, n, count, d, precision, &table, &host, &err, &prefs, &tables);
-    int part_blocks = 0, centre_blocks = 0, hist_blocks = 0;
+    int part_blocks = 0, centre_blocks = 0, pass_total = 0, digit_total = 0;
     for (int32_t b = 0; b < count; ++b) {
         host[b].X = X + xoff[b];
         host[b].S = S + soff[b];
         host[b].lds = lds[b];
+        host[b].sel.S = host[b].S;
+        host[b].sel.lds = lds[b];
         part_blocks += host[b].nb;
         centre_blocks += host[b].centre_nb;
-        hist_blocks += host[b].hist_nb;
+        pass_total += host[b].sel.nb;
+        digit_total += host[b].sel.dn;
     }
     const int di = (int)d, dpad = pad_dim(di);
     const bool bf16 = precision != AP_PREC_FP32;
@@ -897,17 +1177,15 @@ APGB_API int32_t ap_similarity_batched(const float* X, const int64_t* xoff, cons
     // 4-5. the preferences and the diagonals
     const int dgy = (int)std::min<int64_t>((nmax + 255) / 256, 65535);
     if (pref_mode == AP_PREF_MEDIAN) {
-        select_init_batched_kernel<<<count, 256, 0, s>>>(table);
-        const int shifts[3] = {21, 10, 0}, bits[3] = {11, 11, 10};
+        sample_batched_kernel<<<count, kSampleThreads, 0, s>>>(table);
+        if (vec) bracket_batched_kernel<true><<<pass_total, 32 * kPassWarps, 0, s>>>(table, count);
+        else bracket_batched_kernel<false><<<pass_total, 32 * kPassWarps, 0, s>>>(table, count);
         for (int p = 0; p < 3; ++p) {
-            if (vec)
-                radix_hist_batched_kernel<true><<<hist_blocks, 256, 0, s>>>(table, count, shifts[p], bits[p]);
-            else
-                radix_hist_batched_kernel<false><<<hist_blocks, 256, 0, s>>>(table, count, shifts[p], bits[p]);
-            radix_scan_batched_kernel<<<count, 1024, 0, s>>>(table, shifts[p], bits[p]);
+            if (vec) digit_batched_kernel<true><<<digit_total, 256, 0, s>>>(table, count, p);
+            else digit_batched_kernel<false><<<digit_total, 256, 0, s>>>(table, count, p);
         }
         diag_batched_kernel<<<dim3(count, dgy), 256, 0, s>>>(table, 1, 0.f);
-        note_launches(8);
+        note_launches(6);
     } else {
         diag_batched_kernel<<<dim3(count, dgy), 256, 0, s>>>(table, 0, pref[0]);
         note_launches(1);
@@ -927,10 +1205,11 @@ APGB_API int32_t ap_similarity_batched(const float* X, const int64_t* xoff, cons
 }
 
 APGB_API size_t ap_preference_median_workspace_size(int64_t n) {
-    if (n < 2) return 0;
+    if (n < 2 || n > INT_MAX / 2) return 0;
     Carver c(nullptr);
     c.take<SelectState>(1);
     c.take<unsigned long long>(4096);
+    c.take<uint32_t>(cand_cap((int)n));
     c.take<float>(1);
     return c.used;
 }
@@ -944,8 +1223,12 @@ APGB_API int32_t ap_preference_median(const float* S, int64_t n, int64_t ld, flo
     Carver c(ws);
     SelectState* sel = c.take<SelectState>(1);
     unsigned long long* hist = c.take<unsigned long long>(4096);
+    uint32_t* cand = c.take<uint32_t>(cand_cap((int)n));
     float* pref = c.take<float>(1);
-    AP_TRY(median_offdiag(S, (int)n, ld, sel, hist, pref, s));
+    AP_TRY(median_offdiag(S, (int)n, ld, sel, hist, cand, s));
+    select_finish_kernel<<<1, 1, 0, s>>>(sel, pref);
+    note_launches(1);
+    AP_TRY(last_error());
     float v = NAN;
     AP_CUDA_TRY(cudaMemcpyAsync(&v, pref, sizeof(float), cudaMemcpyDeviceToHost, s));
     AP_CUDA_TRY(cudaStreamSynchronize(s));

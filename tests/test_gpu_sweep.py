@@ -376,6 +376,28 @@ def test_preference_median_exact():
         assert got == np.float32(oap.offdiag_median(S))
 
 
+@pytest.mark.parametrize("ld_pad", [0, 1])
+@pytest.mark.parametrize("kind", ["spread", "equal", "two", "steps", "half", "wide", "outliers"])
+@pytest.mark.parametrize("n", [2, 5, 130, 1001, 2048])
+def test_preference_median_of_awkward_distributions(n, kind, ld_pad):
+    """The selection is exact whatever the entries: a mass of equal entries
+    that overflows the candidate buffer or holds the median, two values, a
+    value whose share is just about half, positive and negative entries over
+    60 decades, a few extreme ones; rows 16-byte aligned or not."""
+    g = np.random.default_rng(n)
+    u = g.random((n, n))
+    S = {"spread": lambda: -u * 7,
+         "equal": lambda: np.full((n, n), -2.5),
+         "two": lambda: np.where(u < 0.5, -1.0, -2.0),
+         "steps": lambda: -np.floor(u * 9),
+         "half": lambda: np.where(u < 0.4999, -1.0, -1.0 - u),
+         "wide": lambda: np.where(g.random((n, n)) < 0.5, 1, -1) * 10.0 ** g.uniform(-30, 30, (n, n)),
+         "outliers": lambda: np.where(u < 0.001, -1e30, -u)}[kind]()
+    S = S.astype(np.float32).astype(np.float64)
+    got = capi.ap_preference_median(dev_square(S, capi.padded_ld(n) + ld_pad))
+    assert got == np.float32(oap.offdiag_median(S))
+
+
 def test_tiebreak_noise_uses_the_counter_generator():
     X, _ = synth.gaussian_mixture_2d(per_cluster=30)
     Sd, p = capi.ap_similarity(torch.from_numpy(X).cuda(), precision="fp32",
