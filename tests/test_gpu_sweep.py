@@ -367,6 +367,22 @@ def test_similarity_fp32_matches_oracle(wl):
     assert (np.diag(S) == np.float32(p)).all()
 
 
+@pytest.mark.parametrize("d", [1, 8, 9, 24, 65])
+@pytest.mark.parametrize("n", [2, 127, 129, 258, 385])
+def test_similarity_fp32_mirrored_tiles(n, d):
+    """The float32 product at the edges of its 128-point tiles and 8- and
+    16-feature steps: below the diagonal every value is its mirror image up to
+    the order in which the two norms are subtracted."""
+    g = np.random.default_rng(100 * n + d)
+    X = g.normal(size=(n, d)).astype(np.float32)
+    S = host(capi.ap_similarity(torch.from_numpy(X).cuda(), precision="fp32", pref=-1.0)[0])
+    So = oap.build_similarity(X, pref=-1.0)[0]
+    assert (np.abs(S - So) <= _sim_bound(X)).all()
+    scale = np.abs(So).max() + 4 * (X.astype(np.float64) ** 2).sum(1).max()
+    assert np.abs(S - S.T).max() <= 2.0 ** -22 * scale
+    assert (np.diag(S) == -1.0).all()
+
+
 def test_preference_median_exact():
     for n in (2, 3, 100, 1001):
         g = np.random.default_rng(n)
