@@ -103,3 +103,26 @@ def test_bf16_and_fp32_paths_give_same_exemplars():
         res[prec] = (idx.cpu().numpy(), ex["netsim"])
     assert np.array_equal(res["fp32"][0], res["bf16"][0])
     assert abs(res["fp32"][1] - res["bf16"][1]) <= 1e-3 * abs(res["fp32"][1])
+
+
+@pytest.mark.parametrize("d", [3, 64, 200])
+@pytest.mark.parametrize("n", [2, 5, 127, 128, 129, 255, 257, 385, 513, 770])
+def test_similarity_bf16_mirrored_tiles(n, d):
+    """The bf16 product at the edges of its 128 x 256 tiles, against float64 on
+    the bf16-rounded centred features: entries above and below the diagonal
+    alike, padding columns untouched.  Bound: 64-bit sums of exact products
+    against float32 accumulation, (d + 4) 2^-23 of the norms."""
+    g = np.random.default_rng(1000 * n + d)
+    X = g.normal(size=(n, d)).astype(np.float32)
+    Xd = torch.from_numpy(X).cuda()
+    ld = capi.padded_ld(n) + 4
+    base = torch.full((n, ld), float("nan"), dtype=torch.float32, device="cuda")
+    S, p = capi.ap_similarity(Xd, base[:, :n], precision="bf16")
+    B = (Xd - Xd.double().mean(0).float()).to(torch.bfloat16).double()
+    nrm = (B * B).sum(1)
+    want = (2 * (B @ B.T) - nrm[:, None] - nrm[None, :]).clamp(max=0)
+    off = ~torch.eye(n, dtype=torch.bool, device="cuda")
+    bound = (d + 4) * 2.0 ** -23 * (nrm[:, None] + nrm[None, :])
+    assert bool(((S.double() - want).abs() <= bound)[off].all())
+    assert p == float(np.float32(np.median(S[off].double().cpu().numpy())))
+    assert torch.isnan(base[:, n:]).all()
