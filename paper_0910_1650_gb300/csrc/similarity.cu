@@ -37,67 +37,112 @@ int32_t tc_similarity_bf16_grouped(const __nv_bfloat16* Xb, const float* nrm, in
 size_t tc_similarity_pad_rows();
 
 // ---- 1. column means -----------------------------------------------------------
-// Column sums of X in float64 over blocks of `rows` rows.  Block: 32
-// columns x 8 row lanes; lane y sums rows y, y+8, ... of the row block, and
-// the 8 lane sums are added in a fixed tree (deterministic).  Grid:
-// (ceil(d/32), ceil(n/rows)).  part[row block][j].
+// Column sums of X over blocks of `rows` rows, bound by reading X.  Block: 32
+// column lanes x 8 row lanes; row lane y sums rows y, y+8, ... of the row
+// block, and the 8 lane sums are added in a fixed tree (deterministic).  VEC
+// (X 16-byte aligned, ldx % 4 == 0): a column lane owns four columns and reads
+// 16 bytes a row (10^6 x 128: 90 us where 4-byte loads took 119 us); else
+// one.  A column's sum is the same bits either way.  Grid: (ceil(d / 32 or
+// 128), ceil(n/rows)).  part[row block][j].
 constexpr int kMeanRows = 256;
 
-// One block of the column sums: columns bx*32 .. bx*32+31, row block by.
+// One block of the column sums: column group bx, row block by.
+template <bool VEC>
 __device__ __forceinline__ void colsum_block(const float* __restrict__ X, int64_t n, int d, int64_t ldx,
                                              int64_t rows, double* part, int bx, int by) {
+    constexpr int W = VEC ? 4 : 1;
     const int cx = threadIdx.x & 31, ry = threadIdx.x >> 5;
-    const int j = bx * 32 + cx;
+    const int j = (bx * 32 + cx) * W;
     const int64_t r0 = (int64_t)by * rows;
     const int64_t r1 = min(n, r0 + rows);
-    __shared__ double ps[8][32];
+    __shared__ double ps[8][32 * W];
     // Neumaier-compensated float32 sum of the lane's rows (float64 arithmetic is
     // scarce on this part); (s, c) carries the sum to well below float32 rounding
-    float sm = 0.f, cm = 0.f;
-    if (j < d) {
+    float sm[W], cm[W];
+#pragma unroll
+    for (int e = 0; e < W; ++e) sm[e] = cm[e] = 0.f;
+    auto add = [&](int e, float x) {
+        const float t = sm[e] + x;
+        cm[e] += (fabsf(sm[e]) >= fabsf(x)) ? (sm[e] - t) + x : (x - t) + sm[e];
+        sm[e] = t;
+    };
+    if (VEC && j + 3 < d) {
 #pragma unroll 8
         for (int64_t i = r0 + ry; i < r1; i += 8) {
-            const float x = X[i * ldx + j];
-            const float t = sm + x;
-            cm += (fabsf(sm) >= fabsf(x)) ? (sm - t) + x : (x - t) + sm;
-            sm = t;
+            const float4 x = __ldg(reinterpret_cast<const float4*>(X + i * ldx + j));
+            add(0, x.x);
+            add(W > 1 ? 1 : 0, x.y);
+            add(W > 2 ? 2 : 0, x.z);
+            add(W > 3 ? 3 : 0, x.w);
+        }
+    } else if (j < d) {
+        for (int e = 0; e < W && j + e < d; ++e) {
+            float s1 = 0.f, c1 = 0.f;
+#pragma unroll 8
+            for (int64_t i = r0 + ry; i < r1; i += 8) {
+                const float x = X[i * ldx + j + e];
+                const float t = s1 + x;
+                c1 += (fabsf(s1) >= fabsf(x)) ? (s1 - t) + x : (x - t) + s1;
+                s1 = t;
+            }
+#pragma unroll
+            for (int q = 0; q < W; ++q)
+                if (q == e) { sm[q] = s1; cm[q] = c1; }
         }
     }
-    ps[ry][cx] = (double)sm + (double)cm;
+#pragma unroll
+    for (int e = 0; e < W; ++e) ps[ry][cx * W + e] = (double)sm[e] + (double)cm[e];
     __syncthreads();
-    if (ry == 0 && j < d)
-        part[(int64_t)by * d + j] = ((ps[0][cx] + ps[1][cx]) + (ps[2][cx] + ps[3][cx])) +
-                                    ((ps[4][cx] + ps[5][cx]) + (ps[6][cx] + ps[7][cx]));
+    for (int c = threadIdx.x; c < 32 * W; c += blockDim.x) {
+        const int k = bx * 32 * W + c;
+        if (k < d)
+            part[(int64_t)by * d + k] = ((ps[0][c] + ps[1][c]) + (ps[2][c] + ps[3][c])) +
+                                        ((ps[4][c] + ps[5][c]) + (ps[6][c] + ps[7][c]));
+    }
 }
 
+template <bool VEC>
 __global__ void __launch_bounds__(256) colsum_partial_kernel(const float* __restrict__ X, int64_t n, int d,
                                                              int64_t ldx, int64_t rows, double* part) {
-    colsum_block(X, n, d, ldx, rows, part, blockIdx.x, blockIdx.y);
+    colsum_block<VEC>(X, n, d, ldx, rows, part, blockIdx.x, blockIdx.y);
 }
 
-// The means from the row blocks' sums: columns bx*32 .. bx*32+31, in the
-// layout of colsum_block (32 columns x 8 lanes; lane y adds blocks y, y+8,
-// ... in order, then the 8 lane sums meet in the same fixed tree), so the
-// float64 chain per thread is nb/8 long (float64 is scarce on this part).
+// The means from the row blocks' sums: 256 threads on LANES row lanes x 256 /
+// LANES columns; lane y adds blocks y, y + LANES, ... in order, then the lane
+// sums meet in a fixed tree.  Bound by float64 adds, of which an SM makes two
+// a clock: 32 lanes x 8 columns spread many blocks (nb > 64) over 4 times the
+// SMs that 8 x 32 reach (2048 blocks, d = 128: 15 us where 8 x 32 took 37 us).
+template <int LANES>
 __device__ __forceinline__ void colmean_block(const double* __restrict__ part, int nb, int d, int64_t n,
                                               float* mean, int bx) {
-    const int cx = threadIdx.x & 31, ry = threadIdx.x >> 5;
-    const int j = bx * 32 + cx;
-    __shared__ double ps[8][32];
+    constexpr int COLS = 256 / LANES;
+    const int cx = threadIdx.x % COLS, ry = threadIdx.x / COLS;
+    const int j = bx * COLS + cx;
+    __shared__ double ps[LANES][COLS];
     double sm = 0.0;
-    if (j < d)
-        for (int b = ry; b < nb; b += 8) sm += part[(int64_t)b * d + j];
+    if (j < d) {
+#pragma unroll 8
+        for (int b = ry; b < nb; b += LANES) sm += part[(int64_t)b * d + j];
+    }
     ps[ry][cx] = sm;
     __syncthreads();
-    if (ry == 0 && j < d)
-        mean[j] = (float)((((ps[0][cx] + ps[1][cx]) + (ps[2][cx] + ps[3][cx])) +
-                           ((ps[4][cx] + ps[5][cx]) + (ps[6][cx] + ps[7][cx]))) / (double)n);
+    if (ry == 0 && j < d) {
+        double v[LANES];
+#pragma unroll
+        for (int l = 0; l < LANES; ++l) v[l] = ps[l][cx];
+#pragma unroll
+        for (int w = LANES / 2; w > 0; w >>= 1)
+#pragma unroll
+            for (int e = 0; e < w; ++e) v[e] = v[2 * e] + v[2 * e + 1];
+        mean[j] = (float)(v[0] / (double)n);
+    }
 }
 
-// grid ceil(d/32), 256 threads
+// grid ceil(d / (256 / LANES)), 256 threads
+template <int LANES>
 __global__ void __launch_bounds__(256) colmean_kernel(const double* __restrict__ part, int nb, int d,
                                                       int64_t n, float* mean) {
-    colmean_block(part, nb, d, n, mean, blockIdx.x);
+    colmean_block<LANES>(part, nb, d, n, mean, blockIdx.x);
 }
 
 // ---- 2. centring, norms -----------------------------------------------------------
@@ -814,8 +859,12 @@ size_t column_mean_part_doubles(int64_t n, int d) { return (size_t)mean_blocks(n
 int32_t column_means(const float* X, int64_t n, int d, int64_t ldx, double* part, float* mean,
                      cudaStream_t s) {
     const int nb = mean_blocks(n);
-    colsum_partial_kernel<<<dim3((d + 31) / 32, nb), 256, 0, s>>>(X, n, d, ldx, mean_rows(n), part);
-    colmean_kernel<<<(d + 31) / 32, 256, 0, s>>>(part, nb, d, n, mean);
+    if (aligned16(X) && (ldx & 3) == 0)
+        colsum_partial_kernel<true><<<dim3((d + 127) / 128, nb), 256, 0, s>>>(X, n, d, ldx, mean_rows(n), part);
+    else
+        colsum_partial_kernel<false><<<dim3((d + 31) / 32, nb), 256, 0, s>>>(X, n, d, ldx, mean_rows(n), part);
+    if (nb > 64) colmean_kernel<32><<<(d + 7) / 8, 256, 0, s>>>(part, nb, d, n, mean);
+    else colmean_kernel<8><<<(d + 31) / 32, 256, 0, s>>>(part, nb, d, n, mean);
     note_launches(2);
     return last_error();
 }
@@ -889,18 +938,26 @@ __device__ __forceinline__ int sim_problem_of(const SimProblem* P, int count, in
     return lo;
 }
 
-// grid (sum of column-sum blocks, ceil(d/32))
+// grid (sum of column-sum blocks, ceil(d / 32, or 128 for VEC))
+template <bool VEC>
 __global__ void __launch_bounds__(256) colsum_batched_kernel(const SimProblem* __restrict__ P, int count,
                                                              int d, int64_t ldx) {
     const int b = sim_problem_of(P, count, blockIdx.x, [](const SimProblem& q) { return q.part_b0; });
     const SimProblem& q = P[b];
-    colsum_block(q.X, q.n, d, ldx, q.mrows, q.part, blockIdx.y, blockIdx.x - q.part_b0);
+    colsum_block<VEC>(q.X, q.n, d, ldx, q.mrows, q.part, blockIdx.y, blockIdx.x - q.part_b0);
 }
 
 // grid (problems, ceil(d/32)), 256 threads
 __global__ void __launch_bounds__(256) colmean_batched_kernel(const SimProblem* __restrict__ P, int d) {
     const SimProblem& q = P[blockIdx.x];
-    colmean_block(q.part, q.nb, d, q.n, q.mean, blockIdx.y);
+    if (q.nb > 64) {                        // the sums of colmean_kernel<32>: 8 columns at a time
+        for (int t = 0; t < 4; ++t) {
+            colmean_block<32>(q.part, q.nb, d, q.n, q.mean, 4 * blockIdx.y + t);
+            __syncthreads();
+        }
+    } else {
+        colmean_block<8>(q.part, q.nb, d, q.n, q.mean, blockIdx.y);
+    }
 }
 
 // grid (sum of centring blocks)
@@ -1186,10 +1243,11 @@ APGB_API int32_t ap_similarity_batched(const float* X, const int64_t* xoff, cons
     AP_CUDA_TRY(cudaMemcpyAsync(table, host.data(), sizeof(SimProblem) * count, cudaMemcpyHostToDevice, s));
     AP_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(int32_t) * count, s));
     // 1-2. column means and the centred copies of every problem
-    colsum_batched_kernel<<<dim3(part_blocks, (di + 31) / 32), 256, 0, s>>>(table, count, di, ldx);
-    colmean_batched_kernel<<<dim3(count, (di + 31) / 32), 256, 0, s>>>(table, di);
     bool vx = (ldx & 3) == 0;
     for (int32_t b = 0; b < count; ++b) vx = vx && aligned16(X + xoff[b]);
+    if (vx) colsum_batched_kernel<true><<<dim3(part_blocks, (di + 127) / 128), 256, 0, s>>>(table, count, di, ldx);
+    else colsum_batched_kernel<false><<<dim3(part_blocks, (di + 31) / 32), 256, 0, s>>>(table, count, di, ldx);
+    colmean_batched_kernel<<<dim3(count, (di + 31) / 32), 256, 0, s>>>(table, di);
     if (bf16) {
         if (vx) centre_batched_kernel<true, true><<<centre_blocks, 256, 0, s>>>(table, count, di, ldx, dpad);
         else centre_batched_kernel<true, false><<<centre_blocks, 256, 0, s>>>(table, count, di, ldx, dpad);
