@@ -390,15 +390,18 @@ __device__ __forceinline__ float key_float(uint32_t k) {
 // buffer, starting at the bracket's own highest bit.  Where the bracket missed
 // or the buffer overflowed (a large share of equal entries), the digit passes
 // read S itself from the top bit, so the result is exact either way.  The
-// decision stays on the device.  20000 points (1.6 GB): 445 us, of which the
-// pass is 374, the digits 52 and the sample 18, where three radix passes over
-// S took 1025 us; 1000 points: 62 us where they took 144 us (16 blocks, most of
+// decision stays on the device.  20000 points (1.6 GB): 386 us, of which the
+// pass is 322, the digits 53 and the sample 11, where three radix passes over
+// S took 1025 us; 1000 points: 55 us where they took 144 us (16 blocks, most of
 // the time waiting on shared-memory atomics).
 constexpr int kSampleThreads = 1024;
 constexpr int kSamplePer = 16;          // entries drawn per thread
 constexpr int kSample = kSampleThreads * kSamplePer, kSampleHalfWidth = 288;
 constexpr int kSampleBins = 1024;       // two digits of 10 bits settle the bracket
-constexpr int kChunk = 512;             // buffer entries a warp takes at a time (its hits of one step, at most)
+// Buffer entries a warp takes at a time (more if a step's hits need it): enough
+// that few of its steps wait for the atomic, few enough, where a warp has only
+// a few rows, that the digit passes do not read mostly unused chunk ends.
+__host__ __device__ constexpr int chunk_of(int n) { return n < 4096 ? 128 : 512; }
 constexpr int kPassWarps = 8;           // warps per block of the pass
 
 struct SelectState {
@@ -426,19 +429,37 @@ struct Select {
     float* pref;
 };
 
-// Blocks of the pass over S: about 32K entries each, at most 8 blocks per SM; half
-// of them for the digits of the buffer.
+// Blocks of the pass over S: about 32K entries each, at most 8 per SM; of the
+// digits of the buffer: about 8K of its entries each, at most 4 per SM (a block
+// clears and adds up to 4096 bins).
 static int pass_blocks(int n) {
     return (int)std::max<int64_t>(1, std::min<int64_t>(1216, ((int64_t)n * n + 32767) / 32768));
 }
-static int digit_blocks(int n) { return std::max(1, pass_blocks(n) / 2); }
+static int digit_blocks(int n) {
+    return (int)std::max<int64_t>(1, std::min<int64_t>(608, (int64_t)n * n / (8192 * 28)));
+}
 // A 16th of the entries (the bracket holds 3.5 % on average), and every warp's last chunk.
 static unsigned long long cand_cap(int n) {
-    return (unsigned long long)n * (unsigned long long)n / 16 + (unsigned long long)pass_blocks(n) * kPassWarps * kChunk;
+    return (unsigned long long)n * (unsigned long long)n / 16 +
+           (unsigned long long)std::max(pass_blocks(n), 8) * kPassWarps * 512;
 }
 
-// The bracket of one problem (one block of kSampleThreads): kSample entries at
-// seeded random places off the diagonal, and the keys around the two ranks by
+// The sample: kSample entries of S at seeded random places off the diagonal, read
+// by block bx of gx into the start of the candidate buffer (many blocks: one
+// SM has too few reads in flight for 16384 scattered ones: 3.5 us and 7.7 for the
+// bracket, together 17 when one block did both).
+__device__ __forceinline__ void draw_block(const Select& q, int bx, int gx) {
+    for (int e = bx * blockDim.x + threadIdx.x; e < kSample; e += gx * blockDim.x) {
+        const uint64_t u = splitmix64_at(0x6d656469616eull, (uint64_t)e + 1);
+        const int i = (int)(((u >> 32) * (uint64_t)q.n) >> 32);
+        int k = (int)(((u & 0xffffffffull) * (uint64_t)(q.n - 1)) >> 32);
+        k += k >= i;
+        q.cand[e] = __float_as_uint(__ldg(q.S + (int64_t)i * q.lds + k));
+    }
+}
+
+// The bracket of one problem (one block of kSampleThreads) from the drawn
+// entries: the keys around the two ranks by
 // two radix passes of 10 bits below the sample's own highest differing bit
 // (the digits spread: a fixed top byte would put nearly every entry in one
 // bin, whose shared-memory atomics wait for one another).  What the digits
@@ -454,11 +475,7 @@ __device__ __forceinline__ void sample_block(const Select& q) {
     uint32_t kmin = 0xffffffffu, kmax = 0;
 #pragma unroll
     for (int e = 0; e < kSamplePer; ++e) {
-        const uint64_t u = splitmix64_at(0x6d656469616eull, (uint64_t)(e * kSampleThreads + t) + 1);
-        const int i = (int)(((u >> 32) * (uint64_t)q.n) >> 32);
-        int k = (int)(((u & 0xffffffffull) * (uint64_t)(q.n - 1)) >> 32);
-        k += k >= i;
-        key[e] = float_key(__ldg(q.S + (int64_t)i * q.lds + k));
+        key[e] = float_key(__uint_as_float(q.cand[e * kSampleThreads + t]));
     }
 #pragma unroll
     for (int e = 0; e < kSamplePer; ++e) {
@@ -551,12 +568,26 @@ __device__ __forceinline__ float4 entries4(const float* __restrict__ row, int f,
     }
 }
 
+// One entry of the pass: below the bracket, less grows by 1; not settled by the
+// two comparisons (inside the bracket, a zero or infinity at its edge, NaN),
+// mask grows by bit.  Counts are float32 (exact: at most 16 bits a mask, a row's
+// entries a count), because the additions then go to the FMA pipe and leave the
+// half-rate ALU pipe to the comparisons.
+__device__ __forceinline__ void look(float v, float lo, float hi, float bit, float& less, float& mask) {
+    asm("{\n\t.reg .pred p, r;\n\t"
+        "setp.lt.f32 p, %2, %3;\n\t"
+        "setp.gt.or.f32 r, %2, %4, p;\n\t"
+        "@p add.f32 %0, %0, 0f3F800000;\n\t"
+        "@!r add.f32 %1, %1, %5;\n\t}"
+        : "+f"(less), "+f"(mask)
+        : "f"(v), "f"(lo), "f"(hi), "f"(bit));
+}
+
 // The pass over S: warps take rows in turn; block bx of gx.  A step is 512
 // entries of a row, 16 per lane: two float comparisons each settle all but
-// the bracket's own; these (3.5 %) are looked at again as keys, so that NaN
-// and signed zeros fall where their keys do, and written behind one another
-// by a scan of the lanes' counts.  About 9 instructions an entry, so the pass
-// runs at the rate S can be read.
+// the bracket's own; these (3.5 %) are read again as keys, so that NaN and
+// signed zeros fall where their keys do, and written behind one another by a
+// scan of the lanes' counts.
 template <bool VEC>
 __device__ __forceinline__ void bracket_pass(const Select& q, int bx, int gx) {
     const int lane = threadIdx.x & 31;
@@ -567,9 +598,11 @@ __device__ __forceinline__ void bracket_pass(const Select& q, int bx, int gx) {
     // the warp's current chunk of the buffer: entries [at, end)
     unsigned long long at = 0, end = 0;
     bool full = false;
+    const int chunk = chunk_of(n);
     for (int i = bx * kPassWarps + (threadIdx.x >> 5); i < n; i += gx * kPassWarps) {
         const float* row = q.S + (int64_t)i * q.lds;
         const int fi = i >> 2;
+        float fless = 0.f;
         for (int f0 = 0; f0 < n4; f0 += 128) {
             float4 x[4];
 #pragma unroll
@@ -577,7 +610,7 @@ __device__ __forceinline__ void bracket_pass(const Select& q, int bx, int gx) {
                 const int f = f0 + 32 * u + lane;
                 x[u] = f < n4 ? entries4<VEC>(row, f, n) : make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
             }
-            unsigned mask = 0;
+            float fmask = 0.f;
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int f = f0 + 32 * u + lane;
@@ -589,23 +622,11 @@ __device__ __forceinline__ void bracket_pass(const Select& q, int bx, int gx) {
                         if (4 * f + e == i || 4 * f + e >= n) v[e] = INFINITY;
                 }
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const bool below = v[e] < flo;
-                    less += below;
-                    if (!below && !(v[e] > fhi)) mask |= 1u << (4 * u + e);
-                }
+                for (int e = 0; e < 4; ++e) look(v[e], flo, fhi, (float)(1 << (4 * u + e)), fless, fmask);
             }
+            unsigned mask = (unsigned)fmask;
             if (!__any_sync(0xffffffffu, mask != 0)) continue;
-            // the candidates again, as keys
-            unsigned keep = 0;
-            for (unsigned m = mask; m; m &= m - 1) {
-                const int b = __ffs((int)m) - 1, k = 4 * (f0 + 32 * (b >> 2) + lane) + (b & 3);
-                if (k == i || k >= n) continue;
-                const uint32_t key = float_key(__ldg(row + k));
-                if (key - lo <= range) keep |= 1u << b;
-                else less += key < lo;
-            }
-            const int own = __popc(keep);
+            const int own = __popc(mask);
             int incl = own;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
@@ -613,31 +634,41 @@ __device__ __forceinline__ void bracket_pass(const Select& q, int bx, int gx) {
                 if (lane >= o) incl += y;
             }
             const int total = __shfl_sync(0xffffffffu, incl, 31);
-            inside += total;
-            if (full || total == 0) continue;
-            unsigned long long pos = at + (incl - own), fresh = 0;
-            if (at + total > end) {                         // the entries past `end` open a new chunk
-                if (lane == 0) fresh = atomicAdd(&q.st->slots, (unsigned long long)kChunk);
+            unsigned long long pos = at + (incl - own), fresh = 0, take = 0;
+            if (!full && at + total > end) {                // the entries past `end` open a new chunk
+                // (a multiple of 4: the digit passes read 16 bytes at a time)
+                take = max((unsigned long long)chunk, (at + total - end + 3) & ~3ull);
+                if (lane == 0) fresh = atomicAdd(&q.st->slots, take);
                 fresh = __shfl_sync(0xffffffffu, fresh, 0);
-                if (fresh + kChunk > q.cap) {
-                    full = true;                            // the digit passes will read S
-                    continue;
+                full = fresh + take > q.cap;                // then the digit passes will read S
+            }
+            for (; mask; mask &= mask - 1, ++pos) {
+                const int b = __ffs((int)mask) - 1, k = 4 * (f0 + 32 * (b >> 2) + lane) + (b & 3);
+                uint32_t rel = 0xffffffffu;                 // beyond every range: does not count
+                if (k != i && k < n) {
+                    const uint32_t key = float_key(__ldg(row + k));
+                    less += key < lo;
+                    if (key - lo <= range) {
+                        rel = key - lo;
+                        ++inside;
+                    }
                 }
+                if (!full) q.cand[pos < end ? pos : fresh + (pos - end)] = rel;
             }
-            for (unsigned m = keep; m; m &= m - 1, ++pos) {
-                const int b = __ffs((int)m) - 1, k = 4 * (f0 + 32 * (b >> 2) + lane) + (b & 3);
-                q.cand[pos < end ? pos : fresh + (pos - end)] = float_key(__ldg(row + k)) - lo;
-            }
+            if (full) continue;
             if (at + total > end) {
                 at = fresh + (at + total - end);
-                end = fresh + kChunk;
+                end = fresh + take;
             } else {
                 at += total;
             }
         }
+        less += (unsigned)fless;
     }
-    for (unsigned long long x = at + lane; x < end; x += 32) q.cand[x] = 0xffffffffu;   // beyond every range
+    if (!full)
+        for (unsigned long long x = at + lane; x < end; x += 32) q.cand[x] = 0xffffffffu;
     less = __reduce_add_sync(0xffffffffu, less);
+    inside = __reduce_add_sync(0xffffffffu, inside);
     if (lane == 0) {
         if (less) atomicAdd(&q.st->less, (unsigned long long)less);
         if (inside) atomicAdd(&q.st->inside, (unsigned long long)inside);
@@ -724,7 +755,7 @@ __device__ __forceinline__ void digit_pass(const Select& q, int p, int bx, int g
     };
     if (!direct) {
         const unsigned long long slots = st->slots;
-        const uint4* c4 = reinterpret_cast<const uint4*>(q.cand);      // slots is a multiple of kChunk
+        const uint4* c4 = reinterpret_cast<const uint4*>(q.cand);
         const unsigned long long n4 = slots / 4, step = (unsigned long long)gx * blockDim.x;
         for (unsigned long long x0 = (unsigned long long)bx * blockDim.x + threadIdx.x; x0 < n4; x0 += 4 * step) {
             uint4 v[4];                     // four loads in flight before the first count
@@ -793,6 +824,10 @@ __device__ __forceinline__ float select_result(const SelectState* st) {
     return (float)(0.5 * (a + b));
 }
 
+constexpr int kDrawBlocks = 64;
+
+__global__ void __launch_bounds__(256) draw_kernel(Select q) { draw_block(q, blockIdx.x, gridDim.x); }
+
 __global__ void __launch_bounds__(kSampleThreads) sample_kernel(Select q) { sample_block(q); }
 
 template <bool VEC>
@@ -813,11 +848,12 @@ __global__ void select_finish_kernel(const SelectState* st, float* pref) {
 // p(i) from a device vector, a finished selection (whose result goes to pref)
 // or a by-value scalar (in that order).
 __global__ void diag_kernel(float* S, int n, int64_t lds, const float* __restrict__ pvec,
-                            const SelectState* __restrict__ st, float* pref, float pval) {
+                            const SelectState* __restrict__ st, float* pref, float pval, float zero) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const float p = st ? select_result(st) : pval;
     if (st && i == 0) *pref = p;
-    if (i < n) S[(int64_t)i * lds + i] = pvec ? pvec[i] : p;
+    // zero: -0 (p as it is) or +0 (a preference of -0 becomes +0, as the noise makes it)
+    if (i < n) S[(int64_t)i * lds + i] = (pvec ? pvec[i] : p) + zero;
 }
 
 __global__ void noise_kernel(float* S, int n, int64_t lds, double rel, uint64_t seed) {
@@ -851,18 +887,22 @@ static int pad_rows(int n) {
 static int pad_dim(int d) { return (d + 63) / 64 * 64; }
 // Row blocks of the column means: 256 rows, or more so that there are at most
 // 2048 blocks (the float64 combine of the partials is sequential per column).
-static int64_t mean_rows(int64_t n) { return std::max<int64_t>(kMeanRows, (n + 2047) / 2048); }
-static int mean_blocks(int64_t n) { return (int)((n + mean_rows(n) - 1) / mean_rows(n)); }
+static int64_t mean_rows(int64_t n, int64_t d) {
+    // fewer rows where few columns leave most SMs without a block
+    const int64_t spread = (n * ((d + 127) / 128) + 151) / 152;
+    return std::max<int64_t>(std::max<int64_t>(32, std::min<int64_t>(kMeanRows, spread)), (n + 2047) / 2048);
+}
+static int mean_blocks(int64_t n, int64_t d) { return (int)((n + mean_rows(n, d) - 1) / mean_rows(n, d)); }
 
-size_t column_mean_part_doubles(int64_t n, int d) { return (size_t)mean_blocks(n) * (size_t)d; }
+size_t column_mean_part_doubles(int64_t n, int d) { return (size_t)mean_blocks(n, d) * (size_t)d; }
 
 int32_t column_means(const float* X, int64_t n, int d, int64_t ldx, double* part, float* mean,
                      cudaStream_t s) {
-    const int nb = mean_blocks(n);
+    const int nb = mean_blocks(n, d);
     if (aligned16(X) && (ldx & 3) == 0)
-        colsum_partial_kernel<true><<<dim3((d + 127) / 128, nb), 256, 0, s>>>(X, n, d, ldx, mean_rows(n), part);
+        colsum_partial_kernel<true><<<dim3((d + 127) / 128, nb), 256, 0, s>>>(X, n, d, ldx, mean_rows(n, d), part);
     else
-        colsum_partial_kernel<false><<<dim3((d + 31) / 32, nb), 256, 0, s>>>(X, n, d, ldx, mean_rows(n), part);
+        colsum_partial_kernel<false><<<dim3((d + 31) / 32, nb), 256, 0, s>>>(X, n, d, ldx, mean_rows(n, d), part);
     if (nb > 64) colmean_kernel<32><<<(d + 7) / 8, 256, 0, s>>>(part, nb, d, n, mean);
     else colmean_kernel<8><<<(d + 31) / 32, 256, 0, s>>>(part, nb, d, n, mean);
     note_launches(2);
@@ -892,6 +932,7 @@ static int32_t median_offdiag(const float* S, int n, int64_t lds, SelectState* s
     const int dgrid = digit_blocks(n);
     const Select q{S, lds, n, 0, grid, 0, dgrid, sel, hist, cand, cand_cap(n), nullptr};
     const bool vec = aligned16(S) && (lds & 3) == 0;
+    draw_kernel<<<kDrawBlocks, 256, 0, s>>>(q);
     sample_kernel<<<1, kSampleThreads, 0, s>>>(q);
     if (vec) bracket_kernel<true><<<grid, 32 * kPassWarps, 0, s>>>(q);
     else bracket_kernel<false><<<grid, 32 * kPassWarps, 0, s>>>(q);
@@ -899,7 +940,7 @@ static int32_t median_offdiag(const float* S, int n, int64_t lds, SelectState* s
         if (vec) digit_kernel<true><<<dgrid, 256, 0, s>>>(q, p);
         else digit_kernel<false><<<dgrid, 256, 0, s>>>(q, p);
     }
-    note_launches(5);
+    note_launches(6);
     return last_error();
 }
 
@@ -974,6 +1015,11 @@ __global__ void centre_batched_kernel(const SimProblem* __restrict__ P, int coun
                           q.centre_nb);
 }
 
+// grid (problems, blocks of each)
+__global__ void __launch_bounds__(256) draw_batched_kernel(const SimProblem* __restrict__ P) {
+    draw_block(P[blockIdx.x].sel, blockIdx.y, gridDim.y);
+}
+
 // grid (problems)
 __global__ void __launch_bounds__(kSampleThreads) sample_batched_kernel(const SimProblem* __restrict__ P) {
     sample_block(P[blockIdx.x].sel);
@@ -1041,15 +1087,20 @@ static int32_t similarity_enqueue(const float* X, int ni, int di, int64_t ldx, f
         AP_TRY(tc_similarity_bf16(static_cast<const __nv_bfloat16*>(w.xc), w.nrm, ni, dpad, S, lds,
                                   err, s));
     }
+    const float zero = noise_rel > 0.0 ? 0.f : -0.f;
     if (pref_mode == AP_PREF_MEDIAN) {
         AP_TRY(median_offdiag(S, ni, lds, w.sel, w.hist, w.cand, s));
-        diag_kernel<<<(ni + 255) / 256, 256, 0, s>>>(S, ni, lds, nullptr, w.sel, pref_dev, 0.f);
+        diag_kernel<<<(ni + 255) / 256, 256, 0, s>>>(S, ni, lds, nullptr, w.sel, pref_dev, 0.f, zero);
     } else if (pref_mode == AP_PREF_SCALAR) {
-        diag_kernel<<<(ni + 255) / 256, 256, 0, s>>>(S, ni, lds, nullptr, nullptr, nullptr, pref[0]);
+        diag_kernel<<<(ni + 255) / 256, 256, 0, s>>>(S, ni, lds, nullptr, nullptr, nullptr, pref[0], zero);
     } else {
-        diag_kernel<<<(ni + 255) / 256, 256, 0, s>>>(S, ni, lds, pref, nullptr, nullptr, 0.f);
+        diag_kernel<<<(ni + 255) / 256, 256, 0, s>>>(S, ni, lds, pref, nullptr, nullptr, 0.f, zero);
     }
-    if (noise_rel > 0.0) {
+    // s + noise_rel |s| u with u < 1 and noise_rel <= 2^-26 lies within half a
+    // float32 ulp of s (at least 2^-25 |s|), so it rounds to s itself: the pass
+    // (float64 arithmetic on every entry; 14.6 us at 1000 points) would change
+    // nothing but a -0 on the diagonal, which diag_kernel has made +0
+    if (noise_rel > 0x1p-26) {
         noise_kernel<<<std::min(ni, 8192), 256, 0, s>>>(S, ni, lds, noise_rel, seed);
         note_launches(1);
     }
@@ -1146,8 +1197,8 @@ static size_t carve_batched(void* ws, const int64_t* n, int32_t count, int64_t d
         SimProblem q{};
         q.n = (int)n[b];
         q.npad = pad_rows(q.n);
-        q.mrows = mean_rows(n[b]);
-        q.nb = mean_blocks(n[b]);
+        q.mrows = mean_rows(n[b], d);
+        q.nb = mean_blocks(n[b], d);
         q.part_b0 = part_b0;
         part_b0 += q.nb;
         q.centre_nb = std::min((q.npad + 7) / 8, 65535);
@@ -1309,6 +1360,7 @@ APGB_API int32_t ap_similarity_batched(const float* X, const int64_t* xoff, cons
     // 4-5. the preferences and the diagonals
     const int dgy = (int)std::min<int64_t>((nmax + 255) / 256, 65535);
     if (pref_mode == AP_PREF_MEDIAN) {
+        draw_batched_kernel<<<dim3(count, 16), 256, 0, s>>>(table);
         sample_batched_kernel<<<count, kSampleThreads, 0, s>>>(table);
         if (vec) bracket_batched_kernel<true><<<pass_total, 32 * kPassWarps, 0, s>>>(table, count);
         else bracket_batched_kernel<false><<<pass_total, 32 * kPassWarps, 0, s>>>(table, count);
@@ -1317,7 +1369,7 @@ APGB_API int32_t ap_similarity_batched(const float* X, const int64_t* xoff, cons
             else digit_batched_kernel<false><<<digit_total, 256, 0, s>>>(table, count, p);
         }
         diag_batched_kernel<<<dim3(count, dgy), 256, 0, s>>>(table, 1, 0.f);
-        note_launches(6);
+        note_launches(7);
     } else {
         diag_batched_kernel<<<dim3(count, dgy), 256, 0, s>>>(table, 0, pref[0]);
         note_launches(1);

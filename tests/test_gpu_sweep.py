@@ -383,6 +383,18 @@ def test_similarity_fp32_mirrored_tiles(n, d):
     assert (np.diag(S) == -1.0).all()
 
 
+def test_tiebreak_noise_below_half_an_ulp_changes_nothing():
+    """noise_rel <= 2^-26 rounds away on every entry; 2^-23 does not on all."""
+    X, _ = synth.gaussian_mixture_2d(per_cluster=30)
+    Xd = torch.from_numpy(X).cuda()
+    S0, p0 = capi.ap_similarity(Xd, precision="fp32")
+    for rel in (1e-12, 2.0 ** -26):
+        S1, p1 = capi.ap_similarity(Xd, precision="fp32", noise_rel=rel, seed=3)
+        assert torch.equal(S0, S1) and p0 == p1
+    S2, _ = capi.ap_similarity(Xd, precision="fp32", noise_rel=2.0 ** -23, seed=3)
+    assert not torch.equal(S0, S2)
+
+
 def test_preference_median_exact():
     for n in (2, 3, 100, 1001):
         g = np.random.default_rng(n)

@@ -126,3 +126,22 @@ def test_similarity_bf16_mirrored_tiles(n, d):
     assert bool(((S.double() - want).abs() <= bound)[off].all())
     assert p == float(np.float32(np.median(S[off].double().cpu().numpy())))
     assert torch.isnan(base[:, n:]).all()
+
+
+@pytest.mark.parametrize("kind", ["blocks", "equal", "line"])
+def test_similarity_bf16_median_of_clustered_rows(kind):
+    """The median where its neighbourhood is dense in few rows (points sorted by
+    cluster), where most similarities are equal, and for points on a line (a
+    skewed distribution): exact on the matrix made."""
+    g = np.random.default_rng(7)
+    n = 1500
+    if kind == "blocks":
+        X = np.repeat(g.normal(size=(6, 20)) * 9, n // 6, axis=0) + 0.01 * g.normal(size=(n, 20))
+    elif kind == "equal":
+        X = np.tile(np.eye(2, 20), (n // 2, 1))
+    else:
+        X = np.linspace(0, 1, n)[:, None] * np.ones((1, 20))
+    S, p = capi.ap_similarity(torch.from_numpy(X.astype(np.float32)).cuda(), precision="bf16")
+    off = S[~torch.eye(n, dtype=torch.bool, device="cuda")].double().cpu().numpy()
+    assert p == float(np.float32(np.median(off)))
+    assert bool((torch.diagonal(S) == p).all())
