@@ -123,5 +123,15 @@ __device__ __forceinline__ void st_async_b32(uint32_t addr, uint32_t a, uint32_t
         : "memory");
 }
 
+// Programmatic dependent launch: from here on the next kernel of the stream may
+// be scheduled, if its launch allows it; and the wait of such a kernel for every
+// earlier kernel's results (nothing to wait for in an ordinary launch).
+__device__ __forceinline__ void grid_launch_dependents() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void grid_dependency_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 }  // namespace ptx
 }  // namespace apgb

@@ -199,7 +199,7 @@ sweep_kernel(SweepLaunch L) {
     const int csize = (int)cluster.num_blocks();
     const int crank = (int)cluster.block_rank();
     const int gc = blockIdx.x / csize;
-    const int u_begin = L.ubeg[gc], u_end = L.ubeg[gc + 1];
+    ptx::grid_launch_dependents();
     const int T = (int)blockDim.x - 32;         // compute threads
     const int tid = threadIdx.x;
     const int wid = tid >> 5, lid = tid & 31;
@@ -224,6 +224,10 @@ sweep_kernel(SweepLaunch L) {
     }
     __syncthreads();
     if (csize > 1) cluster.sync();              // peers' barriers exist before any st.async
+    // everything above overlaps the previous kernel's end where this launch was
+    // allowed to start early (ptx.cuh); from here on its results are needed
+    ptx::grid_dependency_wait();
+    const int u_begin = L.ubeg[gc], u_end = L.ubeg[gc + 1];
 
     auto sS = [&](int s) { return stage + ((size_t)s * 3 + 0) * w4s; };
     auto sR = [&](int s) { return stage + ((size_t)s * 3 + 1) * w4s; };
@@ -663,6 +667,8 @@ __device__ __forceinline__ void apply_stop_rule(SweepState* st) {
 }
 
 __global__ void __launch_bounds__(kFinCols * kFinLanes) finalize_kernel(const SweepArgs* __restrict__ table) {
+    ptx::grid_launch_dependents();
+    ptx::grid_dependency_wait();
     const SweepArgs& a = table[blockIdx.y];
     const int cx = threadIdx.x % kFinCols, gy = threadIdx.x / kFinCols;
     const int k = blockIdx.x * kFinCols + cx;
@@ -1090,21 +1096,46 @@ static size_t carve_sweep(void* ws, const Problem* P, int count, const Plan& pla
     return cv.used;
 }
 
+// The launches of a chunk alternate sweep and finalize, each needing all of the
+// one before.  `early` lets a launch start while its predecessor drains
+// (programmatic dependent launch): its blocks are scheduled, set up their
+// barriers and wait there, so that launch latency and set-up leave the chain.
+// For one problem only: 5003 points 92.6 -> 91.8 us an iteration, 2021 points
+// about 3 % of a run; the classes of a batch run side by side, and early blocks
+// that wait hold room the other classes could use (48 problems: 3 % slower).
+static void early_launch(cudaLaunchAttribute* a) {
+    a->id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a->val.programmaticStreamSerializationAllowed = 1;
+}
+
+static int32_t launch_finalize(dim3 grid, const SweepArgs* table, cudaStream_t s, bool early) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(kFinCols * kFinLanes, 1, 1);
+    cfg.stream = s;
+    cudaLaunchAttribute attr;
+    early_launch(&attr);
+    cfg.attrs = &attr;
+    cfg.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, finalize_kernel, table) == cudaSuccess ? AP_OK : AP_ERR_CUDA;
+}
+
 static int32_t launch_sweep(const SweepConfig& c, int clusters, const SweepLaunch& L, cudaStream_t s,
-                            bool set_attr = true) {
+                            bool set_attr = true, bool early = false) {
     if (set_attr) AP_TRY(prepare_sweep_fn(c.EPT));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(c.C * clusters, 1, 1);
     cfg.blockDim = dim3(c.T + 32, 1, 1);       // compute warps + the producer warp
     cfg.dynamicSmemBytes = c.smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = c.C;
-    attr.val.clusterDim.y = 1;
-    attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = c.C;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    early_launch(&attr[1]);
+    cfg.attrs = attr;
+    cfg.numAttrs = early ? 2 : 1;
     void* args[] = {const_cast<SweepLaunch*>(&L)};
     const cudaError_t e = cudaLaunchKernelExC(&cfg, sweep_ptr(c.EPT), args);
     return e == cudaSuccess ? AP_OK : AP_ERR_CUDA;
@@ -1146,8 +1177,9 @@ constexpr size_t kMaxGraphs = 32;
 static int32_t enqueue_chunk(const SweepConfig& c, const Plan& plan, const SweepLaunch& L,
                              int64_t m, dim3 fin_grid, cudaStream_t s) {
     for (int64_t j = 0; j < m; ++j) {
-        AP_TRY(launch_sweep(c, plan.clusters, L, s, false));
-        finalize_kernel<<<fin_grid, kFinCols * kFinLanes, 0, s>>>(L.table);
+        // (the first launch of a chunk follows copies and other kernels: no early start)
+        AP_TRY(launch_sweep(c, plan.clusters, L, s, false, L.count == 1 && j > 0));
+        AP_TRY(launch_finalize(fin_grid, L.table, s, L.count == 1));
     }
     return last_error();
 }
@@ -1279,9 +1311,9 @@ static int32_t run_batch(const Problem* P, int count, const ap_params* p, ap_res
         } else {
             for (int64_t j = 0; j < m; ++j) {
                 if (timed) AP_CUDA_TRY(cudaEventRecord(ev.start[j], s));
-                AP_TRY(launch_sweep(c, cur.clusters, L, s));
+                AP_TRY(launch_sweep(c, cur.clusters, L, s, true, !timed && count == 1 && j > 0));
                 if (timed) AP_CUDA_TRY(cudaEventRecord(ev.stop[j], s));
-                finalize_kernel<<<fin_grid, kFinCols * kFinLanes, 0, s>>>(w.table);
+                AP_TRY(launch_finalize(fin_grid, w.table, s, !timed && count == 1));
             }
         }
         note_launches(2 * (uint64_t)m);
