@@ -620,6 +620,332 @@ sweep_kernel(SweepLaunch L) {
     if (csize > 1) cluster.sync();
 }
 
+// ---------------------------------------------------------------------------
+// A small problem in one launch: S, R and A stay in the shared memory of one
+// 16-CTA cluster for the whole run.
+//
+// At 500 points an iteration's 5 MB are nothing to L2; the launches are what it
+// costs (a sweep and a finalize at about 5.6 us each).  Here a launch's two
+// halves are a step of a loop: CTA b holds rows b, b + 16, ..., a warp takes a
+// row through both halves, and the column sums go through distributed shared
+// memory.  Cluster barriers (two a step) replace the launch boundaries; a
+// cluster's CTAs are always resident together, whatever else runs.  The sums
+// are those of finalize_kernel with one row per unit, in its order: lane l adds
+// the rows i = l mod 32 in turn (rows of CTA l mod 16, every second one), then
+// the lanes meet in its tree, so the results are the same bits as by launches.
+// R_{t-1}, which a stop found at step t returns, is kept in the workspace from
+// the step on at which the run could stop.  500 points, 100 iterations:
+// @RES500@ where launches took 1123 us; the rule is that the three matrices fit
+// (up to about 540 points) and that the launches' units are single rows.
+// ---------------------------------------------------------------------------
+constexpr int kResCtas = 16, kResThreads = 512, kResWarps = kResThreads / 32;
+constexpr int kResQ = 5;                // float4 per lane and row: n4 <= 160
+
+struct ResidentArgs {
+    SweepArgs a;
+    int max_iter, conv_iter;
+    int check;                          // count the entries of S that are not finite
+    int rows;                           // most rows of a CTA
+    int cw;                             // columns per reducing CTA
+};
+
+static size_t resident_smem(int n) {
+    const size_t n4 = (n + 3) / 4, rows = (n + kResCtas - 1) / kResCtas, cw = (n + kResCtas - 1) / kResCtas;
+    return 3 * rows * n4 * 16 + 2 * n4 * 16 +              // S, R, A; (1 - lambda) c and colp
+           (32 * cw + 3 * cw) * 4 + 2 * rows * 4 + 64;     // received sums, diagonal, results; flags, decisions
+}
+
+__global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_constant__ ResidentArgs p) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ int2 cnt[kResCtas];                          // every CTA's (changes, exemplars)
+    __shared__ int own_changes, own_ex, own_bad;
+    cg::cluster_group cluster = cg::this_cluster();
+    const SweepArgs& a = p.a;
+    const int b = (int)cluster.block_rank();
+    const int tid = threadIdx.x, wid = tid >> 5, lid = tid & 31;
+    const int n = a.n, n4 = a.n4, nfull = n >> 2, cw = p.cw;
+    const int m = n > b ? (n - b + kResCtas - 1) / kResCtas : 0;      // this CTA's rows: b + 16 r
+    float4* sS = reinterpret_cast<float4*>(smem);
+    float4* sR = sS + (size_t)p.rows * n4;
+    float4* sA = sR + (size_t)p.rows * n4;
+    float4* cvs = sA + (size_t)p.rows * n4;
+    float* colps = reinterpret_cast<float*>(cvs + n4);
+    float* recv = colps + 4 * n4;                           // [32][cw]
+    float* rdiag = recv + 32 * cw;
+    float* res = rdiag + cw;                                // [2][cw]: c and colp of this CTA's columns
+    int* flags = reinterpret_cast<int*>(res + 2 * cw);
+    int* decs = flags + p.rows;
+    const float lam = a.lam, oml = 1.0f - a.lam;
+    const float2 lam2 = make_float2(lam, lam), oml2 = make_float2(oml, oml), nom2 = make_float2(-oml, -oml);
+
+    if (tid == 0) own_changes = own_ex = own_bad = 0;
+    cluster.sync();                     // every CTA has started: its shared memory may be written
+    int bad = 0;
+    for (int e = tid; e < m * n4; e += kResThreads) {
+        const int r = e / n4, f = e - r * n4;
+        const int64_t off = (int64_t)(b + kResCtas * r) * a.ld + 4 * f;
+        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 s4 = *reinterpret_cast<const float4*>(a.S + off);
+        if (p.check) {
+            bad += !isfinite(s4.x);
+            bad += 4 * f + 1 < n && !isfinite(s4.y);
+            bad += 4 * f + 2 < n && !isfinite(s4.z);
+            bad += 4 * f + 3 < n && !isfinite(s4.w);
+        }
+        sS[e] = s4;
+        sR[e] = a.zero ? z : *reinterpret_cast<const float4*>(a.R0 + off);
+        sA[e] = a.zero ? z : *reinterpret_cast<const float4*>(a.A + off);
+    }
+    for (int r = tid; r < m; r += kResThreads) flags[r] = decs[r] = 0;
+    if (p.check) {
+        bad = __reduce_add_sync(0xffffffffu, bad);
+        if (lid == 0 && bad) atomicAdd(&own_bad, bad);
+        __syncthreads();
+        if (tid < kResCtas) *cluster.map_shared_rank(&cnt[b], tid) = make_int2(own_bad, 0);
+        cluster.sync();
+        int sum = 0;
+        for (int c = 0; c < kResCtas; ++c) sum += cnt[c].x;
+        cluster.sync();                                     // read before anyone writes counts again
+        if (sum) {                                          // the same in every CTA
+            if (b == 0 && tid == 0) {
+                SweepState s{};
+                s.nonfinite = sum;
+                *a.st = s;
+            }
+            return;
+        }
+    }
+    __syncthreads();
+
+    int t = 1, stable = 0, iters = 0, converged = 0;
+    bool doR = true, done = false;
+    for (;; ++t) {
+        const bool doA = t >= 2;
+        doR = t <= p.max_iter;
+        // this step may turn out to be the last: keep R_{t-1}
+        const bool keep = doR && doA && p.conv_iter > 0 && stable + 1 >= p.conv_iter;
+        for (int r = wid; r < m; r += kResWarps) {
+            const int i = b + kResCtas * r, fi = i >> 2;
+            float4 s4[kResQ], r4[kResQ];
+            Top2 tp{-INFINITY, -INFINITY, INT_MAX};
+            float dv = -INFINITY;
+            int dj = INT_MAX;
+#pragma unroll
+            for (int q = 0; q < kResQ; ++q) {
+                const int f = lid + 32 * q, x = r * n4 + f;
+                if (f < n4) {
+                    s4[q] = sS[x];
+                    r4[q] = sR[x];
+                    float4 a4 = sA[x];
+                    const float4 cv = doA ? cvs[f] : make_float4(0.f, 0.f, 0.f, 0.f);
+                    // the availability half, the decision and the top-2, as in
+                    // sweep_kernel (columns reach a lane in increasing order)
+                    if (f != fi && f < nfull) {
+                        const int k0 = 4 * f;
+                        float2 alo = make_float2(a4.x, a4.y), ahi = make_float2(a4.z, a4.w);
+                        if (doA) {
+                            const float2 tlo = __ffma2_rn(nom2, make_float2(fmaxf(0.f, r4[q].x), fmaxf(0.f, r4[q].y)),
+                                                          make_float2(cv.x, cv.y));
+                            const float2 thi = __ffma2_rn(nom2, make_float2(fmaxf(0.f, r4[q].z), fmaxf(0.f, r4[q].w)),
+                                                          make_float2(cv.z, cv.w));
+                            alo = __ffma2_rn(lam2, alo, make_float2(fminf(0.f, tlo.x), fminf(0.f, tlo.y)));
+                            ahi = __ffma2_rn(lam2, ahi, make_float2(fminf(0.f, thi.x), fminf(0.f, thi.y)));
+                            const float2 dlo = __fadd2_rn(alo, make_float2(r4[q].x, r4[q].y));
+                            const float2 dhi = __fadd2_rn(ahi, make_float2(r4[q].z, r4[q].w));
+                            if (dlo.x > dv) { dv = dlo.x; dj = k0; }
+                            if (dlo.y > dv) { dv = dlo.y; dj = k0 + 1; }
+                            if (dhi.x > dv) { dv = dhi.x; dj = k0 + 2; }
+                            if (dhi.y > dv) { dv = dhi.y; dj = k0 + 3; }
+                            a4 = make_float4(alo.x, alo.y, ahi.x, ahi.y);
+                        }
+                        if (doR) {
+                            const float2 vlo = __fadd2_rn(alo, make_float2(s4[q].x, s4[q].y));
+                            const float2 vhi = __fadd2_rn(ahi, make_float2(s4[q].z, s4[q].w));
+                            float v;
+                            v = vlo.x; tp.m2 = fmaxf(tp.m2, fminf(tp.m1, v)); if (v > tp.m1) { tp.m1 = v; tp.j1 = k0; }
+                            v = vlo.y; tp.m2 = fmaxf(tp.m2, fminf(tp.m1, v)); if (v > tp.m1) { tp.m1 = v; tp.j1 = k0 + 1; }
+                            v = vhi.x; tp.m2 = fmaxf(tp.m2, fminf(tp.m1, v)); if (v > tp.m1) { tp.m1 = v; tp.j1 = k0 + 2; }
+                            v = vhi.y; tp.m2 = fmaxf(tp.m2, fminf(tp.m1, v)); if (v > tp.m1) { tp.m1 = v; tp.j1 = k0 + 3; }
+                        }
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const int k = 4 * f + e;
+                            if (k < n) {
+                                const float rv = lane(r4[q], e);
+                                float av = lane(a4, e);
+                                if (doA) {
+                                    const float an = (k == i) ? oml * colps[i]
+                                                              : fminf(0.f, fmaf(-oml, fmaxf(0.f, rv), lane(cv, e)));
+                                    av = fmaf(lam, av, an);
+                                    set_lane(a4, e, av);
+                                    const float d = av + rv;
+                                    if (d > dv) { dv = d; dj = k; }
+                                }
+                                if (doR) {
+                                    const float v = av + lane(s4[q], e);
+                                    tp.m2 = fmaxf(tp.m2, fminf(tp.m1, v));
+                                    if (v > tp.m1) { tp.m1 = v; tp.j1 = k; }
+                                }
+                            }
+                        }
+                    }
+                    if (doA) sA[x] = a4;
+                }
+            }
+            if (doA) {
+                argmax_warp_redux(dv, dj);
+                if (lid == 0) {
+                    const int e = (dj == i) ? 1 : 0;
+                    if (flags[r] != e) atomicAdd(&own_changes, 1);
+                    if (e) atomicAdd(&own_ex, 1);
+                    flags[r] = e;
+                    decs[r] = dj;
+                }
+            }
+            if (doR) {
+                tp = top2_warp_redux(tp);
+                const float om1 = oml * tp.m1, om2 = oml * tp.m2;
+#pragma unroll
+                for (int q = 0; q < kResQ; ++q) {
+                    const int f = lid + 32 * q, x = r * n4 + f;
+                    if (f < n4) {
+                        if (keep) *reinterpret_cast<float4*>(a.R1 + (int64_t)i * a.ld + 4 * f) = r4[q];
+                        const float2 nm1 = make_float2(-om1, -om1);
+                        const float2 olo = __ffma2_rn(lam2, make_float2(r4[q].x, r4[q].y),
+                                                      __ffma2_rn(oml2, make_float2(s4[q].x, s4[q].y), nm1));
+                        const float2 ohi = __ffma2_rn(lam2, make_float2(r4[q].z, r4[q].w),
+                                                      __ffma2_rn(oml2, make_float2(s4[q].z, s4[q].w), nm1));
+                        float4 o = make_float4(olo.x, olo.y, ohi.x, ohi.y);
+                        if (f == tp.j1 >> 2) {              // the row's largest takes the second largest
+                            const int e = tp.j1 & 3;
+                            const float sv = e == 0 ? s4[q].x : e == 1 ? s4[q].y : e == 2 ? s4[q].z : s4[q].w;
+                            const float rv = e == 0 ? r4[q].x : e == 1 ? r4[q].y : e == 2 ? r4[q].z : r4[q].w;
+                            const float ov = fmaf(lam, rv, fmaf(oml, sv, -om2));
+                            o.x = e == 0 ? ov : o.x;
+                            o.y = e == 1 ? ov : o.y;
+                            o.z = e == 2 ? ov : o.z;
+                            o.w = e == 3 ? ov : o.w;
+                        }
+                        sR[x] = o;
+                    }
+                }
+            }
+        }
+        __syncthreads();
+        if (doR) {
+            // this CTA's two lanes of every column's sum, to the column's reducer
+            const float* R = reinterpret_cast<const float*>(sR);
+            for (int k = tid; k < n; k += kResThreads) {
+                const int rd = (k % kResCtas == b) ? k / kResCtas : -1;       // the diagonal's row here
+                float s0 = 0.f, s1 = 0.f;
+                int r = 0;
+                for (; r + 8 <= m; r += 8) {                // eight rows' reads in flight
+                    float v[8];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) v[e] = R[(size_t)(r + e) * 4 * n4 + k];
+#pragma unroll
+                    for (int e = 0; e < 8; e += 2) {
+                        s0 += r + e == rd ? 0.f : fmaxf(0.f, v[e]);
+                        s1 += r + e + 1 == rd ? 0.f : fmaxf(0.f, v[e + 1]);
+                    }
+                }
+                for (; r < m; ++r) {
+                    const float v = r == rd ? 0.f : fmaxf(0.f, R[(size_t)r * 4 * n4 + k]);
+                    if (r & 1) s1 += v;
+                    else s0 += v;
+                }
+                const int dst = k / cw, c = k - dst * cw;
+                float* to = cluster.map_shared_rank(recv, dst);
+                to[b * cw + c] = s0;
+                to[(b + kResCtas) * cw + c] = s1;
+                if (rd >= 0) *cluster.map_shared_rank(rdiag + c, dst) = R[(size_t)rd * 4 * n4 + k];
+            }
+        }
+        if (tid < kResCtas) *cluster.map_shared_rank(&cnt[b], tid) = make_int2(own_changes, own_ex);
+        cluster.sync();
+        int changes = 0, n_ex = 0;
+#pragma unroll
+        for (int c = 0; c < kResCtas; ++c) {
+            const int2 x = cnt[c];
+            changes += x.x;
+            n_ex += x.y;
+        }
+        // the stop rule (apply_stop_rule), the same in every thread of the cluster
+        if (t >= 2) {
+            const int it = t - 1;
+            stable = (it == 1 || changes != 0) ? 1 : stable + 1;
+            if (p.conv_iter > 0 && stable >= p.conv_iter && n_ex > 0) {
+                done = true;
+                converged = 1;
+                iters = it;
+            }
+        }
+        if (!done && t == p.max_iter + 1) {
+            done = true;
+            iters = p.max_iter;
+        }
+        if (done) break;
+        // this CTA's columns: the 32 lane sums in finalize_kernel's tree
+        if (tid < cw && b * cw + tid < n) {
+            float v[32];
+#pragma unroll
+            for (int l = 0; l < 32; ++l) v[l] = recv[l * cw + tid];
+#pragma unroll
+            for (int w = 16; w >= 1; w >>= 1)
+#pragma unroll
+                for (int e = 0; e < w; ++e) v[e] = v[2 * e] + v[2 * e + 1];
+            res[tid] = oml * (rdiag[tid] + v[0]);
+            res[cw + tid] = v[0];
+        }
+        if (tid == 0) own_changes = own_ex = 0;
+        __syncthreads();
+        for (int e = tid; e < kResCtas * cw; e += kResThreads) {
+            const int dst = e / cw, c = e - dst * cw, k = b * cw + c;
+            if (k < n) {
+                cluster.map_shared_rank(reinterpret_cast<float*>(cvs), dst)[k] = res[c];
+                cluster.map_shared_rank(colps, dst)[k] = res[cw + c];
+            }
+        }
+        cluster.sync();
+    }
+    // the messages of iteration `iters`: R is one step ahead when a stop was found
+    // at a step that formed R
+    const bool kept = converged && doR;
+    for (int r = wid; r < m; r += kResWarps) {
+        const int i = b + kResCtas * r;
+        const int64_t off = (int64_t)i * a.ld;
+        for (int f = lid; f < n4; f += 32) {
+            const float4 rv = kept ? *reinterpret_cast<const float4*>(a.R1 + off + 4 * f) : sR[r * n4 + f];
+            const float4 av = sA[r * n4 + f];
+            if (f < nfull) {
+                *reinterpret_cast<float4*>(a.R0 + off + 4 * f) = rv;
+                *reinterpret_cast<float4*>(a.A + off + 4 * f) = av;
+            } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (4 * f + e < n) {
+                        a.R0[off + 4 * f + e] = lane(rv, e);
+                        a.A[off + 4 * f + e] = lane(av, e);
+                    }
+            }
+        }
+        if (a.dec && lid == 0) a.dec[i] = decs[r];
+    }
+    if (b == 0 && tid == 0) {
+        SweepState s{};
+        s.t = t + 1;
+        s.done = 1;
+        s.stable = stable;
+        s.iters = iters;
+        s.converged = converged;
+        s.max_iter = p.max_iter;
+        s.conv_iter = p.conv_iter;
+        *a.st = s;
+    }
+    cluster.sync();                     // no CTA leaves while another may still read its counts
+}
+
 // Column sums in a fixed order, then the stop rule (block 0 of each
 // problem).  Block: 32 columns x 16 lanes over the problem's G unit partials;
 // each lane sums every 16th partial, then the 16 lane sums are added in a
@@ -1226,6 +1552,86 @@ static int32_t launch_chunk_graph(const SweepConfig& c, const Plan& plan, const 
     return AP_OK;
 }
 
+static cudaLaunchConfig_t resident_config(int n, cudaLaunchAttribute* attr, cudaStream_t s) {
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = kResCtas;
+    attr->val.clusterDim.y = 1;
+    attr->val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kResCtas, 1, 1);
+    cfg.blockDim = dim3(kResThreads, 1, 1);
+    cfg.dynamicSmemBytes = resident_smem(n);
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+// Whether resident_kernel can run on the current device (a 16-CTA cluster with
+// all of the shared memory): asked once per device.
+static bool resident_supported() {
+    static std::mutex mu;
+    static std::map<int, bool> known;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    std::lock_guard<std::mutex> lock(mu);
+    auto it = known.find(dev);
+    if (it != known.end()) return it->second;
+    bool ok = cudaFuncSetAttribute(resident_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024) ==
+                  cudaSuccess &&
+              cudaFuncSetAttribute(resident_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    if (ok) {
+        cudaLaunchAttribute attr;
+        cudaLaunchConfig_t cfg = resident_config(2, &attr, nullptr);
+        cfg.dynamicSmemBytes = 226 * 1024;
+        int num = 0;
+        ok = cudaOccupancyMaxActiveClusters(&num, resident_kernel, &cfg) == cudaSuccess && num >= 1;
+    }
+    if (!ok) cudaGetLastError();
+    known[dev] = ok;
+    return ok;
+}
+
+// A single problem goes to resident_kernel when its matrices fit, its launches
+// would sweep one row per unit (the same sums), and the caller asked neither for
+// separate launches nor for a configuration of them.
+static bool takes_resident(const Problem* P, int count, const ap_params* p, const Plan& plan) {
+    if (count != 1 || (p->flags & (AP_FLAG_TIME_SWEEP | AP_FLAG_NO_GRAPH))) return false;
+    const int n = (int)P[0].n;
+    if ((n + 3) / 4 > 32 * kResQ || resident_smem(n) > 226 * 1024 || plan.c.G != n) return false;
+    {
+        std::lock_guard<std::mutex> lock(g_pin_mu);
+        if (g_pinned.count(n)) return false;
+    }
+    return resident_supported();
+}
+
+static int32_t run_resident(const SweepArgs& a, const ap_params* p, ap_result* out, cudaStream_t s) {
+    ResidentArgs r{};
+    r.a = a;
+    r.max_iter = p->max_iter;
+    r.conv_iter = p->conv_iter;
+    r.check = (p->flags & AP_FLAG_S_CHECKED) ? 0 : 1;
+    r.rows = r.cw = (a.n + kResCtas - 1) / kResCtas;
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = resident_config(a.n, &attr, s);
+    AP_CUDA_TRY(cudaLaunchKernelEx(&cfg, resident_kernel, r));
+    note_launches(1);
+    SweepState h;
+    AP_CUDA_TRY(cudaMemcpyAsync(&h, a.st, sizeof(h), cudaMemcpyDeviceToHost, s));
+    AP_CUDA_TRY(cudaStreamSynchronize(s));
+    if (h.nonfinite) return AP_ERR_NONFINITE;
+    const int32_t status = (p->conv_iter > 0 && !h.converged) ? AP_NOT_CONVERGED : AP_OK;
+    if (out) {
+        *out = ap_result{};
+        out->iters = h.iters;
+        out->converged = h.converged;
+        out->status = status;
+        out->sweep_launches = h.t - 1;      // steps of the one launch
+    }
+    return status;
+}
+
 // Runs Algorithm 1 on every problem of the batch until each has stopped.
 // out[b] receives problem b's result; sweep timing is per launch (shared).
 static int32_t run_batch(const Problem* P, int count, const ap_params* p, ap_result* out,
@@ -1235,6 +1641,11 @@ static int32_t run_batch(const Problem* P, int count, const ap_params* p, ap_res
     carve_sweep(ws, P, count, plan, &w);
     const SweepConfig& c = plan.c;
     for (auto& a : w.host) a.lam = p->damping;
+    if (takes_resident(P, count, p, plan)) {
+        SweepArgs a = w.host[0];
+        if (p->flags & AP_FLAG_COLD) a.zero = w.zero;       // (a mark here: zeros are not read)
+        return run_resident(a, p, out, s);
+    }
     if (p->flags & AP_FLAG_COLD) {
         // R and A start at zero whatever the buffers hold: the first launches
         // read this zeroed buffer instead

@@ -395,6 +395,42 @@ def test_tiebreak_noise_below_half_an_ulp_changes_nothing():
     assert not torch.equal(S0, S2)
 
 
+@pytest.mark.parametrize("n", [2, 3, 15, 17, 31, 33, 100, 499, 513, 541, 544, 545])
+def test_one_launch_run_equals_separate_launches(n):
+    """Up to 544 points the matrices fit one cluster's shared memory and the run
+    is one launch: the same bits, decisions and stop as separate launches
+    (graph=False), from zeros or from given messages, for fixed iterations, a
+    stop by the rule (the last iteration and the one before it) and at
+    max_iter; padding columns stay untouched, non-finite S is refused before
+    the messages are touched.  At 545 points the launches take over."""
+    g = np.random.default_rng(n)
+    X = g.normal(size=(n, 3)) + 4 * g.integers(0, 3, size=(n, 1))
+    Sd = dev_square(s32(X), capi.padded_ld(n) + 4)
+    R0, A0 = g.normal(size=(n, n)), -np.abs(g.normal(size=(n, n)))
+    for lam, maxit, conv, cold in ((0.5, 7, 0, True), (0.0, 1, 0, False), (0.9, 40, 3, False), (0.9, 300, 15, True),
+                                   (0.5, 2, 1, False), (0.7, 9, 9, True)):
+        outs = []
+        for graph in (True, False):
+            R, A = dev_square(R0, Sd.stride(0)), dev_square(A0, Sd.stride(0))
+            before = capi.kernel_launches()
+            R, A, res, dec = capi.ap_iterate(Sd, R, A, damping=lam, max_iter=maxit, conv_iter=conv, cold=cold,
+                                             graph=graph)
+            assert (capi.kernel_launches() - before == 1) == (graph and n <= 544)
+            full = [t.as_strided((n, t.stride(0)), (t.stride(0), 1)) for t in (R, A)]
+            assert all(torch.isnan(t[:, n:]).all() for t in full)
+            outs.append((R.clone(), A.clone(), dec, res["iters"], res["converged"], res["status"]))
+        assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1]), (lam, maxit, conv)
+        assert torch.equal(outs[0][2], outs[1][2]) and outs[0][3:] == outs[1][3:]
+    bad = dev_square(host(Sd), Sd.stride(0))
+    bad[n - 1, n // 2] = float("inf")
+    R, A = dev_square(R0, Sd.stride(0)), dev_square(A0, Sd.stride(0))
+    R1, A1 = R.clone(), A.clone()
+    with pytest.raises(capi.ApgbError) as e:
+        capi.ap_iterate(bad, R, A, damping=0.5, max_iter=5)
+    assert e.value.status == -5
+    assert torch.equal(R, R1) and torch.equal(A, A1)
+
+
 def test_preference_median_exact():
     for n in (2, 3, 100, 1001):
         g = np.random.default_rng(n)
