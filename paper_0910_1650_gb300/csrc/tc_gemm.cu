@@ -106,6 +106,33 @@ __device__ __forceinline__ void select8(float* r, const float* v, uint32_t take)
         : "r"(take), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]));
 }
 
+// Running arg-max over 32-column chunks: a chunk's maximum by a tree of
+// three-input maxima; where it beats the running best (strictly: chunks arrive
+// in increasing column order, so a tie keeps the earlier chunk) the chunk's
+// scores replace the kept ones by predicated selects.  The column inside the
+// kept chunk is found once per row block (argmax_column).
+__device__ __forceinline__ void argmax_chunk(const float (&sc)[32], int kcol, float& best, int& bchunk,
+                                             float (&keep)[32]) {
+    float t[11];
+#pragma unroll
+    for (int e = 0; e < 10; ++e) t[e] = max3f(sc[3 * e], sc[3 * e + 1], sc[3 * e + 2]);
+    t[10] = fmaxf(sc[30], sc[31]);
+    const float m = fmaxf(max3f(max3f(t[0], t[1], t[2]), max3f(t[3], t[4], t[5]), max3f(t[6], t[7], t[8])),
+                          fmaxf(t[9], t[10]));
+    const uint32_t imp = m > best ? 1u : 0u;
+#pragma unroll
+    for (int h = 0; h < 4; ++h) select8(keep + 8 * h, sc + 8 * h, imp);
+    best = imp ? m : best;
+    bchunk = imp ? kcol : bchunk;
+}
+// The first column of the kept chunk that attains the best.
+__device__ __forceinline__ int argmax_column(float best, int bchunk, const float (&keep)[32]) {
+    int j = 31;
+#pragma unroll
+    for (int e = 30; e >= 0; --e) j = (keep[e] == best) ? e : j;
+    return bchunk + j;
+}
+
 __device__ __forceinline__ bool aborted(const Ctl& c) {
     return *reinterpret_cast<const volatile int*>(&c.abort) != 0;
 }
@@ -265,14 +292,25 @@ __device__ __forceinline__ uint64_t smem_desc(const void* base) {
 //                          float); zero past `ncols`.
 // One K = 16 MMA over block q % 4 of A' and of B' group q / 4 adds -|b|^2/2
 // to every row of column tile q.
-__device__ void build_augmented(uint8_t* aug, const float* bnrm, int ncols, int groups) {
-    auto pack = [](__nv_bfloat16 lo, __nv_bfloat16 hi) -> uint32_t {
-        return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
-    };
+__device__ __forceinline__ uint32_t pack_bf16(__nv_bfloat16 lo, __nv_bfloat16 hi) {
+    return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
+}
+__device__ __forceinline__ uint4 ones_unit() {
     const __nv_bfloat16 one = __float2bfloat16_rn(1.f), zero = __float2bfloat16_rn(0.f);
+    return make_uint4(pack_bf16(one, one), pack_bf16(one, zero), 0, 0);
+}
+__device__ __forceinline__ uint4 norm_unit(float nrm) {
+    const float x = 0.5f * nrm;
+    const __nv_bfloat16 h = __float2bfloat16_rn(x);
+    const float r1 = x - __bfloat162float(h);                // exact
+    const __nv_bfloat16 m = __float2bfloat16_rn(r1);
+    const __nv_bfloat16 l = __float2bfloat16_rn(r1 - __bfloat162float(m));   // exact
+    return make_uint4(pack_bf16(__hneg(h), __hneg(m)), pack_bf16(__hneg(l), __float2bfloat16_rn(0.f)), 0, 0);
+}
+__device__ void build_augmented(uint8_t* aug, const float* bnrm, int ncols, int groups) {
     for (int i = threadIdx.x; i < BM * 8; i += blockDim.x) {
         const int r = i >> 3, c = i & 7;
-        const uint4 v = (c & 1) ? make_uint4(0, 0, 0, 0) : make_uint4(pack(one, one), pack(one, zero), 0, 0);
+        const uint4 v = (c & 1) ? make_uint4(0, 0, 0, 0) : ones_unit();
         *reinterpret_cast<uint4*>(aug + r * 128 + ((c ^ (r & 7)) << 4)) = v;
     }
     uint8_t* bb = aug + A_BYTES;
@@ -280,15 +318,7 @@ __device__ void build_augmented(uint8_t* aug, const float* bnrm, int ncols, int 
         const int k = i & 3, r = (i >> 2) % BN, g = (i >> 2) / BN;
         const int col = g * 4 * BN + k * BN + r;
         uint4 v = make_uint4(0, 0, 0, 0);
-        if (col < ncols) {
-            const float x = 0.5f * __ldg(bnrm + col);
-            const __nv_bfloat16 h = __float2bfloat16_rn(x);
-            const float r1 = x - __bfloat162float(h);                // exact
-            const __nv_bfloat16 m = __float2bfloat16_rn(r1);
-            const __nv_bfloat16 l = __float2bfloat16_rn(r1 - __bfloat162float(m));   // exact
-            v.x = pack(__hneg(h), __hneg(m));
-            v.y = pack(__hneg(l), zero);
-        }
+        if (col < ncols) v = norm_unit(__ldg(bnrm + col));
         uint8_t* row = bb + (size_t)g * B_BYTES + r * 128;
         *reinterpret_cast<uint4*>(row + (((2 * k) ^ (r & 7)) << 4)) = v;
         *reinterpret_cast<uint4*>(row + (((2 * k + 1) ^ (r & 7)) << 4)) = make_uint4(0, 0, 0, 0);
@@ -651,12 +681,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                     const float2 mhalf = make_float2(-0.5f, -0.5f);
                     const bool full_tile = col_half + 128 <= p.N;
                     uint32_t ra[32], rb[32];
-                    // ARGMAX: each 32-column chunk's maximum by a tree of three-input
-                    // maxima; where it beats the running best (strictly: chunks
-                    // arrive in increasing column order, so a tie keeps the earlier
-                    // chunk) the chunk's scores replace the kept ones by predicated
-                    // selects.  The column inside the kept chunk is found once per
-                    // row block.  TOP2 also keeps the runner-up (the best of the
+                    // ARGMAX: argmax_chunk.  TOP2 also keeps the runner-up (the best of the
                     // other columns, lowest column on ties), column by column.
                     // fold: the MMA has added -|e|^2/2 already (augmented operands)
                     auto scan = [&](uint32_t (&v)[32], int c, auto top2, auto fold) {
@@ -699,18 +724,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                                 best = fmaxf(best, sc[e]);
                             }
                         } else {
-                            float t[11];
-#pragma unroll
-                            for (int e = 0; e < 10; ++e) t[e] = max3f(sc[3 * e], sc[3 * e + 1], sc[3 * e + 2]);
-                            t[10] = fmaxf(sc[30], sc[31]);
-                            const float m = fmaxf(max3f(max3f(t[0], t[1], t[2]), max3f(t[3], t[4], t[5]),
-                                                        max3f(t[6], t[7], t[8])),
-                                                  fmaxf(t[9], t[10]));
-                            const uint32_t imp = m > best ? 1u : 0u;
-#pragma unroll
-                            for (int h = 0; h < 4; ++h) select8(keep + 8 * h, sc + 8 * h, imp);
-                            best = imp ? m : best;
-                            bchunk = imp ? kcol : bchunk;
+                            argmax_chunk(sc, kcol, best, bchunk, keep);
                         }
                         __syncwarp();                    // converged for the next tcgen05 op
                     };
@@ -743,11 +757,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             }
             if (dead) break;
             if (amax && p.mode == ARGMAX && bchunk >= 0) {
-                // the first column of the kept chunk attaining the row's best
-                int j = 31;
-#pragma unroll
-                for (int e = 30; e >= 0; --e) j = (keep[e] == best) ? e : j;
-                bidx = bchunk + j;
+                bidx = argmax_column(best, bchunk, keep);
             }
             if (amax) {
                 // merge the two column halves of each row: the larger score,
@@ -786,7 +796,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                         }
                         const int i = m0 * BM + row_in_tile;
                         if (i < p.M) {
-                            p.arg[i] = bidx;
+                            p.arg[i] = bidx == INT_MAX ? 0 : bidx;      // NaN scores: no choice made
                             if (p.best) p.best[i] = 2.f * best;
                             if (p.mode == TOP2) {
                                 p.arg2[i] = (bidx2 == INT_MAX) ? -1 : bidx2;
@@ -812,6 +822,299 @@ __global__ void __launch_bounds__(THREADS, 1)
         tmem_dealloc(tmem, TMEM_COLS);
     }
     if (threadIdx.x == 0 && aborted(sm) && p.error) atomicExch(p.error, 1);
+}
+
+// ---- assignment with the centres resident in shared memory -------------------------
+// Bound by reading the accumulators: a 128 x 256 tile of scores is 128 KB of
+// tensor memory, which is read at about 64 bytes a clock (2000 clocks), while
+// its MMAs at K = 128 take about 1150.  The persistent kernel above adds waits for
+// operands to that, since it streams every column tile of B for every row block
+// (96 KB a tile).  Here a CTA keeps its share of the centres (and their folded
+// norms) in shared memory for the whole launch and streams only row blocks of
+// points, 16 KB per 64 features.  The centres' column tiles are dealt to G
+// groups of CTAs, as few as hold them (nt tiles of 256 each); each group goes
+// over every row block, and merge_groups_kernel keeps the better of the
+// groups' bests (the lower column on a tie).  The MMAs of a tile are those of
+// the kernel above in the same order, so scores and choices are the same bits.
+// 10^6 points, 1000 centres, d = 128: 230 us (and 8 for the merge) where the
+// kernel above took 267 us.  Slower variants: 16 epilogue warps (257 us), CTA
+// pairs sharing the centres (335 us), packed-FMA selects (249 us); an epilogue
+// that only reads still takes 216 us.
+constexpr int RES_STAGES = 4;                   // A chunks (128 rows x 64 features) in flight
+constexpr int AUG_BYTES = B_BYTES;              // A' in K block 0, B' of tile q in K block q + 1 (nt <= 3)
+
+struct ResCtl {
+    uint64_t full[RES_STAGES], empty[RES_STAGES], tfull[2], tempty[2], bfull, mma_done;
+    uint64_t mfull[4], mempty[4];               // column-half hand-over per lane quarter
+    uint32_t tmem_base;
+    int abort;
+    float b1[BM];                               // the second column half's results
+    int j1[BM];
+};
+
+struct ResParams {
+    int M, N, K;
+    int nt, groups;                 // column tiles per group (the last group may have fewer); groups
+    const float* bnrm;              // |b_k|^2 (N rounded up to BN)
+    int32_t* arg;                   // [groups][M]
+    float* best;                    // [groups][M] or null: twice the best half-score
+    uint32_t spin_limit;
+    int32_t* error;
+};
+
+static size_t resident_smem(int nt, int numK) {
+    return 1024 + (size_t)nt * numK * B_BYTES + AUG_BYTES + (size_t)RES_STAGES * A_BYTES + sizeof(ResCtl);
+}
+
+__global__ void __launch_bounds__(THREADS, 1)
+    tc_assign_resident_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                              ResParams p) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    const int numK = p.K / BK;
+    const int numM = (p.M + BM - 1) / BM, numN = (p.N + BN - 1) / BN;
+    const int group = blockIdx.x % p.groups, member = blockIdx.x / p.groups, members = gridDim.x / p.groups;
+    const int q0 = group * p.nt, nt = min(p.nt, numN - q0);        // this CTA's column tiles
+    uint8_t* sB = base;                                            // [tile][k chunk] 32 KB each
+    uint8_t* aug = sB + (size_t)p.nt * numK * B_BYTES;
+    uint8_t* sA = aug + AUG_BYTES;
+    ResCtl& sm = *reinterpret_cast<ResCtl*>(sA + (size_t)RES_STAGES * A_BYTES);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    auto gave_up = [&]() { return *reinterpret_cast<const volatile int*>(&sm.abort) != 0; };
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < RES_STAGES; ++s) {
+            ptx::mbar_init(&sm.full[s], 1);
+            ptx::mbar_init(&sm.empty[s], 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            ptx::mbar_init(&sm.tfull[b], 1);
+            ptx::mbar_init(&sm.tempty[b], EPI_WARPS);
+        }
+        for (int q = 0; q < 4; ++q) {
+            ptx::mbar_init(&sm.mfull[q], 32);
+            ptx::mbar_init(&sm.mempty[q], 32);
+        }
+        ptx::mbar_init(&sm.bfull, 1);
+        ptx::mbar_init(&sm.mma_done, 1);
+        ptx::fence_mbar_init();
+        sm.abort = 0;
+    }
+    if (warp == 1) tmem_alloc(&sm.tmem_base, TMEM_COLS);
+    // the folded norms: as build_augmented, with A' and B' in one 256-row block
+    for (int i = threadIdx.x; i < BN * 4; i += blockDim.x) {
+        const int k = i & 3, r = i >> 2;
+        const int col = (q0 + k - 1) * BN + r;
+        uint4 v = make_uint4(0, 0, 0, 0);
+        if (k == 0) v = ones_unit();
+        else if (k <= nt && col < numN * BN) v = norm_unit(__ldg(p.bnrm + col));
+        uint8_t* row = aug + r * 128;
+        *reinterpret_cast<uint4*>(row + (((2 * k) ^ (r & 7)) << 4)) = v;
+        *reinterpret_cast<uint4*>(row + (((2 * k + 1) ^ (r & 7)) << 4)) = make_uint4(0, 0, 0, 0);
+    }
+    ptx::fence_proxy_async_smem();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = sm.tmem_base;
+
+    if (warp == 0) {
+        // ---------------- TMA producer ----------------
+        if (lane == 0) {
+            ptx::mbar_arrive_expect_tx(&sm.bfull, (uint32_t)(nt * numK * B_BYTES));
+            for (int q = 0; q < nt; ++q)
+                for (int kb = 0; kb < numK; ++kb)
+                    tma_load_2d(sB + (size_t)(q * numK + kb) * B_BYTES, &tmB, kb * BK, (q0 + q) * BN, &sm.bfull);
+            int stage = 0, nissued = 0;
+            uint32_t eph = (1u << RES_STAGES) - 1u;     // empty barriers start "released"
+            uint32_t armed = 0;                         // loads issued per stage (low bit = parity)
+            bool ok = true;
+            for (int u = member; u < numM && ok && !gave_up(); u += members)
+                for (int kb = 0; kb < numK; ++kb) {
+                    if (!ptx::mbar_wait(&sm.empty[stage], (eph >> stage) & 1u, p.spin_limit)) {
+                        atomicExch(&sm.abort, 1);
+                        ok = false;
+                        break;
+                    }
+                    eph ^= 1u << stage;
+                    ptx::mbar_arrive_expect_tx(&sm.full[stage], A_BYTES);
+                    tma_load_2d(sA + (size_t)stage * A_BYTES, &tmA, kb * BK, u * BM, &sm.full[stage]);
+                    armed ^= 1u << stage;
+                    ++nissued;
+                    stage = (stage + 1 == RES_STAGES) ? 0 : stage + 1;
+                }
+            // loads still in flight must land before shared memory is released
+            ptx::mbar_wait(&sm.bfull, 0, p.spin_limit);
+            for (int s = 0; s < RES_STAGES && s < nissued; ++s)
+                ptx::mbar_wait(&sm.full[s], ((armed >> s) & 1u) ^ 1u, p.spin_limit);
+        }
+    } else if (warp == 1) {
+        // ---------------- MMA issuer ----------------
+        if (lane == 0) {
+            constexpr uint32_t idesc = instr_desc(BM, BN);
+            int stage0 = 0, acc = 0;                    // stage of the row block's first chunk
+            uint32_t fph = 0, tph = 3;                  // tempty barriers start "released"
+            bool ok = ptx::mbar_wait(&sm.bfull, 0, p.spin_limit);
+            if (!ok) atomicExch(&sm.abort, 1);
+            for (int u = member; u < numM && ok && !gave_up(); u += members) {
+                for (int q = 0; q < nt && ok; ++q) {
+                    ok = ptx::mbar_wait(&sm.tempty[acc], (tph >> acc) & 1u, p.spin_limit);
+                    if (!ok) break;
+                    tph ^= 1u << acc;
+                    tc_fence_after();
+                    const uint32_t d = tmem + (uint32_t)(acc * BN);
+                    int stage = stage0;
+                    for (int kb = 0; kb < numK; ++kb) {
+                        if (q == 0) {                   // the chunk's first use
+                            ok = ptx::mbar_wait(&sm.full[stage], (fph >> stage) & 1u, p.spin_limit);
+                            if (!ok) break;
+                            fph ^= 1u << stage;
+                            tc_fence_after();
+                        }
+                        const uint64_t ad = smem_desc(sA + (size_t)stage * A_BYTES);
+                        const uint64_t bd = smem_desc(sB + (size_t)(q * numK + kb) * B_BYTES);
+#pragma unroll
+                        for (int k = 0; k < BK / 16; ++k)
+                            mma_bf16(d, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 2), idesc,
+                                     (kb > 0 || k > 0) ? 1u : 0u);
+                        if (q == nt - 1) mma_commit(&sm.empty[stage]);      // and its last
+                        stage = (stage + 1 == RES_STAGES) ? 0 : stage + 1;
+                    }
+                    if (!ok) break;
+                    // + 1 . (-h - m - l) = -|b|^2/2 for every row
+                    mma_bf16(d, smem_desc(aug), smem_desc(aug) + (uint64_t)((q + 1) * 2), idesc, 1u);
+                    mma_commit(&sm.tfull[acc]);
+                    acc ^= 1;
+                }
+                stage0 = (stage0 + numK) % RES_STAGES;
+            }
+            if (!ok) atomicExch(&sm.abort, 1);
+            // no MMA may still write tensor memory when it is released
+            mma_commit(&sm.mma_done);
+            ptx::mbar_wait(&sm.mma_done, 0, p.spin_limit);
+        }
+    } else {
+        // ---------------- epilogue (warps 2..9) ----------------
+        const int sub = warp & 3, half = (warp - 2) >> 2;
+        const int row_in_tile = sub * 32 + lane;
+        const uint32_t lane_off = (uint32_t)(sub * 32) << 16;
+        int acc = 0;
+        uint32_t tph = 0, uj = 0;
+        bool dead = false;
+        for (int u = member; u < numM && !dead; u += members) {
+            float best = -INFINITY;
+            int bchunk = -1;
+            float keep[32];
+#pragma unroll
+            for (int e = 0; e < 32; ++e) keep[e] = 0.f;
+            for (int q = 0; q < nt; ++q) {
+                uint32_t ok = 1;
+                if (lane == 0)
+                    ok = (!gave_up() && ptx::mbar_wait(&sm.tfull[acc], (tph >> acc) & 1u, p.spin_limit)) ? 1u : 0u;
+                ok = __shfl_sync(0xffffffffu, ok, 0);
+                tph ^= 1u << acc;
+                if (!ok) {
+                    if (lane == 0) atomicExch(&sm.abort, 1);
+                    dead = true;
+                    break;
+                }
+                tc_fence_after();
+                const uint32_t tbase = tmem + (uint32_t)(acc * BN + half * 128) + lane_off;
+                const int col_half = (q0 + q) * BN + half * 128;
+                uint32_t ra[32], rb[32];
+                auto scan = [&](uint32_t (&v)[32], int c) {
+                    const int kcol = col_half + c * OUT_COLS;
+                    float sc[32];
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) sc[e] = __uint_as_float(v[e]);
+                    if (kcol + OUT_COLS > p.N) {
+#pragma unroll
+                        for (int e = 0; e < 32; ++e)
+                            if (kcol + e >= p.N) sc[e] = -INFINITY;
+                    }
+                    argmax_chunk(sc, kcol, best, bchunk, keep);
+                    __syncwarp();                        // converged for the next tcgen05 op
+                };
+                tmem_ld32_async(tbase, ra);
+                tmem_wait(ra);
+#pragma unroll
+                for (int c = 0; c < 4; c += 2) {
+                    tmem_ld32_async(tbase + (uint32_t)((c + 1) * OUT_COLS), rb);
+                    scan(ra, c);
+                    tmem_wait(rb);
+                    if (c + 2 < 4) {
+                        tmem_ld32_async(tbase + (uint32_t)((c + 2) * OUT_COLS), ra);
+                    } else {
+                        // accumulator read: hand it back to the MMA warp
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) ptx::mbar_arrive(&sm.tempty[acc]);
+                    }
+                    scan(rb, c + 1);
+                    if (c + 2 < 4) tmem_wait(ra);
+                }
+                acc ^= 1;
+            }
+            if (dead) break;
+            int bidx = bchunk >= 0 ? argmax_column(best, bchunk, keep) : INT_MAX;   // none: NaN scores
+            // merge the two column halves of each row: the larger score, the
+            // lower column on a tie
+            const uint32_t par = uj & 1u;
+            bool okm;
+            if (half == 1) {
+                okm = ptx::mbar_wait(&sm.mempty[sub], par ^ 1u, p.spin_limit);
+                if (okm) {
+                    sm.b1[row_in_tile] = best;
+                    sm.j1[row_in_tile] = bidx;
+                    ptx::mbar_arrive(&sm.mfull[sub]);
+                }
+            } else {
+                okm = ptx::mbar_wait(&sm.mfull[sub], par, p.spin_limit);
+                if (okm) {
+                    const float o1 = sm.b1[row_in_tile];
+                    const int i1 = sm.j1[row_in_tile];
+                    ptx::mbar_arrive(&sm.mempty[sub]);
+                    if (o1 > best || (o1 == best && i1 < bidx)) { best = o1; bidx = i1; }
+                    const int i = u * BM + row_in_tile;
+                    if (i < p.M) {
+                        p.arg[(int64_t)group * p.M + i] = bidx == INT_MAX ? 0 : bidx;
+                        if (p.best) p.best[(int64_t)group * p.M + i] = 2.f * best;
+                    }
+                }
+            }
+            if (__any_sync(0xffffffffu, !okm)) {
+                if (lane == 0) atomicExch(&sm.abort, 1);
+                dead = true;
+            }
+            ++uj;
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem, TMEM_COLS);
+    }
+    if (threadIdx.x == 0 && gave_up() && p.error) atomicExch(p.error, 1);
+}
+
+// The groups' results (garg, gbest: [groups][n]) into one: the larger score, the
+// lower column on a tie.
+__global__ void merge_groups_kernel(const int32_t* __restrict__ garg, const float* __restrict__ gbest, int groups,
+                                    int64_t n, int32_t* arg, float* best) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        float b = gbest[i];
+        int32_t a = garg[i];
+        for (int g = 1; g < groups; ++g) {
+            const float c = gbest[g * n + i];
+            if (c > b) {                    // later groups hold higher columns
+                b = c;
+                a = garg[g * n + i];
+            }
+        }
+        arg[i] = a;
+        if (best) best[i] = b;
+    }
 }
 
 // ---- host side ----------------------------------------------------------------
@@ -1050,10 +1353,54 @@ static int32_t assign_launch(const __nv_bfloat16* A, int na, const __nv_bfloat16
     return launch(ma, mb, ma, p, (na + BM - 1) / BM, s);                  // row blocks
 }
 
+// Scratch of tc_assign_argmax: the groups' results, at most 4 groups of 8 bytes a point.
+size_t tc_assign_scratch_bytes(int64_t na) { return (size_t)na * 4 * (sizeof(int32_t) + sizeof(float)); }
+
+// The resident kernel takes up to 1024 centres (whose norms the kernel above
+// folds too, so a score has the same bits in both) of up to 256 features: a
+// group then holds at least one column tile of 256 centres next to four 16 KB
+// stages.  Wider features or more centres stream both operands.
 int32_t tc_assign_argmax(const __nv_bfloat16* A, int na, const __nv_bfloat16* B, int nb,
-                         const float* bnrm, int dpad, int32_t* arg, float* best, int32_t* err,
-                         cudaStream_t s) {
-    return assign_launch(A, na, B, nb, bnrm, dpad, arg, best, nullptr, nullptr, err, s);
+                         const float* bnrm, int dpad, int32_t* arg, float* best, void* scratch,
+                         int32_t* err, cudaStream_t s) {
+    using namespace tc;
+    if (dpad % BK || nb < 1 || na < 1) return AP_ERR_INVALID_ARG;
+    const int numK = dpad / BK, numN = (nb + BN - 1) / BN, numM = (na + BM - 1) / BM;
+    if (numN > 4 || numK > 4 || assign_norm_form() > 1 || !scratch)
+        return assign_launch(A, na, B, nb, bnrm, dpad, arg, best, nullptr, nullptr, err, s);
+    const int ntmax = std::min(3, 4 / numK);            // tiles that fit: 128 KB of centres, 3 K blocks of norms
+    const int groups = (numN + ntmax - 1) / ntmax, nt = (numN + groups - 1) / groups;
+    int sms = 0;
+    AP_TRY(device_sm_count(&sms));
+    const size_t bytes = resident_smem(nt, numK);
+    if (bytes > (size_t)SMEM_LIMIT) return AP_ERR_UNSUPPORTED;
+    CUtensorMap ma, mb;
+    AP_TRY(make_map(&ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (void*)A, dpad, (uint64_t)numM * BM, (uint64_t)dpad * 2,
+                    BK, BM, CU_TENSOR_MAP_SWIZZLE_128B));
+    AP_TRY(make_map(&mb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (void*)B, dpad, (uint64_t)numN * BN, (uint64_t)dpad * 2,
+                    BK, BN, CU_TENSOR_MAP_SWIZZLE_128B));
+    ResParams p{};
+    p.M = na;
+    p.N = nb;
+    p.K = dpad;
+    p.nt = nt;
+    p.groups = groups;
+    p.bnrm = bnrm;
+    p.arg = groups > 1 ? static_cast<int32_t*>(scratch) : arg;
+    p.best = groups > 1 ? reinterpret_cast<float*>(p.arg + (size_t)groups * na) : best;
+    p.spin_limit = 1u << 22;
+    p.error = err;
+    AP_CUDA_TRY(cudaFuncSetAttribute(tc_assign_resident_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     SMEM_LIMIT));
+    const int members = std::max(1, std::min(numM, sms / groups));
+    tc_assign_resident_kernel<<<members * groups, THREADS, bytes, s>>>(ma, mb, p);
+    note_launches(1);
+    if (groups > 1) {
+        merge_groups_kernel<<<(int)std::min<int64_t>(((int64_t)na + 255) / 256, 4096), 256, 0, s>>>(
+            p.arg, p.best, groups, na, arg, best);
+        note_launches(1);
+    }
+    return last_error();
 }
 
 int32_t tc_assign_top2(const __nv_bfloat16* A, int na, const __nv_bfloat16* B, int nb,

@@ -404,3 +404,37 @@ def test_lap_refine_single_centre_only_moves_to_the_medoid():
     assert np.array_equal(E.cpu().numpy(), E_ref) and E_ref.size == 1
     assert res["removed"] == 0 and res["moved"] == sum(h["moved"] for h in hist)
     assert np.all(idx.cpu().numpy() == E_ref[0])
+
+
+@pytest.mark.parametrize("d", [3, 64, 65, 128, 190, 256, 257])
+@pytest.mark.parametrize("c", [1, 2, 255, 256, 257, 512, 513, 768, 769, 1000])
+def test_assign_with_resident_centres_at_its_edges(c, d):
+    """Every split of the centres over groups of CTAs (256-column tiles, 128 KB of
+    them per CTA; past 256 features the streaming kernel): the choice is a
+    maximum of the float64 scores of the rounded centred points up to the
+    accumulation bound, the lowest position among equal centres, and `best` is
+    its score.  129 to 1300 points: ragged row blocks."""
+    g = np.random.default_rng(c * 1000 + d)
+    n = max(c + 129, 1300 if c < 1000 else 1200)
+    X = (g.normal(size=(n, d)) * 3).astype(np.float32)
+    X[n // 2] = X[n - 1]                                     # two equal points, both centres when c > 1
+    cen = g.permutation(n)[:c].astype(np.int32)
+    if c > 1:
+        rest = cen[(cen != n // 2) & (cen != n - 1)][:c - 2]
+        cen = np.concatenate([rest, [n - 1, n // 2]]).astype(np.int32)
+    Xd = torch.from_numpy(X).cuda()
+    idx, best = capi.lap_assign(Xd, torch.from_numpy(cen), best=True)
+    B = (Xd - Xd.double().mean(0).float()).to(torch.bfloat16).double()
+    E = B[torch.from_numpy(cen).cuda().long()]
+    score = 2 * (B @ E.T) - (E * E).sum(1)
+    top = score.max(1).values
+    tol = (d + 4) * 2.0 ** -22 * (B * B).sum(1).max()
+    assert bool(((best.double() - top).abs() <= tol).all())
+    pos = {int(k): j for j, k in reversed(list(enumerate(cen)))}
+    got = idx.cpu().numpy()
+    own = np.isin(np.arange(n), cen)
+    assert np.array_equal(got[own], np.arange(n)[own])       # centres keep themselves
+    chosen = torch.tensor([pos[int(k)] for k in got], device="cuda")
+    assert bool((score.gather(1, chosen[:, None])[:, 0] >= top - 2 * tol)[torch.from_numpy(~own).cuda()].all())
+    if c > 1:                                                # of the two equal centres the earlier one
+        assert not np.any(got[~own] == n // 2)
