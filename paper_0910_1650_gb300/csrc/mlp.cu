@@ -389,11 +389,16 @@ __global__ void standardisation_kernel(const float* __restrict__ F, int64_t rows
 // gradients stay float32, weights are bf16: about 74000 multiply-adds per row
 // and direction), not by memory.  rows_kernel therefore takes a tile of 32
 // rows through all three layers -- and, in training, back through them -- with
-// the activations in shared memory: 128 threads own 8 rows x 8 columns of the
-// 256-wide layers each (64 accumulators against 16 shared-memory words per
-// step of k, so the FMA pipe and not shared memory is the limit), multiply in
-// packed f32x2, and prefetch the next 16 x 256 weights into registers while
-// the current ones are used.  A thread owns the same elements in every layer,
+// the activations in shared memory: a thread owns 8 rows x 2 JC columns of the
+// 256-wide layers, multiplies in packed f32x2, and prefetches the next 16 x 256
+// weights into registers while the current ones are used.  The forward pass has
+// several tiles per SM and JC = 4 (64 accumulators against 16 shared-memory
+// words per step of k, so the FMA pipe and not shared memory is the limit); in
+// training, where a batch has about one tile per SM, 256 threads with JC = 2 give
+// every scheduler a second warp to fill the first one's waits (74 us a step
+// where 128 threads took 80).  Every sum runs over k in turn from zero, so that
+// a unit's sign, which decides where gradients flow, does not depend on the
+// split.  A thread owns the same elements in every layer,
 // so the ReLU masks stay in registers.  In training the block leaves its
 // tiles' share of every gradient but W2's in one partial slot, and the rows'
 // H1 and G2 for w2_grad_kernel, which splits the rows of G2^T H1 over blocks;
@@ -405,7 +410,6 @@ __global__ void standardisation_kernel(const float* __restrict__ F, int64_t rows
 constexpr int TR = 32;                 // rows per tile
 constexpr int RS = 36;                 // their stride in shared memory (16-byte groups, fewer bank conflicts)
 constexpr int KC = 16;                 // weights staged per step: KC x 256
-constexpr int RT = 128;                // threads of rows_kernel
 constexpr int kMaxSlots = 608;         // gradient partial slots: 4 tiles in flight per SM
 constexpr int NSMALL = NP - 2 * IN - HID * HID;   // gradients but W2's, in parameter order
 constexpr int SLOT = (NSMALL + 3) / 4 * 4;
@@ -434,86 +438,85 @@ __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w 
 // The next KC x 256 weights of W2 [256 x 256], k from k0: columns of the
 // product are W2's rows going forward (k along a row), its columns going back
 // (BACK: k is W2's row).
-template <bool BACK>
-__device__ __forceinline__ void fetch_w2(const __nv_bfloat16* __restrict__ W, int k0, int vec, uint4 (&pf)[4]) {
-    const int tid = threadIdx.x;
+template <bool BACK, int RT>
+__device__ __forceinline__ void fetch_w2(const __nv_bfloat16* __restrict__ W, int k0, int vec, uint4 (&pf)[512 / RT]) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        if (BACK) {
-            const int e = tid + q * RT;                    // 16 rows x 32 groups of eight
-            pf[q] = load8(W + (int64_t)(k0 + (e >> 5)) * HID + 8 * (e & 31), vec);
-        } else {
-            pf[q] = load8(W + (int64_t)(tid + (q >> 1) * RT) * HID + k0 + 8 * (q & 1), vec);
-        }
+    for (int q = 0; q < 512 / RT; ++q) {
+        const int e = threadIdx.x + q * RT;
+        // 16 rows x 32 groups of eight; or 256 rows x 2 groups (a warp on 32 rows)
+        if (BACK) pf[q] = load8(W + (int64_t)(k0 + (e >> 5)) * HID + 8 * (e & 31), vec);
+        else pf[q] = load8(W + (int64_t)(e & 255) * HID + k0 + 8 * (e >> 8), vec);
     }
 }
-template <bool BACK>
-__device__ __forceinline__ void put_w2(float (*ws)[HID], const uint4 (&pf)[4]) {
-    const int tid = threadIdx.x;
+template <bool BACK, int RT>
+__device__ __forceinline__ void put_w2(float (*ws)[HID], const uint4 (&pf)[512 / RT]) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < 512 / RT; ++q) {
+        const int e = threadIdx.x + q * RT;
         const float v[8] = {bf16_lo(pf[q].x), bf16_hi(pf[q].x), bf16_lo(pf[q].y), bf16_hi(pf[q].y),
                             bf16_lo(pf[q].z), bf16_hi(pf[q].z), bf16_lo(pf[q].w), bf16_hi(pf[q].w)};
         if (BACK) {
-            const int e = tid + q * RT;
             float* at = &ws[e >> 5][8 * (e & 31)];
             *reinterpret_cast<float4*>(at) = make_float4(v[0], v[1], v[2], v[3]);
             *reinterpret_cast<float4*>(at + 4) = make_float4(v[4], v[5], v[6], v[7]);
         } else {
-            const int o = tid + (q >> 1) * RT;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) ws[8 * (q & 1) + j][o] = v[j];
+            for (int j = 0; j < 8; ++j) ws[8 * (e >> 8) + j][e & 255] = v[j];
         }
     }
 }
 
 // acc += (column k of act) x (row k of w): this thread's rows 8 wid .. and
-// columns 2 lid + 64 j, + 1.
-__device__ __forceinline__ void rank1(const float* act, const float* w, int wid, int lid, float2 (&acc)[8][4]) {
+// columns col + 64 j, + 1 (col: 2 lid, + 128 for the second four warps of eight).
+template <int JC>
+__device__ __forceinline__ void rank1(const float* act, const float* w, int wid, int col, float2 (&acc)[8][JC]) {
     const float4 a0 = *reinterpret_cast<const float4*>(act + 8 * wid);
     const float4 a1 = *reinterpret_cast<const float4*>(act + 8 * wid + 4);
-    float2 b[4];
+    float2 b[JC];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const float2*>(w + 64 * j + 2 * lid);
+    for (int j = 0; j < JC; ++j) b[j] = *reinterpret_cast<const float2*>(w + 64 * j + col);
     const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
 #pragma unroll
     for (int r = 0; r < 8; ++r)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[r][j] = __ffma2_rn(make_float2(a[r], a[r]), b[j], acc[r][j]);
+        for (int j = 0; j < JC; ++j) acc[r][j] = __ffma2_rn(make_float2(a[r], a[r]), b[j], acc[r][j]);
 }
 
-__device__ __forceinline__ void clear(float2 (&acc)[8][4]) {
+template <int JC>
+__device__ __forceinline__ void clear(float2 (&acc)[8][JC]) {
 #pragma unroll
     for (int r = 0; r < 8; ++r)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[r][j] = make_float2(0.f, 0.f);
+        for (int j = 0; j < JC; ++j) acc[r][j] = make_float2(0.f, 0.f);
 }
 
 // acc = hs x W2 (or its transpose); leaves the block synchronised, hs free.
-template <bool BACK>
-__device__ __forceinline__ void layer2(RowsSmem& sm, const __nv_bfloat16* __restrict__ W, int vec, int wid, int lid,
-                                       float2 (&acc)[8][4]) {
-    uint4 pf[4];
+template <bool BACK, int JC>
+__device__ __forceinline__ void layer2(RowsSmem& sm, const __nv_bfloat16* __restrict__ W, int vec, int wid, int col,
+                                       float2 (&acc)[8][JC]) {
+    constexpr int RT = 512 / JC;
+    uint4 pf[JC];
     clear(acc);
-    fetch_w2<BACK>(W, 0, vec, pf);
-    put_w2<BACK>(sm.ws[0], pf);
+    fetch_w2<BACK, RT>(W, 0, vec, pf);
+    put_w2<BACK, RT>(sm.ws[0], pf);
     __syncthreads();
     for (int c = 0; c < HID / KC; ++c) {
-        if (c + 1 < HID / KC) fetch_w2<BACK>(W, (c + 1) * KC, vec, pf);
+        if (c + 1 < HID / KC) fetch_w2<BACK, RT>(W, (c + 1) * KC, vec, pf);
 #pragma unroll
-        for (int kk = 0; kk < KC; ++kk) rank1(sm.hs + (c * KC + kk) * RS, sm.ws[c & 1][kk], wid, lid, acc);
-        if (c + 1 < HID / KC) put_w2<BACK>(sm.ws[(c + 1) & 1], pf);
+        for (int kk = 0; kk < KC; ++kk) rank1(sm.hs + (c * KC + kk) * RS, sm.ws[c & 1][kk], wid, col, acc);
+        if (c + 1 < HID / KC) put_w2<BACK, RT>(sm.ws[(c + 1) & 1], pf);
         __syncthreads();
     }
 }
 
-// The thread's 8 x 8 elements into hs, and (out != null) into row-major
+// The thread's 8 x 2 JC elements into hs, and (out != null) into row-major
 // out [rows x 256].
-__device__ __forceinline__ void put_tile(float* hs, float* out, const float2 (&v)[8][4], int wid, int lid, int64_t r0,
+template <int JC>
+__device__ __forceinline__ void put_tile(float* hs, float* out, const float2 (&v)[8][JC], int wid, int col, int64_t r0,
                                          int rows) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        float* x = hs + (64 * j + 2 * lid) * RS + 8 * wid;
+    for (int j = 0; j < JC; ++j) {
+        float* x = hs + (64 * j + col) * RS + 8 * wid;
         *reinterpret_cast<float4*>(x) = make_float4(v[0][j].x, v[1][j].x, v[2][j].x, v[3][j].x);
         *reinterpret_cast<float4*>(x + 4) = make_float4(v[4][j].x, v[5][j].x, v[6][j].x, v[7][j].x);
         *reinterpret_cast<float4*>(x + RS) = make_float4(v[0][j].y, v[1][j].y, v[2][j].y, v[3][j].y);
@@ -525,18 +528,19 @@ __device__ __forceinline__ void put_tile(float* hs, float* out, const float2 (&v
             const int64_t row = r0 + 8 * wid + r;
             if (row < rows)
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    *reinterpret_cast<float2*>(out + row * HID + 64 * j + 2 * lid) = v[r][j];
+                for (int j = 0; j < JC; ++j)
+                    *reinterpret_cast<float2*>(out + row * HID + 64 * j + col) = v[r][j];
         }
     }
 }
 
 // Bias and ReLU; the mask has bit 8 r + 2 j + e for row r, column pair j, element e.
-__device__ __forceinline__ uint64_t bias_relu(float2 (&acc)[8][4], const float* __restrict__ b, int lid) {
+template <int JC>
+__device__ __forceinline__ uint64_t bias_relu(float2 (&acc)[8][JC], const float* __restrict__ b, int col) {
     uint64_t m = 0;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const float b0 = b[64 * j + 2 * lid], b1 = b[64 * j + 2 * lid + 1];
+    for (int j = 0; j < JC; ++j) {
+        const float b0 = b[64 * j + col], b1 = b[64 * j + col + 1];
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
             acc[r][j].x = fmaxf(acc[r][j].x + b0, 0.f);
@@ -556,12 +560,14 @@ struct TrainOut {
 };
 
 template <bool TRAIN>
-__global__ void __launch_bounds__(RT) rows_kernel(const float* __restrict__ P, const __nv_bfloat16* __restrict__ P16,
+__global__ void __launch_bounds__(TRAIN ? 256 : 128) rows_kernel(const float* __restrict__ P, const __nv_bfloat16* __restrict__ P16,
                                                   const float* __restrict__ F, int rows, int vec, float* Y,
                                                   TrainOut t) {
     extern __shared__ __align__(16) unsigned char rows_smem[];
     RowsSmem& sm = *reinterpret_cast<RowsSmem*>(rows_smem);
-    const int tid = threadIdx.x, wid = tid >> 5, lid = tid & 31;
+    constexpr int JC = TRAIN ? 2 : 4, RT = 512 / JC;
+    const int tid = threadIdx.x, wid = (tid >> 5) & 3, lid = tid & 31;
+    const int col = 2 * lid + (tid >> 7) * 128;            // (128 threads: 2 lid)
     const int tiles = (rows + TR - 1) / TR;
     for (int e = tid; e < OUT * HID; e += RT) (&sm.w3[0][0])[e] = __bfloat162float(P16[OFF_W3 + e]);
     float* part = TRAIN ? t.part + (int64_t)blockIdx.x * SLOT : nullptr;
@@ -580,16 +586,16 @@ __global__ void __launch_bounds__(RT) rows_kernel(const float* __restrict__ P, c
             w1[e] = __bfloat162float(P16[OFF_W1 + o * IN + k]);
         }
         __syncthreads();
-        float2 acc[8][4];
+        float2 acc[8][JC];
         clear(acc);
 #pragma unroll 5
-        for (int k = 0; k < IN; ++k) rank1(sm.xs + k * RS, w1 + k * HID, wid, lid, acc);
-        const uint64_t m1 = bias_relu(acc, P + OFF_B1, lid);
-        put_tile(sm.hs, TRAIN ? t.H1 : nullptr, acc, wid, lid, r0, rows);
+        for (int k = 0; k < IN; ++k) rank1(sm.xs + k * RS, w1 + k * HID, wid, col, acc);
+        const uint64_t m1 = bias_relu(acc, P + OFF_B1, col);
+        put_tile(sm.hs, TRAIN ? t.H1 : nullptr, acc, wid, col, r0, rows);
         __syncthreads();
-        layer2<false>(sm, P16 + OFF_W2, vec, wid, lid, acc);
-        const uint64_t m2 = bias_relu(acc, P + OFF_B2, lid);
-        put_tile(sm.hs, nullptr, acc, wid, lid, r0, rows);
+        layer2<false>(sm, P16 + OFF_W2, vec, wid, col, acc);
+        const uint64_t m2 = bias_relu(acc, P + OFF_B2, col);
+        put_tile(sm.hs, nullptr, acc, wid, col, r0, rows);
         __syncthreads();
         if (tid < OUT * TR) {                              // warp o: output o of the 32 rows
             float y0 = 0.f, y1 = 0.f, y2 = 0.f, y3 = 0.f;
@@ -607,7 +613,7 @@ __global__ void __launch_bounds__(RT) rows_kernel(const float* __restrict__ P, c
         }
         if (!TRAIN) continue;
         __syncthreads();
-        if (wid == 0) {
+        if (tid < TR) {
             // the row's loss and dL/dY (divided by the row count)
             const bool in = r0 + lid < rows;
             const float inv = 1.f / (float)rows;
@@ -655,8 +661,8 @@ __global__ void __launch_bounds__(RT) rows_kernel(const float* __restrict__ P, c
         for (int r = 0; r < 8; ++r) {
             const float g0 = sm.gs[0][8 * wid + r], g1 = sm.gs[1][8 * wid + r], g2 = sm.gs[2][8 * wid + r];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int c = 64 * j + 2 * lid;
+            for (int j = 0; j < JC; ++j) {
+                const int c = 64 * j + col;
                 const float2 w0 = *reinterpret_cast<const float2*>(&sm.w3[0][c]);
                 const float2 w1v = *reinterpret_cast<const float2*>(&sm.w3[1][c]);
                 const float2 w2v = *reinterpret_cast<const float2*>(&sm.w3[2][c]);
@@ -667,7 +673,7 @@ __global__ void __launch_bounds__(RT) rows_kernel(const float* __restrict__ P, c
             }
         }
         __syncthreads();                                   // H2 has been read
-        put_tile(sm.hs, t.G2, acc, wid, lid, r0, rows);
+        put_tile(sm.hs, t.G2, acc, wid, col, r0, rows);
         __syncthreads();
 #pragma unroll
         for (int h = 0; h < HID / RT; ++h) {               // gb2
@@ -681,15 +687,15 @@ __global__ void __launch_bounds__(RT) rows_kernel(const float* __restrict__ P, c
             add(S_B2 + c, g);
         }
         // G1 = (G2 W2) where H1 > 0, then gW1 = G1^T X and gb1
-        layer2<true>(sm, P16 + OFF_W2, vec, wid, lid, acc);
+        layer2<true>(sm, P16 + OFF_W2, vec, wid, col, acc);
 #pragma unroll
         for (int r = 0; r < 8; ++r)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
+            for (int j = 0; j < JC; ++j) {
                 if (!((m1 >> (8 * r + 2 * j)) & 1)) acc[r][j].x = 0.f;
                 if (!((m1 >> (8 * r + 2 * j + 1)) & 1)) acc[r][j].y = 0.f;
             }
-        put_tile(sm.hs, nullptr, acc, wid, lid, r0, rows);
+        put_tile(sm.hs, nullptr, acc, wid, col, r0, rows);
         __syncthreads();
 #pragma unroll
         for (int h = 0; h < HID / RT; ++h) {
@@ -923,7 +929,7 @@ static int32_t launch_rows(const float* P, const __nv_bfloat16* P16, const float
                            const TrainOut& t, int grid, cudaStream_t s) {
     AP_CUDA_TRY(cudaFuncSetAttribute(rows_kernel<TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)sizeof(RowsSmem)));
-    rows_kernel<TRAIN><<<grid, RT, sizeof(RowsSmem), s>>>(P, P16, F, rows, aligned16(P16) ? 1 : 0, Y, t);
+    rows_kernel<TRAIN><<<grid, TRAIN ? 256 : 128, sizeof(RowsSmem), s>>>(P, P16, F, rows, aligned16(P16) ? 1 : 0, Y, t);
     note_launches(1);
     return last_error();
 }
