@@ -60,15 +60,18 @@ constexpr int TOPK = 16;
 // Writes features 0-15 and 18-22, the 16 neighbour indices (problem-local)
 // and the sums, from which features_finish_row makes 16-17 with whole warps
 // of rows (a float64 division by one lane costs what 32 cost).
-// 48 problems of 200-4000 points (2.7e8 entries): 637 us (+ 29 us for the second
-// pass), where one block per row with 16 block-wide arg-max rounds and float64
-// sums took 8.1 ms.
-constexpr int kListCap = 128;      // entries listed per warp
+// The listing takes places by a shared atomic (the ranking does not depend on
+// their order) and the counts are float32, whose additions are full rate.
+// 48 problems of 200-4000 points (2.7e8 entries): 544 us (+ 27 us for the second
+// pass; 637 us with ballots, prefix counts and integer sums), where one block per
+// row with 16 block-wide arg-max rounds and float64 sums took 8.1 ms.
+constexpr int kListCap = 256;      // entries listed per warp
 constexpr int kFeatWarps = 8;      // rows per block
 
 struct FeatList {
     float v[kListCap];
     int j[kListCap];
+    int have;
     float bv[TOPK];
     int bj[TOPK];
 };
@@ -88,6 +91,12 @@ __device__ __forceinline__ void two_add(float2& s, float2& c, float2 x) {
     c = __fadd2_rn(c, __fadd2_rn(__ffma2_rn(mone, ap, s), __ffma2_rn(mone, bp, x)));
     s = t;
 }
+// c += 1 where v >= t.
+__device__ __forceinline__ void count_if_ge(float& c, float v, float t) {
+    asm("{\n\t.reg .pred p;\n\tsetp.ge.f32 p, %1, %2;\n\t@p add.f32 %0, %0, 0f3F800000;\n\t}"
+        : "+f"(c)
+        : "f"(v), "f"(t));
+}
 __device__ __forceinline__ void two_add1(float& s, float& c, float x) {
     const float t = s + x, bp = t - s;
     c += (s - (t - bp)) + (x - bp);
@@ -95,28 +104,23 @@ __device__ __forceinline__ void two_add1(float& s, float& c, float x) {
 }
 
 // The 16 best of the list's cnt entries (cnt <= kListCap) to bv, bj, best first.
+// The order in which the entries were listed does not matter.
 __device__ __forceinline__ void rank_list(FeatList& L, int cnt, int lid) {
-    float v[kListCap / 32];
-    int j[kListCap / 32], rank[kListCap / 32];
-#pragma unroll
-    for (int q = 0; q < kListCap / 32; ++q) {
-        const int e = lid + 32 * q;
-        v[q] = e < cnt ? L.v[e] : -INFINITY;
-        j[q] = e < cnt ? L.j[e] : INT_MAX;
-        rank[q] = 0;
-    }
-    for (int e = 0; e < cnt; ++e) {
-        const float w = L.v[e];
-        const int i = L.j[e];
-#pragma unroll
-        for (int q = 0; q < kListCap / 32; ++q) rank[q] += w > v[q] || (w == v[q] && i < j[q]);
-    }
-#pragma unroll
-    for (int q = 0; q < kListCap / 32; ++q)
-        if (lid + 32 * q < cnt && rank[q] < TOPK) {
-            L.bv[rank[q]] = v[q];
-            L.bj[rank[q]] = j[q];
+    for (int e0 = 0; e0 < cnt; e0 += 32) {
+        const int at = e0 + lid;
+        const float v = at < cnt ? L.v[at] : -INFINITY;
+        const int j = at < cnt ? L.j[at] : INT_MAX;
+        int rank = 0;
+#pragma unroll 4
+        for (int e = 0; e < cnt; ++e) {
+            const float w = L.v[e];
+            rank += w > v || (w == v && L.j[e] < j);
         }
+        if (at < cnt && rank < TOPK) {
+            L.bv[rank] = v;
+            L.bj[rank] = j;
+        }
+    }
     __syncwarp();
 }
 
@@ -140,7 +144,9 @@ __device__ __forceinline__ void features_row(const float* __restrict__ S, int n,
     for (int q = 0; q < 4; ++q) thr[q] = -(scale * (0.125f * (float)(1 << q)));   // exact: powers of 2
     const int n4 = (n + 3) >> 2, fk = k >> 2, nfull = n >> 2;
     float2 s1 = make_float2(0.f, 0.f), c1 = s1, s2 = s1, c2 = s1;
-    int cnt[4] = {0, 0, 0, 0};
+    // float32 counts (exact: a lane has at most n / 32 + 4 entries), since their
+    // additions then go to the FMA pipe and not to the half-rate ALU pipe
+    float fcnt[4] = {0.f, 0.f, 0.f, 0.f};
     float mx = -INFINITY;
 #pragma unroll 2
     for (int f = lid; f < n4; f += 32) {
@@ -167,9 +173,9 @@ __device__ __forceinline__ void features_row(const float* __restrict__ S, int n,
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) cnt[q] += v[e] >= thr[q];
-            mx = fmaxf(mx, v[e]);
+            for (int q = 0; q < 4; ++q) count_if_ge(fcnt[q], v[e], thr[q]);
         }
+        mx = fmaxf(mx, fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])));
     }
     // the sums over the warp, in a fixed order
     float t1 = s1.x, d1 = c1.x, t2 = s2.x, d2 = c2.x;
@@ -186,8 +192,9 @@ __device__ __forceinline__ void features_row(const float* __restrict__ S, int n,
         d1 += e1;
         d2 += e2;
     }
+    int cnt[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) cnt[q] = __reduce_add_sync(0xffffffffu, cnt[q]);
+    for (int q = 0; q < 4; ++q) cnt[q] = __reduce_add_sync(0xffffffffu, (int)fcnt[q]);
     // the 16th largest lane maximum: sort the 32 of them, largest first
 #pragma unroll
     for (int w = 2; w <= 32; w <<= 1)
@@ -199,7 +206,9 @@ __device__ __forceinline__ void features_row(const float* __restrict__ S, int n,
         }
     float bar = __shfl_sync(0xffffffffu, mx, TOPK - 1);
     int barj = INT_MAX;                             // an entry equal to bar must come before barj
-    int have = 0;
+    if (lid == 0) L.have = 0;
+    __syncwarp();
+#pragma unroll 2
     for (int f0 = 0; f0 < n4; f0 += 32) {
         const int f = f0 + lid;
         float v[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
@@ -207,34 +216,37 @@ __device__ __forceinline__ void features_row(const float* __restrict__ S, int n,
             const float4 x = row4(row, f, n, vec);
             v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
         }
-        const bool maybe = v[0] >= bar || v[1] >= bar || v[2] >= bar || v[3] >= bar;
+        const bool maybe = fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])) >= bar;
         if (!__any_sync(0xffffffffu, maybe)) continue;
+        if (maybe) {
+            // few lanes: each takes its places by an atomic (the ranking does not
+            // depend on the order)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int j = 4 * f + e;
-            const bool in = v[e] > -INFINITY && (v[e] > bar || (v[e] == bar && j < barj)) && j != k && j < n;
-            const unsigned m = __ballot_sync(0xffffffffu, in);
-            if (in) {
-                const int at = have + __popc(m & ((1u << lid) - 1u));
-                L.v[at] = v[e];
-                L.j[at] = j;
-            }
-            have += __popc(m);
-            if (have > kListCap - 32) {             // room for the next 32: keep the best 16
-                __syncwarp();
-                rank_list(L, have, lid);
-                if (lid < TOPK) {
-                    L.v[lid] = L.bv[lid];
-                    L.j[lid] = L.bj[lid];
+            for (int e = 0; e < 4; ++e) {
+                const int j = 4 * f + e;
+                if (v[e] > -INFINITY && (v[e] > bar || (v[e] == bar && j < barj)) && j != k && j < n) {
+                    const int at = atomicAdd(&L.have, 1);
+                    L.v[at] = v[e];
+                    L.j[at] = j;
                 }
-                __syncwarp();
-                have = TOPK;
-                bar = L.v[TOPK - 1];
-                barj = L.j[TOPK - 1];
             }
+        }
+        __syncwarp();
+        if (L.have > kListCap - 128) {                  // room for the next 128: keep the best 16
+            rank_list(L, L.have, lid);
+            if (lid < TOPK) {
+                L.v[lid] = L.bv[lid];
+                L.j[lid] = L.bj[lid];
+            }
+            if (lid == 0) L.have = TOPK;
+            __syncwarp();
+            bar = L.v[TOPK - 1];
+            barj = L.j[TOPK - 1];
+            __syncwarp();
         }
     }
     __syncwarp();
+    const int have = L.have;
     rank_list(L, have, lid);
     float* out = F + (int64_t)k * IN;
     if (lid < TOPK) {
