@@ -22,11 +22,15 @@
 //
 // Persistent, warp-specialised kernel (one CTA per SM, 320 threads):
 //   warp 0      TMA producer: the A tile (128 x 64) and the B tile (256 x 64)
-//               of each K step into a ring of 2-4 stages (mbarriers
+//               of each K step into a ring of 2-6 stages (mbarriers
 //               full/empty);
 //   warp 1      allocates 512 TMEM columns and issues tcgen05.mma
 //               (M=128, N=256, K=16) from one elected thread into two
 //               256-column accumulators (mbarriers tfull/tempty);
+//               long similarities (see pairs()): two CTAs pair up (cta_group::2,
+//               M=256), each with its own 128 rows of A and half of B's rows,
+//               which the product is bound by fetching from L2 (32 image
+//               problems, d = 4096: 542 us where lone CTAs took 605 us);
 //   warps 2..9  epilogue, two warps per TMEM lane quarter (column halves of
 //               128).  Each warp works on its own: it waits for the
 //               accumulator itself, reads it with pipelined tcgen05.ld, and
@@ -40,6 +44,7 @@
 // store buffering where it is short (bound by writing S).
 // Every mbarrier wait is bounded; on expiry the kernel records an error and
 // all roles stop issuing new work.
+#include <cooperative_groups.h>
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
@@ -55,14 +60,17 @@
 #include "common.cuh"
 #include "ptx.cuh"
 
+namespace cg = cooperative_groups;
+
 namespace apgb {
 namespace tc {
 
 constexpr int BM = 128, BN = 256, BK = 64;
-constexpr int MAX_STAGES = 4;
+constexpr int MAX_STAGES = 6;
 constexpr int A_BYTES = BM * BK * 2;            // 16 KB
 constexpr int B_BYTES = BN * BK * 2;            // 32 KB
 constexpr int STAGE_BYTES = A_BYTES + B_BYTES;  // 48 KB
+constexpr int PAIR_STAGE_BYTES = 2 * A_BYTES;   // 32 KB: a pair's CTA loads half of B's rows
 constexpr int OUT_COLS = 32;                    // fp32 columns per store block (128 B)
 constexpr int WBUF_BYTES = 32 * OUT_COLS * 4;   // one warp's 32 rows x 32 columns: 4 KB
 constexpr int EPI_WARPS = 8;                    // two per TMEM lane quarter: column halves
@@ -230,6 +238,60 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64
         : "memory");
 }
 
+// ---- the same for a pair of CTAs (cta_group::2): one thread of the even CTA issues
+// MMAs of twice the rows; each CTA holds its 128 rows of A and D and half of B's rows.
+// A tile into this CTA's shared memory, completing on the even CTA's barrier
+// (`bar`: a cluster address).
+__device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, "
+        "{%2, %3}], [%4];" ::"r"(ptx::smem_u32(dst)),
+        "l"(map), "r"(x), "r"(y), "r"(bar)
+        : "memory");
+}
+
+__device__ __forceinline__ void tmem_alloc_pair(uint32_t* dst_smem, uint32_t ncols) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(ptx::smem_u32(dst_smem)),
+                 "r"(ncols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+}
+
+__device__ __forceinline__ void mma_bf16_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                              uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+// Arrives on `bar` of both CTAs once the MMAs issued so far are done.
+__device__ __forceinline__ void mma_commit_pair(uint64_t* bar) {
+    asm volatile(
+        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+            ptx::smem_u32(bar)),
+        "h"((uint16_t)3)
+        : "memory");
+}
+
+// Arrives on this CTA's `bar` only.
+__device__ __forceinline__ void mma_commit_pair_local(uint64_t* bar) {
+    asm volatile(
+        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(ptx::smem_u32(bar))
+        : "memory");
+}
+
+// Arrives on a barrier of a CTA of the cluster (a cluster address).
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
 // Arrives on `bar` once every tcgen05.mma issued so far by this thread is done.
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
     asm volatile(
@@ -340,12 +402,29 @@ struct Tile {
     int arow, brow, m, n, prob;
 };
 
-template <bool AMAX>
-__device__ __forceinline__ Tile tile_of(const Params& p, int numN, int u, int q) {
+template <bool AMAX, bool PAIR>
+__device__ __forceinline__ Tile tile_of(const Params& p, int numN, int u, int q, int rank) {
     Tile t;
     if (AMAX) {
         t.m = u; t.n = q; t.prob = 0;
         t.arow = u * BM; t.brow = q * BN;
+    } else if (PAIR) {
+        // 256 x 256 tiles of a CTA pair on or above the diagonal; this CTA has the 128
+        // rows `rank` of the tile's, and loads that half of B's rows
+        int m, roff = 0;
+        if (p.tiles) {
+            const int4 e = p.tiles[u];
+            roff = p.probs[e.x].roff;
+            t.prob = e.x; m = e.y; t.n = e.z;
+        } else {
+            // column block c has the row blocks 0 .. c: c (c + 1) / 2 units before it
+            int c = (int)((sqrtf(8.f * (float)u + 1.f) - 1.f) * 0.5f);
+            while ((c + 1) * (c + 2) / 2 <= u) ++c;
+            while (c * (c + 1) / 2 > u) --c;
+            m = u - c * (c + 1) / 2; t.n = c; t.prob = 0;
+        }
+        t.m = 2 * m + rank;
+        t.arow = roff + t.m * BM; t.brow = roff + t.n * BN + rank * BM;
     } else if (p.tiles) {
         const int4 e = p.tiles[u];
         const int roff = p.probs[e.x].roff;
@@ -374,14 +453,18 @@ __device__ __forceinline__ void wait_store_slot(int nob) {
 
 // AMAX: the ARGMAX and TOP2 modes (one instantiation for SIM, one for these, so
 // that neither epilogue's registers limit the other).
-template <bool AMAX>
+template <bool AMAX, bool PAIR>
 __global__ void __launch_bounds__(THREADS, 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                    const __grid_constant__ CUtensorMap tmOut, Params p) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                ~uintptr_t(1023));
-    uint8_t* out_base = base + (size_t)p.stages * STAGE_BYTES;
+    // PAIR (SIM): rank 0 issues the pair's MMAs and holds the barriers of what both
+    // CTAs load and read
+    constexpr int SB = PAIR ? PAIR_STAGE_BYTES : STAGE_BYTES;
+    const int rank = PAIR ? (int)(blockIdx.x & 1) : 0;
+    uint8_t* out_base = base + (size_t)p.stages * SB;
     // ARGMAX/TOP2 with folded norms: the augmented operands (A' then the B'
     // groups, 1024-byte aligned) sit between the store buffers and Ctl
     uint8_t* aug_base = out_base + (size_t)EPI_WARPS * p.nob * WBUF_BYTES;
@@ -395,7 +478,8 @@ __global__ void __launch_bounds__(THREADS, 1)
     // work units: one tile (SIM) or one row block with all its column tiles (ARGMAX, TOP2)
     constexpr bool amax = AMAX;
     // (SIM: without the last row block where the rows end in an odd one)
-    const int units = amax ? numM : (p.tiles ? p.ntiles : numN * (numN + 1) - (numM & 1));
+    const int u0 = PAIR ? blockIdx.x >> 1 : blockIdx.x, ustep = PAIR ? gridDim.x >> 1 : gridDim.x;
+    const int units = amax ? numM : p.tiles ? p.ntiles : PAIR ? numN * (numN + 1) / 2 : numN * (numN + 1) - (numM & 1);
     const int tiles_per_unit = amax ? numN : 1;
     const int ns = p.stages;
 
@@ -406,7 +490,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
         for (int b = 0; b < 2; ++b) {
             ptx::mbar_init(&sm.tfull[b], 1);
-            ptx::mbar_init(&sm.tempty[b], EPI_WARPS);
+            ptx::mbar_init(&sm.tempty[b], PAIR ? 2 * EPI_WARPS : EPI_WARPS);
         }
         for (int q = 0; q < 4; ++q) {
             ptx::mbar_init(&sm.mfull[q], 32);
@@ -416,13 +500,17 @@ __global__ void __launch_bounds__(THREADS, 1)
         ptx::fence_mbar_init();
         sm.abort = 0;
     }
-    if (warp == 1) tmem_alloc(&sm.tmem_base, TMEM_COLS);
+    if (warp == 1) {
+        if (PAIR) tmem_alloc_pair(&sm.tmem_base, TMEM_COLS);
+        else tmem_alloc(&sm.tmem_base, TMEM_COLS);
+    }
     if (p.aug > 0) {
         build_augmented(aug_base, p.bnrm, numN * BN, p.aug);
         ptx::fence_proxy_async_smem();               // generic stores -> the MMA's reads
     }
     tc_fence_before();
     __syncthreads();
+    if constexpr (PAIR) cg::this_cluster().sync();      // both CTAs' barriers are there
     tc_fence_after();
     const uint32_t tmem = sm.tmem_base;
 
@@ -430,39 +518,52 @@ __global__ void __launch_bounds__(THREADS, 1)
         // ---------------- TMA producer ----------------
         if (lane == 0) {
             int stage = 0;
-            uint32_t eph = 0xFu;                    // empty barriers start "released"
+            uint32_t eph = (1u << MAX_STAGES) - 1u; // empty barriers start "released"
             uint32_t armed = 0;                     // loads issued per stage (low bit = parity)
             int nissued = 0;
-            for (int u = blockIdx.x; u < units && !aborted(sm); u += gridDim.x) {
+            for (int u = u0; u < units && !aborted(sm); u += ustep) {
                 for (int q = 0; q < tiles_per_unit && !aborted(sm); ++q) {
-                    const Tile t = tile_of<AMAX>(p, numN, u, q);
+                    const Tile t = tile_of<AMAX, PAIR>(p, numN, u, q, rank);
                     for (int kb = 0; kb < numK; ++kb) {
                         if (!ptx::mbar_wait(&sm.empty[stage], (eph >> stage) & 1u, p.spin_limit)) {
                             atomicExch(&sm.abort, 1);
                             break;
                         }
                         eph ^= 1u << stage;
-                        uint8_t* st = base + (size_t)stage * STAGE_BYTES;
-                        ptx::mbar_arrive_expect_tx(&sm.full[stage], STAGE_BYTES);
-                        tma_load_2d(st, &tmA, kb * BK, t.arow, &sm.full[stage]);
-                        tma_load_2d(st + A_BYTES, &tmB, kb * BK, t.brow, &sm.full[stage]);
+                        uint8_t* st = base + (size_t)stage * SB;
+                        if constexpr (PAIR) {
+                            if (rank == 0) ptx::mbar_arrive_expect_tx(&sm.full[stage], 2 * SB);
+                            const uint32_t bar = ptx::mapa(&sm.full[stage], 0);
+                            tma_load_2d_pair(st, &tmA, kb * BK, t.arow, bar);
+                            tma_load_2d_pair(st + A_BYTES, &tmB, kb * BK, t.brow, bar);
+                        } else {
+                            ptx::mbar_arrive_expect_tx(&sm.full[stage], SB);
+                            tma_load_2d(st, &tmA, kb * BK, t.arow, &sm.full[stage]);
+                            tma_load_2d(st + A_BYTES, &tmB, kb * BK, t.brow, &sm.full[stage]);
+                        }
                         armed ^= 1u << stage;
                         ++nissued;
                         stage = (stage + 1 == ns) ? 0 : stage + 1;
                     }
                 }
             }
-            // loads still in flight must land before shared memory is released
-            for (int s = 0; s < ns && s < nissued; ++s)
-                ptx::mbar_wait(&sm.full[s], ((armed >> s) & 1u) ^ 1u, p.spin_limit);
+            // PAIR: every release has arrived here before this CTA may leave
+            if (PAIR)
+                for (int s = 0; s < ns && s < nissued && !aborted(sm); ++s)
+                    ptx::mbar_wait(&sm.empty[s], (eph >> s) & 1u, p.spin_limit);
+            // loads still in flight must land before shared memory is released (a
+            // pair's complete on rank 0's barriers, and the pair leaves together)
+            if (rank == 0)
+                for (int s = 0; s < ns && s < nissued; ++s)
+                    ptx::mbar_wait(&sm.full[s], ((armed >> s) & 1u) ^ 1u, p.spin_limit);
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
-        if (lane == 0) {
-            constexpr uint32_t idesc = instr_desc(BM, BN);
+        if (lane == 0 && rank == 0) {
+            constexpr uint32_t idesc = instr_desc(PAIR ? 2 * BM : BM, BN);
             int stage = 0, acc = 0;
             uint32_t fph = 0, tph = 3;              // tempty barriers start "released"
-            for (int u = blockIdx.x; u < units && !aborted(sm); u += gridDim.x) {
+            for (int u = u0; u < units && !aborted(sm); u += ustep) {
                 for (int q = 0; q < tiles_per_unit && !aborted(sm); ++q) {
                     if (!ptx::mbar_wait(&sm.tempty[acc], (tph >> acc) & 1u, p.spin_limit)) {
                         atomicExch(&sm.abort, 1);
@@ -478,19 +579,25 @@ __global__ void __launch_bounds__(THREADS, 1)
                         }
                         fph ^= 1u << stage;
                         tc_fence_after();
-                        const uint8_t* st = base + (size_t)stage * STAGE_BYTES;
+                        const uint8_t* st = base + (size_t)stage * SB;
                         const uint64_t ad = smem_desc(st);
                         const uint64_t bd = smem_desc(st + A_BYTES);
 #pragma unroll
                         for (int k = 0; k < BK / 16; ++k) {
                             // advance 16 bf16 (32 B) along K inside the swizzle atom
-                            mma_bf16(d, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 2), idesc,
-                                     (kb > 0 || k > 0) ? 1u : 0u);
+                            if (PAIR)
+                                mma_bf16_pair(d, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 2), idesc,
+                                              (kb > 0 || k > 0) ? 1u : 0u);
+                            else
+                                mma_bf16(d, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 2), idesc,
+                                         (kb > 0 || k > 0) ? 1u : 0u);
                         }
-                        mma_commit(&sm.empty[stage]);  // frees the stage once these MMAs are done
+                        // frees the stage once these MMAs are done
+                        if (PAIR) mma_commit_pair(&sm.empty[stage]);
+                        else mma_commit(&sm.empty[stage]);
                         stage = (stage + 1 == ns) ? 0 : stage + 1;
                     }
-                    if (p.aug > 0) {
+                    if (AMAX && p.aug > 0) {
                         // + 1 . (-h - m - l) = -|b|^2/2 for every row: column tile q is
                         // K block q % 4 of B' group q / 4 (A' holds the ones in every block)
                         const uint64_t ad = smem_desc(aug_base) + (uint64_t)((q & 3) * 2);
@@ -498,12 +605,14 @@ __global__ void __launch_bounds__(THREADS, 1)
                                             (uint64_t)((q & 3) * 2);
                         mma_bf16(d, ad, bd, idesc, 1u);
                     }
-                    mma_commit(&sm.tfull[acc]);        // accumulator ready for the epilogue
+                    if (PAIR) mma_commit_pair(&sm.tfull[acc]);     // accumulator ready for the epilogue
+                    else mma_commit(&sm.tfull[acc]);
                     acc ^= 1;
                 }
             }
             // no MMA may still write tensor memory when it is released
-            mma_commit(&sm.mma_done);
+            if (PAIR) mma_commit_pair_local(&sm.mma_done);
+            else mma_commit(&sm.mma_done);
             ptx::mbar_wait(&sm.mma_done, 0, p.spin_limit);
         }
     } else {
@@ -530,7 +639,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             asm volatile("bar.sync 1, %0;" ::"n"(32 * EPI_WARPS) : "memory");
         }
         const float* nrm = (amax && p.snrm > 0) ? snrm : p.bnrm;
-        for (int u = blockIdx.x; u < units && !dead; u += gridDim.x) {
+        for (int u = u0; u < units && !dead; u += ustep) {
             float best = -INFINITY;                  // ARGMAX/TOP2: max of x.e - |e|^2/2
             int bidx = INT_MAX;
             int bchunk = -1;                         // ARGMAX: first column of the chunk holding best
@@ -541,7 +650,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             int bidx2 = INT_MAX;
             int m0 = 0;
             for (int q = 0; q < tiles_per_unit; ++q) {
-                const Tile t = tile_of<AMAX>(p, numN, u, q);
+                const Tile t = tile_of<AMAX, PAIR>(p, numN, u, q, rank);
                 m0 = t.m;
                 uint32_t ok = 1;
                 if (lane == 0)
@@ -624,7 +733,8 @@ __global__ void __launch_bounds__(THREADS, 1)
                         ptx::fence_proxy_async_smem();
                         __syncwarp();
                         if (lane == 0) {
-                            if (kcol < n4) tma_store_2d(omap, kcol, t.m * BM + sub * 32, buf);
+                            if (kcol < n4 && t.m * BM + sub * 32 < Mloc)
+                                tma_store_2d(omap, kcol, t.m * BM + sub * 32, buf);
                             ptx::bulk_commit();
                         }
                         ob = (ob + 1 == p.nob) ? 0 : ob + 1;
@@ -752,7 +862,10 @@ __global__ void __launch_bounds__(THREADS, 1)
                 // accumulator drained: hand it back to the MMA warp
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(&sm.tempty[acc]);
+                if (lane == 0) {
+                    if (PAIR) mbar_arrive_cluster(ptx::mapa(&sm.tempty[acc], 0));
+                    else ptx::mbar_arrive(&sm.tempty[acc]);
+                }
                 acc ^= 1;
             }
             if (dead) break;
@@ -817,9 +930,11 @@ __global__ void __launch_bounds__(THREADS, 1)
 
     tc_fence_before();
     __syncthreads();
+    if constexpr (PAIR) cg::this_cluster().sync();      // the peer's loads, MMAs and arrivals are done with this CTA
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem, TMEM_COLS);
+        if (PAIR) tmem_dealloc_pair(tmem, TMEM_COLS);
+        else tmem_dealloc(tmem, TMEM_COLS);
     }
     if (threadIdx.x == 0 && aborted(sm) && p.error) atomicExch(p.error, 1);
 }
@@ -1155,17 +1270,27 @@ static int32_t make_out_map(CUtensorMap* map, float* S, int n, int64_t lds) {
                     (uint64_t)lds * 4, OUT_COLS, 32, CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
+// Whether the similarity goes by CTA pairs (half of B's traffic from L2 per CTA):
+// products long enough to be bound by that, with enough of the lone CTAs'
+// 128 x 256 tiles that a pair's coarser ones fill the SMs.  Measured calls, pairs
+// against lone CTAs: 8000 points, d = 4096 427 to 446 us, d = 2048 327 to 336; a batch
+// of 32, d = 4096 1410 to 1478; but 2000 points, d = 4096 184 to 177, and 20000
+// points, d = 300 802 to 787.
+static bool pairs(int numK, int64_t tiles) { return numK >= 32 && tiles >= 608; }
+
 // Operand stages and store buffers: a long product (K >= 256) wants a deep
 // operand ring and writes S slowly; a short one is bound by writing S.
-static void layout_for(int mode, int numK, int* stages, int* nob) {
+static void layout_for(int mode, int numK, bool pair, int* stages, int* nob) {
     if (mode != SIM) { *stages = 3; *nob = 0; }   // (measured no slower than 4 at K = 128)
+    else if (pair) { *stages = 6; *nob = 1; }
     else if (numK >= 4) { *stages = 4; *nob = 1; }
     else if (numK >= 2) { *stages = 3; *nob = 2; }
     else { *stages = 2; *nob = 4; }
 }
 
-static size_t smem_bytes(int mode, int stages, int nob) {
-    return 1024 + (size_t)stages * STAGE_BYTES + (size_t)EPI_WARPS * nob * WBUF_BYTES + sizeof(Ctl) +
+static size_t smem_bytes(int mode, bool pair, int stages, int nob) {
+    return 1024 + (size_t)stages * (pair ? PAIR_STAGE_BYTES : STAGE_BYTES) +
+           (size_t)EPI_WARPS * nob * WBUF_BYTES + sizeof(Ctl) +
            (mode != SIM ? sizeof(Slots) : 0);
 }
 
@@ -1183,11 +1308,11 @@ static int assign_norm_form() {
 }
 
 static int32_t launch(const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& o, Params p,
-                      int units, cudaStream_t s) {
+                      int units, cudaStream_t s, bool pair = false) {
     int sms = 0;
     AP_TRY(device_sm_count(&sms));
-    layout_for(p.mode, p.K / BK, &p.stages, &p.nob);
-    size_t bytes = smem_bytes(p.mode, p.stages, p.nob);
+    layout_for(p.mode, p.K / BK, pair, &p.stages, &p.nob);
+    size_t bytes = smem_bytes(p.mode, pair, p.stages, p.nob);
     if (bytes > (size_t)SMEM_LIMIT) return AP_ERR_UNSUPPORTED;
     // ARGMAX/TOP2: how -|b|^2/2 enters the scores.  Folded into the product
     // by one extra K = 16 MMA per tile where the augmented operands fit
@@ -1209,11 +1334,25 @@ static int32_t launch(const CUtensorMap& a, const CUtensorMap& b, const CUtensor
             bytes += npad * 4;
         }
     }
-    const auto kernel = p.mode == SIM ? tc_gemm_kernel<false> : tc_gemm_kernel<true>;
+    const auto kernel = p.mode != SIM ? tc_gemm_kernel<true, false>
+                        : pair        ? tc_gemm_kernel<false, true>
+                                      : tc_gemm_kernel<false, false>;
     AP_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT));
-    // persistent: one CTA per SM, each taking every gridDim-th unit
-    const int grid = std::max(1, std::min(units, sms));
-    kernel<<<grid, THREADS, bytes, s>>>(a, b, o, p);
+    // persistent: one CTA per SM (or a pair on two), each taking every gridDim-th unit
+    const int per = pair ? 2 : 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(per * std::max(1, std::min(units, sms / per))), 1, 1);
+    cfg.blockDim = dim3(THREADS, 1, 1);
+    cfg.dynamicSmemBytes = bytes;
+    cfg.stream = s;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)per;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = pair ? 1 : 0;
+    AP_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, a, b, o, p));
     note_launches(1);
     return last_error();
 }
@@ -1230,11 +1369,13 @@ int32_t tc_similarity_bf16(const __nv_bfloat16* Xb, const float* nrm, int n, int
     using namespace tc;
     if (dpad % BK || (lds & 3) || !aligned16(S)) return AP_ERR_INVALID_ARG;
     const int npad = (n + BN - 1) / BN * BN;
+    const int nm = (n + BM - 1) / BM, nn = (n + BN - 1) / BN;
+    const bool pair = pairs(dpad / BK, (int64_t)nn * (nn + 1));
     CUtensorMap ma, mb, mo;
     AP_TRY(make_map(&ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (void*)Xb, dpad, npad, (uint64_t)dpad * 2,
                     BK, BM, CU_TENSOR_MAP_SWIZZLE_128B));
     AP_TRY(make_map(&mb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (void*)Xb, dpad, npad, (uint64_t)dpad * 2,
-                    BK, BN, CU_TENSOR_MAP_SWIZZLE_128B));
+                    BK, pair ? BM : BN, CU_TENSOR_MAP_SWIZZLE_128B));
     AP_TRY(make_out_map(&mo, S, n, lds));
     Params p{};
     p.M = n;
@@ -1249,8 +1390,7 @@ int32_t tc_similarity_bf16(const __nv_bfloat16* Xb, const float* nrm, int n, int
     p.lds = lds;
     p.spin_limit = 1u << 22;
     p.error = err;
-    const int nm = (n + BM - 1) / BM, nn = (n + BN - 1) / BN;
-    return launch(ma, mb, mo, p, nn * (nn + 1) - (nm & 1), s);
+    return launch(ma, mb, mo, p, pair ? nn * (nn + 1) / 2 : nn * (nn + 1) - (nm & 1), s, pair);
 }
 
 // Device bytes of the tables of a grouped similarity over problems of sizes
@@ -1286,6 +1426,9 @@ int32_t tc_similarity_bf16_grouped(const __nv_bfloat16* Xb, const float* nrm, in
     std::vector<CUtensorMap> maps(count);
     std::vector<GroupProblem> probs(count);
     std::vector<int4> tiles;
+    int64_t lone = 0;
+    for (int32_t b = 0; b < count; ++b) lone += (n[b] + BN - 1) / BN * ((n[b] + BN - 1) / BN + 1);
+    const bool pair = pairs(dpad / BK, lone);
     for (int32_t b = 0; b < count; ++b) {
         const int nb = (int)n[b];
         if ((lds[b] & 3) || !aligned16(S[b]) || roff[b] % BN || roff[b] + (nb + BN - 1) / BN * BN > rows)
@@ -1294,7 +1437,7 @@ int32_t tc_similarity_bf16_grouped(const __nv_bfloat16* Xb, const float* nrm, in
         probs[b] = GroupProblem{dmaps + b, S[b], lds[b], (int32_t)roff[b], nb, nb & ~3, 0};
         const int mb = (nb + BM - 1) / BM, nbk = (nb + BN - 1) / BN;
         for (int j = 0; j < nbk; ++j)
-            for (int i = 0; i < std::min(mb, 2 * j + 2); ++i) tiles.push_back(make_int4(b, i, j, 0));
+            for (int i = 0; i < (pair ? j + 1 : std::min(mb, 2 * j + 2)); ++i) tiles.push_back(make_int4(b, i, j, 0));
     }
     int4* dtiles = c.take<int4>(tiles.size());
     AP_CUDA_TRY(cudaMemcpyAsync(dmaps, maps.data(), sizeof(CUtensorMap) * count, cudaMemcpyHostToDevice, s));
@@ -1303,8 +1446,8 @@ int32_t tc_similarity_bf16_grouped(const __nv_bfloat16* Xb, const float* nrm, in
     CUtensorMap ma, mb;
     AP_TRY(make_map(&ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (void*)Xb, dpad, rows, (uint64_t)dpad * 2, BK, BM,
                     CU_TENSOR_MAP_SWIZZLE_128B));
-    AP_TRY(make_map(&mb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (void*)Xb, dpad, rows, (uint64_t)dpad * 2, BK, BN,
-                    CU_TENSOR_MAP_SWIZZLE_128B));
+    AP_TRY(make_map(&mb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (void*)Xb, dpad, rows, (uint64_t)dpad * 2, BK,
+                    pair ? BM : BN, CU_TENSOR_MAP_SWIZZLE_128B));
     Params p{};
     p.M = p.N = 0;
     p.K = dpad;
@@ -1318,7 +1461,7 @@ int32_t tc_similarity_bf16_grouped(const __nv_bfloat16* Xb, const float* nrm, in
     p.spin_limit = 1u << 22;
     p.error = err;
     // the output map argument is unused in grouped mode (each problem has its own)
-    return launch(ma, mb, maps[0], p, p.ntiles, s);
+    return launch(ma, mb, maps[0], p, p.ntiles, s, pair);
 }
 
 // arg[i] = argmax_j (2 a_i . b_j - bnrm_j), j < nb; A [>= na rows x dpad],

@@ -121,3 +121,24 @@ def test_full_size_batch_sampled_problems_match_oracle():
         ref = oap.run(ref_S[b].astype(np.float64), lam=0.9, fixed_iters=10)
         for got, want in ((R, ref["R"]), (A, ref["A"])):
             assert np.abs(got - want).max() <= 1e-4 * np.abs(want).max(), b
+
+
+@pytest.mark.parametrize("d", [2000, 2048, 4100])
+def test_similarity_batched_by_pairs_equals_single(d):
+    """Enough tiles of long products go by CTA pairs (256 x 256 tiles); a problem
+    alone goes by lone CTAs (128 x 256): the same bits at the tiles' edges."""
+    g = np.random.default_rng(d)
+    n = [3000, 2, 127, 128, 129, 255, 2817, 256, 257, 385, 2945, 512, 3073]
+    xoff = np.concatenate([[0], np.cumsum(n)[:-1]]) * d
+    X = torch.from_numpy(g.normal(size=(sum(n), d)).astype(np.float32)).cuda()
+    ld = [capi.padded_ld(v) for v in n]
+    off = [int(v) for v in np.concatenate([[0], np.cumsum([a * b for a, b in zip(n, ld)])[:-1]])]
+    S = torch.full((sum(a * b for a, b in zip(n, ld)),), float("nan"), device="cuda")
+    prefs = capi.ap_similarity_batched(X, [int(v) for v in xoff], n, S, off, ld, precision="bf16")
+    at = 0
+    for b, v in enumerate(n):
+        Sb = S[off[b]:off[b] + v * ld[b]].view(v, ld[b])
+        one, p = capi.ap_similarity(X[at:at + v], precision="bf16")
+        assert torch.equal(Sb[:, :v], one) and prefs[b] == p
+        assert torch.isnan(Sb[:, v:]).all()
+        at += v
