@@ -634,9 +634,14 @@ sweep_kernel(SweepLaunch L) {
 // the rows i = l mod 32 in turn (rows of CTA l mod 16, every second one), then
 // the lanes meet in its tree, so the results are the same bits as by launches.
 // R_{t-1}, which a stop found at step t returns, is kept in the workspace from
-// the step on at which the run could stop.  500 points, 100 iterations:
-// 697 us for the whole call where launches took 1147 us; the rule is that the three matrices fit
-// (up to about 540 points) and that the launches' units are single rows.
+// the step on at which the run could stop.  A row's inner loop has no special
+// elements: the diagonal's new value is patched in by its lane, R_ii lives in
+// rdg between row phases (sR has a zero there, which is what the column sums
+// take), and what lies past the row's end is -inf.  500 points, 100 iterations:
+// 635 us for the whole call where launches took 1147 us (697 us with separate
+// code for the diagonal's float4 and arg-max selects for every element); the rule
+// is that the three matrices fit (up to 544 points) and that the launches' units
+// are single rows.
 // ---------------------------------------------------------------------------
 constexpr int kResCtas = 16, kResThreads = 512, kResWarps = kResThreads / 32;
 constexpr int kResQ = 5;                // float4 per lane and row: n4 <= 160
@@ -652,13 +657,15 @@ struct ResidentArgs {
 static size_t resident_smem(int n) {
     const size_t n4 = (n + 3) / 4, rows = (n + kResCtas - 1) / kResCtas, cw = (n + kResCtas - 1) / kResCtas;
     return 3 * rows * n4 * 16 + 2 * n4 * 16 +              // S, R, A; (1 - lambda) c and colp
-           (32 * cw + 3 * cw) * 4 + 2 * rows * 4 + 64;     // received sums, diagonal, results; flags, decisions
+           (32 * (cw | 1) + 3 * cw) * 4 + 2 * rows * 4 + 64;   // received sums (odd stride), diagonal, results;
+                                                            // flags, the rows' diagonals of R
 }
 
 __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_constant__ ResidentArgs p) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int2 cnt[kResCtas];                          // every CTA's (changes, exemplars)
     __shared__ int own_changes, own_ex, own_bad;
+    __shared__ int2 total;                                  // their sum
     cg::cluster_group cluster = cg::this_cluster();
     const SweepArgs& a = p.a;
     const int b = (int)cluster.block_rank();
@@ -670,11 +677,14 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
     float4* sA = sR + (size_t)p.rows * n4;
     float4* cvs = sA + (size_t)p.rows * n4;
     float* colps = reinterpret_cast<float*>(cvs + n4);
-    float* recv = colps + 4 * n4;                           // [32][cw]
-    float* rdiag = recv + 32 * cw;
+    const int rs = cw | 1;                                  // (odd: lanes read a column of it)
+    float* recv = colps + 4 * n4;                           // [32][rs]
+    float* rdiag = recv + 32 * rs;
     float* res = rdiag + cw;                                // [2][cw]: c and colp of this CTA's columns
     int* flags = reinterpret_cast<int*>(res + 2 * cw);
-    int* decs = flags + p.rows;
+    float* rdg = reinterpret_cast<float*>(flags + p.rows);  // R_ii: sR has a zero there, for the column sums
+    // the reducer of column tid, and of column tid + 512
+    const int dst0 = tid / cw, c0 = tid - dst0 * cw, dst1 = (tid + kResThreads) / cw, c1 = tid + kResThreads - dst1 * cw;
     const float lam = a.lam, oml = 1.0f - a.lam;
     const float2 lam2 = make_float2(lam, lam), oml2 = make_float2(oml, oml), nom2 = make_float2(-oml, -oml);
 
@@ -692,11 +702,29 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
             bad += 4 * f + 2 < n && !isfinite(s4.z);
             bad += 4 * f + 3 < n && !isfinite(s4.w);
         }
-        sS[e] = s4;
-        sR[e] = a.zero ? z : *reinterpret_cast<const float4*>(a.R0 + off);
-        sA[e] = a.zero ? z : *reinterpret_cast<const float4*>(a.A + off);
+        float4 r4 = a.zero ? z : *reinterpret_cast<const float4*>(a.R0 + off);
+        float4 a4 = a.zero ? z : *reinterpret_cast<const float4*>(a.A + off);
+        float4 t4 = s4;
+        // past the row's end: never a maximum, and finite where it is added
+#pragma unroll
+        for (int x = 1; x < 4; ++x)
+            if (4 * f + x >= n) {
+                set_lane(t4, x, -INFINITY);
+                set_lane(r4, x, -INFINITY);
+                set_lane(a4, x, 0.f);
+            }
+        sS[e] = t4;
+        sR[e] = r4;
+        sA[e] = a4;
     }
-    for (int r = tid; r < m; r += kResThreads) flags[r] = decs[r] = 0;
+    for (int k = tid; k < n4; k += kResThreads) cvs[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    __syncthreads();
+    for (int r = tid; r < m; r += kResThreads) {
+        const int at = r * 4 * n4 + b + kResCtas * r;
+        flags[r] = 0;
+        rdg[r] = reinterpret_cast<float*>(sR)[at];
+        reinterpret_cast<float*>(sR)[at] = 0.f;
+    }
     if (p.check) {
         bad = __reduce_add_sync(0xffffffffu, bad);
         if (lid == 0 && bad) atomicAdd(&own_bad, bad);
@@ -725,152 +753,184 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
         // this step may turn out to be the last: keep R_{t-1}
         const bool keep = doR && doA && p.conv_iter > 0 && stable + 1 >= p.conv_iter;
         for (int r = wid; r < m; r += kResWarps) {
-            const int i = b + kResCtas * r, fi = i >> 2;
+            const int i = b + kResCtas * r, di4 = i >> 2, de = i & 3;     // the diagonal: float4 di4 of the row
+            float* Sr = reinterpret_cast<float*>(sS + r * n4);
+            float* Rr = reinterpret_cast<float*>(sR + r * n4);
+            float* Ar = reinterpret_cast<float*>(sA + r * n4);
+            const float rii = rdg[r];
+            const float aii = doA ? fmaf(lam, Ar[i], oml * colps[i]) : Ar[i];
+            const float di = aii + rii;
+            if (lid == 0) Rr[i] = rii;
+            __syncwarp();                                   // Ar[i] has been read, Rr[i] written
             float4 s4[kResQ], r4[kResQ];
-            Top2 tp{-INFINITY, -INFINITY, INT_MAX};
-            float dv = -INFINITY;
-            int dj = INT_MAX;
+            // the lane's largest and second largest a + s, and the float4 of the
+            // first; the largest a + r
+            float m1 = -INFINITY, m2 = -INFINITY, dv = -INFINITY;
+            int jq = 0;
 #pragma unroll
             for (int q = 0; q < kResQ; ++q) {
-                const int f = lid + 32 * q, x = r * n4 + f;
+                const int f = lid + 32 * q;
                 if (f < n4) {
-                    s4[q] = sS[x];
-                    r4[q] = sR[x];
-                    float4 a4 = sA[x];
-                    const float4 cv = doA ? cvs[f] : make_float4(0.f, 0.f, 0.f, 0.f);
-                    // the availability half, the decision and the top-2, as in
-                    // sweep_kernel (columns reach a lane in increasing order)
-                    if (f != fi && f < nfull) {
-                        const int k0 = 4 * f;
-                        float2 alo = make_float2(a4.x, a4.y), ahi = make_float2(a4.z, a4.w);
-                        if (doA) {
-                            const float2 tlo = __ffma2_rn(nom2, make_float2(fmaxf(0.f, r4[q].x), fmaxf(0.f, r4[q].y)),
-                                                          make_float2(cv.x, cv.y));
-                            const float2 thi = __ffma2_rn(nom2, make_float2(fmaxf(0.f, r4[q].z), fmaxf(0.f, r4[q].w)),
-                                                          make_float2(cv.z, cv.w));
-                            alo = __ffma2_rn(lam2, alo, make_float2(fminf(0.f, tlo.x), fminf(0.f, tlo.y)));
-                            ahi = __ffma2_rn(lam2, ahi, make_float2(fminf(0.f, thi.x), fminf(0.f, thi.y)));
-                            const float2 dlo = __fadd2_rn(alo, make_float2(r4[q].x, r4[q].y));
-                            const float2 dhi = __fadd2_rn(ahi, make_float2(r4[q].z, r4[q].w));
-                            if (dlo.x > dv) { dv = dlo.x; dj = k0; }
-                            if (dlo.y > dv) { dv = dlo.y; dj = k0 + 1; }
-                            if (dhi.x > dv) { dv = dhi.x; dj = k0 + 2; }
-                            if (dhi.y > dv) { dv = dhi.y; dj = k0 + 3; }
-                            a4 = make_float4(alo.x, alo.y, ahi.x, ahi.y);
-                        }
-                        if (doR) {
-                            const float2 vlo = __fadd2_rn(alo, make_float2(s4[q].x, s4[q].y));
-                            const float2 vhi = __fadd2_rn(ahi, make_float2(s4[q].z, s4[q].w));
-                            float v;
-                            v = vlo.x; tp.m2 = fmaxf(tp.m2, fminf(tp.m1, v)); if (v > tp.m1) { tp.m1 = v; tp.j1 = k0; }
-                            v = vlo.y; tp.m2 = fmaxf(tp.m2, fminf(tp.m1, v)); if (v > tp.m1) { tp.m1 = v; tp.j1 = k0 + 1; }
-                            v = vhi.x; tp.m2 = fmaxf(tp.m2, fminf(tp.m1, v)); if (v > tp.m1) { tp.m1 = v; tp.j1 = k0 + 2; }
-                            v = vhi.y; tp.m2 = fmaxf(tp.m2, fminf(tp.m1, v)); if (v > tp.m1) { tp.m1 = v; tp.j1 = k0 + 3; }
-                        }
-                    } else {
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const int k = 4 * f + e;
-                            if (k < n) {
-                                const float rv = lane(r4[q], e);
-                                float av = lane(a4, e);
-                                if (doA) {
-                                    const float an = (k == i) ? oml * colps[i]
-                                                              : fminf(0.f, fmaf(-oml, fmaxf(0.f, rv), lane(cv, e)));
-                                    av = fmaf(lam, av, an);
-                                    set_lane(a4, e, av);
-                                    const float d = av + rv;
-                                    if (d > dv) { dv = d; dj = k; }
-                                }
-                                if (doR) {
-                                    const float v = av + lane(s4[q], e);
-                                    tp.m2 = fmaxf(tp.m2, fminf(tp.m1, v));
-                                    if (v > tp.m1) { tp.m1 = v; tp.j1 = k; }
-                                }
-                            }
-                        }
+                    s4[q] = sS[r * n4 + f];
+                    r4[q] = sR[r * n4 + f];
+                    float4 a4 = sA[r * n4 + f];
+                    if (doA) {
+                        // the arithmetic of sweep_kernel
+                        const float4 cv = cvs[f];
+                        const float2 tlo = __ffma2_rn(nom2, make_float2(fmaxf(0.f, r4[q].x), fmaxf(0.f, r4[q].y)),
+                                                      make_float2(cv.x, cv.y));
+                        const float2 thi = __ffma2_rn(nom2, make_float2(fmaxf(0.f, r4[q].z), fmaxf(0.f, r4[q].w)),
+                                                      make_float2(cv.z, cv.w));
+                        const float2 alo = __ffma2_rn(lam2, make_float2(a4.x, a4.y),
+                                                      make_float2(fminf(0.f, tlo.x), fminf(0.f, tlo.y)));
+                        const float2 ahi = __ffma2_rn(lam2, make_float2(a4.z, a4.w),
+                                                      make_float2(fminf(0.f, thi.x), fminf(0.f, thi.y)));
+                        a4 = make_float4(alo.x, alo.y, ahi.x, ahi.y);
                     }
-                    if (doA) sA[x] = a4;
+                    if (q == di4 >> 5 && lid == (di4 & 31)) {         // the diagonal's own value
+                        a4.x = de == 0 ? aii : a4.x;
+                        a4.y = de == 1 ? aii : a4.y;
+                        a4.z = de == 2 ? aii : a4.z;
+                        a4.w = de == 3 ? aii : a4.w;
+                    }
+                    if (doA) {
+                        sA[r * n4 + f] = a4;
+                        const float2 dlo = __fadd2_rn(make_float2(a4.x, a4.y), make_float2(r4[q].x, r4[q].y));
+                        const float2 dhi = __fadd2_rn(make_float2(a4.z, a4.w), make_float2(r4[q].z, r4[q].w));
+                        dv = fmaxf(fmaxf(dv, fmaxf(dlo.x, dlo.y)), fmaxf(dhi.x, dhi.y));
+                    }
+                    if (doR) {
+                        const float2 vlo = __fadd2_rn(make_float2(a4.x, a4.y), make_float2(s4[q].x, s4[q].y));
+                        const float2 vhi = __fadd2_rn(make_float2(a4.z, a4.w), make_float2(s4[q].z, s4[q].w));
+                        const float h0 = fmaxf(vlo.x, vlo.y), l0 = fminf(vlo.x, vlo.y);
+                        const float h1 = fmaxf(vhi.x, vhi.y), l1 = fminf(vhi.x, vhi.y);
+                        const float hi = fmaxf(h0, h1);
+                        const float second = fmaxf(fminf(h0, h1), fmaxf(l0, l1));
+                        m2 = fmaxf(fmaxf(m2, second), fminf(m1, hi));
+                        if (hi > m1) { m1 = hi; jq = q; }
+                    }
                 }
             }
             if (doA) {
-                argmax_warp_redux(dv, dj);
+                // the point chose itself: nothing is larger than the diagonal's a + r,
+                // and nothing before it as large
+                int self = di == warp_max_f32(dv) && di > -INFINITY ? 1 : 0;
+                if (self) {
+                    bool before = false;
+                    __syncwarp();
+                    for (int k = lid; k < i; k += 32) before = before || Ar[k] + Rr[k] == di;
+                    self = __any_sync(0xffffffffu, before) ? 0 : 1;
+                }
                 if (lid == 0) {
-                    const int e = (dj == i) ? 1 : 0;
-                    if (flags[r] != e) atomicAdd(&own_changes, 1);
-                    if (e) atomicAdd(&own_ex, 1);
-                    flags[r] = e;
-                    decs[r] = dj;
+                    if (flags[r] != self) atomicAdd(&own_changes, 1);
+                    if (self) atomicAdd(&own_ex, 1);
+                    flags[r] = self;
                 }
             }
             if (doR) {
-                tp = top2_warp_redux(tp);
+                // the row's largest, the lowest index that attains it, and the second largest
+                Top2 tp;
+                tp.m1 = warp_max_f32(m1);
+                int j = INT_MAX;
+                if (m1 == tp.m1 && lid + 32 * jq < n4) {
+                    const int f = lid + 32 * jq;
+                    const float4 a4 = sA[r * n4 + f], q4 = sS[r * n4 + f];
+                    const float v[4] = {a4.x + q4.x, a4.y + q4.y, a4.z + q4.z, a4.w + q4.w};
+#pragma unroll
+                    for (int e = 3; e >= 0; --e)
+                        if (v[e] == m1 && 4 * f + e < n) j = 4 * f + e;
+                }
+                tp.j1 = __reduce_min_sync(0xffffffffu, j);
+                tp.m2 = warp_max_f32(j == tp.j1 ? m2 : m1);
                 const float om1 = oml * tp.m1, om2 = oml * tp.m2;
+                const float2 nm1 = make_float2(-om1, -om1);
+                // the row's largest takes the second largest
+                const int jj = min(tp.j1, n - 1);           // (no largest among NaNs)
+                const float ov = fmaf(lam, Rr[jj], fmaf(oml, Sr[jj], -om2));
+                __syncwarp();                               // Rr[jj] has been read
 #pragma unroll
                 for (int q = 0; q < kResQ; ++q) {
-                    const int f = lid + 32 * q, x = r * n4 + f;
+                    const int f = lid + 32 * q;
                     if (f < n4) {
                         if (keep) *reinterpret_cast<float4*>(a.R1 + (int64_t)i * a.ld + 4 * f) = r4[q];
-                        const float2 nm1 = make_float2(-om1, -om1);
                         const float2 olo = __ffma2_rn(lam2, make_float2(r4[q].x, r4[q].y),
                                                       __ffma2_rn(oml2, make_float2(s4[q].x, s4[q].y), nm1));
                         const float2 ohi = __ffma2_rn(lam2, make_float2(r4[q].z, r4[q].w),
                                                       __ffma2_rn(oml2, make_float2(s4[q].z, s4[q].w), nm1));
-                        float4 o = make_float4(olo.x, olo.y, ohi.x, ohi.y);
-                        if (f == tp.j1 >> 2) {              // the row's largest takes the second largest
-                            const int e = tp.j1 & 3;
-                            const float sv = e == 0 ? s4[q].x : e == 1 ? s4[q].y : e == 2 ? s4[q].z : s4[q].w;
-                            const float rv = e == 0 ? r4[q].x : e == 1 ? r4[q].y : e == 2 ? r4[q].z : r4[q].w;
-                            const float ov = fmaf(lam, rv, fmaf(oml, sv, -om2));
-                            o.x = e == 0 ? ov : o.x;
-                            o.y = e == 1 ? ov : o.y;
-                            o.z = e == 2 ? ov : o.z;
-                            o.w = e == 3 ? ov : o.w;
-                        }
-                        sR[x] = o;
+                        sR[r * n4 + f] = make_float4(olo.x, olo.y, ohi.x, ohi.y);
                     }
                 }
+                // (by the lanes that wrote these float4)
+                if (lid == ((tp.j1 >> 2) & 31) && tp.j1 < n) Rr[jj] = ov;
+                if (lid == (di4 & 31)) rdg[r] = Rr[i];
             }
+            if (lid == (di4 & 31)) Rr[i] = 0.f;
+            __syncwarp();
         }
         __syncthreads();
         if (doR) {
             // this CTA's two lanes of every column's sum, to the column's reducer
             const float* R = reinterpret_cast<const float*>(sR);
-            for (int k = tid; k < n; k += kResThreads) {
-                const int rd = (k % kResCtas == b) ? k / kResCtas : -1;       // the diagonal's row here
-                float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int k = tid + h * kResThreads, dst = h ? dst1 : dst0, c = h ? c1 : c0;
+                if (k >= n) break;
+                float s0 = 0.f, s1 = 0.f;                   // (the diagonal is a zero here)
                 int r = 0;
                 for (; r + 8 <= m; r += 8) {                // eight rows' reads in flight
                     float v[8];
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) v[e] = R[(size_t)(r + e) * 4 * n4 + k];
+                    for (int e = 0; e < 8; ++e) v[e] = R[(r + e) * 4 * n4 + k];
 #pragma unroll
                     for (int e = 0; e < 8; e += 2) {
-                        s0 += r + e == rd ? 0.f : fmaxf(0.f, v[e]);
-                        s1 += r + e + 1 == rd ? 0.f : fmaxf(0.f, v[e + 1]);
+                        s0 += fmaxf(0.f, v[e]);
+                        s1 += fmaxf(0.f, v[e + 1]);
                     }
                 }
                 for (; r < m; ++r) {
-                    const float v = r == rd ? 0.f : fmaxf(0.f, R[(size_t)r * 4 * n4 + k]);
+                    const float v = fmaxf(0.f, R[r * 4 * n4 + k]);
                     if (r & 1) s1 += v;
                     else s0 += v;
                 }
-                const int dst = k / cw, c = k - dst * cw;
                 float* to = cluster.map_shared_rank(recv, dst);
-                to[b * cw + c] = s0;
-                to[(b + kResCtas) * cw + c] = s1;
-                if (rd >= 0) *cluster.map_shared_rank(rdiag + c, dst) = R[(size_t)rd * 4 * n4 + k];
+                to[b * rs + c] = s0;
+                to[(b + kResCtas) * rs + c] = s1;
+                if (k % kResCtas == b) *cluster.map_shared_rank(rdiag + c, dst) = rdg[k / kResCtas];
             }
         }
         if (tid < kResCtas) *cluster.map_shared_rank(&cnt[b], tid) = make_int2(own_changes, own_ex);
         cluster.sync();
-        int changes = 0, n_ex = 0;
-#pragma unroll
-        for (int c = 0; c < kResCtas; ++c) {
-            const int2 x = cnt[c];
-            changes += x.x;
-            n_ex += x.y;
+        if (wid == kResWarps - 1) {
+            const int2 x = cnt[lid & (kResCtas - 1)];
+            const int ch = __reduce_add_sync(0xffffffffu, lid < kResCtas ? x.x : 0);
+            const int ex = __reduce_add_sync(0xffffffffu, lid < kResCtas ? x.y : 0);
+            if (lid == 0) total = make_int2(ch, ex);
         }
+        if (tid == 0) own_changes = own_ex = 0;
+        if (doR) {
+            // this CTA's columns: the 32 lane sums in finalize_kernel's tree (neighbours
+            // first), a warp a column; the results to every CTA
+            for (int c = wid; c < cw && b * cw + c < n; c += kResWarps) {
+                float v = recv[lid * rs + c];
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                if (lid == 0) {
+                    res[c] = oml * (rdiag[c] + v);
+                    res[cw + c] = v;
+                }
+            }
+            __syncthreads();
+            // to every CTA, a warp each
+            static_assert(kResWarps == kResCtas, "a warp a CTA");
+            float* to = cluster.map_shared_rank(reinterpret_cast<float*>(cvs), wid) + b * cw;
+            float* tp = cluster.map_shared_rank(colps, wid) + b * cw;
+            for (int c = lid; c < cw && b * cw + c < n; c += 32) {
+                to[c] = res[c];
+                tp[c] = res[cw + c];
+            }
+        }
+        cluster.sync();
+        const int changes = total.x, n_ex = total.y;
         // the stop rule (apply_stop_rule), the same in every thread of the cluster
         if (t >= 2) {
             const int it = t - 1;
@@ -886,28 +946,6 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
             iters = p.max_iter;
         }
         if (done) break;
-        // this CTA's columns: the 32 lane sums in finalize_kernel's tree
-        if (tid < cw && b * cw + tid < n) {
-            float v[32];
-#pragma unroll
-            for (int l = 0; l < 32; ++l) v[l] = recv[l * cw + tid];
-#pragma unroll
-            for (int w = 16; w >= 1; w >>= 1)
-#pragma unroll
-                for (int e = 0; e < w; ++e) v[e] = v[2 * e] + v[2 * e + 1];
-            res[tid] = oml * (rdiag[tid] + v[0]);
-            res[cw + tid] = v[0];
-        }
-        if (tid == 0) own_changes = own_ex = 0;
-        __syncthreads();
-        for (int e = tid; e < kResCtas * cw; e += kResThreads) {
-            const int dst = e / cw, c = e - dst * cw, k = b * cw + c;
-            if (k < n) {
-                cluster.map_shared_rank(reinterpret_cast<float*>(cvs), dst)[k] = res[c];
-                cluster.map_shared_rank(colps, dst)[k] = res[cw + c];
-            }
-        }
-        cluster.sync();
     }
     // the messages of iteration `iters`: R is one step ahead when a stop was found
     // at a step that formed R
@@ -915,9 +953,17 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
     for (int r = wid; r < m; r += kResWarps) {
         const int i = b + kResCtas * r;
         const int64_t off = (int64_t)i * a.ld;
+        float dv = -INFINITY;               // the decision: the lowest index of the largest a + r
+        int dj = INT_MAX;
         for (int f = lid; f < n4; f += 32) {
-            const float4 rv = kept ? *reinterpret_cast<const float4*>(a.R1 + off + 4 * f) : sR[r * n4 + f];
+            float4 rv = kept ? *reinterpret_cast<const float4*>(a.R1 + off + 4 * f) : sR[r * n4 + f];
+            if (!kept && f == i >> 2) set_lane(rv, i & 3, rdg[r]);
             const float4 av = sA[r * n4 + f];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float d = lane(av, e) + lane(rv, e);
+                if (4 * f + e < n && d > dv) { dv = d; dj = 4 * f + e; }
+            }
             if (f < nfull) {
                 *reinterpret_cast<float4*>(a.R0 + off + 4 * f) = rv;
                 *reinterpret_cast<float4*>(a.A + off + 4 * f) = av;
@@ -930,7 +976,8 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
                     }
             }
         }
-        if (a.dec && lid == 0) a.dec[i] = decs[r];
+        argmax_warp_redux(dv, dj);
+        if (a.dec && lid == 0) a.dec[i] = dj;
     }
     if (b == 0 && tid == 0) {
         SweepState s{};
@@ -1577,7 +1624,7 @@ static bool resident_supported() {
     std::lock_guard<std::mutex> lock(mu);
     auto it = known.find(dev);
     if (it != known.end()) return it->second;
-    bool ok = cudaFuncSetAttribute(resident_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024) ==
+    bool ok = cudaFuncSetAttribute(resident_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 512) ==
                   cudaSuccess &&
               cudaFuncSetAttribute(resident_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
     if (ok) {
@@ -1598,7 +1645,7 @@ static bool resident_supported() {
 static bool takes_resident(const Problem* P, int count, const ap_params* p, const Plan& plan) {
     if (count != 1 || (p->flags & (AP_FLAG_TIME_SWEEP | AP_FLAG_NO_GRAPH))) return false;
     const int n = (int)P[0].n;
-    if ((n + 3) / 4 > 32 * kResQ || resident_smem(n) > 226 * 1024 || plan.c.G != n) return false;
+    if ((n + 3) / 4 > 32 * kResQ || resident_smem(n) > 227 * 1024 - 512 || plan.c.G != n) return false;
     {
         std::lock_guard<std::mutex> lock(g_pin_mu);
         if (g_pinned.count(n)) return false;
