@@ -634,17 +634,23 @@ sweep_kernel(SweepLaunch L) {
 // the rows i = l mod 32 in turn (rows of CTA l mod 16, every second one), then
 // the lanes meet in its tree, so the results are the same bits as by launches.
 // R_{t-1}, which a stop found at step t returns, is kept in the workspace from
-// the step on at which the run could stop.  A row's inner loop has no special
-// elements: the diagonal's new value is patched in by its lane, R_ii lives in
-// rdg between row phases (sR has a zero there, which is what the column sums
-// take), and what lies past the row's end is -inf.  500 points, 100 iterations:
-// 635 us for the whole call where launches took 1147 us (697 us with separate
-// code for the diagonal's float4 and arg-max selects for every element); the rule
-// is that the three matrices fit (up to 544 points) and that the launches' units
-// are single rows.
+// the step on at which the run could stop.  The half-rate pipe of comparisons,
+// maxima and selects bounds a step, so a row's loop has few of them: max(0, r)
+// and min(0, t) are additions (below), the diagonal is kept apart in sdg, rdg
+// and adg (the matrices have -inf, 0 and -inf there; the column sums want the
+// 0), what lies past the row's end is -inf, only the largest a + s is carried
+// along (the lane that has it is looked at again by all lanes together, for
+// its index and the second largest), and decisions are formed only for the
+// stop rule.  500 points, 100 iterations: 589 us for the whole call where
+// launches took 1147 us (697 us with arg-max selects for every element); the
+// rule is that the three matrices fit (up to 544 points) and that the launches'
+// units are single rows.  Up to 512 points a warp's two rows of S and A stay
+// in registers.  Slower: 1024 threads (644 us), one lane alone looking again
+// (693 us).
 // ---------------------------------------------------------------------------
 constexpr int kResCtas = 16, kResThreads = 512, kResWarps = kResThreads / 32;
 constexpr int kResQ = 5;                // float4 per lane and row: n4 <= 160
+constexpr int kResRegN = 512;           // two rows a warp and four float4 a lane: S and A in registers
 
 struct ResidentArgs {
     SweepArgs a;
@@ -656,11 +662,12 @@ struct ResidentArgs {
 
 static size_t resident_smem(int n) {
     const size_t n4 = (n + 3) / 4, rows = (n + kResCtas - 1) / kResCtas, cw = (n + kResCtas - 1) / kResCtas;
-    return 3 * rows * n4 * 16 + 2 * n4 * 16 +              // S, R, A; (1 - lambda) c and colp
-           (32 * (cw | 1) + 3 * cw) * 4 + 2 * rows * 4 + 64;   // received sums (odd stride), diagonal, results;
-                                                            // flags, the rows' diagonals of R
+    return 3 * rows * n4 * 16 + 2 * n4 * 16 +              // S, R, A; half (1 - lambda) c, and colp
+           (32 * (cw | 1) + 3 * cw) * 4 + 4 * rows * 4 + 64;   // received sums (odd stride), diagonal, results;
+                                                            // flags, the rows' diagonals of S, R and A
 }
 
+template <bool REG>
 __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_constant__ ResidentArgs p) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int2 cnt[kResCtas];                          // every CTA's (changes, exemplars)
@@ -680,13 +687,15 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
     const int rs = cw | 1;                                  // (odd: lanes read a column of it)
     float* recv = colps + 4 * n4;                           // [32][rs]
     float* rdiag = recv + 32 * rs;
-    float* res = rdiag + cw;                                // [2][cw]: c and colp of this CTA's columns
+    float* res = rdiag + cw;                                // [2][cw]: half (1 - lambda) c, and colp, of its columns
     int* flags = reinterpret_cast<int*>(res + 2 * cw);
     float* rdg = reinterpret_cast<float*>(flags + p.rows);  // R_ii: sR has a zero there, for the column sums
+    float* adg = rdg + p.rows;                              // A_ii and S_ii: sA and sS have -inf there
+    float* sdg = adg + p.rows;
     // the reducer of column tid, and of column tid + 512
     const int dst0 = tid / cw, c0 = tid - dst0 * cw, dst1 = (tid + kResThreads) / cw, c1 = tid + kResThreads - dst1 * cw;
     const float lam = a.lam, oml = 1.0f - a.lam;
-    const float2 lam2 = make_float2(lam, lam), oml2 = make_float2(oml, oml), nom2 = make_float2(-oml, -oml);
+    const float2 lam2 = make_float2(lam, lam), oml2 = make_float2(oml, oml), noq2 = make_float2(-0.25f * oml, -0.25f * oml);
 
     if (tid == 0) own_changes = own_ex = own_bad = 0;
     cluster.sync();                     // every CTA has started: its shared memory may be written
@@ -719,11 +728,32 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
     }
     for (int k = tid; k < n4; k += kResThreads) cvs[k] = make_float4(0.f, 0.f, 0.f, 0.f);
     __syncthreads();
-    for (int r = tid; r < m; r += kResThreads) {
+    for (int r = tid; r < p.rows; r += kResThreads) {
         const int at = r * 4 * n4 + b + kResCtas * r;
         flags[r] = 0;
-        rdg[r] = reinterpret_cast<float*>(sR)[at];
-        reinterpret_cast<float*>(sR)[at] = 0.f;
+        rdg[r] = adg[r] = sdg[r] = 0.f;
+        if (r < m) {
+            rdg[r] = reinterpret_cast<float*>(sR)[at];
+            adg[r] = reinterpret_cast<float*>(sA)[at];
+            sdg[r] = reinterpret_cast<float*>(sS)[at];
+            reinterpret_cast<float*>(sR)[at] = 0.f;
+            reinterpret_cast<float*>(sA)[at] = reinterpret_cast<float*>(sS)[at] = -INFINITY;
+        }
+    }
+    __syncthreads();
+    // REG: a warp's two rows of S and A, for the whole run
+    constexpr int NR = REG ? 2 : 1, Q = REG ? 4 : kResQ;
+    float4 sr[NR][Q], ar[NR][Q];
+    if (REG) {
+#pragma unroll
+        for (int j = 0; j < NR; ++j)
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const int r = wid + kResWarps * j, f = lid + 32 * q;
+                const bool in = r < m && f < n4;
+                sr[j][q] = in ? sS[r * n4 + f] : make_float4(0.f, 0.f, 0.f, 0.f);
+                ar[j][q] = in ? sA[r * n4 + f] : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
     }
     if (p.check) {
         bad = __reduce_add_sync(0xffffffffu, bad);
@@ -748,124 +778,188 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
     int t = 1, stable = 0, iters = 0, converged = 0;
     bool doR = true, done = false;
     for (;; ++t) {
-        const bool doA = t >= 2;
+        const bool doA = t >= 2, doD = doA && p.conv_iter > 0;    // (only the stop rule asks for decisions)
         doR = t <= p.max_iter;
         // this step may turn out to be the last: keep R_{t-1}
         const bool keep = doR && doA && p.conv_iter > 0 && stable + 1 >= p.conv_iter;
-        for (int r = wid; r < m; r += kResWarps) {
-            const int i = b + kResCtas * r, di4 = i >> 2, de = i & 3;     // the diagonal: float4 di4 of the row
-            float* Sr = reinterpret_cast<float*>(sS + r * n4);
-            float* Rr = reinterpret_cast<float*>(sR + r * n4);
-            float* Ar = reinterpret_cast<float*>(sA + r * n4);
-            const float rii = rdg[r];
-            const float aii = doA ? fmaf(lam, Ar[i], oml * colps[i]) : Ar[i];
-            const float di = aii + rii;
-            if (lid == 0) Rr[i] = rii;
-            __syncwarp();                                   // Ar[i] has been read, Rr[i] written
-            float4 s4[kResQ], r4[kResQ];
-            // the lane's largest and second largest a + s, and the float4 of the
-            // first; the largest a + r
-            float m1 = -INFINITY, m2 = -INFINITY, dv = -INFINITY;
-            int jq = 0;
+        // N rows r0, r0 + 16 of this warp together (a slot past the CTA's rows is
+        // computed and ignored)
+        auto rows_step = [&](auto count, int r0) {
+            constexpr int N = decltype(count)::value;
+            float rii[N], aii[N], sii[N];
+            int i[N];
+            float m1[N], dv[N];                             // the lane's largest a + s, a + r off the diagonal
 #pragma unroll
-            for (int q = 0; q < kResQ; ++q) {
+            for (int j = 0; j < N; ++j) {
+                const int r = r0 + kResWarps * j;
+                i[j] = r < m ? b + kResCtas * r : 0;
+                rii[j] = rdg[r];
+                sii[j] = sdg[r];
+                aii[j] = doA ? fmaf(lam, adg[r], oml * colps[i[j]]) : adg[r];
+                m1[j] = dv[j] = -INFINITY;
+            }
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
                 const int f = lid + 32 * q;
                 if (f < n4) {
-                    s4[q] = sS[r * n4 + f];
-                    r4[q] = sR[r * n4 + f];
-                    float4 a4 = sA[r * n4 + f];
-                    if (doA) {
-                        // the arithmetic of sweep_kernel
-                        const float4 cv = cvs[f];
-                        const float2 tlo = __ffma2_rn(nom2, make_float2(fmaxf(0.f, r4[q].x), fmaxf(0.f, r4[q].y)),
-                                                      make_float2(cv.x, cv.y));
-                        const float2 thi = __ffma2_rn(nom2, make_float2(fmaxf(0.f, r4[q].z), fmaxf(0.f, r4[q].w)),
-                                                      make_float2(cv.z, cv.w));
-                        const float2 alo = __ffma2_rn(lam2, make_float2(a4.x, a4.y),
-                                                      make_float2(fminf(0.f, tlo.x), fminf(0.f, tlo.y)));
-                        const float2 ahi = __ffma2_rn(lam2, make_float2(a4.z, a4.w),
-                                                      make_float2(fminf(0.f, thi.x), fminf(0.f, thi.y)));
-                        a4 = make_float4(alo.x, alo.y, ahi.x, ahi.y);
-                    }
-                    if (q == di4 >> 5 && lid == (di4 & 31)) {         // the diagonal's own value
-                        a4.x = de == 0 ? aii : a4.x;
-                        a4.y = de == 1 ? aii : a4.y;
-                        a4.z = de == 2 ? aii : a4.z;
-                        a4.w = de == 3 ? aii : a4.w;
-                    }
-                    if (doA) {
-                        sA[r * n4 + f] = a4;
-                        const float2 dlo = __fadd2_rn(make_float2(a4.x, a4.y), make_float2(r4[q].x, r4[q].y));
-                        const float2 dhi = __fadd2_rn(make_float2(a4.z, a4.w), make_float2(r4[q].z, r4[q].w));
-                        dv = fmaxf(fmaxf(dv, fmaxf(dlo.x, dlo.y)), fmaxf(dhi.x, dhi.y));
-                    }
-                    if (doR) {
-                        const float2 vlo = __fadd2_rn(make_float2(a4.x, a4.y), make_float2(s4[q].x, s4[q].y));
-                        const float2 vhi = __fadd2_rn(make_float2(a4.z, a4.w), make_float2(s4[q].z, s4[q].w));
-                        const float h0 = fmaxf(vlo.x, vlo.y), l0 = fminf(vlo.x, vlo.y);
-                        const float h1 = fmaxf(vhi.x, vhi.y), l1 = fminf(vhi.x, vhi.y);
-                        const float hi = fmaxf(h0, h1);
-                        const float second = fmaxf(fminf(h0, h1), fmaxf(l0, l1));
-                        m2 = fmaxf(fmaxf(m2, second), fminf(m1, hi));
-                        if (hi > m1) { m1 = hi; jq = q; }
+                    const float4 cv = cvs[f];
+#pragma unroll
+                    for (int j = 0; j < N; ++j) {
+                        const int x = (r0 + kResWarps * j) * n4 + f;
+                        if (!REG) {
+                            sr[j][q] = sS[x];
+                            ar[j][q] = sA[x];
+                        }
+                        float4 a4 = ar[j][q];
+                        const float4 rv = sR[x], sv = sr[j][q];
+                        if (doA) {
+                            // the arithmetic of sweep_kernel at half size: 2 max(0, r) = r + |r|
+                            // and 2 min(0, t) = t - |t|, additions at full rate where
+                            // maxima take the half-rate pipe
+                            const float2 tlo = __ffma2_rn(noq2, make_float2(rv.x + fabsf(rv.x), rv.y + fabsf(rv.y)),
+                                                          make_float2(cv.x, cv.y));
+                            const float2 thi = __ffma2_rn(noq2, make_float2(rv.z + fabsf(rv.z), rv.w + fabsf(rv.w)),
+                                                          make_float2(cv.z, cv.w));
+                            const float2 alo = __ffma2_rn(lam2, make_float2(a4.x, a4.y),
+                                                          make_float2(tlo.x - fabsf(tlo.x), tlo.y - fabsf(tlo.y)));
+                            const float2 ahi = __ffma2_rn(lam2, make_float2(a4.z, a4.w),
+                                                          make_float2(thi.x - fabsf(thi.x), thi.y - fabsf(thi.y)));
+                            a4 = make_float4(alo.x, alo.y, ahi.x, ahi.y);
+                            ar[j][q] = a4;
+                            sA[x] = a4;
+                        }
+                        if (doD) {
+                            const float2 dlo = __fadd2_rn(make_float2(a4.x, a4.y), make_float2(rv.x, rv.y));
+                            const float2 dhi = __fadd2_rn(make_float2(a4.z, a4.w), make_float2(rv.z, rv.w));
+                            dv[j] = fmaxf(fmaxf(dv[j], fmaxf(dlo.x, dlo.y)), fmaxf(dhi.x, dhi.y));
+                        }
+                        const float2 vlo = __fadd2_rn(make_float2(a4.x, a4.y), make_float2(sv.x, sv.y));
+                        const float2 vhi = __fadd2_rn(make_float2(a4.z, a4.w), make_float2(sv.z, sv.w));
+                        m1[j] = fmaxf(fmaxf(m1[j], fmaxf(vlo.x, vlo.y)), fmaxf(vhi.x, vhi.y));
                     }
                 }
             }
-            if (doA) {
-                // the point chose itself: nothing is larger than the diagonal's a + r,
+            if (doD) {
+                // the point chose itself: nothing else is larger than the diagonal's a + r,
                 // and nothing before it as large
-                int self = di == warp_max_f32(dv) && di > -INFINITY ? 1 : 0;
-                if (self) {
-                    bool before = false;
-                    __syncwarp();
-                    for (int k = lid; k < i; k += 32) before = before || Ar[k] + Rr[k] == di;
-                    self = __any_sync(0xffffffffu, before) ? 0 : 1;
-                }
-                if (lid == 0) {
-                    if (flags[r] != self) atomicAdd(&own_changes, 1);
-                    if (self) atomicAdd(&own_ex, 1);
-                    flags[r] = self;
+                float top[N];
+#pragma unroll
+                for (int j = 0; j < N; ++j) top[j] = warp_max_f32(dv[j]);
+#pragma unroll
+                for (int j = 0; j < N; ++j) {
+                    const int r = r0 + kResWarps * j;
+                    const float di = aii[j] + rii[j];
+                    int self = di > top[j] ? 1 : 0;
+                    if (di == top[j] && di > -INFINITY) {
+                        bool before = false;
+#pragma unroll
+                        for (int q = 0; q < Q; ++q)
+                            if (lid + 32 * q < n4) {
+                                const float4 a4 = ar[j][q], rv = sR[r * n4 + lid + 32 * q];
+                                const int k = 4 * (lid + 32 * q);
+                                before = before || (k < i[j] && a4.x + rv.x == di) || (k + 1 < i[j] && a4.y + rv.y == di) ||
+                                         (k + 2 < i[j] && a4.z + rv.z == di) || (k + 3 < i[j] && a4.w + rv.w == di);
+                            }
+                        self = __any_sync(0xffffffffu, before) ? 0 : 1;
+                    }
+                    if (lid == 0 && r < m) {
+                        if (flags[r] != self) atomicAdd(&own_changes, 1);
+                        if (self) atomicAdd(&own_ex, 1);
+                        flags[r] = self;
+                    }
                 }
             }
             if (doR) {
-                // the row's largest, the lowest index that attains it, and the second largest
-                Top2 tp;
-                tp.m1 = warp_max_f32(m1);
-                int j = INT_MAX;
-                if (m1 == tp.m1 && lid + 32 * jq < n4) {
-                    const int f = lid + 32 * jq;
-                    const float4 a4 = sA[r * n4 + f], q4 = sS[r * n4 + f];
-                    const float v[4] = {a4.x + q4.x, a4.y + q4.y, a4.z + q4.z, a4.w + q4.w};
+                // the rows' largest, the lowest index that attains it, and the second
+                // largest: of the lane that has the largest all lanes look at an entry each
+                float off[N], sec[N], x[N];
+                int jo[N];
+                unsigned mask[N];
 #pragma unroll
-                    for (int e = 3; e >= 0; --e)
-                        if (v[e] == m1 && 4 * f + e < n) j = 4 * f + e;
+                for (int j = 0; j < N; ++j) off[j] = warp_max_f32(m1[j]);
+                __syncwarp();                               // sA is written
+#pragma unroll
+                for (int j = 0; j < N; ++j) {
+                    const float* Ar = reinterpret_cast<const float*>(sA + (r0 + kResWarps * j) * n4);
+                    const float* Sr = reinterpret_cast<const float*>(sS + (r0 + kResWarps * j) * n4);
+                    mask[j] = __ballot_sync(0xffffffffu, m1[j] == off[j]);
+                    const int own = __ffs((int)mask[j]) - 1, k = 4 * own + (lid & 3) + 128 * (lid >> 2);
+                    const float v = lid < 4 * Q && k < n ? Ar[k] + Sr[k] : -INFINITY;
+                    jo[j] = __reduce_min_sync(0xffffffffu, v == off[j] ? k : INT_MAX);
+                    x[j] = fmaxf(lid == own ? -INFINITY : m1[j], k == jo[j] ? -INFINITY : v);
                 }
-                tp.j1 = __reduce_min_sync(0xffffffffu, j);
-                tp.m2 = warp_max_f32(j == tp.j1 ? m2 : m1);
-                const float om1 = oml * tp.m1, om2 = oml * tp.m2;
-                const float2 nm1 = make_float2(-om1, -om1);
-                // the row's largest takes the second largest
-                const int jj = min(tp.j1, n - 1);           // (no largest among NaNs)
-                const float ov = fmaf(lam, Rr[jj], fmaf(oml, Sr[jj], -om2));
-                __syncwarp();                               // Rr[jj] has been read
 #pragma unroll
-                for (int q = 0; q < kResQ; ++q) {
-                    const int f = lid + 32 * q;
-                    if (f < n4) {
-                        if (keep) *reinterpret_cast<float4*>(a.R1 + (int64_t)i * a.ld + 4 * f) = r4[q];
-                        const float2 olo = __ffma2_rn(lam2, make_float2(r4[q].x, r4[q].y),
-                                                      __ffma2_rn(oml2, make_float2(s4[q].x, s4[q].y), nm1));
-                        const float2 ohi = __ffma2_rn(lam2, make_float2(r4[q].z, r4[q].w),
-                                                      __ffma2_rn(oml2, make_float2(s4[q].z, s4[q].w), nm1));
-                        sR[r * n4 + f] = make_float4(olo.x, olo.y, ohi.x, ohi.y);
+                for (int j = 0; j < N; ++j) sec[j] = warp_max_f32(x[j]);
+#pragma unroll
+                for (int j = 0; j < N; ++j) {
+                    // several lanes have it: the lowest index of all of them
+                    for (unsigned rest = mask[j] & (mask[j] - 1); rest; rest &= rest - 1) {
+                        const float* Ar = reinterpret_cast<const float*>(sA + (r0 + kResWarps * j) * n4);
+                        const float* Sr = reinterpret_cast<const float*>(sS + (r0 + kResWarps * j) * n4);
+                        const int k = 4 * (__ffs((int)rest) - 1) + (lid & 3) + 128 * (lid >> 2);
+                        const float v = lid < 4 * Q && k < n ? Ar[k] + Sr[k] : -INFINITY;
+                        jo[j] = min(jo[j], __reduce_min_sync(0xffffffffu, v == off[j] ? k : INT_MAX));
                     }
                 }
-                // (by the lanes that wrote these float4)
-                if (lid == ((tp.j1 >> 2) & 31) && tp.j1 < n) Rr[jj] = ov;
-                if (lid == (di4 & 31)) rdg[r] = Rr[i];
+#pragma unroll
+                for (int j = 0; j < N; ++j) {
+                    const int r = r0 + kResWarps * j;
+                    float* Rr = reinterpret_cast<float*>(sR + r * n4);
+                    const float* Sr = reinterpret_cast<const float*>(sS + r * n4);
+                    const float vii = aii[j] + sii[j];      // the diagonal joins
+                    float first = off[j], second = sec[j];
+                    int j1 = jo[j];
+                    if (vii > first) {
+                        second = first;
+                        first = vii;
+                        j1 = i[j];
+                    } else if (vii == first) {
+                        second = first;
+                        j1 = min(j1, i[j]);
+                    } else {
+                        second = fmaxf(second, vii);
+                    }
+                    const float om1 = oml * first, om2 = oml * second;
+                    const float2 nm1 = make_float2(-om1, -om1);
+                    const int jj = min(j1, n - 1);          // (no largest among NaNs)
+                    // the row's largest takes the second largest
+                    const float ov = fmaf(lam, Rr[jj], fmaf(oml, Sr[jj], -om2));
+                    __syncwarp();                           // Rr[jj] has been read
+#pragma unroll
+                    for (int q = 0; q < Q; ++q) {
+                        const int f = lid + 32 * q;
+                        if (f < n4) {
+                            const float4 rv = sR[r * n4 + f], sv = sr[j][q];
+                            if (keep && r < m) *reinterpret_cast<float4*>(a.R1 + (int64_t)i[j] * a.ld + 4 * f) = rv;
+                            const float2 olo = __ffma2_rn(lam2, make_float2(rv.x, rv.y),
+                                                          __ffma2_rn(oml2, make_float2(sv.x, sv.y), nm1));
+                            const float2 ohi = __ffma2_rn(lam2, make_float2(rv.z, rv.w),
+                                                          __ffma2_rn(oml2, make_float2(sv.z, sv.w), nm1));
+                            sR[r * n4 + f] = make_float4(olo.x, olo.y, ohi.x, ohi.y);
+                        }
+                    }
+                    // (by the lanes that wrote these float4)
+                    if (lid == ((j1 >> 2) & 31) && j1 < n) Rr[jj] = ov;
+                    if (lid == ((i[j] >> 2) & 31)) {
+                        Rr[i[j]] = 0.f;
+                        if (keep && r < m) a.R1[(int64_t)i[j] * a.ld + i[j]] = rii[j];
+                    }
+                    rii[j] = fmaf(lam, rii[j], fmaf(oml, sii[j], j1 == i[j] ? -om2 : -om1));
+                }
             }
-            if (lid == (di4 & 31)) Rr[i] = 0.f;
+#pragma unroll
+            for (int j = 0; j < N; ++j)
+                if (lid == 0) {
+                    rdg[r0 + kResWarps * j] = rii[j];
+                    adg[r0 + kResWarps * j] = aii[j];
+                }
             __syncwarp();
+        };
+        if constexpr (REG) {
+            if (wid + kResWarps < p.rows) rows_step(std::integral_constant<int, 2>{}, wid);
+            else if (wid < p.rows) rows_step(std::integral_constant<int, 1>{}, wid);
+        } else {
+            for (int r = wid; r < m; r += kResWarps) rows_step(std::integral_constant<int, 1>{}, r);
         }
         __syncthreads();
         if (doR) {
@@ -875,7 +969,7 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
             for (int h = 0; h < 2; ++h) {
                 const int k = tid + h * kResThreads, dst = h ? dst1 : dst0, c = h ? c1 : c0;
                 if (k >= n) break;
-                float s0 = 0.f, s1 = 0.f;                   // (the diagonal is a zero here)
+                float s0 = 0.f, s1 = 0.f;                   // twice the sums (the diagonal is a zero here)
                 int r = 0;
                 for (; r + 8 <= m; r += 8) {                // eight rows' reads in flight
                     float v[8];
@@ -883,12 +977,12 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
                     for (int e = 0; e < 8; ++e) v[e] = R[(r + e) * 4 * n4 + k];
 #pragma unroll
                     for (int e = 0; e < 8; e += 2) {
-                        s0 += fmaxf(0.f, v[e]);
-                        s1 += fmaxf(0.f, v[e + 1]);
+                        s0 += v[e] + fabsf(v[e]);
+                        s1 += v[e + 1] + fabsf(v[e + 1]);
                     }
                 }
                 for (; r < m; ++r) {
-                    const float v = fmaxf(0.f, R[r * 4 * n4 + k]);
+                    const float x = R[r * 4 * n4 + k], v = x + fabsf(x);
                     if (r & 1) s1 += v;
                     else s0 += v;
                 }
@@ -915,7 +1009,8 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
                 if (lid == 0) {
-                    res[c] = oml * (rdiag[c] + v);
+                    v *= 0.5f;
+                    res[c] = 0.5f * (oml * (rdiag[c] + v));
                     res[cw + c] = v;
                 }
             }
@@ -958,7 +1053,8 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
         for (int f = lid; f < n4; f += 32) {
             float4 rv = kept ? *reinterpret_cast<const float4*>(a.R1 + off + 4 * f) : sR[r * n4 + f];
             if (!kept && f == i >> 2) set_lane(rv, i & 3, rdg[r]);
-            const float4 av = sA[r * n4 + f];
+            float4 av = sA[r * n4 + f];
+            if (f == i >> 2) set_lane(av, i & 3, adg[r]);
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const float d = lane(av, e) + lane(rv, e);
@@ -1599,6 +1695,8 @@ static int32_t launch_chunk_graph(const SweepConfig& c, const Plan& plan, const 
     return AP_OK;
 }
 
+static auto resident_ptr(int n) { return n <= kResRegN ? resident_kernel<true> : resident_kernel<false>; }
+
 static cudaLaunchConfig_t resident_config(int n, cudaLaunchAttribute* attr, cudaStream_t s) {
     attr->id = cudaLaunchAttributeClusterDimension;
     attr->val.clusterDim.x = kResCtas;
@@ -1624,15 +1722,16 @@ static bool resident_supported() {
     std::lock_guard<std::mutex> lock(mu);
     auto it = known.find(dev);
     if (it != known.end()) return it->second;
-    bool ok = cudaFuncSetAttribute(resident_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 512) ==
-                  cudaSuccess &&
-              cudaFuncSetAttribute(resident_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
-    if (ok) {
+    bool ok = true;
+    for (const auto fn : {resident_kernel<true>, resident_kernel<false>}) {
+        ok = ok && cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 512) == cudaSuccess &&
+             cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+        if (!ok) break;
         cudaLaunchAttribute attr;
         cudaLaunchConfig_t cfg = resident_config(2, &attr, nullptr);
-        cfg.dynamicSmemBytes = 226 * 1024;
+        cfg.dynamicSmemBytes = 227 * 1024 - 512;
         int num = 0;
-        ok = cudaOccupancyMaxActiveClusters(&num, resident_kernel, &cfg) == cudaSuccess && num >= 1;
+        ok = cudaOccupancyMaxActiveClusters(&num, fn, &cfg) == cudaSuccess && num >= 1;
     }
     if (!ok) cudaGetLastError();
     known[dev] = ok;
@@ -1662,7 +1761,7 @@ static int32_t run_resident(const SweepArgs& a, const ap_params* p, ap_result* o
     r.rows = r.cw = (a.n + kResCtas - 1) / kResCtas;
     cudaLaunchAttribute attr;
     const cudaLaunchConfig_t cfg = resident_config(a.n, &attr, s);
-    AP_CUDA_TRY(cudaLaunchKernelEx(&cfg, resident_kernel, r));
+    AP_CUDA_TRY(cudaLaunchKernelEx(&cfg, resident_ptr(a.n), r));
     note_launches(1);
     SweepState h;
     AP_CUDA_TRY(cudaMemcpyAsync(&h, a.st, sizeof(h), cudaMemcpyDeviceToHost, s));
