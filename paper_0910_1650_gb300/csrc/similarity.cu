@@ -395,8 +395,8 @@ __device__ __forceinline__ float key_float(uint32_t k) {
 // S took 1025 us; 1000 points: 55 us where they took 144 us (16 blocks, most of
 // the time waiting on shared-memory atomics).
 constexpr int kSampleThreads = 1024;
-constexpr int kSamplePer = 16;          // entries drawn per thread
-constexpr int kSample = kSampleThreads * kSamplePer, kSampleHalfWidth = 288;
+constexpr int kSamplePer = 16;          // entries per thread (small selections: 4)
+constexpr int kSample = kSampleThreads * kSamplePer;
 constexpr int kSampleBins = 1024;       // two digits of 10 bits settle the bracket
 // Buffer entries a warp takes at a time (more if a step's hits need it): enough
 // that few of its steps wait for the atomic, few enough, where a warp has only
@@ -429,6 +429,13 @@ struct Select {
     float* pref;
 };
 
+// Up to this many points a selection's latency is what counts, and three launches
+// do all of it: the sample's block draws it (a quarter of the entries), the pass
+// over S has smaller blocks and counts the first digit of what it keeps, and
+// one block takes the other digits and writes the diagonal (1000 points: the
+// three 35 us and the whole call 111 us, where six launches took 58 and 126 us).
+constexpr int kSmallSelect = 1500;
+
 // Blocks of the pass over S: about 32K entries each, at most 8 per SM; of the
 // digits of the buffer: about 8K of its entries each, at most 4 per SM (a block
 // clears and adds up to 4096 bins).
@@ -448,14 +455,16 @@ static unsigned long long cand_cap(int n) {
 // by block bx of gx into the start of the candidate buffer (many blocks: one
 // SM has too few reads in flight for 16384 scattered ones: 3.5 us and 7.7 for the
 // bracket, together 17 when one block did both).
+__device__ __forceinline__ float drawn(const Select& q, int e) {
+    const uint64_t u = splitmix64_at(0x6d656469616eull, (uint64_t)e + 1);
+    const int i = (int)(((u >> 32) * (uint64_t)q.n) >> 32);
+    int k = (int)(((u & 0xffffffffull) * (uint64_t)(q.n - 1)) >> 32);
+    k += k >= i;
+    return __ldg(q.S + (int64_t)i * q.lds + k);
+}
 __device__ __forceinline__ void draw_block(const Select& q, int bx, int gx) {
-    for (int e = bx * blockDim.x + threadIdx.x; e < kSample; e += gx * blockDim.x) {
-        const uint64_t u = splitmix64_at(0x6d656469616eull, (uint64_t)e + 1);
-        const int i = (int)(((u >> 32) * (uint64_t)q.n) >> 32);
-        int k = (int)(((u & 0xffffffffull) * (uint64_t)(q.n - 1)) >> 32);
-        k += k >= i;
-        q.cand[e] = __float_as_uint(__ldg(q.S + (int64_t)i * q.lds + k));
-    }
+    for (int e = bx * blockDim.x + threadIdx.x; e < kSample; e += gx * blockDim.x)
+        q.cand[e] = __float_as_uint(drawn(q, e));
 }
 
 // The bracket of one problem (one block of kSampleThreads) from the drawn
@@ -464,21 +473,27 @@ __device__ __forceinline__ void draw_block(const Select& q, int bx, int gx) {
 // (the digits spread: a fixed top byte would put nearly every entry in one
 // bin, whose shared-memory atomics wait for one another).  What the digits
 // leave open widens the bracket.  The state and histograms start from here.
+// PER entries per thread, drawn here (SELF) or before.
+template <int PER, bool SELF>
 __device__ __forceinline__ void sample_block(const Select& q) {
+    // 4.5 standard deviations of a median's rank, sqrt(sample) / 2
+    constexpr int SAMPLE = kSampleThreads * PER, HALF = PER == 16 ? 288 : 144;
+    static_assert(PER == 16 || PER == 4, "half widths");
     __shared__ unsigned int h[2][kSampleBins];
     __shared__ unsigned int wsum[32];
     __shared__ uint32_t wmin[32], wmax[32];
     __shared__ int found[2];
     __shared__ unsigned int rem[2];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    uint32_t key[kSamplePer];
+    uint32_t key[PER];
     uint32_t kmin = 0xffffffffu, kmax = 0;
 #pragma unroll
-    for (int e = 0; e < kSamplePer; ++e) {
-        key[e] = float_key(__uint_as_float(q.cand[e * kSampleThreads + t]));
+    for (int e = 0; e < PER; ++e) {
+        key[e] = float_key(SELF ? drawn(q, e * kSampleThreads + t)
+                                : __uint_as_float(q.cand[e * kSampleThreads + t]));
     }
 #pragma unroll
-    for (int e = 0; e < kSamplePer; ++e) {
+    for (int e = 0; e < PER; ++e) {
         kmin = min(kmin, key[e]);
         kmax = max(kmax, key[e]);
     }
@@ -491,7 +506,7 @@ __device__ __forceinline__ void sample_block(const Select& q) {
     kmax = __reduce_max_sync(0xffffffffu, wmax[lane]);
     const int bits = 32 - __clz((int)(kmax - kmin));
     uint32_t pre[2] = {0, 0}, km = 0;
-    unsigned int rank[2] = {kSample / 2 - kSampleHalfWidth, kSample / 2 + kSampleHalfWidth};
+    unsigned int rank[2] = {SAMPLE / 2 - HALF, SAMPLE / 2 + HALF};
     int shift = bits;
 #pragma unroll
     for (int pass = 0; pass < 2; ++pass) {
@@ -502,7 +517,7 @@ __device__ __forceinline__ void sample_block(const Select& q) {
         h[1][t] = 0;
         __syncthreads();
 #pragma unroll
-        for (int e = 0; e < kSamplePer; ++e) {
+        for (int e = 0; e < PER; ++e) {
             const uint32_t rel = key[e] - kmin, dg = (rel >> shift) & dm;
             if ((rel & km) == pre[0]) atomicAdd(&h[0][dg], 1u);
             if ((rel & km) == pre[1]) atomicAdd(&h[1][dg], 1u);
@@ -588,7 +603,8 @@ __device__ __forceinline__ void look(float v, float lo, float hi, float bit, flo
 // the bracket's own; these (3.5 %) are read again as keys, so that NaN and
 // signed zeros fall where their keys do, and written behind one another by a
 // scan of the lanes' counts.
-template <bool VEC>
+// HIST: counts the first digit of select_small_kernel along the way.
+template <bool VEC, bool HIST = false>
 __device__ __forceinline__ void bracket_pass(const Select& q, int bx, int gx) {
     const int lane = threadIdx.x & 31;
     const uint32_t lo = q.st->lo, range = q.st->range;
@@ -598,7 +614,8 @@ __device__ __forceinline__ void bracket_pass(const Select& q, int bx, int gx) {
     // the warp's current chunk of the buffer: entries [at, end)
     unsigned long long at = 0, end = 0;
     bool full = false;
-    const int chunk = chunk_of(n);
+    const int chunk = HIST ? 32 : chunk_of(n);              // (a warp has one or two rows there)
+    const int bits = 32 - __clz((int)range), shift = bits > 11 ? bits - 11 : 0;
     for (int i = bx * kPassWarps + (threadIdx.x >> 5); i < n; i += gx * kPassWarps) {
         const float* row = q.S + (int64_t)i * q.lds;
         const int fi = i >> 2;
@@ -651,6 +668,7 @@ __device__ __forceinline__ void bracket_pass(const Select& q, int bx, int gx) {
                     if (key - lo <= range) {
                         rel = key - lo;
                         ++inside;
+                        if (HIST) atomicAdd(reinterpret_cast<unsigned int*>(q.hist) + ((rel >> shift) & 2047u), 1u);
                     }
                 }
                 if (!full) q.cand[pos < end ? pos : fresh + (pos - end)] = rel;
@@ -818,6 +836,115 @@ __device__ __forceinline__ void digit_pass(const Select& q, int p, int bx, int g
     }
 }
 
+// All digits of a small selection in one block, histograms in shared memory, then
+// the result and (diag not null) the diagonal.
+template <bool VEC>
+__global__ void __launch_bounds__(1024) select_small_kernel(Select q, float* diag, float* pref, float zero) {
+    __shared__ unsigned int h[2][2048];
+    __shared__ unsigned long long wsum[32];
+    __shared__ int found[2];
+    __shared__ uint64_t rem[2];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const SelectState s = *q.st;
+    // as pass 0 of digit_pass
+    const bool direct = s.slots > q.cap || s.rank[0] < s.less || s.rank[1] >= s.less + s.inside || s.range == 0xffffffffu;
+    const uint32_t lo = direct ? 0u : s.lo, range = direct ? 0xffffffffu : s.range;
+    uint64_t rank[2] = {direct ? s.rank[0] : s.rank[0] - s.less, direct ? s.rank[1] : s.rank[1] - s.less};
+    uint32_t pre[2] = {0, 0}, km = 0;
+    int shift = 32 - __clz((int)range);
+    while (shift > 0) {
+        const int width = min(11, shift);
+        shift -= width;
+        const uint32_t dm = (1u << width) - 1u;
+        const bool same = pre[0] == pre[1];
+        const bool counted = km == 0 && !direct;            // the first digit of the buffer's entries
+        for (int b = t; b < 2 * 2048; b += 1024)
+            (&h[0][0])[b] = counted && b < 2048 ? __ldcg(reinterpret_cast<const unsigned int*>(q.hist) + b) : 0u;
+        __syncthreads();
+        auto count = [&](uint32_t rel) {
+            const uint32_t dg = (rel >> shift) & dm;
+            if ((rel & km) == pre[0]) atomicAdd(&h[0][dg], 1u);
+            if (!same && (rel & km) == pre[1]) atomicAdd(&h[1][dg], 1u);
+        };
+        if (counted) {
+        } else if (!direct) {
+            const uint4* c4 = reinterpret_cast<const uint4*>(q.cand);
+            const unsigned n4 = (unsigned)(s.slots / 4);
+            for (unsigned x0 = t; x0 < n4; x0 += 4 * 1024) {
+                uint4 v[4];                         // four loads in flight before the first count
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    v[u] = x0 + 1024 * u < n4 ? c4[x0 + 1024 * u]
+                                              : make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    if (v[u].x <= range) count(v[u].x);
+                    if (v[u].y <= range) count(v[u].y);
+                    if (v[u].z <= range) count(v[u].z);
+                    if (v[u].w <= range) count(v[u].w);
+                }
+            }
+        } else {
+            const int n4 = (q.n + 3) >> 2;
+            for (int i = warp; i < q.n; i += 32) {
+                const float* row = q.S + (int64_t)i * q.lds;
+                for (int f = lane; f < n4; f += 32) {
+                    const float4 x = entries4<VEC>(row, f, q.n);
+                    const float v[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if (4 * f + e < q.n && 4 * f + e != i) count(float_key(v[e]));
+                }
+            }
+        }
+        __syncthreads();
+        // thread t owns bins 2t and 2t + 1 of both histograms, scanned together
+        const unsigned a0 = h[0][2 * t], a1 = h[0][2 * t + 1];
+        const unsigned b0 = same ? a0 : h[1][2 * t], b1 = same ? a1 : h[1][2 * t + 1];
+        const unsigned long long own = (unsigned long long)(a0 + a1) | ((unsigned long long)(b0 + b1) << 32);
+        unsigned long long x = own;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) wsum[warp] = x;
+        __syncthreads();
+        unsigned long long w = wsum[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long y = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += y;
+        }
+        const unsigned long long before = __shfl_sync(0xffffffffu, w, warp > 0 ? warp - 1 : 0);
+        x += (warp > 0 ? before : 0ull) - own;              // exclusive
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const uint64_t base = j ? x >> 32 : x & 0xffffffffull;
+            const unsigned c0 = j ? b0 : a0, c1 = j ? b1 : a1;
+            if (rank[j] >= base && rank[j] < base + c0) {
+                found[j] = 2 * t;
+                rem[j] = rank[j] - base;
+            } else if (rank[j] >= base + c0 && rank[j] < base + c0 + c1) {
+                found[j] = 2 * t + 1;
+                rem[j] = rank[j] - base - c0;
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            pre[j] |= (uint32_t)found[j] << shift;
+            rank[j] = rem[j];
+        }
+        km |= dm << shift;
+        __syncthreads();
+    }
+    const float p = (float)(0.5 * ((double)key_float(lo + pre[0]) + (double)key_float(lo + pre[1])));
+    if (t == 0) *pref = p;
+    if (diag)
+        for (int i = t; i < q.n; i += 1024) diag[(int64_t)i * q.lds + i] = p + zero;
+}
+
 __device__ __forceinline__ float select_result(const SelectState* st) {
     const double a = (double)key_float(st->lo + st->prefix[0]);
     const double b = (double)key_float(st->lo + st->prefix[1]);
@@ -828,11 +955,13 @@ constexpr int kDrawBlocks = 64;
 
 __global__ void __launch_bounds__(256) draw_kernel(Select q) { draw_block(q, blockIdx.x, gridDim.x); }
 
-__global__ void __launch_bounds__(kSampleThreads) sample_kernel(Select q) { sample_block(q); }
+__global__ void __launch_bounds__(kSampleThreads) sample_kernel(Select q) { sample_block<kSamplePer, false>(q); }
 
-template <bool VEC>
+__global__ void __launch_bounds__(kSampleThreads) sample_small_kernel(Select q) { sample_block<4, true>(q); }
+
+template <bool VEC, bool HIST>
 __global__ void __launch_bounds__(32 * kPassWarps, 4) bracket_kernel(Select q) {
-    bracket_pass<VEC>(q, blockIdx.x, gridDim.x);
+    bracket_pass<VEC, HIST>(q, blockIdx.x, gridDim.x);
 }
 
 template <bool VEC>
@@ -924,23 +1053,39 @@ static size_t carve_sim(void* ws, int64_t n, int64_t d, SimWs* w) {
     return c.used;
 }
 
-// Enqueues the selection of the two middle order statistics of S's off-diagonal
-// entries; select_result reads them from sel.
+// Enqueues the median of S's off-diagonal entries, to *pref, and (diag: S, for
+// writing) onto the diagonal; zero as in diag_kernel.
 static int32_t median_offdiag(const float* S, int n, int64_t lds, SelectState* sel, unsigned long long* hist,
-                              uint32_t* cand, cudaStream_t s) {
-    const int grid = pass_blocks(n);
-    const int dgrid = digit_blocks(n);
+                              uint32_t* cand, float* diag, float* pref, float zero, cudaStream_t s) {
+    const int grid = n <= kSmallSelect ? (n * n + 8191) / 8192 : pass_blocks(n), dgrid = digit_blocks(n);
     const Select q{S, lds, n, 0, grid, 0, dgrid, sel, hist, cand, cand_cap(n), nullptr};
-    const bool vec = aligned16(S) && (lds & 3) == 0;
-    draw_kernel<<<kDrawBlocks, 256, 0, s>>>(q);
-    sample_kernel<<<1, kSampleThreads, 0, s>>>(q);
-    if (vec) bracket_kernel<true><<<grid, 32 * kPassWarps, 0, s>>>(q);
-    else bracket_kernel<false><<<grid, 32 * kPassWarps, 0, s>>>(q);
+    const bool vec = aligned16(S) && (lds & 3) == 0, small = n <= kSmallSelect;
+    if (small) {
+        sample_small_kernel<<<1, kSampleThreads, 0, s>>>(q);
+    } else {
+        draw_kernel<<<kDrawBlocks, 256, 0, s>>>(q);
+        sample_kernel<<<1, kSampleThreads, 0, s>>>(q);
+    }
+    if (small) {
+        if (vec) bracket_kernel<true, true><<<grid, 32 * kPassWarps, 0, s>>>(q);
+        else bracket_kernel<false, true><<<grid, 32 * kPassWarps, 0, s>>>(q);
+    } else {
+        if (vec) bracket_kernel<true, false><<<grid, 32 * kPassWarps, 0, s>>>(q);
+        else bracket_kernel<false, false><<<grid, 32 * kPassWarps, 0, s>>>(q);
+    }
+    if (small) {
+        if (vec) select_small_kernel<true><<<1, 1024, 0, s>>>(q, diag, pref, zero);
+        else select_small_kernel<false><<<1, 1024, 0, s>>>(q, diag, pref, zero);
+        note_launches(3);
+        return last_error();
+    }
     for (int p = 0; p < 3; ++p) {
         if (vec) digit_kernel<true><<<dgrid, 256, 0, s>>>(q, p);
         else digit_kernel<false><<<dgrid, 256, 0, s>>>(q, p);
     }
-    note_launches(6);
+    if (diag) diag_kernel<<<(n + 255) / 256, 256, 0, s>>>(diag, n, lds, nullptr, sel, pref, 0.f, zero);
+    else select_finish_kernel<<<1, 1, 0, s>>>(sel, pref);
+    note_launches(7);
     return last_error();
 }
 
@@ -1022,7 +1167,7 @@ __global__ void __launch_bounds__(256) draw_batched_kernel(const SimProblem* __r
 
 // grid (problems)
 __global__ void __launch_bounds__(kSampleThreads) sample_batched_kernel(const SimProblem* __restrict__ P) {
-    sample_block(P[blockIdx.x].sel);
+    sample_block<kSamplePer, false>(P[blockIdx.x].sel);
 }
 
 // grid (sum of the problems' pass blocks)
@@ -1089,8 +1234,7 @@ static int32_t similarity_enqueue(const float* X, int ni, int di, int64_t ldx, f
     }
     const float zero = noise_rel > 0.0 ? 0.f : -0.f;
     if (pref_mode == AP_PREF_MEDIAN) {
-        AP_TRY(median_offdiag(S, ni, lds, w.sel, w.hist, w.cand, s));
-        diag_kernel<<<(ni + 255) / 256, 256, 0, s>>>(S, ni, lds, nullptr, w.sel, pref_dev, 0.f, zero);
+        AP_TRY(median_offdiag(S, ni, lds, w.sel, w.hist, w.cand, S, pref_dev, zero, s));
     } else if (pref_mode == AP_PREF_SCALAR) {
         diag_kernel<<<(ni + 255) / 256, 256, 0, s>>>(S, ni, lds, nullptr, nullptr, nullptr, pref[0], zero);
     } else {
@@ -1104,7 +1248,8 @@ static int32_t similarity_enqueue(const float* X, int ni, int di, int64_t ldx, f
         noise_kernel<<<std::min(ni, 8192), 256, 0, s>>>(S, ni, lds, noise_rel, seed);
         note_launches(1);
     }
-    note_launches(precision == AP_PREC_FP32 ? 3 : 2);   // centre, GEMM, diagonal
+    // centre, GEMM (the tensor-core one counts itself), a diagonal not written by the median
+    note_launches((precision == AP_PREC_FP32 ? 2 : 1) + (pref_mode == AP_PREF_MEDIAN ? 0 : 1));
     return last_error();
 }
 
@@ -1409,10 +1554,7 @@ APGB_API int32_t ap_preference_median(const float* S, int64_t n, int64_t ld, flo
     unsigned long long* hist = c.take<unsigned long long>(4096);
     uint32_t* cand = c.take<uint32_t>(cand_cap((int)n));
     float* pref = c.take<float>(1);
-    AP_TRY(median_offdiag(S, (int)n, ld, sel, hist, cand, s));
-    select_finish_kernel<<<1, 1, 0, s>>>(sel, pref);
-    note_launches(1);
-    AP_TRY(last_error());
+    AP_TRY(median_offdiag(S, (int)n, ld, sel, hist, cand, nullptr, pref, 0.f, s));
     float v = NAN;
     AP_CUDA_TRY(cudaMemcpyAsync(&v, pref, sizeof(float), cudaMemcpyDeviceToHost, s));
     AP_CUDA_TRY(cudaStreamSynchronize(s));

@@ -568,3 +568,28 @@ def test_autotune_pins_a_configuration_that_matches_oracle_and_is_not_slower():
         assert t_tuned <= 1.10 * t_default
     finally:
         capi.ap_sweep_set_config(n)
+
+
+@pytest.mark.parametrize("pad", [0, 1])
+@pytest.mark.parametrize("kind", ["spread", "ties", "one value", "specials"])
+@pytest.mark.parametrize("n", [2, 90, 91, 1499, 1500, 1501])
+def test_preference_median_at_the_small_selection_edge(n, kind, pad):
+    """Up to 1500 points one block settles the digits: exact order statistics on
+    both sides of the rule, for 16-byte rows and others, where most entries are
+    equal, and with infinities and zeros of both signs."""
+    g = np.random.default_rng(n + pad)
+    S = (-g.random((n, n)) * 7).astype(np.float32)
+    if kind == "ties":
+        S[g.random((n, n)) < 0.6] = -3.5
+    elif kind == "one value":
+        S[:] = -2.25
+    elif kind == "specials":
+        S[g.random((n, n)) < 0.2] = -np.inf
+        S[g.random((n, n)) < 0.2] = 0.0
+        S[g.random((n, n)) < 0.3] = -0.0
+    buf = torch.full((n, capi.padded_ld(n) + pad), float("nan"), dtype=torch.float32, device="cuda")
+    buf[:, :n] = torch.from_numpy(S).cuda()
+    got = capi.ap_preference_median(buf[:, :n])
+    x = np.sort(S[~np.eye(n, dtype=bool)].astype(np.float64))
+    m = x.size
+    assert got == np.float32(0.5 * (x[(m - 1) // 2] + x[m // 2]))
