@@ -3,6 +3,7 @@
 //   idx(i) = i for i in E, else argmax_{k in E} s(i,k)  (lowest index on ties)
 //   dpsim  = sum_{i not in E} s(i, idx(i)),  expref = sum_{k in E} s(k,k),
 //   netsim = dpsim + expref                             (float64, fixed order)
+#include <cstring>
 #include <algorithm>
 #include <climits>
 #include <mutex>
@@ -119,7 +120,7 @@ __global__ void sum2_kernel(const double* __restrict__ a, const double* __restri
 struct ExWs {
     int32_t* flag;
     int32_t* list;
-    int32_t* count;
+    int32_t* count;         // behind sums, so that one copy brings both
     double* dp;
     double* ep;
     double* sums;
@@ -129,10 +130,10 @@ static size_t carve_ex(void* ws, int64_t n, ExWs* w) {
     Carver c(ws);
     w->flag = c.take<int32_t>(n);
     w->list = c.take<int32_t>(n);
-    w->count = c.take<int32_t>(1);
     w->dp = c.take<double>(n);
     w->ep = c.take<double>(n);
-    w->sums = c.take<double>(2);
+    w->sums = c.take<double>(3);
+    w->count = reinterpret_cast<int32_t*>(w->sums + 2);
     return c.used;
 }
 
@@ -154,11 +155,11 @@ int32_t exemplars_impl(const float* S, const float* R, const float* A, int64_t n
     sum2_kernel<<<1, 1024, 0, s>>>(w.dp, w.ep, ni, w.sums);
     note_launches(4);
     AP_TRY(last_error());
-    double h[2];
-    int32_t cnt = 0;
+    double h[3];
     AP_CUDA_TRY(cudaMemcpyAsync(h, w.sums, sizeof(h), cudaMemcpyDeviceToHost, s));
-    AP_CUDA_TRY(cudaMemcpyAsync(&cnt, w.count, sizeof(cnt), cudaMemcpyDeviceToHost, s));
     AP_CUDA_TRY(cudaStreamSynchronize(s));
+    int32_t cnt = 0;
+    std::memcpy(&cnt, h + 2, sizeof(cnt));
     const int32_t status = cnt > 0 ? AP_OK : AP_NO_EXEMPLARS;
     out->n_exemplars = cnt;
     out->status = status;

@@ -13,6 +13,7 @@
 //      bracket, one pass over S, and radix digits over what it encloses;
 //   5. diagonal <- p, then s <- s + noise_rel*|s|*u(i,k) on every entry.
 #include <algorithm>
+#include <cstring>
 #include <mutex>
 #include <map>
 #include <array>
@@ -1048,8 +1049,8 @@ static size_t carve_sim(void* ws, int64_t n, int64_t d, SimWs* w) {
     w->sel = c.take<SelectState>(1);
     w->hist = c.take<unsigned long long>(4096);
     w->cand = c.take<uint32_t>(cand_cap((int)n));
-    w->pref = c.take<float>(1);
-    w->err = c.take<int32_t>(1);
+    w->pref = c.take<float>(2);
+    w->err = reinterpret_cast<int32_t*>(w->pref + 1);       // one copy brings both
     return c.used;
 }
 
@@ -1278,14 +1279,12 @@ APGB_API int32_t ap_similarity(const float* X, int64_t n, int64_t d, int64_t ldx
     AP_CUDA_TRY(cudaMemsetAsync(w.err, 0, sizeof(int32_t), s));
     AP_TRY(similarity_enqueue(X, (int)n, (int)d, ldx, S, lds, precision, pref_mode, pref, noise_rel,
                               seed, w, w.pref, w.err, s));
-    float v = pref_mode == AP_PREF_SCALAR ? pref[0] : NAN;
-    int32_t err = 0;
-    if (pref_mode == AP_PREF_MEDIAN)
-        AP_CUDA_TRY(cudaMemcpyAsync(&v, w.pref, sizeof(float), cudaMemcpyDeviceToHost, s));
-    AP_CUDA_TRY(cudaMemcpyAsync(&err, w.err, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    struct { float pref; int32_t err; } h;
+    AP_CUDA_TRY(cudaMemcpyAsync(&h, w.pref, sizeof(h), cudaMemcpyDeviceToHost, s));
     AP_CUDA_TRY(cudaStreamSynchronize(s));
-    if (err) return AP_ERR_TIMEOUT;
-    if (pref_out) *pref_out = v;
+    if (h.err) return AP_ERR_TIMEOUT;
+    if (pref_out)
+        *pref_out = pref_mode == AP_PREF_MEDIAN ? h.pref : pref_mode == AP_PREF_SCALAR ? pref[0] : NAN;
     return AP_OK;
 }
 
@@ -1324,8 +1323,8 @@ static size_t carve_batched(void* ws, const int64_t* n, int32_t count, int64_t d
                             float** prefs, void** tables) {
     Carver c(ws);
     SimProblem* t = c.take<SimProblem>((size_t)count);
-    int32_t* e = c.take<int32_t>((size_t)count);
-    float* pv = c.take<float>((size_t)count);
+    float* pv = c.take<float>(2 * (size_t)count);           // the preferences, then the errors: one copy
+    int32_t* e = pv ? reinterpret_cast<int32_t*>(pv + count) : nullptr;
     const int dpad = pad_dim((int)d);
     const size_t esz = precision == AP_PREC_FP32 ? sizeof(float) : sizeof(__nv_bfloat16);
     // every problem's centred rows (and norms) in one arena, problem b from row
@@ -1520,16 +1519,17 @@ APGB_API int32_t ap_similarity_batched(const float* X, const int64_t* xoff, cons
         note_launches(1);
     }
     AP_TRY(last_error());
-    std::vector<float> v(count, pref_mode == AP_PREF_SCALAR ? pref[0] : NAN);
-    std::vector<int32_t> e(count, 0);
-    if (pref_mode == AP_PREF_MEDIAN)
-        AP_CUDA_TRY(cudaMemcpyAsync(v.data(), prefs, sizeof(float) * count, cudaMemcpyDeviceToHost, s));
-    AP_CUDA_TRY(cudaMemcpyAsync(e.data(), err, sizeof(int32_t) * count, cudaMemcpyDeviceToHost, s));
+    std::vector<float> v(2 * (size_t)count);                // preferences, errors
+    AP_CUDA_TRY(cudaMemcpyAsync(v.data(), prefs, sizeof(float) * v.size(), cudaMemcpyDeviceToHost, s));
     AP_CUDA_TRY(cudaStreamSynchronize(s));
-    for (int32_t b = 0; b < count; ++b)
-        if (e[b]) return AP_ERR_TIMEOUT;
+    for (int32_t b = 0; b < count; ++b) {
+        int32_t e;
+        std::memcpy(&e, &v[(size_t)count + b], sizeof(e));
+        if (e) return AP_ERR_TIMEOUT;
+    }
     if (pref_out)
-        for (int32_t b = 0; b < count; ++b) pref_out[b] = v[b];
+        for (int32_t b = 0; b < count; ++b)
+            pref_out[b] = pref_mode == AP_PREF_MEDIAN ? v[b] : pref_mode == AP_PREF_SCALAR ? pref[0] : NAN;
     return AP_OK;
 }
 
