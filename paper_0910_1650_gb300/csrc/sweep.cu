@@ -1569,9 +1569,20 @@ static size_t carve_sweep(void* ws, const Problem* P, int count, const Plan& pla
 // one before.  `early` lets a launch start while its predecessor drains
 // (programmatic dependent launch): its blocks are scheduled, set up their
 // barriers and wait there, so that launch latency and set-up leave the chain.
-// For one problem only: 5003 points 92.6 -> 91.8 us an iteration, 2021 points
-// about 3 % of a run; the classes of a batch run side by side, and early blocks
-// that wait hold room the other classes could use (48 problems: 3 % slower).
+// A sweep that starts early shares the SMs with the finalize blocks before it,
+// and its clusters are then placed around them: from clusters of four CTAs on
+// they no longer fit side by side, which costs far more than the gap
+// (microseconds an iteration, early against not: 5500 points 162 to 103, 8192
+// points 284 to 226, 20000 points 1470 to 1361).  With one or two CTAs a
+// cluster it gains where the launches are short or the sweep long (600 points
+// 12.0 to 12.4, 1000 points 15.7 to 16.5, 4000 points 60.6 to 61.6, 5003 points
+// 92.3 to 93.4) and not between (2021 points 24.9 to 24.0, 3000 points 41 to
+// 39.5).  The classes of a batch run side by side, and early blocks that wait
+// hold room the other classes could use (48 problems: 3 % slower).
+static bool starts_early(int count, int nmax, int cluster) {
+    return count == 1 && cluster <= 2 && (nmax <= 1024 || nmax >= 4096);
+}
+
 static void early_launch(cudaLaunchAttribute* a) {
     a->id = cudaLaunchAttributeProgrammaticStreamSerialization;
     a->val.programmaticStreamSerializationAllowed = 1;
@@ -1645,10 +1656,11 @@ constexpr size_t kMaxGraphs = 32;
 
 static int32_t enqueue_chunk(const SweepConfig& c, const Plan& plan, const SweepLaunch& L,
                              int64_t m, dim3 fin_grid, cudaStream_t s) {
+    const bool early = starts_early(L.count, plan.nmax, c.C);
     for (int64_t j = 0; j < m; ++j) {
         // (the first launch of a chunk follows copies and other kernels: no early start)
-        AP_TRY(launch_sweep(c, plan.clusters, L, s, false, L.count == 1 && j > 0));
-        AP_TRY(launch_finalize(fin_grid, L.table, s, L.count == 1));
+        AP_TRY(launch_sweep(c, plan.clusters, L, s, false, early && j > 0));
+        AP_TRY(launch_finalize(fin_grid, L.table, s, early));
     }
     return last_error();
 }
