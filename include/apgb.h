@@ -81,7 +81,8 @@ typedef struct ap_params {
  * each chunk of check_every iterations (m sweep + m column-sum launches, when
  * m >= 4) is one CUDA graph: captured on a library-owned stream the first time
  * a workspace address and launch shape are seen, kept (up to 32 per process),
- * and launched on the caller's stream. */
+ * and launched on the caller's stream; a single problem of at most 544 points
+ * (without a pinned configuration) is one kernel launch for the whole run. */
 #define AP_FLAG_NO_GRAPH   2
 /* ap_params.flags, pap_run only: Step 4 starts from the block-diagonal R of
  * the sub-problems as well as A' (the paper carries availabilities only, so
@@ -156,9 +157,10 @@ int32_t   ap_similarity(const float* X, int64_t n, int64_t d, int64_t ldx,
  *           for every problem; AP_PREF_VECTOR is not accepted).  No noise.
  *  pref_out host float[count] (may be NULL): the preference of each problem.
  *  Each stage (column means, centring, median passes, diagonal) is one
- *  launch for every problem of the batch on ``stream``; the Gram products
- *  are launched per problem, round-robin over 4 library-owned streams that
- *  fork from and join back to ``stream`` by events.  The workspace holds
+ *  launch for every problem of the batch on ``stream``, and so are the bf16
+ *  Gram products; the float32 ones are launched per problem, round-robin over
+ *  4 library-owned streams that fork from and join back to ``stream`` by
+ *  events.  The workspace holds
  *  every problem's scratch (its centred copy included, sized for float32).
  *  The stream is synchronised once, at the end.  Results equal ap_similarity
  *  on each problem bit for bit.
@@ -177,7 +179,9 @@ int32_t   ap_similarity_batched(const float* X, const int64_t* xoff, const int64
  * "adjust the input preference" to a common value (Section 5): the exact
  * median of the n(n-1) off-diagonal entries of S (the diagonal is ignored;
  * mean of the two middle order statistics in double, rounded to float, when
- * n(n-1) is even).  Exact selection on the float32 bit patterns, 3 passes.
+ * n(n-1) is even).  Exact selection on the float32 bit patterns: a drawn sample
+ * brackets the middle ranks, one pass over S collects what lies between (more
+ * passes only where the bracket misses).
  *
  *  S        device float32 [n x ld], n >= 2.
  *  median   host float* out (required); the call is synchronous.
