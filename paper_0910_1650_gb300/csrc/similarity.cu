@@ -1018,9 +1018,10 @@ static int pad_dim(int d) { return (d + 63) / 64 * 64; }
 // Row blocks of the column means: 256 rows, or more so that there are at most
 // 2048 blocks (the float64 combine of the partials is sequential per column).
 static int64_t mean_rows(int64_t n, int64_t d) {
-    // fewer rows where few columns leave most SMs without a block
+    // fewer rows where few columns leave most SMs without a block; not below 128 up
+    // to 2048 points, where combining many partials costs more than it saves
     const int64_t spread = (n * ((d + 127) / 128) + 151) / 152;
-    return std::max<int64_t>(std::max<int64_t>(32, std::min<int64_t>(kMeanRows, spread)), (n + 2047) / 2048);
+    return std::max<int64_t>(std::max<int64_t>(n <= 2048 ? 128 : 32, std::min<int64_t>(kMeanRows, spread)), (n + 2047) / 2048);
 }
 static int mean_blocks(int64_t n, int64_t d) { return (int)((n + mean_rows(n, d) - 1) / mean_rows(n, d)); }
 
@@ -1033,7 +1034,7 @@ int32_t column_means(const float* X, int64_t n, int d, int64_t ldx, double* part
         colsum_partial_kernel<true><<<dim3((d + 127) / 128, nb), 256, 0, s>>>(X, n, d, ldx, mean_rows(n, d), part);
     else
         colsum_partial_kernel<false><<<dim3((d + 31) / 32, nb), 256, 0, s>>>(X, n, d, ldx, mean_rows(n, d), part);
-    if (nb > 64) colmean_kernel<32><<<(d + 7) / 8, 256, 0, s>>>(part, nb, d, n, mean);
+    if (nb > 8) colmean_kernel<32><<<(d + 7) / 8, 256, 0, s>>>(part, nb, d, n, mean);
     else colmean_kernel<8><<<(d + 31) / 32, 256, 0, s>>>(part, nb, d, n, mean);
     note_launches(2);
     return last_error();

@@ -157,6 +157,7 @@ struct GroupProblem {
 
 struct Params {
     int M, N, K;                    // rows of A, rows of B, padded K (multiple of 64)
+    int square;                     // SIM: every tile of the square, none mirrored
     int mode;
     int stages, nob;                // operand stages; store buffers per epilogue warp
     const float* anrm;              // SIM: |a_i|^2 (length >= M)
@@ -430,6 +431,9 @@ __device__ __forceinline__ Tile tile_of(const Params& p, int numN, int u, int q,
         const int roff = p.probs[e.x].roff;
         t.prob = e.x; t.m = e.y; t.n = e.z;
         t.arow = roff + e.y * BM; t.brow = roff + e.z * BN;
+    } else if (p.square) {
+        t.n = u % numN; t.m = u / numN; t.prob = 0;
+        t.arow = t.m * BM; t.brow = t.n * BN;
     } else {
         // column block q has the row blocks 0 .. 2 q + 1: q (q + 1) units before it
         int c = (int)((sqrtf(4.f * (float)u + 1.f) - 1.f) * 0.5f);
@@ -479,7 +483,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     constexpr bool amax = AMAX;
     // (SIM: without the last row block where the rows end in an odd one)
     const int u0 = PAIR ? blockIdx.x >> 1 : blockIdx.x, ustep = PAIR ? gridDim.x >> 1 : gridDim.x;
-    const int units = amax ? numM : p.tiles ? p.ntiles : PAIR ? numN * (numN + 1) / 2 : numN * (numN + 1) - (numM & 1);
+    const int units = amax ? numM : p.tiles ? p.ntiles : p.square ? numM * numN : PAIR ? numN * (numN + 1) / 2 : numN * (numN + 1) - (numM & 1);
     const int tiles_per_unit = amax ? numN : 1;
     const int ns = p.stages;
 
@@ -687,7 +691,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                     const float2 nai = make_float2(-ai, -ai), two = make_float2(2.f, 2.f),
                                  mone = make_float2(-1.f, -1.f);
                     const float* bn = p.bnrm + roff + col_half;
-                    const bool mirror = t.m < 2 * t.n;     // wholly above the diagonal (rows < columns)
+                    const bool mirror = t.m < 2 * t.n && !p.square;     // wholly above the diagonal (rows < columns)
                     uint32_t ra[32], rb[32];
                     auto emit = [&](uint32_t (&v)[32], int c) {
                         const int kcol = col_half + c * OUT_COLS;
@@ -1371,6 +1375,8 @@ int32_t tc_similarity_bf16(const __nv_bfloat16* Xb, const float* nrm, int n, int
     const int npad = (n + BN - 1) / BN * BN;
     const int nm = (n + BM - 1) / BM, nn = (n + BN - 1) / BN;
     const bool pair = pairs(dpad / BK, (int64_t)nn * (nn + 1));
+    int sms = 0;
+    AP_TRY(device_sm_count(&sms));
     CUtensorMap ma, mb, mo;
     AP_TRY(make_map(&ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (void*)Xb, dpad, npad, (uint64_t)dpad * 2,
                     BK, BM, CU_TENSOR_MAP_SWIZZLE_128B));
@@ -1390,7 +1396,12 @@ int32_t tc_similarity_bf16(const __nv_bfloat16* Xb, const float* nrm, int n, int
     p.lds = lds;
     p.spin_limit = 1u << 22;
     p.error = err;
-    return launch(ma, mb, mo, p, pair ? nn * (nn + 1) / 2 : nn * (nn + 1) - (nm & 1), s, pair);
+    // Where the whole square is one tile per SM at most, all of it is multiplied: a
+    // tile's time is then the call's, and a mirrored tile's second store adds to it
+    // (1500 points, d = 64, given preference: call 64 us against 67.5, together with fewer, larger blocks of column sums).
+    p.square = !pair && (int64_t)nm * nn <= sms;
+    const int units = pair ? nn * (nn + 1) / 2 : p.square ? nm * nn : nn * (nn + 1) - (nm & 1);
+    return launch(ma, mb, mo, p, units, s, pair);
 }
 
 // Device bytes of the tables of a grouped similarity over problems of sizes
