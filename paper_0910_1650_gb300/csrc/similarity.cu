@@ -1025,7 +1025,18 @@ static int64_t mean_rows(int64_t n, int64_t d) {
 }
 static int mean_blocks(int64_t n, int64_t d) { return (int)((n + mean_rows(n, d) - 1) / mean_rows(n, d)); }
 
-size_t column_mean_part_doubles(int64_t n, int d) { return (size_t)mean_blocks(n, d) * (size_t)d; }
+// The largest mean_blocks(m, d) of any m <= n: callers size for their largest
+// set and then take the means of subsets in the same buffer, and mean_blocks
+// falls at many n (d <= 128: 152 blocks at 4864 points, 148 at 4865).  Up to 2048
+// points a block has at least 128 rows; beyond, rows >= m ceil(d / 128) / 152
+// unless they are 256 or more.
+static int64_t mean_blocks_cap(int64_t n, int64_t d) {
+    if (n <= 2048) return (n + 127) / 128;
+    const int64_t wide = (d + 127) / 128, spread = (151 + wide) / wide;
+    return std::max({int64_t(16), spread, std::min<int64_t>((n + kMeanRows - 1) / kMeanRows, 2048)});
+}
+
+size_t column_mean_part_doubles(int64_t n, int d) { return (size_t)mean_blocks_cap(n, d) * (size_t)d; }
 
 int32_t column_means(const float* X, int64_t n, int d, int64_t ldx, double* part, float* mean,
                      cudaStream_t s) {

@@ -438,3 +438,36 @@ def test_assign_with_resident_centres_at_its_edges(c, d):
     assert bool((score.gather(1, chosen[:, None])[:, 0] >= top - 2 * tol)[torch.from_numpy(~own).cuda()].all())
     if c > 1:                                                # of the two equal centres the earlier one
         assert not np.any(got[~own] == n // 2)
+
+
+def test_lap_full_level_with_more_column_blocks_than_the_whole_set():
+    """The column means of 4864 points (one recursion level) take 152 row blocks,
+    those of all 7000 points 149, in one scratch sized for the whole set.  The
+    landmarks and 2136 points lie together, the other 4864 far from them in ten
+    groups: the first level leaves exactly those, the second settles them as
+    the oracle does wherever its decision is clear of rounding (1e-4 of the
+    gates; nearly all points)."""
+    n, far, L, seed = 7000, 4864, 100, 5
+    g = np.random.default_rng(12)
+    lm = olap.uniform_landmarks(n, L, seed)
+    out = g.permutation(np.setdiff1d(np.arange(n), lm))[:far]
+    X = 0.1 * g.normal(size=(n, 8))
+    X[lm] = g.normal(size=(L, 8))
+    C = g.normal(size=(10, 8))
+    X[out] = 200.0 + 60.0 * C[g.integers(0, 10, far)] + 0.5 * g.normal(size=(far, 8))
+    X = X.astype(np.float32)
+    kw = dict(max_iter=1000, max_levels=2)
+    ref = olap.run_full(X, L, seed, 2, lam=0.9, convits=15, **kw)
+    l1 = ref["levels"][1]
+    assert l1["n"] == far
+    idx, level_of, res = capi.lap_run_full(torch.from_numpy(X).cuda(), L, 2, seed=seed, precision="fp32",
+                                           damping=0.9, conv_iter=15, **kw)
+    level_of = level_of.cpu().numpy()
+    assert res["levels"] == 2 and res["unassigned"][0] == far
+    assert res["exemplars_at"] == [e["E"].size for e in ref["levels"]]
+    ids = np.sort(out)
+    rest = np.setdiff1d(ids, ids[olap.uniform_landmarks(far, L, seed + 1)])
+    clear = rest[l1["margin"] > 1e-4 * l1["scale"]]
+    assert clear.size > 0.9 * rest.size
+    assert np.array_equal(level_of[clear] == -1, np.isin(clear, l1["unassigned"]))
+    _check_assignment(X, ref["E"], idx.cpu().numpy().astype(np.int64))

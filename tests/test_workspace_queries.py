@@ -1,0 +1,35 @@
+"""Workspace queries (host only): a workspace for n points is enough for every
+smaller n.  Callers rely on it, and so does the library: lap_run_full sizes
+its scratch for all n points once and takes the column means of every level's
+subset in it."""
+import pytest
+
+from paper_0910_1650_gb300 import build as b
+from paper_0910_1650_gb300 import capi
+
+
+@pytest.fixture(scope="module")
+def lib():
+    b.build()
+    return capi.lib()
+
+
+def _never_shrinks(query, sizes):
+    largest = 0
+    for n in sizes:
+        need = query(n)
+        assert need >= largest, n
+        largest = need
+
+
+@pytest.mark.parametrize("d", [1, 64, 129, 300, 4096])
+def test_point_set_queries_never_shrink(lib, d):
+    """The column sums' row blocks are fewer at many larger sizes (d = 64: 152 at
+    4864 points, 148 at 4865); the scratch must not follow them down.  Sizes to
+    10000 one by one, and around the 2048-block limit."""
+    near = [w * 2048 + e for w in (255, 256, 257, 263, 264, 300) for e in (-1, 0, 1)]
+    for sizes in (range(2, 10001), near):
+        _never_shrinks(lambda n: lib.lap_assign_workspace_size(n, d, 2), sizes)
+        _never_shrinks(lambda n: lib.lap_refine_workspace_size(n, d, 2), sizes)
+        _never_shrinks(lambda n: lib.lap_run_full_workspace_size(n, d, 2, 2, 2), sizes)
+        _never_shrinks(lambda n: lib.ap_similarity_workspace_size(n, d), sizes)
