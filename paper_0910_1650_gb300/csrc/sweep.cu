@@ -61,7 +61,8 @@ struct SweepState {
     int32_t final_buf;   // R buffer (0 = caller's R, 1 = workspace) with R_iters
     int32_t nonfinite;   // count of NaN/Inf entries of S
     int32_t error;       // a bounded wait gave up
-    int32_t pad[4];
+    int32_t large;       // resident_kernel: the input is left to the launches
+    int32_t pad[3];
 };
 
 // One problem of a launch (a launch sweeps a table of independent problems;
@@ -632,11 +633,13 @@ sweep_kernel(SweepLaunch L) {
 // cluster's CTAs are always resident together, whatever else runs.  The sums
 // are those of finalize_kernel with one row per unit, in its order: lane l adds
 // the rows i = l mod 32 in turn (rows of CTA l mod 16, every second one), then
-// the lanes meet in its tree, so the results are the same bits as by launches.
+// the lanes meet in its tree, so the results are the same bits as by launches
+// (but for the last bit of messages below 2^-125, which are halved on the way).
 // R_{t-1}, which a stop found at step t returns, is kept in the workspace from
 // the step on at which the run could stop.  The half-rate pipe of comparisons,
 // maxima and selects bounds a step, so a row's loop has few of them: max(0, r)
-// and min(0, t) are additions (below), the diagonal is kept apart in sdg, rdg
+// and min(0, t) are additions (below; what they double must not overflow, so
+// large inputs go by launches: resident_limit), the diagonal is kept apart in sdg, rdg
 // and adg (the matrices have -inf, 0 and -inf there; the column sums want the
 // 0), what lies past the row's end is -inf, only the largest a + s is carried
 // along (the lane that has it is looked at again by all lanes together, for
@@ -656,6 +659,7 @@ struct ResidentArgs {
     SweepArgs a;
     int max_iter, conv_iter;
     int check;                          // count the entries of S that are not finite
+    float limit;                        // resident_limit
     int rows;                           // most rows of a CTA
     int cw;                             // columns per reducing CTA
 };
@@ -671,7 +675,7 @@ template <bool REG>
 __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_constant__ ResidentArgs p) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int2 cnt[kResCtas];                          // every CTA's (changes, exemplars)
-    __shared__ int own_changes, own_ex, own_bad;
+    __shared__ int own_changes, own_ex, own_bad, own_large;
     __shared__ int2 total;                                  // their sum
     cg::cluster_group cluster = cg::this_cluster();
     const SweepArgs& a = p.a;
@@ -697,9 +701,10 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
     const float lam = a.lam, oml = 1.0f - a.lam;
     const float2 lam2 = make_float2(lam, lam), oml2 = make_float2(oml, oml), noq2 = make_float2(-0.25f * oml, -0.25f * oml);
 
-    if (tid == 0) own_changes = own_ex = own_bad = 0;
+    if (tid == 0) own_changes = own_ex = own_bad = own_large = 0;
     cluster.sync();                     // every CTA has started: its shared memory may be written
     int bad = 0;
+    bool fits = true;                   // (a NaN does not)
     for (int e = tid; e < m * n4; e += kResThreads) {
         const int r = e / n4, f = e - r * n4;
         const int64_t off = (int64_t)(b + kResCtas * r) * a.ld + 4 * f;
@@ -714,6 +719,10 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
         float4 r4 = a.zero ? z : *reinterpret_cast<const float4*>(a.R0 + off);
         float4 a4 = a.zero ? z : *reinterpret_cast<const float4*>(a.A + off);
         float4 t4 = s4;
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+            fits = fits && (4 * f + x >= n || (fabsf(lane(s4, x)) <= p.limit && fabsf(lane(r4, x)) <= p.limit &&
+                                               fabsf(lane(a4, x)) <= p.limit));
         // past the row's end: never a maximum, and finite where it is added
 #pragma unroll
         for (int x = 1; x < 4; ++x)
@@ -755,23 +764,26 @@ __global__ void __launch_bounds__(kResThreads, 1) resident_kernel(const __grid_c
                 ar[j][q] = in ? sA[r * n4 + f] : make_float4(0.f, 0.f, 0.f, 0.f);
             }
     }
-    if (p.check) {
-        bad = __reduce_add_sync(0xffffffffu, bad);
-        if (lid == 0 && bad) atomicAdd(&own_bad, bad);
-        __syncthreads();
-        if (tid < kResCtas) *cluster.map_shared_rank(&cnt[b], tid) = make_int2(own_bad, 0);
-        cluster.sync();
-        int sum = 0;
-        for (int c = 0; c < kResCtas; ++c) sum += cnt[c].x;
-        cluster.sync();                                     // read before anyone writes counts again
-        if (sum) {                                          // the same in every CTA
-            if (b == 0 && tid == 0) {
-                SweepState s{};
-                s.nonfinite = sum;
-                *a.st = s;
-            }
-            return;
+    bad = __reduce_add_sync(0xffffffffu, bad);
+    if (lid == 0 && bad) atomicAdd(&own_bad, bad);
+    if (!__all_sync(0xffffffffu, fits) && lid == 0) own_large = 1;
+    __syncthreads();
+    if (tid < kResCtas) *cluster.map_shared_rank(&cnt[b], tid) = make_int2(own_bad, own_large);
+    cluster.sync();
+    int sum = 0, large = 0;
+    for (int c = 0; c < kResCtas; ++c) {
+        sum += cnt[c].x;
+        large |= cnt[c].y;
+    }
+    cluster.sync();                                         // read before anyone writes counts again
+    if (sum || large) {                                     // the same in every CTA
+        if (b == 0 && tid == 0) {
+            SweepState s{};
+            s.nonfinite = sum;
+            s.large = large;
+            *a.st = s;
         }
+        return;
     }
     __syncthreads();
 
@@ -1764,12 +1776,24 @@ static bool takes_resident(const Problem* P, int count, const ap_params* p, cons
     return resident_supported();
 }
 
-static int32_t run_resident(const SweepArgs& a, const ap_params* p, ap_result* out, cudaStream_t s) {
+// The largest magnitude of S, R and A on entry that resident_kernel takes.  With
+// every entry at most u, a run never has (in exact arithmetic; a run damps
+// towards these, so it stays between them and the entry values)
+//   r(k,k) >= -3u    its row's other a + s are at most 2u,
+//   a(i,k) >= -3u    off the diagonal, as min(0, r(k,k) + a sum of max(0, r)),
+//   r(i,k) <=  5u    s minus a maximum over entries of at least -3u - u,
+// so column sums are at most 5nu and the doubled ones 10nu.  Launches do not double:
+// S with larger entries (pairs ruled out by -1e38, say) is theirs.
+static float resident_limit(int n) { return std::ldexp(1.f, 124) / (float)(n + 2); }
+
+// *taken = false: the input is larger than resident_limit, nothing was written.
+static int32_t run_resident(const SweepArgs& a, const ap_params* p, ap_result* out, cudaStream_t s, bool* taken) {
     ResidentArgs r{};
     r.a = a;
     r.max_iter = p->max_iter;
     r.conv_iter = p->conv_iter;
     r.check = (p->flags & AP_FLAG_S_CHECKED) ? 0 : 1;
+    r.limit = resident_limit(a.n);
     r.rows = r.cw = (a.n + kResCtas - 1) / kResCtas;
     cudaLaunchAttribute attr;
     const cudaLaunchConfig_t cfg = resident_config(a.n, &attr, s);
@@ -1779,6 +1803,8 @@ static int32_t run_resident(const SweepArgs& a, const ap_params* p, ap_result* o
     AP_CUDA_TRY(cudaMemcpyAsync(&h, a.st, sizeof(h), cudaMemcpyDeviceToHost, s));
     AP_CUDA_TRY(cudaStreamSynchronize(s));
     if (h.nonfinite) return AP_ERR_NONFINITE;
+    *taken = !h.large;
+    if (h.large) return AP_OK;
     const int32_t status = (p->conv_iter > 0 && !h.converged) ? AP_NOT_CONVERGED : AP_OK;
     if (out) {
         *out = ap_result{};
@@ -1802,7 +1828,9 @@ static int32_t run_batch(const Problem* P, int count, const ap_params* p, ap_res
     if (takes_resident(P, count, p, plan)) {
         SweepArgs a = w.host[0];
         if (p->flags & AP_FLAG_COLD) a.zero = w.zero;       // (a mark here: zeros are not read)
-        return run_resident(a, p, out, s);
+        bool taken = true;
+        const int32_t status = run_resident(a, p, out, s, &taken);
+        if (status < 0 || taken) return status;
     }
     if (p->flags & AP_FLAG_COLD) {
         // R and A start at zero whatever the buffers hold: the first launches

@@ -431,6 +431,45 @@ def test_one_launch_run_equals_separate_launches(n):
     assert torch.equal(R, R1) and torch.equal(A, A1)
 
 
+@pytest.mark.parametrize("n", [3, 17, 300, 512, 544])
+@pytest.mark.parametrize("mask", [-1e30, -1e36, -1e38, float(-np.finfo(np.float32).max)])
+def test_one_launch_run_with_large_masks_equals_separate_launches(n, mask):
+    """S with pairs or candidates ruled out by a large finite value (an infinity is
+    refused), one candidate left or several: the same bits as separate launches,
+    from zeros and from given messages, one of them with messages as large as
+    the mask and one with an infinite message."""
+    g = np.random.default_rng(n)
+    X = g.normal(size=(n, 3)) + 4 * g.integers(0, 3, size=(n, 1))
+    S0 = s32(X)
+    pairs = S0.copy()
+    off = ~np.eye(n, dtype=bool)
+    pairs[(g.random((n, n)) < 0.4) & off] = mask
+    one = S0.copy()                                          # only candidate 0 is left, for itself and every other
+    one[:, 1:] = mask
+    several = S0.copy()
+    np.fill_diagonal(several, np.where(np.arange(n) % 3 == 0, np.diag(S0), mask))
+    row = S0.copy()                                          # one point apart from all others
+    row[n // 2, :] = mask
+    R0, A0 = g.normal(size=(n, n)), -np.abs(g.normal(size=(n, n)))
+    big = R0.copy()
+    big[0, n - 1] = -mask
+    inf = R0.copy()
+    inf[n - 1, 0] = -np.inf
+    for S in (pairs, one, several, row):
+        Sd = dev_square(S)
+        for lam, maxit, conv, start in ((0.9, 60, 5, None), (0.5, 25, 0, R0), (0.7, 10, 0, big), (0.9, 8, 3, inf)):
+            outs = []
+            for graph in (True, False):
+                R, A = dev_square(R0 if start is None else start), dev_square(A0)
+                R, A, res, dec = capi.ap_iterate(Sd, R, A, damping=lam, max_iter=maxit, conv_iter=conv,
+                                                 cold=start is None, graph=graph)
+                outs.append((R.clone(), A.clone(), dec, res["iters"], res["converged"], res["status"]))
+            for a, b in zip(outs[0][:2], outs[1][:2]):
+                assert torch.equal(torch.isnan(a), torch.isnan(b))
+                assert torch.equal(torch.nan_to_num(a, 0.0), torch.nan_to_num(b, 0.0)), (lam, maxit, conv)
+            assert torch.equal(outs[0][2], outs[1][2]) and outs[0][3:] == outs[1][3:]
+
+
 def test_preference_median_exact():
     for n in (2, 3, 100, 1001):
         g = np.random.default_rng(n)
