@@ -1906,11 +1906,12 @@ static int32_t run_batch(const Problem* P, int count, const ap_params* p, ap_res
         if (graph && m >= 4) {
             AP_TRY(launch_chunk_graph(c, cur, L, m, fin_grid, s));
         } else {
+            const bool early = !timed && starts_early(count, cur.nmax, c.C);
             for (int64_t j = 0; j < m; ++j) {
                 if (timed) AP_CUDA_TRY(cudaEventRecord(ev.start[j], s));
-                AP_TRY(launch_sweep(c, cur.clusters, L, s, true, !timed && count == 1 && j > 0));
+                AP_TRY(launch_sweep(c, cur.clusters, L, s, true, early && j > 0));
                 if (timed) AP_CUDA_TRY(cudaEventRecord(ev.stop[j], s));
-                AP_TRY(launch_finalize(fin_grid, w.table, s, !timed && count == 1));
+                AP_TRY(launch_finalize(fin_grid, w.table, s, early));
             }
         }
         note_launches(2 * (uint64_t)m);
