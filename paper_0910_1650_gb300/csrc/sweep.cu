@@ -1586,13 +1586,14 @@ static size_t carve_sweep(void* ws, const Problem* P, int count, const Plan& pla
 // they no longer fit side by side, which costs far more than the gap
 // (microseconds an iteration, early against not: 5500 points 162 to 103, 8192
 // points 284 to 226, 20000 points 1470 to 1361).  With one or two CTAs a
-// cluster it gains where the launches are short or the sweep long (600 points
-// 12.0 to 12.4, 1000 points 15.7 to 16.5, 4000 points 60.6 to 61.6, 5003 points
-// 92.3 to 93.4) and not between (2021 points 24.9 to 24.0, 3000 points 41 to
-// 39.5).  The classes of a batch run side by side, and early blocks that wait
+// cluster it gains where the launches are short (600 points 12.0 to 12.4, 1000
+// points 15.7 to 16.5), loses from there to about 3000 points (2021 points 25.1
+// to 24.0, 3000 points 44.6 to 40.0), and beyond makes no difference that
+// repeats tell from noise (4000 to 5100 points: -1.5 to +3 %, either sign at
+// one size).  The classes of a batch run side by side, and early blocks that wait
 // hold room the other classes could use (48 problems: 3 % slower).
 static bool starts_early(int count, int nmax, int cluster) {
-    return count == 1 && cluster <= 2 && (nmax <= 1024 || nmax >= 4096);
+    return count == 1 && cluster <= 2 && nmax <= 1024;
 }
 
 static void early_launch(cudaLaunchAttribute* a) {
