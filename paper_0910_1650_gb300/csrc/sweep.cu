@@ -200,6 +200,8 @@ sweep_kernel(SweepLaunch L) {
     const int csize = (int)cluster.num_blocks();
     const int crank = (int)cluster.block_rank();
     const int gc = blockIdx.x / csize;
+    // (no kernel writes the list; read here, its latency hides behind the set-up)
+    const int u_begin = L.ubeg[gc], u_end = L.ubeg[gc + 1];
     ptx::grid_launch_dependents();
     const int T = (int)blockDim.x - 32;         // compute threads
     const int tid = threadIdx.x;
@@ -228,7 +230,6 @@ sweep_kernel(SweepLaunch L) {
     // everything above overlaps the previous kernel's end where this launch was
     // allowed to start early (ptx.cuh); from here on its results are needed
     ptx::grid_dependency_wait();
-    const int u_begin = L.ubeg[gc], u_end = L.ubeg[gc + 1];
 
     auto sS = [&](int s) { return stage + ((size_t)s * 3 + 0) * w4s; };
     auto sR = [&](int s) { return stage + ((size_t)s * 3 + 1) * w4s; };
