@@ -1592,7 +1592,8 @@ static size_t carve_sweep(void* ws, const Problem* P, int count, const Plan& pla
 // to 24.0, 3000 points 44.6 to 40.0), and beyond makes no difference that
 // repeats tell from noise (4000 to 5100 points: -1.5 to +3 %, either sign at
 // one size).  The classes of a batch run side by side, and early blocks that wait
-// hold room the other classes could use (48 problems: 3 % slower).
+// hold room the other classes could use (48 problems: 3 % slower; run_batch's
+// beside).
 static bool starts_early(int count, int nmax, int cluster) {
     return count == 1 && cluster <= 2 && nmax <= 1024;
 }
@@ -1656,10 +1657,11 @@ struct GraphKey {
     int count, C, EPT, NS, T, G, clusters, nmax;
     size_t smem;
     int64_t m;
+    bool early;
     bool operator<(const GraphKey& o) const {
-        return std::tie(dev, table, count, C, EPT, NS, T, G, clusters, nmax, smem, m) <
+        return std::tie(dev, table, count, C, EPT, NS, T, G, clusters, nmax, smem, m, early) <
                std::tie(o.dev, o.table, o.count, o.C, o.EPT, o.NS, o.T, o.G, o.clusters, o.nmax,
-                        o.smem, o.m);
+                        o.smem, o.m, o.early);
     }
 };
 
@@ -1669,8 +1671,7 @@ static std::map<int, cudaStream_t> g_capture_stream;
 constexpr size_t kMaxGraphs = 32;
 
 static int32_t enqueue_chunk(const SweepConfig& c, const Plan& plan, const SweepLaunch& L,
-                             int64_t m, dim3 fin_grid, cudaStream_t s) {
-    const bool early = starts_early(L.count, plan.nmax, c.C);
+                             int64_t m, dim3 fin_grid, cudaStream_t s, bool early) {
     for (int64_t j = 0; j < m; ++j) {
         // (the first launch of a chunk follows copies and other kernels: no early start)
         AP_TRY(launch_sweep(c, plan.clusters, L, s, false, early && j > 0));
@@ -1680,11 +1681,11 @@ static int32_t enqueue_chunk(const SweepConfig& c, const Plan& plan, const Sweep
 }
 
 static int32_t launch_chunk_graph(const SweepConfig& c, const Plan& plan, const SweepLaunch& L,
-                                  int64_t m, dim3 fin_grid, cudaStream_t s) {
+                                  int64_t m, dim3 fin_grid, cudaStream_t s, bool early) {
     int dev = 0;
     AP_CUDA_TRY(cudaGetDevice(&dev));
     const GraphKey key{dev, L.table, L.count, c.C, c.EPT, c.NS, c.T, c.G, plan.clusters,
-                       plan.nmax, c.smem, m};
+                       plan.nmax, c.smem, m, early};
     // the shared-memory ceiling is a function attribute, set outside the capture
     AP_TRY(prepare_sweep_fn(c.EPT));
     std::lock_guard<std::mutex> lock(g_graph_mu);
@@ -1699,7 +1700,7 @@ static int32_t launch_chunk_graph(const SweepConfig& c, const Plan& plan, const 
             cs = sit->second;
         }
         AP_CUDA_TRY(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-        const int32_t st = enqueue_chunk(c, plan, L, m, fin_grid, cs);
+        const int32_t st = enqueue_chunk(c, plan, L, m, fin_grid, cs, early);
         cudaGraph_t graph = nullptr;
         const cudaError_t e = cudaStreamEndCapture(cs, &graph);
         if (st != AP_OK || e != cudaSuccess) {
@@ -1820,14 +1821,18 @@ static int32_t run_resident(const SweepArgs& a, const ap_params* p, ap_result* o
 
 // Runs Algorithm 1 on every problem of the batch until each has stopped.
 // out[b] receives problem b's result; sweep timing is per launch (shared).
-static int32_t run_batch(const Problem* P, int count, const ap_params* p, ap_result* out,
-                         void* ws, size_t ws_bytes, cudaStream_t s, const Plan& plan) {
+// beside: other classes of a batch run at the same time, so a single problem
+// takes plain launches: early blocks would hold room the others could use, and
+// resident_kernel's cluster would wait for 16 free SMs of one GPC (36 problems of
+// 500 points and one of 540: 6.85 ms where plain launches take 6.79).
+static int32_t run_batch(const Problem* P, int count, const ap_params* p, ap_result* out, void* ws, size_t ws_bytes,
+                         cudaStream_t s, const Plan& plan, bool beside = false) {
     SweepWs w;
     AP_TRY(check_ws(ws, ws_bytes, carve_sweep(nullptr, P, count, plan, nullptr)));
     carve_sweep(ws, P, count, plan, &w);
     const SweepConfig& c = plan.c;
     for (auto& a : w.host) a.lam = p->damping;
-    if (takes_resident(P, count, p, plan)) {
+    if (!beside && takes_resident(P, count, p, plan)) {
         SweepArgs a = w.host[0];
         if (p->flags & AP_FLAG_COLD) a.zero = w.zero;       // (a mark here: zeros are not read)
         bool taken = true;
@@ -1904,11 +1909,11 @@ static int32_t run_batch(const Problem* P, int count, const ap_params* p, ap_res
     const bool graph = !timed && !(p->flags & AP_FLAG_NO_GRAPH);
     while (launched < total) {
         const int64_t m = std::min<int64_t>(chunk, total - launched);
+        const bool early = !timed && !beside && starts_early(count, cur.nmax, c.C);
         // a graph pays for its capture only over several iterations
         if (graph && m >= 4) {
-            AP_TRY(launch_chunk_graph(c, cur, L, m, fin_grid, s));
+            AP_TRY(launch_chunk_graph(c, cur, L, m, fin_grid, s, early));
         } else {
-            const bool early = !timed && starts_early(count, cur.nmax, c.C);
             for (int64_t j = 0; j < m; ++j) {
                 if (timed) AP_CUDA_TRY(cudaEventRecord(ev.start[j], s));
                 AP_TRY(launch_sweep(c, cur.clusters, L, s, true, early && j > 0));
@@ -2217,7 +2222,7 @@ APGB_API int32_t ap_iterate_batched(const float* S, float* R, float* A, const in
     auto run_class = [&](size_t i, cudaStream_t cs) {
         r[i].assign(cls[i].P.size(), ap_result{});
         st[i] = run_batch(cls[i].P.data(), (int)cls[i].P.size(), p, r[i].data(),
-                          static_cast<char*>(ws) + cls[i].ws_off, cls[i].ws_bytes, cs, cls[i].plan);
+                          static_cast<char*>(ws) + cls[i].ws_off, cls[i].ws_bytes, cs, cls[i].plan, cls.size() > 1);
     };
     if (cls.size() == 1) {
         run_class(0, s);

@@ -142,3 +142,21 @@ def test_similarity_batched_by_pairs_equals_single(d):
         assert torch.equal(Sb[:, :v], one) and prefs[b] == p
         assert torch.isnan(Sb[:, v:]).all()
         at += v
+
+
+def test_single_problem_class_beside_others_takes_plain_launches():
+    """33 problems of 500 points fill a class and one of 540 is the last: beside
+    other classes it goes by launches (a sweep and a column sum each iteration, one
+    set-up and one finite check per class), not by the one-launch kernel, and
+    its messages are those of a call of its own."""
+    n = [500] * 33 + [540]
+    g = np.random.default_rng(5)
+    off, ns, ld, total = batched.layout(n)
+    S = torch.from_numpy(-g.random(total).astype(np.float32)).cuda()
+    R, A = torch.zeros_like(S), torch.zeros_like(S)
+    before = capi.kernel_launches()
+    capi.ap_iterate_batched(S, R, A, off, ns, ld, damping=0.9, max_iter=10, conv_iter=0)
+    assert capi.kernel_launches() - before == 2 * (2 + 2 * 11)
+    view = [batched.view(t, off, ns, ld, 33) for t in (S, R, A)]
+    R1, A1, _, _ = capi.ap_iterate(view[0], damping=0.9, max_iter=10, conv_iter=0)
+    assert torch.equal(view[1], R1) and torch.equal(view[2], A1)
