@@ -111,8 +111,13 @@ __global__ void __launch_bounds__(256) colsum_partial_kernel(const float* __rest
 // The means from the row blocks' sums: 256 threads on LANES row lanes x 256 /
 // LANES columns; lane y adds blocks y, y + LANES, ... in order, then the lane
 // sums meet in a fixed tree.  Bound by float64 adds, of which an SM makes two
-// a clock: 32 lanes x 8 columns spread many blocks (nb > 64) over 4 times the
-// SMs that 8 x 32 reach (2048 blocks, d = 128: 15 us where 8 x 32 took 37 us).
+// a clock: 32 lanes x 8 columns spread many blocks over 4 times the SMs that 8
+// x 32 reach (2048 blocks, d = 128: 15 us where 8 x 32 took 37 us; 50 blocks, d =
+// 300: 4.7 and 6.0 us), but have the longer tree (16 blocks, d = 100: 4.0 us where
+// 8 x 32 take 3.5).  The choice is the order of the sums, so the batched build
+// makes the same one.
+static __host__ __device__ __forceinline__ bool mean_by_32_lanes(int nb) { return nb > 16; }
+
 template <int LANES>
 __device__ __forceinline__ void colmean_block(const double* __restrict__ part, int nb, int d, int64_t n,
                                               float* mean, int bx) {
@@ -1045,7 +1050,7 @@ int32_t column_means(const float* X, int64_t n, int d, int64_t ldx, double* part
         colsum_partial_kernel<true><<<dim3((d + 127) / 128, nb), 256, 0, s>>>(X, n, d, ldx, mean_rows(n, d), part);
     else
         colsum_partial_kernel<false><<<dim3((d + 31) / 32, nb), 256, 0, s>>>(X, n, d, ldx, mean_rows(n, d), part);
-    if (nb > 8) colmean_kernel<32><<<(d + 7) / 8, 256, 0, s>>>(part, nb, d, n, mean);
+    if (mean_by_32_lanes(nb)) colmean_kernel<32><<<(d + 7) / 8, 256, 0, s>>>(part, nb, d, n, mean);
     else colmean_kernel<8><<<(d + 31) / 32, 256, 0, s>>>(part, nb, d, n, mean);
     note_launches(2);
     return last_error();
@@ -1149,7 +1154,7 @@ __global__ void __launch_bounds__(256) colsum_batched_kernel(const SimProblem* _
 // grid (problems, ceil(d/32)), 256 threads
 __global__ void __launch_bounds__(256) colmean_batched_kernel(const SimProblem* __restrict__ P, int d) {
     const SimProblem& q = P[blockIdx.x];
-    if (q.nb > 64) {                        // the sums of colmean_kernel<32>: 8 columns at a time
+    if (mean_by_32_lanes(q.nb)) {           // 8 columns at a time
         for (int t = 0; t < 4; ++t) {
             colmean_block<32>(q.part, q.nb, d, q.n, q.mean, 4 * blockIdx.y + t);
             __syncthreads();

@@ -160,3 +160,23 @@ def test_single_problem_class_beside_others_takes_plain_launches():
     view = [batched.view(t, off, ns, ld, 33) for t in (S, R, A)]
     R1, A1, _, _ = capi.ap_iterate(view[0], damping=0.9, max_iter=10, conv_iter=0)
     assert torch.equal(view[1], R1) and torch.equal(view[2], A1)
+
+
+@pytest.mark.parametrize("d,n", [(64, 1100), (64, 1500), (64, 2000), (64, 2049), (64, 2500), (4096, 2100),
+                                  (4096, 4000), (4096, 4400)])
+def test_similarity_batched_column_means_are_the_single_ones(d, n):
+    """9 to 79 row blocks of column sums, on both sides of the line between the two
+    ways to add them: both entry points take the same one.
+    Columns whose blocks 0 and 1 hold a large pair that cancels show the order:
+    what the other blocks hold is lost beside it or not, so the means and the
+    centred features of the other points would differ, and S with them."""
+    block = 256 if d > 64 else 128 if n <= 2048 else 32
+    g = np.random.default_rng(n)
+    X = (g.random((n, d)) * 2.0 ** -10).astype(np.float32)
+    X[0], X[block] = 2.0 ** 45, -2.0 ** 45
+    Xd = torch.from_numpy(X).cuda()
+    one, p = capi.ap_similarity(Xd, precision="fp32")
+    ld = capi.padded_ld(n)
+    S = torch.empty(n * ld, device="cuda")
+    prefs = capi.ap_similarity_batched(Xd, [0], [n], S, [0], [ld], precision="fp32")
+    assert torch.equal(S.view(n, ld)[:, :n], one) and prefs == [p]
