@@ -48,23 +48,32 @@ constexpr int TOPK = 16;
 // One warp per row of one problem.  The pass is bound by reading S (twice:
 // the second time mostly from L2) and by about 25 instructions an entry, not
 // by the selection:
-//   scan 1  sums of v and v^2 (two-float accumulators, packed f32x2: float64
-//           arithmetic is scarce on this part), the four counts, and every
-//           lane's largest entry.  The 16th largest of the 32 lane maxima is
-//           a value that at least 16 entries reach;
+//   scan 1  sums of e and e^2, where e = v - (a value inside the row): the mean
+//           of 32 entries spread over it.  Entries close to one another lose
+//           nothing to cancellation then, and e^2 exceeds the variance by a
+//           factor of at most 1 + n / 32 on average, whatever the entries.  e is
+//           a two-float difference (exact), the sums are two-float accumulators
+//           (about 48 bits; packed f32x2: float64 arithmetic is scarce on this
+//           part).  Also the four counts, and every lane's largest entry: the
+//           16th largest of the 32 lane maxima is a value that at least 16
+//           entries reach;
 //   scan 2  the entries that reach it (about 22 on unordered data) go to a
 //           list in shared memory; if the list fills up it is cut to its 16
 //           best and the bar rises to the 16th of them;
 //   then each listed entry's rank is the number of better ones (larger, or
 //   equal with a lower index): ranks 0-15 are features 0-15.
 // Writes features 0-15 and 18-22, the 16 neighbour indices (problem-local)
-// and the sums, from which features_finish_row makes 16-17 with whole warps
-// of rows (a float64 division by one lane costs what 32 cost).
+// and the sums (their pivot and unit in the places of features 16-17), from which
+// features_finish_row makes 16-17 with whole warps of rows (a float64 division by
+// one lane costs what 32 cost).
 // The listing takes places by a shared atomic (the ranking does not depend on
 // their order) and the counts are float32, whose additions are full rate.
-// 48 problems of 200-4000 points (2.7e8 entries): 544 us (+ 27 us for the second
-// pass; 637 us with ballots, prefix counts and integer sums), where one block per
-// row with 16 block-wide arg-max rounds and float64 sums took 8.1 ms.
+// Six blocks per SM (40 registers) hide the scans' latencies: with the registers
+// that the compiler takes by itself four fit and it takes 638 us.
+// 48 problems of 200-4000 points (2.7e8 entries): 550 us (+ 24 us for the second
+// pass; sums of v and v^2 themselves 543 + 27, but 2e-3 off in feature 17 at mean
+// 1000 and spread 0.001; ballots, prefix counts and integer sums 637), where one
+// block per row with 16 block-wide arg-max rounds and float64 sums took 8.1 ms.
 constexpr int kListCap = 256;      // entries listed per warp
 constexpr int kFeatWarps = 8;      // rows per block
 
@@ -83,6 +92,7 @@ __device__ __forceinline__ float unit_of(float scale) {
 }
 
 // s + c += x, exactly but for c's rounding (Knuth's two-sum), two columns at a time.
+// A lane's c is a float32 sum of n / 64 errors: s + c carries about 48 bits.
 __device__ __forceinline__ void two_add(float2& s, float2& c, float2 x) {
     const float2 mone = make_float2(-1.f, -1.f);
     const float2 t = __fadd2_rn(s, x);
@@ -96,6 +106,15 @@ __device__ __forceinline__ void count_if_ge(float& c, float v, float t) {
     asm("{\n\t.reg .pred p;\n\tsetp.ge.f32 p, %1, %2;\n\t@p add.f32 %0, %0, 0f3F800000;\n\t}"
         : "+f"(c)
         : "f"(v), "f"(t));
+}
+// u v - p = d + e exactly (Knuth's two-sum with -p; u a power of two, nu = -u).
+__device__ __forceinline__ float2 two_diff(float2 v, float2 u, float2 nu, float2 p, float2 np, float2& e) {
+    const float2 mone = make_float2(-1.f, -1.f);
+    const float2 d = __ffma2_rn(u, v, np);
+    const float2 bp = __ffma2_rn(nu, v, d);
+    const float2 nap = __ffma2_rn(mone, d, bp);
+    e = __ffma2_rn(mone, __fadd2_rn(p, bp), __ffma2_rn(u, v, nap));
+    return d;
 }
 __device__ __forceinline__ void two_add1(float& s, float& c, float x) {
     const float t = s + x, bp = t - s;
@@ -138,11 +157,21 @@ __device__ __forceinline__ void features_row(const float* __restrict__ S, int n,
                                              int k, float* F, int32_t* nbr, float4* sums, FeatList& L) {
     const int lid = threadIdx.x & 31;
     const float* row = S + (int64_t)k * ld;
-    const float inv_scale = 1.f / scale, unit = unit_of(scale);
+    const float inv_scale = 1.f / scale;
     float thr[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) thr[q] = -(scale * (0.125f * (float)(1 << q)));   // exact: powers of 2
     const int n4 = (n + 3) >> 2, fk = k >> 2, nfull = n >> 2;
+    // the pivot, and the sums' unit from the entries' size (not far below the scale's)
+    const int at = (int)(((int64_t)lid * n) >> 5);
+    const float sample = row[at == k ? (k > 0 ? k - 1 : 1) : at];
+    float pivot = sample * 0.03125f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) pivot += __shfl_xor_sync(0xffffffffu, pivot, o);
+    const float unit = unit_of(fmaxf(__uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(sample)))),
+                                     scale * 0x1p-40f));
+    const float2 unit2 = make_float2(unit, unit), nunit2 = make_float2(-unit, -unit);
+    const float2 pu = make_float2(pivot * unit, pivot * unit), npu = make_float2(-pu.x, -pu.y);
     float2 s1 = make_float2(0.f, 0.f), c1 = s1, s2 = s1, c2 = s1;
     // float32 counts (exact: a lane has at most n / 32 + 4 entries), since their
     // additions then go to the FMA pipe and not to the half-rate ALU pipe
@@ -158,17 +187,19 @@ __device__ __forceinline__ void features_row(const float* __restrict__ S, int n,
             for (int e = 0; e < 4; ++e)
                 if (4 * f + e == k || 4 * f + e >= n) {
                     v[e] = -INFINITY;
-                    u[e] = 0.f;
+                    u[e] = pivot;
                 }
         }
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const float2 w = make_float2(u[2 * h] * unit, u[2 * h + 1] * unit);
-            const float2 p = __ffma2_rn(w, w, make_float2(0.f, 0.f));
+            float2 l;
+            const float2 w = two_diff(make_float2(u[2 * h], u[2 * h + 1]), unit2, nunit2, pu, npu, l);
+            const float2 p = __fmul2_rn(w, w);
             const float2 e = __ffma2_rn(w, w, make_float2(-p.x, -p.y));     // w^2 = p + e exactly
             two_add(s1, c1, w);
+            c1 = __fadd2_rn(c1, l);
             two_add(s2, c2, p);
-            c2 = __fadd2_rn(c2, e);
+            c2 = __fadd2_rn(c2, __ffma2_rn(__fadd2_rn(w, w), l, e));        // (w + l)^2 but for l^2
         }
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
@@ -208,7 +239,7 @@ __device__ __forceinline__ void features_row(const float* __restrict__ S, int n,
     int barj = INT_MAX;                             // an entry equal to bar must come before barj
     if (lid == 0) L.have = 0;
     __syncwarp();
-#pragma unroll 2
+#pragma unroll 1
     for (int f0 = 0; f0 < n4; f0 += 32) {
         const int f = f0 + lid;
         float v[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
@@ -259,7 +290,11 @@ __device__ __forceinline__ void features_row(const float* __restrict__ S, int n,
 #pragma unroll
     for (int q = 0; q < 4; ++q)
         if (lid == 19 + q) out[19 + q] = log1pf((float)cnt[q]);
-    if (lid == 0) sums[k] = make_float4(t1, d1, t2, d2);
+    if (lid == 0) {
+        sums[k] = make_float4(t1, d1, t2, d2);
+        out[16] = pivot;
+        out[17] = unit;
+    }
     __syncwarp();
 }
 
@@ -267,7 +302,7 @@ static __device__ __forceinline__ int row_vec(const float* S, int64_t ld) {
     return (reinterpret_cast<uintptr_t>(S) & 15) == 0 && (ld & 3) == 0;
 }
 
-__global__ void __launch_bounds__(32 * kFeatWarps) features_kernel(const float* __restrict__ S, int n, int64_t ld,
+__global__ void __launch_bounds__(32 * kFeatWarps, 6) features_kernel(const float* __restrict__ S, int n, int64_t ld,
                                                                    float scale, float* F, int32_t* nbr,
                                                                    float4* sums) {
     __shared__ FeatList lists[kFeatWarps];
@@ -278,18 +313,20 @@ __global__ void __launch_bounds__(32 * kFeatWarps) features_kernel(const float* 
 
 // Features 16-17 of row k from its sums, 23-24 from the densities of its 16
 // neighbours.  Sums out of float32's range (entries that are infinite, NaN or
-// more than about 1e18 times the scale) are taken again in float64.
+// more than about 1e18 times most others) are taken again in float64.
 __device__ __forceinline__ void features_finish_row(const float* __restrict__ S, int64_t ld, int k, int n, float scale,
                                                     const float4* __restrict__ sums, const int32_t* __restrict__ nbr,
                                                     float* F) {
     const float4 t = sums[k];
-    const double unit = (double)unit_of(scale), inv_scale = (double)(1.f / scale);
+    const double inv_scale = (double)(1.f / scale);
+    double pivot = (double)F[(int64_t)k * IN + 16];
+    const double unit = (double)F[(int64_t)k * IN + 17];
     double a = (double)t.x + (double)t.y, b = (double)t.z + (double)t.w;
     if (isfinite(a) && isfinite(b)) {
         a /= unit;
         b /= unit * unit;
     } else {
-        a = b = 0.0;
+        a = b = pivot = 0.0;
         for (int j = 0; j < n; ++j)
             if (j != k) {
                 const double v = (double)S[(int64_t)k * ld + j];
@@ -297,8 +334,8 @@ __device__ __forceinline__ void features_finish_row(const float* __restrict__ S,
                 b += v * v;
             }
     }
-    const double m = a / (double)(n - 1);
-    const double var = fmax(0.0, b / (double)(n - 1) - m * m);
+    const double dm = a / (double)(n - 1), m = pivot + dm;
+    const double var = fmax(0.0, b / (double)(n - 1) - dm * dm);
     F[(int64_t)k * IN + 16] = (float)(m * inv_scale);
     F[(int64_t)k * IN + 17] = (float)(sqrt(var) * inv_scale);
     const float d = F[(int64_t)k * IN + F_DENS];
@@ -344,7 +381,7 @@ __device__ __forceinline__ int batch_problem_of(const BatchProblem* P, int count
     return lo;
 }
 
-__global__ void __launch_bounds__(32 * kFeatWarps) features_batched_kernel(const BatchProblem* __restrict__ P, int count,
+__global__ void __launch_bounds__(32 * kFeatWarps, 6) features_batched_kernel(const BatchProblem* __restrict__ P, int count,
                                                                            float* F, int32_t* nbr, float4* sums) {
     __shared__ FeatList lists[kFeatWarps];
     const int b = batch_problem_of(P, count, blockIdx.x, [](const BatchProblem& q) { return (int64_t)q.b0; });

@@ -102,6 +102,28 @@ def test_features_selection_edges(kind, n, ld_pad):
         assert rel_inf(F[:, 16:18], np.stack([off.mean(1), off.std(1)], 1) / scale) <= 1e-6
 
 
+@pytest.mark.parametrize("mean,spread", [(1000.0, 0.001), (1000.0, 0.01), (1000.0, 1.0), (1.0, 1.0), (1e-3, 30.0),
+                                         (5e-26, 1e-26)])
+@pytest.mark.parametrize("n", [20, 257, 4000])
+def test_feature_moments_of_nearly_equal_entries(n, mean, spread):
+    """Mean and standard deviation of rows whose entries differ by much less than
+    their size, by more, or are far below the scale; in some rows one entry is
+    1e12 times the others.  Exact sums would leave the rounding of the result
+    (2^-24 of it; the scale is a power of two).  Sums of about 48 bits add at most
+    125 roundings of 2^-48 a lane, times 1 + n / 32 where the values are taken from
+    the mean of 32 entries of the row: 2^-23.9, and 2e-12 of the spread."""
+    g = np.random.default_rng(n)
+    S = (-mean + spread * g.normal(size=(n, n))).astype(np.float32)
+    S[::7, n // 3] = np.float32(-1e12 * mean)
+    F = capi.apl_features(_square(S), 512.0).cpu().numpy().astype(np.float64)
+    off = S[~np.eye(n, dtype=bool)].reshape(n, n - 1).astype(np.longdouble)
+    m = off.mean(1)
+    s = np.sqrt(((off - m[:, None]) ** 2).mean(1))
+    for got, want in ((F[:, 16], m / 512), (F[:, 17], s / 512)):
+        bound = 2.0 ** -23.9 * np.abs(want) + 2e-12 * s / 512
+        assert (np.abs(got - want) <= bound).all()
+
+
 def test_forward_matches_oracle():
     P, Pd, P16 = _params()
     F = np.random.default_rng(7).normal(size=(1000, 25)).astype(np.float32)
