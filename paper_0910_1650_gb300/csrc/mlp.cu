@@ -963,12 +963,16 @@ static int w2_splits(int64_t rows) {
     return (int)((rows + per - 1) / per);
 }
 
+// The most splits of any smaller batch: the splits fall where a split grows by a
+// chunk (38 at 1216 rows, 26 at 1217), and a workspace serves smaller batches.
+static int64_t w2_splits_cap(int64_t rows) { return std::min<int64_t>((rows + 31) / 32, 38); }
+
 static size_t carve(void* ws, int64_t rows, MlpWs* w) {
     Carver c(ws);
     w->H1 = c.take<float>((size_t)rows * HID);
     w->G2 = c.take<float>((size_t)rows * HID);
     w->part = c.take<float>((size_t)grad_slots(rows) * SLOT);
-    w->w2part = c.take<float>((size_t)w2_splits(rows) * HID * HID);
+    w->w2part = c.take<float>((size_t)w2_splits_cap(rows) * HID * HID);
     w->lpart = c.take<double>(grad_slots(rows));
     return c.used;
 }

@@ -33,3 +33,9 @@ def test_point_set_queries_never_shrink(lib, d):
         _never_shrinks(lambda n: lib.lap_refine_workspace_size(n, d, 2), sizes)
         _never_shrinks(lambda n: lib.lap_run_full_workspace_size(n, d, 2, 2, 2), sizes)
         _never_shrinks(lambda n: lib.ap_similarity_workspace_size(n, d), sizes)
+
+
+def test_training_query_never_shrinks(lib):
+    """A training loop's last batch is the smallest.  The partial sums of W2's
+    gradient are fewer at many larger batches (38 at 1216 rows, 26 at 1217)."""
+    _never_shrinks(lib.apl_workspace_size, range(1, 25001))
