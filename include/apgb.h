@@ -134,6 +134,10 @@ typedef struct ap_result {
  *           2^-53.  noise_rel = 0 skips the pass.
  *  pref_out host float* (may be NULL): receives the scalar preference used
  *           (NaN for AP_PREF_VECTOR).  The call synchronises ``stream``.
+ *  ws       ap_similarity_workspace_size(n, d) bytes.  Most of it serves the
+ *           median (n^2 / 4 bytes): with a given preference (AP_PREF_SCALAR,
+ *           AP_PREF_VECTOR) ap_preference_median_workspace_size(n) bytes less
+ *           are enough.
  *  Errors: AP_ERR_TIMEOUT if a bounded wait of the tensor-core kernel gave up.
  * ------------------------------------------------------------------------- */
 size_t    ap_similarity_workspace_size(int64_t n, int64_t d);
@@ -162,6 +166,8 @@ int32_t   ap_similarity(const float* X, int64_t n, int64_t d, int64_t ldx,
  *  4 library-owned streams that fork from and join back to ``stream`` by
  *  events.  The workspace holds
  *  every problem's scratch (its centred copy included, sized for float32).
+ *  With AP_PREF_SCALAR the sum of ap_preference_median_workspace_size(n[b])
+ *  over the problems is not needed of ws_bytes.
  *  The stream is synchronised once, at the end.  Results equal ap_similarity
  *  on each problem bit for bit.
  *  Errors: AP_ERR_INVALID_ARG for a bad size or offset; AP_ERR_TIMEOUT as for

@@ -295,7 +295,10 @@ def ap_similarity(X, S=None, precision="fp32", pref="median", noise_rel=0.0, see
     else:
         keep = (C.c_float * 1)(float(pref))
         mode, pptr = AP_PREF_SCALAR, C.cast(keep, C.c_void_p)
-    ws = workspace(lib().ap_similarity_workspace_size(n, d), X.device)
+    need = lib().ap_similarity_workspace_size(n, d)
+    if mode != AP_PREF_MEDIAN:          # the median's selection is most of it
+        need -= lib().ap_preference_median_workspace_size(n)
+    ws = workspace(need, X.device)
     out = C.c_float(0.0)
     st = lib().ap_similarity(C.c_void_p(X.data_ptr()), n, d, X.stride(0),
                              C.c_void_p(S.data_ptr()), S.stride(0), prec, mode, pptr,

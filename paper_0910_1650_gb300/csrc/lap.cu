@@ -24,8 +24,8 @@ int32_t exemplars_impl(const float* S, const float* R, const float* A, int64_t n
 size_t exemplars_ws_bytes(int64_t n);
 int32_t tc_assign_argmax(const __nv_bfloat16* A, int na, const __nv_bfloat16* B, int nb,
                          const float* bnrm, int dpad, int32_t* arg, float* best, void* scratch,
-                         int32_t* err, cudaStream_t s);
-size_t tc_assign_scratch_bytes(int64_t na);
+                         size_t scratch_bytes, int32_t* err, cudaStream_t s);
+size_t tc_assign_scratch_bytes(int64_t na, int64_t nb, int dpad);
 int32_t tc_assign_top2(const __nv_bfloat16* A, int na, const __nv_bfloat16* B, int nb,
                        const float* bnrm, int dpad, int32_t* arg, float* best, int32_t* arg2,
                        float* best2, int32_t* err, cudaStream_t s);
@@ -588,6 +588,7 @@ struct LapWs {
     float* enrm;
     int32_t* arg;
     void* scratch;          // tc_assign_argmax
+    size_t scratch_bytes;
     double* dp;
     double* sums;
     int32_t* err;
@@ -595,7 +596,8 @@ struct LapWs {
 
 static int64_t ld32(int64_t n) { return (n + 31) / 32 * 32; }
 
-static size_t carve_lap(void* ws, int64_t n, int64_t d, int64_t L, LapWs* w) {
+// centres: the most that the points are assigned to in this workspace.
+static size_t carve_lap(void* ws, int64_t n, int64_t d, int64_t L, int64_t centres, LapWs* w) {
     const int dpad = (int)((d + 63) / 64 * 64);
     const int64_t ldL = ld32(L);
     const size_t sub = std::max({ap_similarity_workspace_size(L, d), ap_iterate_workspace_size(L, ldL),
@@ -622,7 +624,8 @@ static size_t carve_lap(void* ws, int64_t n, int64_t d, int64_t L, LapWs* w) {
     w->Eb = c.take<__nv_bfloat16>((size_t)cpad * dpad);
     w->enrm = c.take<float>(cpad);
     w->arg = c.take<int32_t>(n);
-    w->scratch = c.take<char>(tc_assign_scratch_bytes(n));
+    w->scratch_bytes = tc_assign_scratch_bytes(n, centres, dpad);
+    w->scratch = c.take<char>(w->scratch_bytes);
     w->dp = c.take<double>(n);
     w->sums = c.take<double>(2);
     w->err = c.take<int32_t>(1);
@@ -653,7 +656,7 @@ APGB_API size_t lap_run_workspace_size(int64_t n, int64_t d, int64_t n_landmarks
     if (n < 2 || d < 1 || n_landmarks < 2 || n_landmarks > n || n > INT_MAX / 2 || d > 65536)
         return 0;
     LapWs w;
-    return carve_lap(nullptr, n, d, n_landmarks, &w);
+    return carve_lap(nullptr, n, d, n_landmarks, n_landmarks, &w);
 }
 
 APGB_API int32_t lap_run(const float* X, int64_t n, int64_t d, int64_t ldx, int64_t L,
@@ -671,8 +674,8 @@ APGB_API int32_t lap_run(const float* X, int64_t n, int64_t d, int64_t ldx, int6
     AP_TRY(require_sm103());
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     LapWs w;
-    AP_TRY(check_ws(ws, ws_bytes, carve_lap(nullptr, n, d, L, &w)));
-    carve_lap(ws, n, d, L, &w);
+    AP_TRY(check_ws(ws, ws_bytes, carve_lap(nullptr, n, d, L, L, &w)));
+    carve_lap(ws, n, d, L, L, &w);
     const int di = (int)d;
     const int dpad = (di + 63) / 64 * 64;
     const int64_t ldL = ld32(L);
@@ -746,7 +749,7 @@ APGB_API int32_t lap_run(const float* X, int64_t n, int64_t d, int64_t ldx, int6
     AP_CUDA_TRY(cudaMemsetAsync(w.err, 0, sizeof(int32_t), s));
     note_launches(3);
     AP_TRY(last_error());
-    AP_TRY(tc_assign_argmax(w.Xb, (int)n, w.Eb, c, w.enrm, dpad, w.arg, nullptr, w.scratch, w.err, s));
+    AP_TRY(tc_assign_argmax(w.Xb, (int)n, w.Eb, c, w.enrm, dpad, w.arg, nullptr, w.scratch, w.scratch_bytes, w.err, s));
     const int lgrid = (int)std::min<int64_t>((n + 255) / 256, 4096);
     labels_kernel<<<lgrid, 256, 0, s>>>(w.arg, n, w.epts, idx);
     exemplars_keep_self_kernel<<<(c + 255) / 256, 256, 0, s>>>(w.epts, c, idx);
@@ -787,6 +790,7 @@ struct AssignWs {
     float* enrm;
     int32_t* arg;
     void* scratch;          // tc_assign_argmax
+    size_t scratch_bytes;
     int32_t* err;
 };
 
@@ -801,7 +805,8 @@ static size_t carve_assign(void* ws, int64_t n, int64_t d, int64_t c, AssignWs* 
     w->Eb = cv.take<__nv_bfloat16>((size_t)cpad * dpad);
     w->enrm = cv.take<float>(cpad);
     w->arg = cv.take<int32_t>(n);
-    w->scratch = cv.take<char>(tc_assign_scratch_bytes(n));
+    w->scratch_bytes = tc_assign_scratch_bytes(n, c, dpad);
+    w->scratch = cv.take<char>(w->scratch_bytes);
     w->err = cv.take<int32_t>(1);
     return cv.used;
 }
@@ -834,7 +839,7 @@ APGB_API int32_t lap_assign(const float* X, int64_t n, int64_t d, int64_t ldx, c
     AP_CUDA_TRY(cudaMemsetAsync(w.err, 0, sizeof(int32_t), s));
     note_launches(2);
     AP_TRY(last_error());
-    AP_TRY(tc_assign_argmax(w.Xb, (int)n, w.Eb, (int)c, w.enrm, dpad, w.arg, best, w.scratch, w.err, s));
+    AP_TRY(tc_assign_argmax(w.Xb, (int)n, w.Eb, (int)c, w.enrm, dpad, w.arg, best, w.scratch, w.scratch_bytes, w.err, s));
     const int lgrid = (int)std::min<int64_t>((n + 255) / 256, 4096);
     labels_kernel<<<lgrid, 256, 0, s>>>(w.arg, n, centres, idx);
     exemplars_keep_self_kernel<<<(int)((c + 255) / 256), 256, 0, s>>>(centres, (int)c, idx);
@@ -879,13 +884,14 @@ static size_t carve_lap_full(void* ws, int64_t n, int64_t d, int64_t L, int64_t 
     const int64_t emax = std::min<int64_t>(n, L * max_levels + m0);
     const int64_t epad = (emax + 255) / 256 * 256;
     const int64_t ldm = ld32(m0);
-    const size_t sub = std::max({ap_similarity_workspace_size(m0, d), ap_iterate_workspace_size(m0, ldm),
-                                 exemplars_ws_bytes(m0)});
+    // (the similarities of the points left have a given preference)
+    const size_t sub = std::max({ap_similarity_workspace_size(m0, d) - ap_preference_median_workspace_size(m0),
+                                 ap_iterate_workspace_size(m0, ldm), exemplars_ws_bytes(m0)});
     LapWs tmp;
-    const size_t lap_bytes = carve_lap(nullptr, n, d, L, &tmp);
+    const size_t lap_bytes = carve_lap(nullptr, n, d, L, emax, &tmp);
     Carver c(ws);
     char* lap_base = c.take<char>(lap_bytes);
-    if (ws) carve_lap(lap_base, n, d, L, &w->lap);
+    if (ws) carve_lap(lap_base, n, d, L, emax, &w->lap);
     for (int b = 0; b < 2; ++b) w->Xn[b] = c.take<float>((size_t)n * d);
     for (int b = 0; b < 2; ++b) w->ids[b] = c.take<int32_t>(n);
     w->is_lm = c.take<int32_t>(n);
@@ -1177,7 +1183,7 @@ APGB_API int32_t lap_run_full(const float* X, int64_t n, int64_t d, int64_t ldx,
         note_launches(5);
         AP_TRY(last_error());
         AP_TRY(tc_assign_argmax(w.lap.Xb, (int)nl, w.lap.Eb, c, w.lap.enrm, dpad, w.lap.arg, w.best,
-                                w.lap.scratch, w.lap.err, s));
+                                w.lap.scratch, w.lap.scratch_bytes, w.lap.err, s));
         AP_CUDA_TRY(cudaMemsetAsync(w.is_lm, 0, sizeof(int32_t) * nl, s));
         flag_rows_kernel<<<grid_for(Ll), 256, 0, s>>>(w.lap.lm, Ll, w.is_lm);
         gate_kernel<<<grid_for(nl), 256, 0, s>>>(nl, w.lap.arg, w.best, w.xnrm, w.maxd, w.is_lm, ids,
@@ -1234,7 +1240,7 @@ APGB_API int32_t lap_run_full(const float* X, int64_t n, int64_t d, int64_t ldx,
     note_launches(1);
     AP_TRY(last_error());
     AP_TRY(tc_assign_argmax(w.lap.Xb, (int)n, w.Eb, (int)nE, w.enrm, dpad, w.lap.arg, nullptr,
-                            w.lap.scratch, w.lap.err, s));
+                            w.lap.scratch, w.lap.scratch_bytes, w.lap.err, s));
     labels_kernel<<<grid_for(n), 256, 0, s>>>(w.lap.arg, n, w.E, idx);
     exemplars_keep_self_kernel<<<(int)((nE + 255) / 256), 256, 0, s>>>(w.E, (int)nE, idx);
     lap_dpsim_kernel<<<(int)std::min<int64_t>((n + 7) / 8, 65535), 256, 0, s>>>(X, ldx, di, n, idx,
@@ -1272,6 +1278,7 @@ struct RefineWs {
     unsigned long long *delta, *sums, *mind;
     unsigned* absmax;
     void* scratch;          // tc_assign_argmax
+    size_t scratch_bytes;
     int32_t* err;
 };
 
@@ -1297,7 +1304,8 @@ static size_t carve_refine(void* ws, int64_t n, int64_t d, int64_t c, RefineWs* 
     w->mind = cv.take<unsigned long long>(c);
     w->sums = cv.take<unsigned long long>((size_t)c * d);
     w->absmax = cv.take<unsigned>(1);
-    w->scratch = cv.take<char>(tc_assign_scratch_bytes(n));
+    w->scratch_bytes = tc_assign_scratch_bytes(n, c, dpad);
+    w->scratch = cv.take<char>(w->scratch_bytes);
     w->err = cv.take<int32_t>(1);
     return cv.used;
 }
@@ -1350,7 +1358,7 @@ APGB_API int32_t lap_refine(const float* X, int64_t n, int64_t d, int64_t ldx, c
         X, ldx, di, w.E, nE, epad, dpad, w.mean, w.Eb, w.enrm);
     note_launches(1);
     AP_TRY(last_error());
-    AP_TRY(tc_assign_argmax(w.Xb, (int)n, w.Eb, (int)nE, w.enrm, dpad, w.j1, nullptr, w.scratch, w.err, s));
+    AP_TRY(tc_assign_argmax(w.Xb, (int)n, w.Eb, (int)nE, w.enrm, dpad, w.j1, nullptr, w.scratch, w.scratch_bytes, w.err, s));
     labels_kernel<<<grid_for(n), 256, 0, s>>>(w.j1, n, w.E, idx);
     exemplars_keep_self_kernel<<<(int)((nE + 255) / 256), 256, 0, s>>>(w.E, (int)nE, idx);
     lap_dpsim_kernel<<<(int)std::min<int64_t>((n + 7) / 8, 65535), 256, 0, s>>>(X, ldx, di, n, idx, w.dp);

@@ -1056,18 +1056,36 @@ int32_t column_means(const float* X, int64_t n, int d, int64_t ldx, double* part
     return last_error();
 }
 
-static size_t carve_sim(void* ws, int64_t n, int64_t d, SimWs* w) {
+// The median's selection: state and result, histograms, buffer (n^2 / 16 words).
+struct MedianWs {
+    SelectState* sel;
+    float* pref;
+    unsigned long long* hist;
+    uint32_t* cand;
+};
+static void take_median(Carver& c, int64_t n, MedianWs* w) {
+    char* head = c.take<char>(sizeof(SelectState) + sizeof(float));
+    w->sel = reinterpret_cast<SelectState*>(head);
+    w->pref = reinterpret_cast<float*>(head + (head ? sizeof(SelectState) : 0));
+    w->hist = c.take<unsigned long long>(4096);
+    w->cand = c.take<uint32_t>(cand_cap((int)n));
+}
+
+// median: with what only the median preference needs.
+static size_t carve_sim(void* ws, int64_t n, int64_t d, bool median, SimWs* w) {
     Carver c(ws);
     const int npad = pad_rows((int)n), dpad = pad_dim((int)d);
     w->part = c.take<double>(column_mean_part_doubles(n, (int)d));
     w->mean = c.take<float>(d);
     w->xc = c.take<float>((size_t)npad * dpad);   // large enough for either precision
     w->nrm = c.take<float>(npad);
-    w->sel = c.take<SelectState>(1);
-    w->hist = c.take<unsigned long long>(4096);
-    w->cand = c.take<uint32_t>(cand_cap((int)n));
     w->pref = c.take<float>(2);
     w->err = reinterpret_cast<int32_t*>(w->pref + 1);       // one copy brings both
+    MedianWs m{};
+    if (median) take_median(c, n, &m);
+    w->sel = m.sel;
+    w->hist = m.hist;
+    w->cand = m.cand;
     return c.used;
 }
 
@@ -1219,7 +1237,7 @@ using namespace apgb;
 APGB_API size_t ap_similarity_workspace_size(int64_t n, int64_t d) {
     if (n < 2 || d < 1 || n > INT_MAX / 2 || d > 65536) return 0;
     SimWs w;
-    return carve_sim(nullptr, n, d, &w);
+    return carve_sim(nullptr, n, d, true, &w);
 }
 
 namespace apgb {
@@ -1291,8 +1309,9 @@ APGB_API int32_t ap_similarity(const float* X, int64_t n, int64_t d, int64_t ldx
     AP_TRY(require_sm103());
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     SimWs w;
-    AP_TRY(check_ws(ws, ws_bytes, carve_sim(nullptr, n, d, &w)));
-    carve_sim(ws, n, d, &w);
+    const bool median = pref_mode == AP_PREF_MEDIAN;
+    AP_TRY(check_ws(ws, ws_bytes, carve_sim(nullptr, n, d, median, &w)));
+    carve_sim(ws, n, d, median, &w);
     AP_CUDA_TRY(cudaMemsetAsync(w.err, 0, sizeof(int32_t), s));
     AP_TRY(similarity_enqueue(X, (int)n, (int)d, ldx, S, lds, precision, pref_mode, pref, noise_rel,
                               seed, w, w.pref, w.err, s));
@@ -1335,7 +1354,7 @@ static int32_t sim_streams(std::array<cudaStream_t, kSimStreams>* out) {
 // partials, mean, centred copy, norms, select state and histograms, its
 // preference and its Gram product's error flag.  host[b] receives problem b's
 // pointers and block counts (problem fields filled by the caller).
-static size_t carve_batched(void* ws, const int64_t* n, int32_t count, int64_t d, int32_t precision,
+static size_t carve_batched(void* ws, const int64_t* n, int32_t count, int64_t d, int32_t precision, bool median,
                             SimProblem** table, std::vector<SimProblem>* host, int32_t** err,
                             float** prefs, void** tables) {
     Carver c(ws);
@@ -1378,10 +1397,12 @@ static size_t carve_batched(void* ws, const int64_t* n, int32_t count, int64_t d
         q.xc = xc_arena ? xc_arena + (size_t)roff * dpad * esz : nullptr;
         q.nrm = nrm_arena ? nrm_arena + roff : nullptr;
         roff += q.npad;
-        q.sel.st = c.take<SelectState>(1);
-        q.sel.hist = c.take<unsigned long long>(4096);
+        MedianWs m{};
+        if (median) take_median(c, n[b], &m);
+        q.sel.st = m.sel;
+        q.sel.hist = m.hist;
         q.sel.cap = cand_cap(q.n);
-        q.sel.cand = c.take<uint32_t>(q.sel.cap);
+        q.sel.cand = m.cand;
         q.sel.pref = pv ? pv + b : nullptr;
         if (host) (*host)[b] = q;
     }
@@ -1407,8 +1428,7 @@ static bool batched_args_ok(const int64_t* n, int32_t count, int64_t d) {
 APGB_API size_t ap_similarity_batched_workspace_size(const int64_t* n, int32_t count, int64_t d) {
     if (!batched_args_ok(n, count, d)) return 0;
     // the bf16 centred copy is the smaller; size for float32 so one query serves both
-    return carve_batched(nullptr, n, count, d, AP_PREC_FP32, nullptr, nullptr, nullptr, nullptr,
-                         nullptr);
+    return carve_batched(nullptr, n, count, d, AP_PREC_FP32, true, nullptr, nullptr, nullptr, nullptr, nullptr);
 }
 
 APGB_API int32_t ap_similarity_batched(const float* X, const int64_t* xoff, const int64_t* n,
@@ -1431,13 +1451,15 @@ APGB_API int32_t ap_similarity_batched(const float* X, const int64_t* xoff, cons
     if (precision != AP_PREC_FP32 && !vec) return AP_ERR_INVALID_ARG;
     AP_TRY(require_sm103());
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    AP_TRY(check_ws(ws, ws_bytes, ap_similarity_batched_workspace_size(n, count, d)));
+    const bool median = pref_mode == AP_PREF_MEDIAN;
+    AP_TRY(check_ws(ws, ws_bytes, carve_batched(nullptr, n, count, d, AP_PREC_FP32, median, nullptr, nullptr, nullptr,
+                                                nullptr, nullptr)));
     std::vector<SimProblem> host(count);
     SimProblem* table = nullptr;
     int32_t* err = nullptr;
     float* prefs = nullptr;
     void* tables = nullptr;
-    carve_batched(ws, n, count, d, precision, &table, &host, &err, &prefs, &tables);
+    carve_batched(ws, n, count, d, precision, median, &table, &host, &err, &prefs, &tables);
     int part_blocks = 0, centre_blocks = 0, pass_total = 0, digit_total = 0;
     for (int32_t b = 0; b < count; ++b) {
         host[b].X = X + xoff[b];
@@ -1553,10 +1575,8 @@ APGB_API int32_t ap_similarity_batched(const float* X, const int64_t* xoff, cons
 APGB_API size_t ap_preference_median_workspace_size(int64_t n) {
     if (n < 2 || n > INT_MAX / 2) return 0;
     Carver c(nullptr);
-    c.take<SelectState>(1);
-    c.take<unsigned long long>(4096);
-    c.take<uint32_t>(cand_cap((int)n));
-    c.take<float>(1);
+    MedianWs w;
+    take_median(c, n, &w);
     return c.used;
 }
 
@@ -1567,13 +1587,11 @@ APGB_API int32_t ap_preference_median(const float* S, int64_t n, int64_t ld, flo
     AP_TRY(check_ws(ws, ws_bytes, ap_preference_median_workspace_size(n)));
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     Carver c(ws);
-    SelectState* sel = c.take<SelectState>(1);
-    unsigned long long* hist = c.take<unsigned long long>(4096);
-    uint32_t* cand = c.take<uint32_t>(cand_cap((int)n));
-    float* pref = c.take<float>(1);
-    AP_TRY(median_offdiag(S, (int)n, ld, sel, hist, cand, nullptr, pref, 0.f, s));
+    MedianWs w;
+    take_median(c, n, &w);
+    AP_TRY(median_offdiag(S, (int)n, ld, w.sel, w.hist, w.cand, nullptr, w.pref, 0.f, s));
     float v = NAN;
-    AP_CUDA_TRY(cudaMemcpyAsync(&v, pref, sizeof(float), cudaMemcpyDeviceToHost, s));
+    AP_CUDA_TRY(cudaMemcpyAsync(&v, w.pref, sizeof(float), cudaMemcpyDeviceToHost, s));
     AP_CUDA_TRY(cudaStreamSynchronize(s));
     *median = v;
     return AP_OK;

@@ -1507,8 +1507,21 @@ static int32_t assign_launch(const __nv_bfloat16* A, int na, const __nv_bfloat16
     return launch(ma, mb, ma, p, (na + BM - 1) / BM, s);                  // row blocks
 }
 
-// Scratch of tc_assign_argmax: the groups' results, at most 4 groups of 8 bytes a point.
-size_t tc_assign_scratch_bytes(int64_t na) { return (size_t)na * 4 * (sizeof(int32_t) + sizeof(float)); }
+// Groups of CTAs that the resident kernel deals numN column tiles of centres to, and
+// how many tiles each holds at most (128 KB of centres, 3 K blocks of norms).
+static int resident_groups(int numN, int numK) {
+    const int ntmax = std::min(3, 4 / numK);
+    return (numN + ntmax - 1) / ntmax;
+}
+
+// Scratch of tc_assign_argmax on na points and at most nb centres: the groups'
+// results where the resident kernel has more than one, 8 bytes a point each.
+size_t tc_assign_scratch_bytes(int64_t na, int64_t nb, int dpad) {
+    using namespace tc;
+    if (dpad / BK > 4) return 0;
+    const int groups = resident_groups((int)std::min<int64_t>((nb + BN - 1) / BN, 4), dpad / BK);
+    return groups > 1 ? (size_t)na * groups * (sizeof(int32_t) + sizeof(float)) : 0;
+}
 
 // The resident kernel takes up to 1024 centres (whose norms the kernel above
 // folds too, so a score has the same bits in both) of up to 256 features: a
@@ -1516,14 +1529,14 @@ size_t tc_assign_scratch_bytes(int64_t na) { return (size_t)na * 4 * (sizeof(int
 // stages.  Wider features or more centres stream both operands.
 int32_t tc_assign_argmax(const __nv_bfloat16* A, int na, const __nv_bfloat16* B, int nb,
                          const float* bnrm, int dpad, int32_t* arg, float* best, void* scratch,
-                         int32_t* err, cudaStream_t s) {
+                         size_t scratch_bytes, int32_t* err, cudaStream_t s) {
     using namespace tc;
     if (dpad % BK || nb < 1 || na < 1) return AP_ERR_INVALID_ARG;
     const int numK = dpad / BK, numN = (nb + BN - 1) / BN, numM = (na + BM - 1) / BM;
-    if (numN > 4 || numK > 4 || assign_norm_form() > 1 || !scratch)
+    if (numN > 4 || numK > 4 || assign_norm_form() > 1)
         return assign_launch(A, na, B, nb, bnrm, dpad, arg, best, nullptr, nullptr, err, s);
-    const int ntmax = std::min(3, 4 / numK);            // tiles that fit: 128 KB of centres, 3 K blocks of norms
-    const int groups = (numN + ntmax - 1) / ntmax, nt = (numN + groups - 1) / groups;
+    const int groups = resident_groups(numN, numK), nt = (numN + groups - 1) / groups;
+    if (tc_assign_scratch_bytes(na, nb, dpad) > scratch_bytes) return AP_ERR_WORKSPACE;
     int sms = 0;
     AP_TRY(device_sm_count(&sms));
     const size_t bytes = resident_smem(nt, numK);

@@ -6,6 +6,8 @@ values widened back to float64, so the only difference is the arithmetic of
 the updates.  R/A error is the infinity-norm relative error
 max|X_gpu - X_ref| / max|X_ref|, bounded by 1e-4.  Decisions that floating
 point takes (the a+r arg-max) are taken in float32 by both sides."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -492,6 +494,36 @@ def test_iterations_outside_a_graph_take_no_longer_than_in_one(n, kw):
             torch.cuda.synchronize()
             best[name] = min(best.get(name, 1e9), a.elapsed_time(b))
     assert best["plain"] <= 1.2 * best["graph"], best
+
+
+@pytest.mark.parametrize("n,d", [(2, 3), (700, 64), (3000, 65)])
+@pytest.mark.parametrize("precision", [capi.AP_PREC_FP32, capi.AP_PREC_BF16])
+def test_given_preference_needs_no_selection_workspace(n, d, precision):
+    """A build with a given preference takes a workspace without the median's
+    part, stays inside it (a guard behind it is untouched) and gives the
+    entries the median build gives; the median build is refused there."""
+    L = capi.lib()
+    X = torch.from_numpy(np.random.default_rng(n).normal(size=(n, d)).astype(np.float32)).cuda()
+    full = L.ap_similarity_workspace_size(n, d)
+    need = full - L.ap_preference_median_workspace_size(n)
+    ld = capi.padded_ld(n)
+    guard = 1 << 16
+    ws = torch.full((need + guard,), 0x5A, dtype=torch.uint8, device="cuda")
+    p = ctypes.c_float(-3.5)
+    P = ctypes.c_void_p
+
+    def build(S, mode, nbytes):
+        return L.ap_similarity(P(X.data_ptr()), n, d, d, P(S.data_ptr()), ld, precision, mode,
+                               ctypes.cast(ctypes.pointer(p), P), 0.0, 0, None, P(ws.data_ptr()), nbytes,
+                               P(torch.cuda.current_stream().cuda_stream))
+
+    S = torch.zeros((n, ld), device="cuda")
+    assert build(S, capi.AP_PREF_SCALAR, need) == 0
+    assert bool((ws[need:] == 0x5A).all())
+    assert build(S, capi.AP_PREF_SCALAR, need - 256) == -3 and build(S, capi.AP_PREF_MEDIAN, need) == -3
+    M, _ = capi.ap_similarity(X, precision="fp32" if precision == capi.AP_PREC_FP32 else "bf16")
+    off = ~torch.eye(n, dtype=torch.bool, device="cuda")
+    assert torch.equal(S[:, :n][off], M[off]) and bool((torch.diagonal(S[:, :n]) == -3.5).all())
 
 
 def test_preference_median_exact():

@@ -39,3 +39,14 @@ def test_training_query_never_shrinks(lib):
     """A training loop's last batch is the smallest.  The partial sums of W2's
     gradient are fewer at many larger batches (38 at 1216 rows, 26 at 1217)."""
     _never_shrinks(lib.apl_workspace_size, range(1, 25001))
+
+
+@pytest.mark.parametrize("d,c,row", [(300, 10, 644), (300, 1000, 644), (64, 768, 132), (128, 512, 260),
+                                     (128, 513, 276), (64, 769, 148), (256, 1024, 548)])
+def test_assignment_query_counts_the_groups_there_are(lib, d, c, row):
+    """Per point: the bf16 features (d rounded up to 64), the choice, and 8 bytes
+    for each group of CTAs the centres are dealt to where there is more than
+    one (768 centres per group at d <= 64, 512 at 128, 256 at 256; none past it)."""
+    n = 1000000
+    grow = lib.lap_assign_workspace_size(2 * n, d, c) - lib.lap_assign_workspace_size(n, d, c)
+    assert abs(grow / n - row) < 0.1
