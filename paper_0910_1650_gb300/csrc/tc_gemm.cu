@@ -951,7 +951,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 // (96 KB a tile).  Here a CTA keeps its share of the centres (and their folded
 // norms) in shared memory for the whole launch and streams only row blocks of
 // points, 16 KB per 64 features.  The centres' column tiles are dealt to G
-// groups of CTAs, as few as hold them (nt tiles of 256 each); each group goes
+// groups of CTAs, one or two (nt tiles of 256 each; resident_groups); each goes
 // over every row block, and merge_groups_kernel keeps the better of the
 // groups' bests (the lower column on a tie).  The MMAs of a tile are those of
 // the kernel above in the same order, so scores and choices are the same bits.
@@ -1507,35 +1507,44 @@ static int32_t assign_launch(const __nv_bfloat16* A, int na, const __nv_bfloat16
     return launch(ma, mb, ma, p, (na + BM - 1) / BM, s);                  // row blocks
 }
 
-// Groups of CTAs that the resident kernel deals numN column tiles of centres to, and
-// how many tiles each holds at most (128 KB of centres, 3 K blocks of norms).
-static int resident_groups(int numN, int numK) {
+// Groups of CTAs that the resident kernel deals numN column tiles of centres to
+// (a CTA holds at most 128 KB of centres and 3 K blocks of norms); 0: both operands
+// are streamed by the kernel above.
+//
+// The resident kernel takes up to 1024 centres (whose norms the kernel above folds
+// too, so a score has the same bits in both) of up to 256 features, in one group
+// at any size: resident against streaming, 10000 points, 50 centres, d = 64 7.4 us
+// against 12.8; 20000, 700, d = 64 12.1 against 18.0.  A second group reads the points
+// again and needs the merge's launch, so it has to have as many tiles as the first
+// and enough points (1000 centres, d = 128, merge included: 10000 points 14.9 against
+// 15.4 us, calls 3.5 us slower; 80000 30.3 against 34.7, calls the same; 120000 38.7
+// against 44.6, calls 1.02 times as fast; 600 centres, 2 tiles and 1, 200000 points:
+// 56.9 against 55.8).  Three and four groups lose everywhere (d = 250, 1000 centres:
+// 600000 points 247 against 231 us).
+static int resident_groups(int64_t na, int numN, int numK) {
+    if (numN > 4 || numK > 4) return 0;
     const int ntmax = std::min(3, 4 / numK);
-    return (numN + ntmax - 1) / ntmax;
+    if (numN <= ntmax) return 1;
+    return numN == 4 && numK <= 2 && na >= 100000 ? 2 : 0;
 }
 
-// Scratch of tc_assign_argmax on na points and at most nb centres: the groups'
-// results where the resident kernel has more than one, 8 bytes a point each.
+// Scratch of tc_assign_argmax on up to na points and nb centres: the groups' results
+// where the resident kernel has two, 8 bytes a point each.
 size_t tc_assign_scratch_bytes(int64_t na, int64_t nb, int dpad) {
     using namespace tc;
-    if (dpad / BK > 4) return 0;
-    const int groups = resident_groups((int)std::min<int64_t>((nb + BN - 1) / BN, 4), dpad / BK);
+    const int groups = resident_groups(na, (int)std::min<int64_t>((nb + BN - 1) / BN, 4), dpad / BK);
     return groups > 1 ? (size_t)na * groups * (sizeof(int32_t) + sizeof(float)) : 0;
 }
 
-// The resident kernel takes up to 1024 centres (whose norms the kernel above
-// folds too, so a score has the same bits in both) of up to 256 features: a
-// group then holds at least one column tile of 256 centres next to four 16 KB
-// stages.  Wider features or more centres stream both operands.
 int32_t tc_assign_argmax(const __nv_bfloat16* A, int na, const __nv_bfloat16* B, int nb,
                          const float* bnrm, int dpad, int32_t* arg, float* best, void* scratch,
                          size_t scratch_bytes, int32_t* err, cudaStream_t s) {
     using namespace tc;
     if (dpad % BK || nb < 1 || na < 1) return AP_ERR_INVALID_ARG;
     const int numK = dpad / BK, numN = (nb + BN - 1) / BN, numM = (na + BM - 1) / BM;
-    if (numN > 4 || numK > 4 || assign_norm_form() > 1)
-        return assign_launch(A, na, B, nb, bnrm, dpad, arg, best, nullptr, nullptr, err, s);
-    const int groups = resident_groups(numN, numK), nt = (numN + groups - 1) / groups;
+    const int groups = assign_norm_form() > 1 ? 0 : resident_groups(na, numN, numK);
+    if (!groups) return assign_launch(A, na, B, nb, bnrm, dpad, arg, best, nullptr, nullptr, err, s);
+    const int nt = (numN + groups - 1) / groups;
     if (tc_assign_scratch_bytes(na, nb, dpad) > scratch_bytes) return AP_ERR_WORKSPACE;
     int sms = 0;
     AP_TRY(device_sm_count(&sms));

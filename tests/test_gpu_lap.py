@@ -440,6 +440,35 @@ def test_assign_with_resident_centres_at_its_edges(c, d):
         assert not np.any(got[~own] == n // 2)
 
 
+@pytest.mark.parametrize("n", [99999, 100000, 100129])
+@pytest.mark.parametrize("c,d", [(769, 64), (1000, 128), (1024, 65)])
+def test_assign_with_two_groups_of_resident_centres(c, d, n):
+    """Four column tiles of centres are dealt to two groups of CTAs from 100000
+    points on and streamed below: the choice is a maximum of the float64 scores of
+    the rounded centred points up to the accumulation bound, `best` its score,
+    and of two equal centres in different groups the earlier one."""
+    g = np.random.default_rng(c + n)
+    X = (g.normal(size=(n, d)) * 3).astype(np.float32)
+    cen = g.permutation(n)[:c].astype(np.int32)
+    X[cen[c - 1]] = X[cen[3]]                                # tiles 3 and 0
+    Xd = torch.from_numpy(X).cuda()
+    idx, best = capi.lap_assign(Xd, torch.from_numpy(cen), best=True)
+    B = (Xd - Xd.double().mean(0).float()).to(torch.bfloat16).double()
+    cd = torch.from_numpy(cen).cuda().long()
+    score = 2 * (B @ B[cd].T) - (B[cd] * B[cd]).sum(1)
+    top = score.max(1).values
+    tol = (d + 4) * 2.0 ** -22 * (B * B).sum(1).max()
+    assert bool(((best.double() - top).abs() <= tol).all())
+    pos = torch.full((n,), -1, dtype=torch.long, device="cuda")
+    pos[cd] = torch.arange(c, device="cuda")
+    own = pos >= 0
+    assert torch.equal(idx.long()[own], torch.arange(n, device="cuda")[own])
+    chosen = pos[idx.long()]
+    assert bool((chosen >= 0).all())
+    assert bool((score.gather(1, chosen[:, None])[:, 0] >= top - 2 * tol)[~own].all())
+    assert not bool((chosen[~own] == c - 1).any())
+
+
 def test_lap_full_level_with_more_column_blocks_than_the_whole_set():
     """The column means of 4864 points (one recursion level) take 152 row blocks,
     those of all 7000 points 149, in one scratch sized for the whole set.  The

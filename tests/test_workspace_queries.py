@@ -42,11 +42,11 @@ def test_training_query_never_shrinks(lib):
 
 
 @pytest.mark.parametrize("d,c,row", [(300, 10, 644), (300, 1000, 644), (64, 768, 132), (128, 512, 260),
-                                     (128, 513, 276), (64, 769, 148), (256, 1024, 548)])
+                                     (128, 513, 260), (64, 769, 148), (128, 1024, 276), (256, 1024, 516)])
 def test_assignment_query_counts_the_groups_there_are(lib, d, c, row):
     """Per point: the bf16 features (d rounded up to 64), the choice, and 8 bytes
-    for each group of CTAs the centres are dealt to where there is more than
-    one (768 centres per group at d <= 64, 512 at 128, 256 at 256; none past it)."""
+    for each group of CTAs the centres are dealt to where there are two (769 to
+    1024 centres of up to 128 features)."""
     n = 1000000
     grow = lib.lap_assign_workspace_size(2 * n, d, c) - lib.lap_assign_workspace_size(n, d, c)
     assert abs(grow / n - row) < 0.1
