@@ -145,3 +145,12 @@ def test_similarity_bf16_median_of_clustered_rows(kind):
     off = S[~torch.eye(n, dtype=torch.bool, device="cuda")].double().cpu().numpy()
     assert p == float(np.float32(np.median(off)))
     assert bool((torch.diagonal(S) == p).all())
+
+
+@pytest.mark.parametrize("d", [3, 64, 200])
+@pytest.mark.parametrize("n", [2049, 2305, 2431, 2561])
+def test_similarity_bf16_mirrored_tiles_of_a_triangle(n, d):
+    """Squares of more tiles than SMs (17 x 9 and more): only tiles on or above the
+    diagonal are multiplied.  Odd and even numbers of row blocks, last blocks of
+    one row and column, of a part and of all but one."""
+    test_similarity_bf16_mirrored_tiles(n, d)
