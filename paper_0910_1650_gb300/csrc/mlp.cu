@@ -144,7 +144,8 @@ __device__ __forceinline__ void rank_list(FeatList& L, int cnt, int lid) {
 }
 
 // Four consecutive entries 4f .. 4f+3 of a row (vec: 16-byte aligned rows whose
-// stride is a multiple of 4); past the row's end: NaN, which nothing selects.
+// stride is a multiple of 4).  Past the row's end: whatever the padding holds, or
+// 0, the largest similarity there is; the callers mask those out (j < n).
 __device__ __forceinline__ float4 row4(const float* __restrict__ row, int f, int n, int vec) {
     if (vec) return __ldg(reinterpret_cast<const float4*>(row) + f);
     float v[4];
@@ -454,8 +455,8 @@ __global__ void standardisation_kernel(const float* __restrict__ F, int64_t rows
 // adam_reduce_kernel adds the slots in a fixed order and takes the step.
 // A training step on 4096 rows: three launches where separate layer kernels
 // took 15 (weight gradients on at most 16 blocks, bias gradients one thread
-// per column), 80 us where they took 1752 us.  The forward pass alone on
-// 101000 rows: about 390 us where four layer launches took 870 us.
+// per column), 74 us where they took 1752 us.  The forward pass alone on
+// 104000 rows: 408 us where four layer launches took about 870 us.
 constexpr int TR = 32;                 // rows per tile
 constexpr int RS = 36;                 // their stride in shared memory (16-byte groups, fewer bank conflicts)
 constexpr int KC = 16;                 // weights staged per step: KC x 256

@@ -397,9 +397,11 @@ __device__ __forceinline__ float key_float(uint32_t k) {
 // or the buffer overflowed (a large share of equal entries), the digit passes
 // read S itself from the top bit, so the result is exact either way.  The
 // decision stays on the device.  20000 points (1.6 GB): 386 us, of which the
-// pass is 322, the digits 53 and the sample 11, where three radix passes over
-// S took 1025 us; 1000 points: 55 us where they took 144 us (16 blocks, most of
-// the time waiting on shared-memory atomics).
+// pass is 321 (0.75 of the copy rate: with 3.5 % hits nearly every step of 512
+// entries takes the tail of scan, second read and stores, behind four 16-byte
+// loads a lane), the digits 53 and the sample 11, where three radix passes over
+// S took 1025 us; 1000 points: 35 us (kSmallSelect) where they took 144 us (16
+// blocks, most of the time waiting on shared-memory atomics).
 constexpr int kSampleThreads = 1024;
 constexpr int kSamplePer = 16;          // entries per thread (small selections: 4)
 constexpr int kSample = kSampleThreads * kSamplePer;
