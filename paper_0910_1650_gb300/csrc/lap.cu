@@ -22,6 +22,7 @@ namespace apgb {
 int32_t exemplars_impl(const float* S, const float* R, const float* A, int64_t n, int64_t ld,
                        int32_t* idx, ap_result* out, void* ws, size_t ws_bytes, cudaStream_t s);
 size_t exemplars_ws_bytes(int64_t n);
+size_t iterate_bytes_upto(int64_t n, int64_t ld);
 int32_t tc_assign_argmax(const __nv_bfloat16* A, int na, const __nv_bfloat16* B, int nb,
                          const float* bnrm, int dpad, int32_t* arg, float* best, void* scratch,
                          size_t scratch_bytes, int32_t* err, cudaStream_t s);
@@ -884,9 +885,9 @@ static size_t carve_lap_full(void* ws, int64_t n, int64_t d, int64_t L, int64_t 
     const int64_t emax = std::min<int64_t>(n, L * max_levels + m0);
     const int64_t epad = (emax + 255) / 256 * 256;
     const int64_t ldm = ld32(m0);
-    // (the similarities of the points left have a given preference)
+    // (for any number of points left up to m0; their similarities have a given preference)
     const size_t sub = std::max({ap_similarity_workspace_size(m0, d) - ap_preference_median_workspace_size(m0),
-                                 ap_iterate_workspace_size(m0, ldm), exemplars_ws_bytes(m0)});
+                                 iterate_bytes_upto(m0, ldm), exemplars_ws_bytes(m0)});
     LapWs tmp;
     const size_t lap_bytes = carve_lap(nullptr, n, d, L, emax, &tmp);
     Carver c(ws);

@@ -2035,6 +2035,17 @@ APGB_API size_t ap_iterate_workspace_size(int64_t n, int64_t ld) {
     return b;
 }
 
+namespace apgb {
+// Enough for every problem of at most n points (ld: n's leading dimension).  All
+// but the column partials' pool, the work list and the cold start's zeros grows
+// with n; those follow the launch configuration, which changes at many sizes
+// (1024 points need 0.5 MB more than 1025).  R resident clusters of C CTAs hold
+// at least two stages of three 4-byte slices of a row, R C (2 x 12 n / C) bytes of
+// 152 x 228 KB, so the pool (4 R n bytes) is at most 6 MB; the list and the zeros
+// take less than 0.3 MB.
+size_t iterate_bytes_upto(int64_t n, int64_t ld) { return ap_iterate_workspace_size(n, ld) + (size_t(8) << 20); }
+}  // namespace apgb
+
 APGB_API int32_t ap_iterate(const float* S, float* R, float* A, int64_t n, int64_t ld,
                             const ap_params* p, int32_t* decisions, ap_result* out,
                             void* ws, size_t ws_bytes, void* stream) {

@@ -500,3 +500,24 @@ def test_lap_full_level_with_more_column_blocks_than_the_whole_set():
     assert clear.size > 0.9 * rest.size
     assert np.array_equal(level_of[clear] == -1, np.isin(clear, l1["unassigned"]))
     _check_assignment(X, ref["E"], idx.cpu().numpy().astype(np.int64))
+
+
+@pytest.mark.parametrize("far,m0", [(1024, 1030), (1536, 1540), (2048, 2100)])
+def test_lap_full_base_case_smaller_than_m0_fits_its_workspace(far, m0):
+    """The sweep's launch configuration changes just above 1024, 1536 and 2048
+    points, and with it the workspace, which falls: one sized for m0 points has
+    to be enough for the fewer that the gate leaves."""
+    n, L, seed = 3000, 100, 5
+    g = np.random.default_rng(far)
+    lm = olap.uniform_landmarks(n, L, seed)
+    out = g.permutation(np.setdiff1d(np.arange(n), lm))[:far]
+    X = 0.1 * g.normal(size=(n, 8))
+    X[lm] = g.normal(size=(L, 8))
+    X[out] = 200.0 + 60.0 * g.normal(size=(10, 8))[g.integers(0, 10, far)] + 0.5 * g.normal(size=(far, 8))
+    X = X.astype(np.float32)
+    idx, level_of, res = capi.lap_run_full(torch.from_numpy(X).cuda(), L, m0, seed=seed, damping=0.9,
+                                           max_iter=1000, conv_iter=15)
+    assert res["base_case"] == 1 and res["unassigned"] == [far]
+    level_of = level_of.cpu().numpy()
+    assert np.array_equal(np.nonzero(level_of == 1)[0], np.sort(out))
+    assert np.isin(idx.cpu().numpy()[out], out).all()
